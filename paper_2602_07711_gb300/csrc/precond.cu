@@ -21,7 +21,7 @@ __global__ void scale_copy_kernel(const float2* __restrict__ a, float2* __restri
 bool use_tc(const helm_ctx* c) { return c->opt.precision != HELM_PREC_FP32; }
 
 // complex64 -> 16-bit pairs (H = 1 BF16, 2 FP16 clamped to the finite range; round to nearest even), the
-// entry of the 16-bit chain: two points per float4, times s0 and the Arnoldi scale sigma[sidx] (else inv[0])
+// entry of the 16-bit chain: two points per float4, times s0 and the Arnoldi scale sigma[sidx]
 template <int H>
 __device__ __forceinline__ uint32_t cpack16(float lo, float hi) {
     if (H == 2) {
@@ -34,9 +34,8 @@ __device__ __forceinline__ uint32_t cpack16(float lo, float hi) {
 // (nb vectors back to back, vector v scaled by sigma[sidx + v sstride]: blockIdx.y = v)
 template <int H>
 __global__ void c64_to_h16_kernel(const float4* __restrict__ a, uint2* __restrict__ b, size_t n2, float s0,
-                                  const double* __restrict__ sigma, int sidx, const double* __restrict__ inv,
-                                  int sstride = 0) {
-    const float sc = s0 * (sigma ? (float)sigma[sidx + blockIdx.y * sstride] : inv ? (float)inv[0] : 1.f);
+                                  const double* __restrict__ sigma, int sidx, int sstride = 0) {
+    const float sc = s0 * (sigma ? (float)sigma[sidx + blockIdx.y * sstride] : 1.f);
     a += (size_t)blockIdx.y * n2;
     b += (size_t)blockIdx.y * n2;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -55,13 +54,46 @@ __global__ void c64_to_h16_kernel(const float4* __restrict__ a, uint2* __restric
     }
 }
 
-// ||r||_2 of a complex64 grid: per-block FP64 partial sums, then one block writes 1/||r|| (0 for r = 0) and ||r||
-constexpr int NRM_BLOCKS = 1024;
-__global__ void norm_part_kernel(const float2* __restrict__ r, size_t n, double* __restrict__ part) {
+// ||r||_2 of a complex64 grid as per-block FP64 partial sums.  GB300 runs FP64 (and its conversions) at a small
+// fraction of the FP32 rate: one FP64 product and conversion per value bound this kernel at 169 us for 256^3
+// (134 MB).  So a thread squares and sums 8 points in compensated FP32 (the rounding error of each product and
+// sum is carried in a second FP32 number, about 2^-46 relative) and joins them in FP64 once.  The 8 points
+// are scaled by the power of two of their largest magnitude first, so that every finite FP32 input squares
+// without overflow or underflow as it did in FP64; a group with an Inf or NaN takes the FP64 sum, whose result
+// it then decides.  Measured at 256^3: 29 us, 4.7 TB/s.
+constexpr int NRM_BLOCKS = 608;   // four 256-thread CTAs on each of 152 SMs (the scratch holds 1024 partials)
+__global__ void __launch_bounds__(256) norm_part_kernel(const float4* __restrict__ r, size_t n4, double* __restrict__ part) {
     double acc = 0.0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float2 v = r[i];
-        acc += (double)v.x * v.x + (double)v.y * v.y;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i0 < n4; i0 += 4 * stride) {
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const size_t i = i0 + u * stride;
+            const float4 q = i < n4 ? r[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[4 * u] = q.x; v[4 * u + 1] = q.y; v[4 * u + 2] = q.z; v[4 * u + 3] = q.w;
+        }
+        unsigned big = 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) big = max(big, __float_as_uint(v[k]) & 0x7FFFFFFFu);
+        if (big >= 0x7F800000u) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) acc += (double)v[k] * v[k];
+            continue;
+        }
+        const int e = min((int)(big >> 23), 253);              // biased exponent of the largest magnitude
+        const float sc = __uint_as_float((unsigned)(254 - e) << 23);   // 2^(127 - e): |v| sc < 4, exact
+        float hi = 0.f, lo = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const float x = v[k] * sc, p = __fmul_rn(x, x);
+            const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);
+            // rounding errors of the sum (two-sum) and of the product
+            lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z)) + fmaf(x, x, -p);
+            hi = t;
+        }
+        const double back = __longlong_as_double((long long)(1023 + 2 * (e - 127)) << 52);   // sc^-2
+        acc = fma((double)hi, back, fma((double)lo, back, acc));
     }
     __shared__ double sh[256];
     sh[threadIdx.x] = acc;
@@ -72,20 +104,41 @@ __global__ void norm_part_kernel(const float2* __restrict__ r, size_t n, double*
     }
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
-__global__ void norm_final_kernel(const double* __restrict__ part, int nparts, double* __restrict__ out) {
+
+// The FP16 chain's entry without an Arnoldi scale: r times s0 / ||r|| in FP16.  Every block sums the partial
+// norms itself, in the same order (a separate one-block launch cost 6 us); block 0 leaves 1/||r|| (0 for r = 0)
+// and ||r|| in out[0..1] for the last pass.
+__global__ void __launch_bounds__(256) normed_to_h16_kernel(const float4* __restrict__ a, uint2* __restrict__ b, size_t n2,
+                                                            float s0, const double* __restrict__ part,
+                                                            double* __restrict__ out) {
     __shared__ double sh[256];
     double acc = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[i];
+    for (int i = threadIdx.x; i < NRM_BLOCKS; i += 256) acc += part[i];
     sh[threadIdx.x] = acc;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    for (int o = 128; o > 0; o >>= 1) {
         if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        const double nr = sqrt(sh[0]);
-        out[0] = nr > 0.0 ? 1.0 / nr : 0.0;
+    const double nr = sqrt(sh[0]), inv = nr > 0.0 ? 1.0 / nr : 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        out[0] = inv;
         out[1] = nr;
+    }
+    const float sc = s0 * (float)inv;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i0 < n2; i0 += 4 * stride) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const size_t i = i0 + u * stride;
+            v[u] = i < n2 ? a[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const size_t i = i0 + u * stride;
+            if (i < n2) b[i] = make_uint2(cpack16<2>(sc * v[u].x, sc * v[u].y), cpack16<2>(sc * v[u].z, sc * v[u].w));
+        }
     }
 }
 
@@ -131,21 +184,19 @@ helm_status precond_h16(helm_ctx* c, const float2* r, float2* z, const double* s
     uint16_t* T0 = reinterpret_cast<uint16_t*>(c->tmp);
     uint16_t* T1 = T0 + 2 * n;
     const float* sc = c->h16s;
-    const double* inv = nullptr;
     const double* nrm = nullptr;
     prof_begin(c, s, PROF_XPASS);
     if (H == 2 && !sigma) {   // no Arnoldi scale: normalise by ||r|| here, restore it in the last pass
-        norm_part_kernel<<<NRM_BLOCKS, 256, 0, s>>>(r, n, c->h16n + 2);
-        norm_final_kernel<<<1, 256, 0, s>>>(c->h16n + 2, NRM_BLOCKS, c->h16n);
-        inv = c->h16n;
+        norm_part_kernel<<<NRM_BLOCKS, 256, 0, s>>>(reinterpret_cast<const float4*>(r), n / 2, c->h16n + 2);
+        normed_to_h16_kernel<<<NRM_BLOCKS, 256, 0, s>>>(reinterpret_cast<const float4*>(r), reinterpret_cast<uint2*>(T0),
+                                                        n / 2, sc[0], c->h16n + 2, c->h16n);
         nrm = c->h16n + 1;
-    }
-    if (H == 2)
+    } else if (H == 2)
         c64_to_h16_kernel<2><<<2048, 256, 0, s>>>(reinterpret_cast<const float4*>(r), reinterpret_cast<uint2*>(T0), n / 2,
-                                                  sc[0], sigma, sidx, inv);
+                                                  sc[0], sigma, sidx);
     else
         c64_to_h16_kernel<1><<<2048, 256, 0, s>>>(reinterpret_cast<const float4*>(r), reinterpret_cast<uint2*>(T0), n / 2,
-                                                  sc[0], sigma, sidx, inv);
+                                                  sc[0], sigma, sidx);
     HELM_CUDA_TRY(cudaGetLastError());
     prof_end(c, s);
     return h16_chain(c, T0, T1, z, sc[5], nrm, 0, s);
@@ -238,7 +289,7 @@ helm_status precond_h16_basis(helm_ctx* c, const uint16_t* V16, float2* z, const
 helm_status to_h16_basis(helm_ctx* c, const float2* r, uint16_t* V16, const double* sigma, int sidx, cudaStream_t s) {
     prof_begin(c, s, PROF_SMALL);
     c64_to_h16_kernel<2><<<2048, 256, 0, s>>>(reinterpret_cast<const float4*>(r), reinterpret_cast<uint2*>(V16), c->npts / 2,
-                                              c->h16s[0], sigma, sidx, nullptr);
+                                              c->h16s[0], sigma, sidx);
     prof_end(c, s);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
@@ -270,10 +321,10 @@ helm_status precond_apply_nb(helm_ctx* c, const float2* r, float2* z, int nb, co
         prof_begin(c, s, PROF_XPASS);
         if (c->opt.precision == HELM_PREC_FP16)
             c64_to_h16_kernel<2><<<dim3(512, nb), 256, 0, s>>>(reinterpret_cast<const float4*>(r), reinterpret_cast<uint2*>(T0),
-                                                              n / 2, c->h16s[0], sigma, sidx, nullptr, sstride);
+                                                              n / 2, c->h16s[0], sigma, sidx, sstride);
         else
             c64_to_h16_kernel<1><<<dim3(512, nb), 256, 0, s>>>(reinterpret_cast<const float4*>(r), reinterpret_cast<uint2*>(T0),
-                                                              n / 2, c->h16s[0], sigma, sidx, nullptr, sstride);
+                                                              n / 2, c->h16s[0], sigma, sidx, sstride);
         HELM_CUDA_TRY(cudaGetLastError());
         prof_end(c, s);
         return h16_chain(c, T0, T1, z, c->h16s[5], nullptr, 0, s, nb);
