@@ -230,10 +230,16 @@ helm_status zsolve_reserve(helm_ctx* c, int nb);
 helm_status launch_zsolve(helm_ctx* c, const float2* in, float2* out, cudaStream_t s, int nb = 1);
 helm_status zsolve_factor(helm_ctx* c, cudaStream_t s);
 helm_status zsolve_factor_with(helm_ctx* c, const float2* dxs, const float2* dys, float2** m, cudaStream_t s);
-helm_status launch_zsolve_fact(helm_ctx* c, const float2* m, const float2* in, float2* out, const float2* P,
-                               const float2* Q, cudaStream_t s, int nb = 1);
-helm_status launch_zsolve_gen(helm_ctx* c, const float2* in, float2* out, const float2* dxs, const float2* dys,
-                              const float2* P, const float2* Q, cudaStream_t s);
+helm_status launch_zsolve_fact(helm_ctx* c, const float2* m, const float2* in, float2* out, cudaStream_t s, int nb = 1);
+// A generated right-hand side, the sum of four outer products per slice (PFFT):
+//   y[l][j][i] += p0[j] q0[l][i] + p1[j] q1[l][i] + p2[j][l] q2[i] + p3[j][l] q3[i]
+// (q0, q1 [nz][nx]; p2, p3 [ny][nzp], 16-byte aligned)
+struct ZGen {
+    const float2 *p0, *p1, *p2, *p3, *q0, *q1, *q2, *q3;
+    int nzp;
+};
+// factorised solve of in (NULL = 0) plus the generated right-hand side; even N_x
+helm_status launch_zsolve_gen(helm_ctx* c, const float2* m, const float2* in, float2* out, const ZGen& g, cudaStream_t s);
 // pfft.cu
 helm_status pfft_prepare(helm_ctx* c, cudaStream_t s);
 helm_status pfft_apply(helm_ctx* c, const float2* r, float2* z, const double* sigma, int sidx, cudaStream_t s);

@@ -33,7 +33,11 @@ struct PfftState {
     float2* Yh = nullptr;                           // transformed right-hand side (kept for step 3)
     float2 *fa = nullptr, *fb = nullptr, *fc = nullptr;   // frame work vectors [4][nz][nmax]
     float2 *fb1 = nullptr, *fc1 = nullptr;          // second frame layer (zeta = 2): Theta, W
-    float2 *P = nullptr, *Q = nullptr;              // outer-product factors [4][nz][ny], [4][nz][nx]
+    // factors of the four outer products per slice: the two that vary with the slice, Pt [2][ny][nzp] (slice
+    // index fastest, nzp = nz rounded up to 8) and Q [2][nz][nx], and the EigT step's slice-independent ones:
+    // columns 0 and N-1 of Vyi and of Vxi, back to back
+    float2 *Pt = nullptr, *Q = nullptr, *ecol = nullptr;
+    int nzp = 0;
     float2* zfacF = nullptr;                        // Thomas factors of the z-systems of A_p^F
 };
 
@@ -179,125 +183,196 @@ __global__ void __launch_bounds__(256) dst_y_kernel(const float2* __restrict__ i
 }
 
 // ---- frame extraction ------------------------------------------------------------------------------
-// TT[l][i] = sum_j wr0[j] C[l][j][i],  TB[l][i] = sum_j wr1[j] C[l][j][i]   (weights over rows)
-__global__ void frame_cols_kernel(const float2* __restrict__ C, int nx, int ny, const float2* __restrict__ wr0,
-                                  const float2* __restrict__ wr1, float2* __restrict__ TT, float2* __restrict__ TB,
-                                  int ld) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, l = blockIdx.y;
-    if (i >= nx) return;
+// The frame sums of every slice l of C in one read of it:
+//   TT[l][i] = sum_j wr0[j] C[l][j][i],  TB with wr1 (weights over rows)
+//   UL[l][j] = sum_i C[l][j][i] wc0[i],  UR with wc1 (weights over columns)
+// HBM-bound: a CTA takes a slice and streams it through a three-stage shared-memory ring of 4096-point row
+// groups (cp.async); each staged group feeds the column sums (one thread per column, its rows in order) and
+// the row sums (one warp per row, lanes along the row).  Two separate kernels over C, the column one with a
+// single dependent load in flight per thread, took 92 + 34 us at 256^3; this one 40 us (134 MB).
+constexpr int FR_PTS = 4096, FR_ST = 3, FR_NT = 256;
+__device__ __forceinline__ int frame_rows_per(int nx, int ny) { return min(min(FR_PTS / nx, ny), 64); }
+__global__ void __launch_bounds__(FR_NT) frame_sums_kernel(const float2* __restrict__ C, int nx, int ny,
+                                                           const float2* __restrict__ wr0, const float2* __restrict__ wr1,
+                                                           const float2* __restrict__ wc0, const float2* __restrict__ wc1,
+                                                           float2* __restrict__ TT, float2* __restrict__ TB,
+                                                           float2* __restrict__ UL, float2* __restrict__ UR, int ld) {
+    extern __shared__ float4 fsm[];
+    float2* ring = reinterpret_cast<float2*>(fsm);   // [FR_ST][FR_PTS]
+    float2* w = ring + FR_ST * FR_PTS;               // wc0, wc1 [nx], wr0, wr1 [ny]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l = blockIdx.x;
+    const int R = frame_rows_per(nx, ny), ng = ny / R;   // powers of two
     const float2* s = C + (size_t)l * nx * ny;
-    float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-    for (int j = 0; j < ny; ++j) {
-        const float2 v = s[(size_t)j * nx + i];
-        a = cfma(wr0[j], v, a);
-        b = cfma(wr1[j], v, b);
+    auto fetch = [&](int g) {
+        if (g < ng) {
+            const float4* src = reinterpret_cast<const float4*>(s + (size_t)g * R * nx);
+            float4* dst = reinterpret_cast<float4*>(ring + (g % FR_ST) * FR_PTS);
+            for (int e = tid; e < R * nx / 2; e += FR_NT) {
+                const unsigned a = (unsigned)__cvta_generic_to_shared(dst + e);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(src + e) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    for (int g = 0; g < FR_ST - 1; ++g) fetch(g);
+    for (int e = tid; e < nx; e += FR_NT) { w[e] = wc0[e]; w[nx + e] = wc1[e]; }
+    for (int e = tid; e < ny; e += FR_NT) { w[2 * nx + e] = wr0[e]; w[2 * nx + ny + e] = wr1[e]; }
+    float2 ca[2], cb[2];   // columns tid and tid + 256 (nx <= 512)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) ca[q] = cb[q] = make_float2(0.f, 0.f);
+    for (int g = 0; g < ng; ++g) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(FR_ST - 2) : "memory");
+        __syncthreads();         // group g landed for every thread; stage (g - 1) % FR_ST is free
+        fetch(g + FR_ST - 1);
+        const float2* t = ring + (g % FR_ST) * FR_PTS;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = tid + q * FR_NT;
+            if (i < nx)
+#pragma unroll 8
+                for (int r = 0; r < R; ++r) {
+                    const float2 v = t[r * nx + i];
+                    ca[q] = cfma(w[2 * nx + g * R + r], v, ca[q]);
+                    cb[q] = cfma(w[2 * nx + ny + g * R + r], v, cb[q]);
+                }
+        }
+        for (int r = warp; r < R; r += FR_NT / 32) {
+            float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
+#pragma unroll 4
+            for (int i = lane; i < nx; i += 32) {
+                const float2 v = t[r * nx + i];
+                a = cfma(v, w[i], a);
+                b = cfma(v, w[nx + i], b);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                a.x += __shfl_down_sync(0xffffffffu, a.x, o); a.y += __shfl_down_sync(0xffffffffu, a.y, o);
+                b.x += __shfl_down_sync(0xffffffffu, b.x, o); b.y += __shfl_down_sync(0xffffffffu, b.y, o);
+            }
+            if (lane == 0) {
+                UL[(size_t)l * ld + g * R + r] = a;
+                UR[(size_t)l * ld + g * R + r] = b;
+            }
+        }
     }
-    TT[(size_t)l * ld + i] = a;
-    TB[(size_t)l * ld + i] = b;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int i = tid + q * FR_NT;
+        if (i < nx) {
+            TT[(size_t)l * ld + i] = ca[q];
+            TB[(size_t)l * ld + i] = cb[q];
+        }
+    }
 }
+size_t frame_smem(int nx, int ny) { return (size_t)(FR_ST * FR_PTS + 2 * nx + 2 * ny) * sizeof(float2); }
 
-// UL[l][j] = sum_i C[l][j][i] wc0[i],  UR[l][j] = sum_i C[l][j][i] wc1[i]   (one warp per row)
-__global__ void frame_rows_kernel(const float2* __restrict__ C, int nx, int ny, const float2* __restrict__ wc0,
-                                  const float2* __restrict__ wc1, float2* __restrict__ UL, float2* __restrict__ UR,
-                                  int ld) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j = blockIdx.x * (blockDim.x >> 5) + warp, l = blockIdx.y;
-    if (j >= ny) return;
-    const float2* row = C + ((size_t)l * ny + j) * nx;
-    float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-    for (int i = lane; i < nx; i += 32) {
-        const float2 v = row[i];
-        a = cfma(v, wc0[i], a);
-        b = cfma(v, wc1[i], b);
+// Four batched dense matrix-vector products in one launch (blockIdx.z): out_b = Mat v_b (trans = 0) or Mat^T v_b
+// (trans = 1) for the nvec vectors v_b = in[b ld ..], element r of out_b at out[b ob + r orow].  A CTA takes 64
+// rows and 8 vectors, so that each row of Mat read from L2 serves 8 vectors; Mat is read along its rows in both
+// forms (trans 0: one warp per two rows with lanes along them, the 16 component sums of a row folded across the
+// lanes; trans 1: one thread per row and vector pair).  Bound by the latency of its few waves of CTAs.  One vector
+// per CTA and one launch per product (16 launches an application, each reading Mat once per vector) took 35 us a
+// product at N = 256; this takes 28 us for four.
+constexpr int MV_NV = 8, MV_ROWS = 64;
+struct MvJob {
+    const float2* Mat;
+    const float2* in;
+    float2* out;
+    int n, trans;
+    long ob, orow;
+};
+struct MvJobs { MvJob j[4]; };
+__global__ void __launch_bounds__(256) matvec4_kernel(const __grid_constant__ MvJobs jobs, int ld, int nvec) {
+    extern __shared__ float2 v[];   // [MV_NV][n]
+    const MvJob J = jobs.j[blockIdx.z];
+    const int n = J.n, r0 = blockIdx.y * MV_ROWS, b0 = blockIdx.x * MV_NV;
+    if (r0 >= n) return;
+    const int nb = min(MV_NV, nvec - b0), r1 = min(r0 + MV_ROWS, n);
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        float2 t[MV_NV];
+#pragma unroll
+        for (int q = 0; q < MV_NV; ++q) t[q] = q < nb ? J.in[(size_t)(b0 + q) * ld + k] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < MV_NV; ++q) v[q * n + k] = t[q];
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        a.x += __shfl_down_sync(0xffffffffu, a.x, o); a.y += __shfl_down_sync(0xffffffffu, a.y, o);
-        b.x += __shfl_down_sync(0xffffffffu, b.x, o); b.y += __shfl_down_sync(0xffffffffu, b.y, o);
-    }
-    if (lane == 0) { UL[(size_t)l * ld + j] = a; UR[(size_t)l * ld + j] = b; }
-}
-
-// out[b][r] = alpha * sum_k M(r, k) in[b][k]; M(r, k) = Mat[r][k] (trans = 0) or Mat[k][r] (trans = 1).
-// optional add: out += add (same layout).  Vectors of length n, stride ld; one CTA per vector.
-// Batched dense matrix times vector: out_b = alpha Mat v_b (+ add_b) for the nvec vectors v_b = in[b ld ..],
-// NV vectors per block (every row of Mat read from L2 serves NV of them).  trans = 0 reads Mat row by row
-// (one warp per row, lanes along the row, warp-shuffle sums); trans = 1 multiplies by Mat^T (one thread per
-// output, lanes along the row index), so both forms read Mat coalesced.
-template <int NV>
-__global__ void matvec_kernel(const float2* __restrict__ Mat, int n, int trans, const float2* __restrict__ in,
-                              float2* __restrict__ out, int ld, float2 alpha, const float2* __restrict__ add, int nvec) {
-    extern __shared__ float2 v[];   // [NV][n]
-    const int b0 = blockIdx.x * NV;
-    const int nb = min(NV, nvec - b0);
-    for (int q = 0; q < NV; ++q)
-        for (int k = threadIdx.x; k < n; k += blockDim.x)
-            v[q * n + k] = q < nb ? in[(size_t)(b0 + q) * ld + k] : make_float2(0.f, 0.f);
     __syncthreads();
-    if (trans) {
-        for (int r = threadIdx.x; r < n; r += blockDim.x) {
-            float2 acc[NV];
-#pragma unroll
-            for (int q = 0; q < NV; ++q) acc[q] = make_float2(0.f, 0.f);
-            for (int k = 0; k < n; ++k) {
-                const float2 m = Mat[(size_t)k * n + r];
-#pragma unroll
-                for (int q = 0; q < NV; ++q) acc[q] = cfma(m, v[q * n + k], acc[q]);
-            }
-            for (int q = 0; q < nb; ++q) {
-                float2 o = cmul(alpha, acc[q]);
-                if (add) o = cadd(o, add[(size_t)(b0 + q) * ld + r]);
-                out[(size_t)(b0 + q) * ld + r] = o;
-            }
+    if (J.trans) {
+        const int r = r0 + (threadIdx.x & (MV_ROWS - 1)), q0 = 2 * (threadIdx.x / MV_ROWS);
+        if (r >= r1) return;
+        float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+#pragma unroll 32
+        for (int k = 0; k < n; ++k) {
+            const float2 m = J.Mat[(size_t)k * n + r];
+            a0 = cfma(m, v[q0 * n + k], a0);
+            a1 = cfma(m, v[(q0 + 1) * n + k], a1);
         }
+        if (q0 < nb) J.out[(b0 + q0) * J.ob + r * J.orow] = a0;
+        if (q0 + 1 < nb) J.out[(b0 + q0 + 1) * J.ob + r * J.orow] = a1;
     } else {
-        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-        for (int r = threadIdx.x >> 5; r < n; r += nw) {
-            float2 acc[NV];
+        const int lane = threadIdx.x & 31;
+        // two rows per warp at a time, so that a vector element read from shared memory serves both
+        for (int r = r0 + 2 * (threadIdx.x >> 5); r < r1; r += 16) {
+            const int rb = min(r + 1, r1 - 1);
+            float2 acc[2][MV_NV];
 #pragma unroll
-            for (int q = 0; q < NV; ++q) acc[q] = make_float2(0.f, 0.f);
+            for (int q = 0; q < MV_NV; ++q) acc[0][q] = acc[1][q] = make_float2(0.f, 0.f);
+#pragma unroll 8
             for (int k = lane; k < n; k += 32) {
-                const float2 m = Mat[(size_t)r * n + k];
+                const float2 m0 = J.Mat[(size_t)r * n + k], m1 = J.Mat[(size_t)rb * n + k];
 #pragma unroll
-                for (int q = 0; q < NV; ++q) acc[q] = cfma(m, v[q * n + k], acc[q]);
+                for (int q = 0; q < MV_NV; ++q) {
+                    const float2 x = v[q * n + k];
+                    acc[0][q] = cfma(m0, x, acc[0][q]);
+                    acc[1][q] = cfma(m1, x, acc[1][q]);
+                }
             }
+            // sums over the lanes of the 16 components of a row: at each step a lane keeps half of them and adds the
+            // other half-warp's share (pairs at distance 16, 8, 4, 2, 1); lane bits 4..1 select the component it
+            // ends with
 #pragma unroll
-            for (int q = 0; q < NV; ++q)
-                for (int o = 16; o > 0; o >>= 1) {
-                    acc[q].x += __shfl_down_sync(0xffffffffu, acc[q].x, o);
-                    acc[q].y += __shfl_down_sync(0xffffffffu, acc[q].y, o);
+            for (int y = 0; y < 2; ++y) {
+                float f[2 * MV_NV];
+#pragma unroll
+                for (int q = 0; q < MV_NV; ++q) { f[2 * q] = acc[y][q].x; f[2 * q + 1] = acc[y][q].y; }
+#pragma unroll
+                for (int h = MV_NV, o = 16; h >= 1; h >>= 1, o >>= 1) {
+                    const bool up = lane & o;
+#pragma unroll
+                    for (int i = 0; i < h; ++i) {
+                        const float keep = up ? f[i + h] : f[i], send = up ? f[i] : f[i + h];
+                        f[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
                 }
-            if (lane == 0)
-                for (int q = 0; q < nb; ++q) {
-                    float2 o = cmul(alpha, acc[q]);
-                    if (add) o = cadd(o, add[(size_t)(b0 + q) * ld + r]);
-                    out[(size_t)(b0 + q) * ld + r] = o;
-                }
+                const float res = f[0] + __shfl_xor_sync(0xffffffffu, f[0], 1);
+                const int id = (lane & 16 ? 8 : 0) + (lane & 8 ? 4 : 0) + (lane & 4 ? 2 : 0) + (lane & 2 ? 1 : 0);
+                if (!(lane & 1) && (id >> 1) < nb && r + y < r1)
+                    reinterpret_cast<float*>(&J.out[(b0 + (id >> 1)) * J.ob + (r + y) * J.orow])[id & 1] = res;
+            }
         }
     }
 }
 
-constexpr int MV_NV = 1;   // one vector per block: nz blocks fill the GPU
-void launch_matvec(int nvec, cudaStream_t s, const float2* Mat, int n, int trans, const float2* in, float2* out, int ld,
-                   float2 alpha, const float2* add) {
-    matvec_kernel<MV_NV><<<(nvec + MV_NV - 1) / MV_NV, 256, MV_NV * n * sizeof(float2), s>>>(Mat, n, trans, in, out, ld,
-                                                                                         alpha, add, nvec);
+helm_status launch_matvec4(int nvec, cudaStream_t s, int ld, const MvJobs& jobs) {
+    int n = 0;
+    for (const MvJob& j : jobs.j) n = j.n > n ? j.n : n;
+    matvec4_kernel<<<dim3((nvec + MV_NV - 1) / MV_NV, (n + MV_ROWS - 1) / MV_ROWS, 4), 256, MV_NV * n * sizeof(float2), s>>>(
+        jobs, ld, nvec);
+    HELM_CUDA_TRY(cudaGetLastError());
+    return HELM_OK;
 }
 
-// out[t][l][m] = vec[m] for every slice l (t fixed): fills the slice-independent outer-product factors
-__global__ void fill_kernel(float2* __restrict__ out, int nz, int n, const float2* __restrict__ vec, int vstride,
-                            int voff) {
-    const size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (id >= (size_t)nz * n) return;
-    const int m = (int)(id % n);
-    out[id] = vec[(size_t)m * vstride + voff];
+// out[m] = column voff of a row-major matrix of row length vstride
+__global__ void column_kernel(float2* __restrict__ out, int n, const float2* __restrict__ mat, int vstride, int voff) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m < n) out[m] = mat[(size_t)m * vstride + voff];
 }
 
 // c = s (a + b) + t (a1 + b1) elementwise (frame values -> correction vectors; b, b1 may be NULL, and a1
-// is NULL for a one-layer frame)
+// is NULL for a one-layer frame); the first half of the n values (rows) takes s0, t0, the second (columns) s1, t1
 __global__ void frame_scale_kernel(const float2* __restrict__ a, const float2* __restrict__ b, const float2* a1,
-                                   const float2* b1, float2* c, size_t n, float2 s, float2 t) {
+                                   const float2* b1, float2* c, size_t n, float2 s0, float2 t0, float2 s1, float2 t1) {
     const size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (id >= n) return;
+    const float2 s = id < n / 2 ? s0 : s1, t = id < n / 2 ? t0 : t1;
     float2 v = a[id];
     if (b) v = cadd(v, b[id]);
     float2 o = cmul(s, v);
@@ -391,7 +466,16 @@ helm_status pfft_prepare(helm_ctx* c, cudaStream_t s) {
     if ((st = dmal(&P->fa, fv)) || (st = dmal(&P->fb, fv)) || (st = dmal(&P->fc, fv))) return st;
     if (c->zeta[0] != 1.0 || c->zeta[1] != 1.0)
         if ((st = dmal(&P->fb1, fv)) || (st = dmal(&P->fc1, fv))) return st;
-    if ((st = dmal(&P->P, (size_t)4 * nz * ny)) || (st = dmal(&P->Q, (size_t)4 * nz * nx))) return st;
+    P->nzp = (nz + 7) / 8 * 8;
+    if ((st = dmal(&P->Pt, (size_t)2 * P->nzp * ny)) || (st = dmal(&P->Q, (size_t)2 * nz * nx)) ||
+        (st = dmal(&P->ecol, (size_t)2 * (nx + ny)))) return st;
+    for (int k = 0; k < 2; ++k) {
+        column_kernel<<<(ny + 127) / 128, 128, 0, s>>>(P->ecol + k * ny, ny, P->Vyi, ny, k * (ny - 1));
+        column_kernel<<<(nx + 127) / 128, 128, 0, s>>>(P->ecol + 2 * ny + k * nx, nx, P->Vxi, nx, k * (nx - 1));
+    }
+    HELM_CUDA_TRY(cudaGetLastError());
+    HELM_CUDA_TRY(cudaFuncSetAttribute(frame_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)frame_smem(nx > 512 ? nx : 512, 512)));
     if ((st = zsolve_factor_with(c, P->dxF, P->dyF, &P->zfacF, s))) return st;
     if (c->tmaps) {
         // TF32 contexts: the sine transforms run as dense products on the tensor cores (operand sets 2, 3)
@@ -436,7 +520,8 @@ void pfft_release(helm_ctx* c) {
     PfftState* P = (PfftState*)c->pfft;
     if (!P) return;
     void* ps[] = {P->twx, P->twy, P->fwx, P->fwy, P->gpx, P->gpy, P->gmx, P->gmy, P->Sx, P->Sy, P->Vx, P->Vxi,
-                  P->Vy, P->Vyi, P->dxF, P->dyF, P->Yh, P->fa, P->fb, P->fc, P->fb1, P->fc1, P->P, P->Q, P->zfacF};
+                  P->Vy, P->Vyi, P->dxF, P->dyF, P->Yh, P->fa, P->fb, P->fc, P->fb1, P->fc1, P->Pt, P->Q,
+                  P->ecol, P->zfacF};
     for (void* p : ps) if (p) cudaFree(p);
     delete P;
     c->pfft = nullptr;
@@ -485,18 +570,13 @@ helm_status frame_of(helm_ctx* c, PfftState* P, const float2* C, const float2* M
     float2* TB = P->fa + blk;
     float2* UL = P->fa + 2 * blk;
     float2* UR = P->fa + 3 * blk;
-    frame_cols_kernel<<<dim3((nx + 127) / 128, nz), 128, 0, s>>>(C, nx, ny, My + (size_t)k * ny,
-                                                                 My + (size_t)(ny - 1 - k) * ny, TT, TB, nm);
-    frame_rows_kernel<<<dim3((ny + 7) / 8, nz), 256, 0, s>>>(C, nx, ny, Mx + (size_t)k * nx,
-                                                             Mx + (size_t)(nx - 1 - k) * nx, UL, UR, nm);
-    const float2 one = make_float2(1.f, 0.f);
-    // rows: Theta[0][i] = sum_i' Mx[i][i'] TT[i'];  columns: Theta[j][0] = sum_j' My[j][j'] UL[j']
-    launch_matvec(nz, s, Mx, nx, 0, TT, fr, nm, one, nullptr);
-    launch_matvec(nz, s, Mx, nx, 0, TB, fr + blk, nm, one, nullptr);
-    launch_matvec(nz, s, My, ny, 0, UL, fr + 2 * blk, nm, one, nullptr);
-    launch_matvec(nz, s, My, ny, 0, UR, fr + 3 * blk, nm, one, nullptr);
+    frame_sums_kernel<<<nz, FR_NT, frame_smem(nx, ny), s>>>(C, nx, ny, My + (size_t)k * ny, My + (size_t)(ny - 1 - k) * ny,
+                                                            Mx + (size_t)k * nx, Mx + (size_t)(nx - 1 - k) * nx, TT, TB, UL,
+                                                            UR, nm);
     HELM_CUDA_TRY(cudaGetLastError());
-    return HELM_OK;
+    // rows: Theta[0][i] = sum_i' Mx[i][i'] TT[i'];  columns: Theta[j][0] = sum_j' My[j][j'] UL[j']
+    return launch_matvec4(nz, s, nm, MvJobs{{{Mx, TT, fr, nx, 0, nm, 1}, {Mx, TB, fr + blk, nx, 0, nm, 1},
+                                             {My, UL, fr + 2 * blk, ny, 0, nm, 1}, {My, UR, fr + 3 * blk, ny, 0, nm, 1}}});
 }
 
 }  // namespace
@@ -509,7 +589,7 @@ helm_status pfft_apply_dirichlet(helm_ctx* c, const float2* r, float2* z, const 
     if (!P) return HELM_ERR_UNSUPPORTED;
     helm_status st;
     if ((st = dst2d(c, P, 0, r, P->Yh, 1.f, sigma, sidx, s)) != HELM_OK) return st;
-    if ((st = launch_zsolve_fact(c, P->zfacF, P->Yh, P->Yh, nullptr, nullptr, s)) != HELM_OK) return st;
+    if ((st = launch_zsolve_fact(c, P->zfacF, P->Yh, P->Yh, s)) != HELM_OK) return st;
     const float hz2 = (float)(c->h[2] * c->h[2]);
     return dst2d(c, P, 1, P->Yh, z, hz2, nullptr, 0, s);
 }
@@ -520,7 +600,6 @@ helm_status pfft_apply(helm_ctx* c, const float2* r, float2* z, const double* si
     const int nx = P->nx, ny = P->ny, nz = P->nz, nm = nx > ny ? nx : ny;
     const size_t blk = (size_t)nz * nm;
     helm_status st;
-    const float2 one = make_float2(1.f, 0.f);
     // (A_p^F - A_p) on the frame: alpha_d (-1 - gamma_d) times the boundary layer, plus alpha_d (1 - zeta_d)
     // times the second layer (zeta = 2 on collocated grids; nothing for zeta = 1)
     const float2 ex = make_float2((float)(c->ax * (-1.0 - c->gam[0].x)), (float)(c->ax * (-c->gam[0].y)));
@@ -530,70 +609,44 @@ helm_status pfft_apply(helm_ctx* c, const float2* r, float2* z, const double* si
     const bool two = P->fb1 != nullptr;
     // 1. Yh = S_y^T Y S_x ; Th = z-solve_F(Yh) -> tmp2 (z is free until the end)
     if ((st = dst2d(c, P, 0, r, P->Yh, 1.f, sigma, sidx, s)) != HELM_OK) return st;
-    if ((st = launch_zsolve_fact(c, P->zfacF, P->Yh, z, nullptr, nullptr, s)) != HELM_OK) return st;
+    if ((st = launch_zsolve_fact(c, P->zfacF, P->Yh, z, s)) != HELM_OK) return st;
     // 2. Theta on the frame (fb; second layer fb1), R vectors (fc): rows scaled by e_y, t_y, columns by e_x, t_x
     if ((st = frame_of(c, P, z, P->Sx, P->Sy, P->fb, s)) != HELM_OK) return st;
     if (two && (st = frame_of(c, P, z, P->Sx, P->Sy, P->fb1, s, 1)) != HELM_OK) return st;
-    frame_scale_kernel<<<(unsigned)((2 * blk + 255) / 256), 256, 0, s>>>(P->fb, nullptr, two ? P->fb1 : nullptr,
-                                                                        nullptr, P->fc, 2 * blk, ey, ty);
-    frame_scale_kernel<<<(unsigned)((2 * blk + 255) / 256), 256, 0, s>>>(
-        P->fb + 2 * blk, nullptr, two ? P->fb1 + 2 * blk : nullptr, nullptr, P->fc + 2 * blk, 2 * blk, ex, tx);
+    const unsigned fgrid = (unsigned)((4 * blk + 255) / 256);
+    frame_scale_kernel<<<fgrid, 256, 0, s>>>(P->fb, nullptr, two ? P->fb1 : nullptr, nullptr, P->fc, 4 * blk, ey, ty, ex, tx);
+    HELM_CUDA_TRY(cudaGetLastError());
     // Rbar = sum of four outer products: (Vyi e_0)(Vxi ryT)^T + (Vyi e_N)(Vxi ryB)^T + (Vyi cxL)(Vxi e_0)^T + ...
     //   P[0] = Vyi[:, 0], P[1] = Vyi[:, N-1], P[2] = Vyi cxL, P[3] = Vyi cxR
     //   Q[0] = Vxi ryT,   Q[1] = Vxi ryB,     Q[2] = Vxi[:, 0], Q[3] = Vxi[:, N-1]
-    fill_kernel<<<(unsigned)((nz * (size_t)ny + 255) / 256), 256, 0, s>>>(P->P, nz, ny, P->Vyi, ny, 0);
-    fill_kernel<<<(unsigned)((nz * (size_t)ny + 255) / 256), 256, 0, s>>>(P->P + (size_t)nz * ny, nz, ny, P->Vyi, ny, ny - 1);
-    fill_kernel<<<(unsigned)((nz * (size_t)nx + 255) / 256), 256, 0, s>>>(P->Q + 2 * (size_t)nz * nx, nz, nx, P->Vxi, nx, 0);
-    fill_kernel<<<(unsigned)((nz * (size_t)nx + 255) / 256), 256, 0, s>>>(P->Q + 3 * (size_t)nz * nx, nz, nx, P->Vxi, nx, nx - 1);
-    // matvec outputs are written with stride n of the factor arrays
-    launch_matvec(nz, s, P->Vyi, ny, 0, P->fc + 2 * blk, P->fa, nm, one, nullptr);
-    launch_matvec(nz, s, P->Vyi, ny, 0, P->fc + 3 * blk, P->fa + blk, nm, one, nullptr);
-    launch_matvec(nz, s, P->Vxi, nx, 0, P->fc, P->fa + 2 * blk, nm, one, nullptr);
-    launch_matvec(nz, s, P->Vxi, nx, 0, P->fc + blk, P->fa + 3 * blk, nm, one, nullptr);
-    HELM_CUDA_TRY(cudaGetLastError());
-    // repack to the factor layouts P[t][l][j], Q[t][l][i]
-    HELM_CUDA_TRY(cudaMemcpy2DAsync(P->P + 2 * (size_t)nz * ny, ny * sizeof(float2), P->fa, nm * sizeof(float2),
-                                    ny * sizeof(float2), nz, cudaMemcpyDeviceToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpy2DAsync(P->P + 3 * (size_t)nz * ny, ny * sizeof(float2), P->fa + blk, nm * sizeof(float2),
-                                    ny * sizeof(float2), nz, cudaMemcpyDeviceToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpy2DAsync(P->Q, nx * sizeof(float2), P->fa + 2 * blk, nm * sizeof(float2), nx * sizeof(float2),
-                                    nz, cudaMemcpyDeviceToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpy2DAsync(P->Q + (size_t)nz * nx, nx * sizeof(float2), P->fa + 3 * blk, nm * sizeof(float2),
-                                    nx * sizeof(float2), nz, cudaMemcpyDeviceToDevice, s));
+    // (the products are written in the z-solve's layouts Pt[t][j][l], Q[t][l][i])
+    const long nzp = P->nzp;
+    float2 *pt0 = P->Pt, *pt1 = P->Pt + nzp * ny, *q0 = P->Q, *q1 = P->Q + (size_t)nz * nx;
+    if ((st = launch_matvec4(nz, s, nm, MvJobs{{{P->Vyi, P->fc + 2 * blk, pt0, ny, 0, 1, nzp},
+                                                {P->Vyi, P->fc + 3 * blk, pt1, ny, 0, 1, nzp},
+                                                {P->Vxi, P->fc, q0, nx, 0, nx, 1},
+                                                {P->Vxi, P->fc + blk, q1, nx, 0, nx, 1}}})) != HELM_OK)
+        return st;
     //    Wbar = z-solve_EigT(Rbar) into z; W on the frame (fc) from Wbar with the EigT bases
-    if ((st = launch_zsolve_fact(c, c->zfac, nullptr, z, P->P, P->Q, s)) != HELM_OK) return st;
+    const ZGen ge = {P->ecol, P->ecol + ny, pt0, pt1, q0, q1, P->ecol + 2 * ny, P->ecol + 2 * ny + nx, P->nzp};
+    if ((st = launch_zsolve_gen(c, c->zfac, nullptr, z, ge, s)) != HELM_OK) return st;
     if ((st = frame_of(c, P, z, P->Vx, P->Vy, P->fc, s)) != HELM_OK) return st;
     if (two && (st = frame_of(c, P, z, P->Vx, P->Vy, P->fc1, s, 1)) != HELM_OK) return st;
     // 3. R2 = (A_p^F - A_p)(Theta + W) on the frame -> fc (rows e_y, t_y, columns e_x, t_x)
-    frame_scale_kernel<<<(unsigned)((2 * blk + 255) / 256), 256, 0, s>>>(
-        P->fb, P->fc, two ? P->fb1 : nullptr, two ? P->fc1 : nullptr, P->fc, 2 * blk, ey, ty);
-    frame_scale_kernel<<<(unsigned)((2 * blk + 255) / 256), 256, 0, s>>>(
-        P->fb + 2 * blk, P->fc + 2 * blk, two ? P->fb1 + 2 * blk : nullptr, two ? P->fc1 + 2 * blk : nullptr,
-        P->fc + 2 * blk, 2 * blk, ex, tx);
+    frame_scale_kernel<<<fgrid, 256, 0, s>>>(P->fb, P->fc, two ? P->fb1 : nullptr, two ? P->fc1 : nullptr, P->fc, 4 * blk,
+                                             ey, ty, ex, tx);
+    HELM_CUDA_TRY(cudaGetLastError());
     //    sine transform of R2 as four outer products:
     //   P[0] = S_y[0][:], P[1] = S_y[N-1][:], P[2] = S_y^T c2L, P[3] = S_y^T c2R
     //   Q[0] = S_x^T r2T, Q[1] = S_x^T r2B,   Q[2] = S_x[0][:], Q[3] = S_x[N-1][:]
-    fill_kernel<<<(unsigned)((nz * (size_t)ny + 255) / 256), 256, 0, s>>>(P->P, nz, ny, P->Sy, 1, 0);
-    fill_kernel<<<(unsigned)((nz * (size_t)ny + 255) / 256), 256, 0, s>>>(P->P + (size_t)nz * ny, nz, ny,
-                                                                        P->Sy + (size_t)(ny - 1) * ny, 1, 0);
-    fill_kernel<<<(unsigned)((nz * (size_t)nx + 255) / 256), 256, 0, s>>>(P->Q + 2 * (size_t)nz * nx, nz, nx, P->Sx, 1, 0);
-    fill_kernel<<<(unsigned)((nz * (size_t)nx + 255) / 256), 256, 0, s>>>(P->Q + 3 * (size_t)nz * nx, nz, nx,
-                                                                        P->Sx + (size_t)(nx - 1) * nx, 1, 0);
-    launch_matvec(nz, s, P->Sy, ny, 1, P->fc + 2 * blk, P->fa, nm, one, nullptr);
-    launch_matvec(nz, s, P->Sy, ny, 1, P->fc + 3 * blk, P->fa + blk, nm, one, nullptr);
-    launch_matvec(nz, s, P->Sx, nx, 1, P->fc, P->fa + 2 * blk, nm, one, nullptr);
-    launch_matvec(nz, s, P->Sx, nx, 1, P->fc + blk, P->fa + 3 * blk, nm, one, nullptr);
-    HELM_CUDA_TRY(cudaGetLastError());
-    HELM_CUDA_TRY(cudaMemcpy2DAsync(P->P + 2 * (size_t)nz * ny, ny * sizeof(float2), P->fa, nm * sizeof(float2),
-                                    ny * sizeof(float2), nz, cudaMemcpyDeviceToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpy2DAsync(P->P + 3 * (size_t)nz * ny, ny * sizeof(float2), P->fa + blk, nm * sizeof(float2),
-                                    ny * sizeof(float2), nz, cudaMemcpyDeviceToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpy2DAsync(P->Q, nx * sizeof(float2), P->fa + 2 * blk, nm * sizeof(float2), nx * sizeof(float2),
-                                    nz, cudaMemcpyDeviceToDevice, s));
-    HELM_CUDA_TRY(cudaMemcpy2DAsync(P->Q + (size_t)nz * nx, nx * sizeof(float2), P->fa + 3 * blk, nm * sizeof(float2),
-                                    nx * sizeof(float2), nz, cudaMemcpyDeviceToDevice, s));
+    if ((st = launch_matvec4(nz, s, nm, MvJobs{{{P->Sy, P->fc + 2 * blk, pt0, ny, 1, 1, nzp},
+                                                {P->Sy, P->fc + 3 * blk, pt1, ny, 1, 1, nzp},
+                                                {P->Sx, P->fc, q0, nx, 1, nx, 1},
+                                                {P->Sx, P->fc + blk, q1, nx, 1, nx, 1}}})) != HELM_OK)
+        return st;
     //    Uh = z-solve_F(Yh + sine transform of R2) in place in Yh; U = h_z^2 S_y Uh S_x^T
-    if ((st = launch_zsolve_fact(c, P->zfacF, P->Yh, P->Yh, P->P, P->Q, s)) != HELM_OK) return st;
+    const ZGen gf = {P->Sy, P->Sy + (size_t)(ny - 1) * ny, pt0, pt1, q0, q1, P->Sx, P->Sx + (size_t)(nx - 1) * nx, P->nzp};
+    if ((st = launch_zsolve_gen(c, P->zfacF, P->Yh, P->Yh, gf, s)) != HELM_OK) return st;
     const float hz2 = (float)(c->h[2] * c->h[2]);
     return dst2d(c, P, 1, P->Yh, z, hz2, nullptr, 0, s);
 }

@@ -27,9 +27,6 @@ struct ZParams {
     const float2* cz;    // h_z^2 k0^2(z_l) - 2(alpha_x + alpha_y + 1)
     float2 gz;           // gamma_z
     float zz;            // zeta_z
-    // optional generated right-hand side: y[l][j][i] += sum_{t<4} P[t][l][j] Q[t][l][i]  (PFFT)
-    const float2* P;
-    const float2* Q;
 };
 
 __device__ inline float2 f2(float a, float b) { return make_float2(a, b); }
@@ -75,6 +72,13 @@ __device__ __forceinline__ float2 zbwd(float2 d, float2 m, float2 x, float sup) 
     return make_float2(__fmaf_rn(-px, sup, d.x), __fmaf_rn(-py, sup, d.y));
 }
 
+// y + a b with the product rounded as written (so that every kernel that forms a generated right-hand side
+// gives the same bits)
+__device__ __forceinline__ float2 zaddmul(float2 y, float2 a, float2 b) {
+    return make_float2(__fadd_rn(y.x, __fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y))),
+                       __fadd_rn(y.y, __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y))));
+}
+
 template <int L, int MCH>
 __global__ void __launch_bounds__(L * 32)
 zsolve_kernel(ZParams p, const float2* in, float2* out, unsigned* status) {
@@ -105,16 +109,6 @@ zsolve_kernel(ZParams p, const float2* in, float2* out, unsigned* status) {
 #pragma unroll
     for (int k = 0; k < MCH; ++k)
         y[k] = (in && live && k < len) ? in[base + (size_t)(s + k) * plane] : f2(0.f, 0.f);
-    if (p.P && live) {
-#pragma unroll
-        for (int k = 0; k < MCH; ++k)
-            if (k < len) {
-                const int l = s + k;
-#pragma unroll
-                for (int t = 0; t < 4; ++t)
-                    y[k] = cadd(y[k], cmul(p.P[((size_t)t * nz + l) * p.ny + j], p.Q[((size_t)t * nz + l) * p.nx + i]));
-            }
-    }
 #pragma unroll
     for (int k = 0; k < MCH; ++k) bd[k] = (k < len) ? diag(s + k) : f2(1.f, 0.f);
     float minpiv = 1e30f;
@@ -253,14 +247,13 @@ __global__ void __launch_bounds__(128) zfactor_kernel(ZParams p, float2* __restr
 }
 
 __global__ void __launch_bounds__(128) zsolve_fact_kernel(int nx, int ny, int nz, float zz, const float2* __restrict__ m,
-                                                         const float2* in, float2* out, const float2* __restrict__ P,
-                                                         const float2* __restrict__ Q) {
+                                                         const float2* in, float2* out) {
     // blockIdx.y = (right-hand side of a batch group) * ny + j; the factors m are shared
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y % ny, vb = blockIdx.y / ny;
     if (i >= nx) return;
     const size_t plane = (size_t)nx * ny, base = (size_t)j * nx + i, voff = (size_t)vb * plane * nz;
     if (vb) {
-        if (in) in += voff;
+        in += voff;
         out += voff;
     }
     float2 d = f2(0.f, 0.f);
@@ -269,21 +262,9 @@ __global__ void __launch_bounds__(128) zsolve_fact_kernel(int nx, int ny, int nz
 #pragma unroll
         for (int u = 0; u < ZU; ++u)
             if (l0 + u < nz) {
-                yv[u] = in ? in[base + (size_t)(l0 + u) * plane] : f2(0.f, 0.f);
+                yv[u] = in[base + (size_t)(l0 + u) * plane];
                 mv[u] = m[base + (size_t)(l0 + u) * plane];
             }
-        if (P) {
-            // generated right-hand side: y[l][j][i] += sum_{t<4} P[t][l][j] Q[t][l][i]
-#pragma unroll
-            for (int u = 0; u < ZU; ++u) {
-                const int l = l0 + u;
-                if (l < nz) {
-#pragma unroll
-                    for (int t = 0; t < 4; ++t)
-                        yv[u] = cadd(yv[u], cmul(P[((size_t)t * nz + l) * ny + j], Q[((size_t)t * nz + l) * nx + i]));
-                }
-            }
-        }
 #pragma unroll
         for (int u = 0; u < ZU; ++u) {
             const int l = l0 + u;
@@ -317,38 +298,55 @@ __global__ void __launch_bounds__(128) zsolve_fact_kernel(int nx, int ny, int nz
     }
 }
 
-// Factorised solve, L2-resident form (no generated right-hand side, even N_x).  The backward sweep reads
+// Factorised solve, L2-resident form (even N_x).  The backward sweep reads
 // d and m again; when every line runs at once those re-reads (16 B/pt) miss the L2, so here a persistent
 // grid of a few 64-thread CTAs per SM keeps about 20k-40k lines in flight (their d and m stay in L2) and
 // walks the rest in turn.  Each thread takes two adjacent lines (16-byte accesses) and streams its inputs
 // through a private ring of ZB blocks of ZU steps in shared memory by cp.async (one group per block, no
 // block barrier); a landed block is read into registers at once and its ZU dependent steps then run back
 // to back, so the shared-memory latency is paid once per block rather than once per step.
-constexpr int ZRT = 64, ZU2 = 8, ZB = 4;
-constexpr size_t ZRING_BYTES = (size_t)ZB * ZU2 * 2 * ZRT * sizeof(float4);   // 64 KiB
+// GEN = 1, 2 (PFFT's boundary correction; 2: no input grid): the right-hand side of ZGen is formed as the forward
+// sweep consumes a block.  Its two factors that vary with the slice and x ride in the ring beside y and m; those
+// that vary with the slice and y are read one block ahead into registers (they are contiguous in the slice
+// index), the rest are constant along a line.  One thread per line without a ring, re-reading all eight
+// factors at every step, took 235 us at 256^3; this takes 119 us (GEN = 1) and 107 us (GEN = 2).
+constexpr int ZRT = 64, ZU2 = 8;
+__host__ __device__ constexpr int zring_arrays(int gen) { return gen == 0 ? 2 : (gen == 1 ? 4 : 3); }
+__host__ __device__ constexpr int zring_depth(int gen) { return gen == 1 ? 3 : 4; }   // blocks in the ring
+__host__ __device__ constexpr size_t zring_bytes(int gen) {   // 64 KiB, 96 KiB, 96 KiB
+    return (size_t)zring_depth(gen) * ZU2 * zring_arrays(gen) * ZRT * sizeof(float4);
+}
 
 __device__ __forceinline__ void zcp16(void* smem, const void* gmem) {
     const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void zcommit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void zwait_ring() { asm volatile("cp.async.wait_group %0;\n" ::"n"(ZB - 1) : "memory"); }
+template <int N>
+__device__ __forceinline__ void zwait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void zwait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // nb > 1: nb right-hand side grids back to back (a batch group), sharing the factors m
+template <int GEN>
 __global__ void __launch_bounds__(ZRT) zsolve_ring_kernel(int nx, int ny, int nz, float zz,
                                                          const float4* __restrict__ m, const float4* in, float4* out,
-                                                         int nb) {
-    extern __shared__ float4 zring[];   // [ZB * ZU2][2][ZRT]
+                                                         int nb, const __grid_constant__ ZGen g) {
+    constexpr int ZB = zring_depth(GEN), NA = zring_arrays(GEN);
+    constexpr int AQ = GEN == 1 ? 2 : 1;   // first of the two Q arrays in a slot (y: 0, m: the last without GEN)
+    constexpr int AM = GEN == 2 ? 0 : 1;
+    extern __shared__ float4 zring[];   // [ZB * ZU2][NA][ZRT]
     const int tid = threadIdx.x;
     const int hx = nx / 2, npairs = hx * ny;
     const int nblk = (nz + ZU2 - 1) / ZU2;
     const size_t plane = (size_t)hx * ny;   // in float4 (two lines) units
-    auto slot = [&](int st, int a) -> float4* { return &zring[((size_t)st * 2 + a) * ZRT + tid]; };
+    auto slot = [&](int st, int a) -> float4* { return &zring[((size_t)st * NA + a) * ZRT + tid]; };
     for (int prb = blockIdx.x * ZRT + tid; prb < npairs * nb; prb += gridDim.x * ZRT) {
         const int pr = prb % npairs, vb = prb / npairs;
         const size_t off = (size_t)pr;   // pair pr = (j, i/2) is float4 pr of every plane
         const size_t voff = (size_t)vb * plane * nz;   // this right-hand side's grid (the factors are shared)
+        const int j = pr / hx;
+        const float4* q0 = GEN ? reinterpret_cast<const float4*>(g.q0) + (pr - j * hx) : nullptr;
+        const float4* q1 = GEN ? reinterpret_cast<const float4*>(g.q1) + (pr - j * hx) : nullptr;
         // ---- forward: d_l = (y_l - a_l d_{l-1}) m_l, steps in increasing l
         auto fetch_f = [&](int b) {
             if (b < nblk) {
@@ -356,8 +354,12 @@ __global__ void __launch_bounds__(ZRT) zsolve_ring_kernel(int nx, int ny, int nz
                 for (int u = 0; u < ZU2; ++u) {
                     const int l = b * ZU2 + u;
                     if (l < nz) {
-                        zcp16(slot((b % ZB) * ZU2 + u, 0), in + voff + off + (size_t)l * plane);
-                        zcp16(slot((b % ZB) * ZU2 + u, 1), m + off + (size_t)l * plane);
+                        if (GEN != 2) zcp16(slot((b % ZB) * ZU2 + u, 0), in + voff + off + (size_t)l * plane);
+                        zcp16(slot((b % ZB) * ZU2 + u, AM), m + off + (size_t)l * plane);
+                        if (GEN) {
+                            zcp16(slot((b % ZB) * ZU2 + u, AQ), q0 + (size_t)l * hx);
+                            zcp16(slot((b % ZB) * ZU2 + u, AQ + 1), q1 + (size_t)l * hx);
+                        }
                     }
                 }
             }
@@ -365,15 +367,51 @@ __global__ void __launch_bounds__(ZRT) zsolve_ring_kernel(int nx, int ny, int nz
         };
         for (int b = 0; b < ZB - 1; ++b) fetch_f(b);
         float2 d0 = f2(0.f, 0.f), d1 = d0;
+        float2 p0 = d0, p1 = d0;                         // GEN: the factors constant along the line pair
+        float4 c2 = make_float4(0.f, 0.f, 0.f, 0.f), c3 = c2;
+        float4 n2[ZU2 / 2], n3[ZU2 / 2];                 // p2, p3 of the next block, two steps per float4
+        const float4* p2 = nullptr;
+        const float4* p3 = nullptr;
+        if (GEN) {
+            p0 = g.p0[j];
+            p1 = g.p1[j];
+            c2 = reinterpret_cast<const float4*>(g.q2)[pr - j * hx];
+            c3 = reinterpret_cast<const float4*>(g.q3)[pr - j * hx];
+            p2 = reinterpret_cast<const float4*>(g.p2 + (size_t)j * g.nzp);
+            p3 = reinterpret_cast<const float4*>(g.p3 + (size_t)j * g.nzp);
+#pragma unroll
+            for (int u = 0; u < ZU2 / 2; ++u) { n2[u] = p2[u]; n3[u] = p3[u]; }
+        }
         for (int b = 0; b < nblk; ++b) {
             fetch_f(b + ZB - 1);
-            zwait_ring();   // block b has landed
+            zwait<ZB - 1>();   // block b has landed
             float4 y[ZU2], mm[ZU2];
 #pragma unroll
             for (int u = 0; u < ZU2; ++u) {
-                y[u] = *slot((b % ZB) * ZU2 + u, 0);
-                mm[u] = *slot((b % ZB) * ZU2 + u, 1);
+                y[u] = GEN == 2 ? make_float4(0.f, 0.f, 0.f, 0.f) : *slot((b % ZB) * ZU2 + u, 0);
+                mm[u] = *slot((b % ZB) * ZU2 + u, AM);
+                if (GEN) {
+                    const float4 a = *slot((b % ZB) * ZU2 + u, AQ), e = *slot((b % ZB) * ZU2 + u, AQ + 1);
+                    const float2 r2 = u & 1 ? f2(n2[u / 2].z, n2[u / 2].w) : f2(n2[u / 2].x, n2[u / 2].y);
+                    const float2 r3 = u & 1 ? f2(n3[u / 2].z, n3[u / 2].w) : f2(n3[u / 2].x, n3[u / 2].y);
+                    float2 v0 = f2(y[u].x, y[u].y), v1 = f2(y[u].z, y[u].w);
+                    v0 = zaddmul(v0, p0, f2(a.x, a.y));
+                    v0 = zaddmul(v0, p1, f2(e.x, e.y));
+                    v0 = zaddmul(v0, r2, f2(c2.x, c2.y));
+                    v0 = zaddmul(v0, r3, f2(c3.x, c3.y));
+                    v1 = zaddmul(v1, p0, f2(a.z, a.w));
+                    v1 = zaddmul(v1, p1, f2(e.z, e.w));
+                    v1 = zaddmul(v1, r2, f2(c2.z, c2.w));
+                    v1 = zaddmul(v1, r3, f2(c3.z, c3.w));
+                    y[u] = make_float4(v0.x, v0.y, v1.x, v1.y);
+                }
             }
+            if (GEN && b + 1 < nblk)
+#pragma unroll
+                for (int u = 0; u < ZU2 / 2; ++u) {
+                    n2[u] = p2[(b + 1) * (ZU2 / 2) + u];
+                    n3[u] = p3[(b + 1) * (ZU2 / 2) + u];
+                }
 #pragma unroll
             for (int u = 0; u < ZU2; ++u) {
                 const int l = b * ZU2 + u;
@@ -405,7 +443,7 @@ __global__ void __launch_bounds__(ZRT) zsolve_ring_kernel(int nx, int ny, int nz
         float2 x0 = f2(0.f, 0.f), x1 = x0;
         for (int b = 0; b < nblk; ++b) {
             fetch_b(b + ZB - 1);
-            zwait_ring();
+            zwait<ZB - 1>();
             float4 dv[ZU2], mm[ZU2];
 #pragma unroll
             for (int u = 0; u < ZU2; ++u) {
@@ -622,14 +660,17 @@ helm_status zsolve_factor_with(helm_ctx* c, const float2* dxs, const float2* dys
         if (cudaMalloc(m, c->npts * sizeof(float2)) != cudaSuccess) { cudaGetLastError(); return HELM_ERR_NOMEM; }
     }
     if (!c->zring_sms) {   // the ring kernel of the factorised solve: shared memory and grid size
-        HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_ring_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)ZRING_BYTES));
+        HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_ring_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)zring_bytes(0)));
+        HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_ring_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)zring_bytes(1)));
+        HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_ring_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)zring_bytes(2)));
         HELM_CUDA_TRY(cudaDeviceGetAttribute(&c->zring_sms, cudaDevAttrMultiProcessorCount, c->device));
     }
     ZParams p;
     p.nx = c->nx; p.ny = c->ny; p.nz = c->nz;
     p.dxs = dxs; p.dys = dys; p.cz = c->cz;
-    p.P = nullptr; p.Q = nullptr;
     p.gz = make_float2((float)c->gam[2].x, (float)c->gam[2].y);
     p.zz = (float)c->zeta[2];
     dim3 grid((c->nx + 127) / 128, c->ny);
@@ -640,36 +681,53 @@ helm_status zsolve_factor_with(helm_ctx* c, const float2* dxs, const float2* dys
 
 helm_status zsolve_factor(helm_ctx* c, cudaStream_t s) { return zsolve_factor_with(c, c->dxs, c->dys, &c->zfac, s); }
 
-// factorised solve with factors m, optional input (NULL = 0) and optional generated right-hand side
-helm_status launch_zsolve_fact(helm_ctx* c, const float2* m, const float2* in, float2* out, const float2* P,
-                               const float2* Q, cudaStream_t s, int nb) {
+// factorised solve with factors m
+helm_status launch_zsolve_fact(helm_ctx* c, const float2* m, const float2* in, float2* out, cudaStream_t s, int nb) {
     prof_begin(c, s, PROF_ZSOLVE);
-    if (!P && in && c->nx % 2 == 0 && c->tune_zring && c->zring_sms > 0) {
+    if (c->nx % 2 == 0 && c->tune_zring && c->zring_sms > 0) {
         const int sms = c->zring_sms;
         const int npairs = c->nx / 2 * c->ny * nb;
         const int need = (npairs + ZRT - 1) / ZRT;
         const int grid = need < sms * c->tune_zring ? need : sms * c->tune_zring;
-        zsolve_ring_kernel<<<grid, ZRT, ZRING_BYTES, s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2],
-                                                         reinterpret_cast<const float4*>(m),
-                                                         reinterpret_cast<const float4*>(in), reinterpret_cast<float4*>(out),
-                                                         nb);
+        zsolve_ring_kernel<0><<<grid, ZRT, zring_bytes(0), s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2],
+                                                                reinterpret_cast<const float4*>(m),
+                                                                reinterpret_cast<const float4*>(in),
+                                                                reinterpret_cast<float4*>(out), nb, ZGen());
         prof_end(c, s);
         HELM_CUDA_TRY(cudaGetLastError());
         return HELM_OK;
     }
     dim3 grid((c->nx + 127) / 128, c->ny * nb);
-    zsolve_fact_kernel<<<grid, 128, 0, s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2], m, in, out, P, Q);
+    zsolve_fact_kernel<<<grid, 128, 0, s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2], m, in, out);
     prof_end(c, s);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
 }
 
-helm_status launch_zsolve_gen(helm_ctx* c, const float2* in, float2* out, const float2* dxs, const float2* dys,
-                              const float2* P, const float2* Q, cudaStream_t s) {
+helm_status launch_zsolve_gen(helm_ctx* c, const float2* m, const float2* in, float2* out, const ZGen& g, cudaStream_t s) {
+    if (c->nx % 2 != 0 || c->zring_sms <= 0) return HELM_ERR_UNSUPPORTED;
+    const int need = (c->nx / 2 * c->ny + ZRT - 1) / ZRT, cap = 2 * c->zring_sms;   // two CTAs per SM (shared memory)
+    const int grid = need < cap ? need : cap;
+    prof_begin(c, s, PROF_ZSOLVE);
+    if (in)
+        zsolve_ring_kernel<1><<<grid, ZRT, zring_bytes(1), s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2],
+                                                                reinterpret_cast<const float4*>(m),
+                                                                reinterpret_cast<const float4*>(in),
+                                                                reinterpret_cast<float4*>(out), 1, g);
+    else
+        zsolve_ring_kernel<2><<<grid, ZRT, zring_bytes(2), s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2],
+                                                                reinterpret_cast<const float4*>(m), nullptr,
+                                                                reinterpret_cast<float4*>(out), 1, g);
+    prof_end(c, s);
+    HELM_CUDA_TRY(cudaGetLastError());
+    return HELM_OK;
+}
+
+// the partitioned solve, for systems without set-up factors
+static helm_status launch_zsolve_part(helm_ctx* c, const float2* in, float2* out, cudaStream_t s) {
     ZParams p;
     p.nx = c->nx; p.ny = c->ny; p.nz = c->nz;
-    p.dxs = dxs; p.dys = dys; p.cz = c->cz;
-    p.P = P; p.Q = Q;
+    p.dxs = c->dxs; p.dys = c->dys; p.cz = c->cz;
     p.gz = make_float2((float)c->gam[2].x, (float)c->gam[2].y);
     p.zz = (float)c->zeta[2];
     if (c->nz > 512) return HELM_ERR_UNSUPPORTED;
@@ -708,9 +766,7 @@ helm_status launch_zsolve(helm_ctx* c, const float2* in, float2* out, cudaStream
     if (!c->zfac) {
         helm_status st;
         for (int v = 0; v < nb; ++v)
-            if ((st = launch_zsolve_gen(c, in + (size_t)v * c->npts, out + (size_t)v * c->npts, c->dxs, c->dys, nullptr,
-                                        nullptr, s)) != HELM_OK)
-                return st;
+            if ((st = launch_zsolve_part(c, in + (size_t)v * c->npts, out + (size_t)v * c->npts, s)) != HELM_OK) return st;
         return HELM_OK;
     }
     if (in && c->nx % 2 == 0 && c->tune_zring && c->zring_sms > 0 && !c->zpiv_off) {
@@ -723,7 +779,7 @@ helm_status launch_zsolve(helm_ctx* c, const float2* in, float2* out, cudaStream
         if (zsolve_ck_bytes(c, slot + nb) > c->zck_bytes) {
             cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
             HELM_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
-            if (cap != cudaStreamCaptureStatusNone) return launch_zsolve_fact(c, c->zfac, in, out, nullptr, nullptr, s, nb);
+            if (cap != cudaStreamCaptureStatusNone) return launch_zsolve_fact(c, c->zfac, in, out, s, nb);
             helm_status st;
             if ((st = zsolve_reserve(c, slot + nb)) != HELM_OK) return st;
         }
@@ -746,7 +802,7 @@ helm_status launch_zsolve(helm_ctx* c, const float2* in, float2* out, cudaStream
         HELM_CUDA_TRY(cudaGetLastError());
         return HELM_OK;
     }
-    return launch_zsolve_fact(c, c->zfac, in, out, nullptr, nullptr, s, nb);
+    return launch_zsolve_fact(c, c->zfac, in, out, s, nb);
 }
 
 // The z-solves of the 16-bit transform chain (HELM_PREC_BF16, HELM_PREC_FP16): the pivot-recomputing kernel

@@ -3,7 +3,8 @@
 M^-1 is linear and the chain runs on r / ||r||, so scaling r by a power of two must scale z by the same
 power: the sums of squares, which lie outside FP32's range at these scales, are formed on scaled values.  Only
 1/||r|| and ||r|| are rounded (to FP32, 6e-8 each), and a changed rounding of 1/||r|| would move FP16 roundings;
-powers of two change neither significand, so the result is exact.
+powers of two change neither significand, so the result is exact down to 2^-126.  Below that FP32 is subnormal: the
+kernel's product and the reference's scaling each round to a multiple of 2^-149.
 """
 import math
 
@@ -28,7 +29,8 @@ def test_scaling_the_input_scales_the_output(n, exponent):
     s = 2.0 ** exponent
     a = S.apply_precond(r)
     b = S.apply_precond((r * s).contiguous())
-    assert torch.equal(torch.view_as_real(a) * s, torch.view_as_real(b))
+    a, b = torch.view_as_real(a).double() * s, torch.view_as_real(b).double()
+    assert ((a - b).abs() <= torch.where(a.abs() < 2.0 ** -126, 2.0 ** -149, 0.0)).all()
 
 
 def test_zero_stays_zero():
