@@ -1,64 +1,53 @@
 // 3x3x3 convolutions of the learned correction on the tcgen05 tensor cores (BF16 operands, FP32 accumulation
-// in tensor memory), as implicit GEMMs.  An extension of the method (the paper has no network); the
-// network, its layout ([B][C][Z][Y][X], x fastest) and the direct SIMT kernels it replaces live in
-// learned.cu.
+// in tensor memory), as implicit GEMMs.  An extension of the method (the paper has no network); the network
+// itself lives in learned.cu, the activation layout in cells.cuh.
 //
-// Forward (and data gradient, which is the same convolution with flipped, transposed weights):
-//   out[o][p] = act(bias[o] + sum_{t, i} W(o, i, t) in[i][p + off_t]),  zero padding.
-//   A CTA computes CT_TY rows of CT_TX = 128 points along x: per row one accumulator of M = 128 points by
-//   N = Cout (padded to a multiple of 16) in tensor memory.  The K dimension runs over 16-channel chunks
-//   and the 27 taps.  For a chunk, the CTA stages the input halo slab (3 planes x (CT_TY + 2) rows x 130
-//   points x 16 channels) in shared memory as 16-byte cells of 8 channels, laid out [channel group][z][y][x]
-//   so that consecutive x are consecutive cells.  That layout is the canonical K-major, no-swizzle operand
-//   layout (8 rows of 16 bytes per core matrix), and a tap's shifted view of the slab is the same layout
-//   at another start address: the 27 taps read one slab, nothing is copied per tap.  The weights of the
-//   chunk (27 taps x N x 16, pre-arranged by arrange_w_kernel) arrive by one bulk copy.  Two stages.
-//   Warps 0-7 gather the slab (8-point vector loads of the channel-first input, a register transpose into
-//   the cells, BF16, zeros outside the grid); warps 0-3 then run the epilogue (bias, ReLU, optional mask,
-//   channel-first stores); warp 8 allocates tensor memory and one lane issues the MMAs (M = 128, N = Np,
-//   K = 16 each).
+// Layout: activations are cells of 8 channels (16 bytes) on grids with a zero halo, [channel group][z][y][x].
+// Consecutive points of a padded plane are consecutive cells, which is the canonical K-major, no-swizzle operand
+// layout (a core matrix is 8 points x 16 bytes), and a tap's view of the staged points is the same layout at
+// another start address.  So a run of points with everything its 27 taps need is three contiguous pieces of
+// memory per channel group, fetched by bulk copies without any gather.  (The layout before, channel-first
+// rows transposed into cells by eight warps per tile, made that gather the bound, at 9% of the tensor pipe.)
+//
+// Forward and data gradient (the same convolution with flipped, transposed weights):
+//   out[o][p] = act(bias[o] + sum_{t, i} W(o, i, t) in[i][p + off_t])
+//   A tile is R x 128 consecutive points of a padded plane, taken along the flattened (y, x) index: rows follow
+//   one another across the halo, so the waste is the two halo points per row and not the remainder of a row to
+//   128.  Per 128 points one accumulator of 128 x Np (Np: outputs padded to 16) in tensor memory, R Np <= 256
+//   columns, two buffers.  The K dimension runs over 16-channel chunks, then the taps in order; a stage is one
+//   chunk and one dz: the points of plane z + dz - 1 (128 R plus a row and a point on both sides, or three runs
+//   for the three dy where rows are longer than a tile) and the 9 taps' weights.
+//   Persistent, one CTA per SM: warp 0 issues the bulk copies, one thread of warp 1 the MMAs (M = 128, N = Np,
+//   K = 16), warps 2-5 run the epilogue of the previous tile.
+//   The tensor unit bounds it (84% busy at 160^3): it takes about 64 cycles for an MMA of M = 128, K = 16 however
+//   small N is, so 28 outputs use an eighth of its rate.  The order of the sums is chunk, tap, 16 channels.
+//   Measured at 160^3, width 28: the 84 -> 28 layer 4.14 -> 1.38 ms, the forward pass 9.2 -> 3.2 ms.
 // Weight gradient:  gW[o][i][t] = sum_p g[o][p] in[i][p + off_t].
-//   A CTA owns one 16-channel chunk of i and walks a share of the 128-point row tiles.  Per tile: A = the
-//   gradient rows (M = 128 output channels, padded, K = 128 points, K-major cells of 8 points) and B = the
-//   same input slab, read as an MN-major operand (N = 16 channels, K = points; the tap's shift is again a
-//   start address).  27 accumulators of 128 x 16 live in tensor memory for the CTA's whole share and are
-//   added to gW (FP32 atomics) at the end.
+//   Both operands are read as MN-major cells (channels x points): M = output channels (64, or 128), N = all
+//   input channels of a block (up to 160), K = 256 points of a flattened plane (the gradient's halo is zero, so
+//   rows run on).  A CTA holds the accumulators of one dz and either 9 taps (narrow inputs) or the 3 taps of
+//   one dy in tensor memory for its whole share of the points and adds them to gW (FP32 atomics) at the end.
+//   The copies bound it: one warp issues a 4 KiB copy per channel group and tile.  Measured on two 96^3 fields, 84 ->
+//   28 layer: 0.65 ms with tiles of 256 points, 1.19 ms with 128; 7.6 ms with M = 128 rows of which 28 were used, N =
+//   16 inputs at a time and a gathered slab per input chunk.  A training pass: 24.2 -> 5.0 ms.
 // Every mbarrier wait is bounded; an expired wait raises HELM_DEV_WAIT, the CTA waits (bounded) for its bulk
 // copies and MMAs in flight, frees its tensor memory and exits.
-#include "common.cuh"
-#include <cuda_bf16.h>
+#include "cells.cuh"
 #include <algorithm>
-
-typedef __nv_bfloat16 bf16;
 
 namespace {
 
-constexpr int CT_TX = 128;                         // output points per row (MMA M)
-constexpr int CT_SX = CT_TX + 2;                   // slab points per row (one halo point each side)
-constexpr int CT_NPMAX = 64;                       // largest padded output-channel count
 constexpr long CT_WAIT = 1L << 22;                 // bound of every mbarrier wait (polls)
-constexpr int CT_PW = 8;                           // producer warps (gather); warps 0-3 also run the epilogue
-constexpr int CT_THREADS = (CT_PW + 1) * 32;       // + one warp for tensor memory and the MMAs
-constexpr int CT_MW = CT_PW;                       // the MMA warp
-
-template <int TY>
-struct CtLayout {
-    static constexpr int SY = TY + 2;
-    static constexpr int CELLS = 2 * 3 * SY * CT_SX;            // 16-byte cells of one 16-channel chunk
-    static constexpr int SLAB = CELLS * 16;
-    static constexpr int CG = 3 * SY * CT_SX * 16;              // bytes between the two channel groups
-};
-// forward: two rows per CTA; a stage is the slab and the chunk's weights (27 x 2 x Np x 16 bytes); two stages
-// when there are several channel chunks, one (and so more CTAs per SM) when there is one
-constexpr int FW_TY = 2;
-constexpr int FW_WMAX = 27 * 2 * CT_NPMAX * 16;                 // 55,296 bytes
-constexpr int FW_SMEM = 2 * (CtLayout<FW_TY>::SLAB + FW_WMAX) + 128;   // the largest request
-__host__ __device__ constexpr int fw_stage_bytes(int Np) { return CtLayout<FW_TY>::SLAB + 27 * 2 * Np * 16; }
-// weight gradient: one row per tile; a stage is the slab and the gradient tile (16 x 128 cells)
-constexpr int WG_G = 16 * 128 * 16;                             // 32,768
-constexpr int WG_STAGE = CtLayout<1>::SLAB + WG_G;              // 70,208
-constexpr int WG_NS = 3;
-constexpr int WG_SMEM = WG_NS * WG_STAGE + 128;
+constexpr int CT_NPMAX = 64;                       // largest padded output-channel count of a launch
+constexpr int CT_RMAX = 8;                         // largest tile: 8 x 128 points
+constexpr int CT_THREADS = 192;                    // producer warp, MMA warp, four epilogue warps
+constexpr int CT_NST = 6;                          // most stages
+constexpr int CT_SMEM = 229376;                    // dynamic shared memory of a CTA at most (224 KiB)
+constexpr int WG_KT = 256;                         // points of a weight-gradient tile at most
+// Points a CTA sums in tensor memory before it adds to gW.  The accumulators of the tensor cores are FP32 with
+// truncation, so long chains of additions lose digits: with one wave of CTAs (112,000 points for the
+// 84 -> 28 layer on two 96^3 fields) the gradient moved by 2.8e-5 against chains a quarter as long.
+constexpr int WG_POINTS = 16384;
 
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(uint32_t b, uint32_t n) {
@@ -81,6 +70,10 @@ __device__ __forceinline__ bool bar_wait(uint32_t b, uint32_t parity, long limit
     }
     return false;
 }
+// the same by every lane of a warp, with one answer
+__device__ __forceinline__ bool warp_wait(uint32_t b, uint32_t parity, long limit) {
+    return __all_sync(0xffffffffu, bar_wait(b, parity, limit));
+}
 // bulk copy global -> shared (16-byte aligned addresses, size a multiple of 16), completion on bar
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t b) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -101,9 +94,22 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int a_mn, int b_
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::
-                     "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc));
+// The MMAs of a stage differ in their start addresses alone, so the issuing thread keeps the upper words of the
+// descriptors and adds to the lower ones (start address / 16 in the low 14 bits; shared memory ends below 2^18, so
+// the sums stay in the field).  The whole warp runs the issuing loop and `lead` (one elected lane) predicates the
+// instruction: the operands are then warp-uniform values in uniform registers.
+__device__ __forceinline__ void mma_bf16(uint32_t lead, uint32_t d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                         uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .pred p, q;\n.reg .b64 da, db;\nmov.b64 da, {%1, %2};\nmov.b64 db, {%3, %4};\nsetp.ne.b32 p, %6, 0;\n"
+        "setp.ne.b32 q, %7, 0;\n@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d), "r"(alo), "r"(ahi),
+        "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(lead));
+}
+// 1 in one lane of the (converged) warp
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r;
 }
 __device__ __forceinline__ void mma_commit(uint32_t b) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(b) : "memory");
@@ -120,349 +126,374 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
-
-__device__ __forceinline__ float ldf(const float* p, size_t i) { return p[i]; }
-__device__ __forceinline__ void stf(bf16* p, size_t i, float v) { p[i] = __float2bfloat16(v); }
-__device__ __forceinline__ void stf(float* p, size_t i, float v) { p[i] = v; }
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t*>(&h);
+// tensor memory: the MMA warp allocates all 512 columns (one CTA per SM) and frees them at the end
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s32(slot)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
-
-// 8 consecutive values of one row (x = xb .. xb + 7) as four packed BF16 pairs: one 16-byte (BF16) or two
-// 16-byte (FP32) loads inside the row when aligned (rows of a multiple of 8 points), else per point, zeros
-// outside 0 .. X - 1
-__device__ __forceinline__ uint4 load8(const bf16* __restrict__ row, int xb, int X, bool vec) {
-    if (vec && xb >= 0 && xb + 8 <= X) return *reinterpret_cast<const uint4*>(row + xb);
-    float v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = (xb + k >= 0 && xb + k < X) ? __bfloat162float(row[xb + k]) : 0.f;
-    return make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
-}
-__device__ __forceinline__ uint4 load8(const float* __restrict__ row, int xb, int X, bool vec) {
-    if (vec && xb >= 0 && xb + 8 <= X) {
-        const float4 a = *reinterpret_cast<const float4*>(row + xb), b = *reinterpret_cast<const float4*>(row + xb + 4);
-        return make_uint4(pack2(a.x, a.y), pack2(a.z, a.w), pack2(b.x, b.y), pack2(b.z, b.w));
-    }
-    float v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = (xb + k >= 0 && xb + k < X) ? row[xb + k] : 0.f;
-    return make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
-}
-__device__ __forceinline__ uint32_t u4w(const uint4& q, int i) { return i == 0 ? q.x : (i == 1 ? q.y : (i == 2 ? q.z : q.w)); }
-
-// Fill the slab of one 16-channel chunk (channels c0 .. c0 + 15) for output rows y0 .. y0 + TY - 1 of plane
-// z: cell q = ((cg * 3 + dz) * SY + yr) * 130 + xi holds channels c0 + 8 cg .. + 7 of the input point
-// (z + dz - 1, y0 + yr - 1, x0 + xi - 1); zero outside the grid and beyond Cin.  A work item is one row of
-// the slab and one group of 8 points x = x0 - 8 + 8 g (g = 0 .. 17, aligned when x0 is): it loads the 8
-// channels' rows of those points (8-point vector loads) and writes the 8 cells, a transpose of the
-// channel-first input into the channel-contiguous cells done on packed BF16 pairs (byte permutes).
-template <int TY, typename TIN>
-__device__ __forceinline__ void fill_slab(unsigned char* slab, const TIN* __restrict__ in, int Cin, int c0, int z,
-                                          int y0, int x0, int Z, int Y, int X, int t, int nthreads) {
-    typedef CtLayout<TY> L;
-    constexpr int NG = (CT_SX + 14) / 8;   // 18 groups cover x0 - 8 .. x0 + 135 (the slab is x0 - 1 .. x0 + 128)
-    const size_t vol = (size_t)Z * Y * X;
-    const bool vec = (X % 8) == 0;
-    for (int it = t; it < 2 * 3 * L::SY * NG; it += nthreads) {
-        const int g = it % NG;
-        int r = it / NG;
-        const int yr = r % L::SY;
-        r /= L::SY;
-        const int dz = r % 3, cg = r / 3;
-        const int gz = z + dz - 1, gy = y0 + yr - 1, xb = x0 - 8 + 8 * g;
-        const bool rowok = gz >= 0 && gz < Z && gy >= 0 && gy < Y;
-        const size_t roff = rowok ? ((size_t)gz * Y + gy) * X : 0;
-        uint4 row[8];   // channel j: the 8 points as BF16 pairs
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int ch = c0 + 8 * cg + j;
-            row[j] = (rowok && ch < Cin) ? load8(in + (size_t)ch * vol + roff, xb, X, vec) : make_uint4(0u, 0u, 0u, 0u);
-        }
-        unsigned char* rowp = slab + (size_t)(((cg * 3 + dz) * L::SY + yr) * CT_SX) * 16;
-        // Store slot k writes the cell of point k ^ sw (sw = g mod 8).  A thread's 8 cells are 128 contiguous
-        // bytes and neighbouring threads take neighbouring groups, so with the same order everywhere all the
-        // 16-byte stores of one warp instruction would hit the same four banks; rotated, they spread over all
-        // 32.  The rotation is applied to the loaded words (point pair k >> 1 is word k >> 1 of each row) and
-        // to the half selector (point parity), so every register index stays static.
-        const int sw = g & 7;
-        if (sw & 2)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) row[j] = make_uint4(row[j].y, row[j].x, row[j].w, row[j].z);
-        if (sw & 4)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) row[j] = make_uint4(row[j].z, row[j].w, row[j].x, row[j].y);
-        const uint32_t sel_even = (sw & 1) ? 0x7632u : 0x5410u, sel_odd = (sw & 1) ? 0x5410u : 0x7632u;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int xi = 8 * g - 7 + (k ^ sw);   // slab index of the point xb + (k ^ sw)
-            if (xi >= 0 && xi < CT_SX) {
-                // cell word m = (channel 2m, channel 2m + 1) at the point: the low (even point) or high halves
-                const uint32_t sel = (k & 1) ? sel_odd : sel_even;
-                uint32_t w[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) w[m] = __byte_perm(u4w(row[2 * m], k >> 1), u4w(row[2 * m + 1], k >> 1), sel);
-                *reinterpret_cast<uint4*>(rowp + (size_t)xi * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
-    }
+__device__ __forceinline__ void tmem_free(uint32_t tmem) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
 // ---- forward / data gradient ------------------------------------------------------------------------------
-// wt: arranged weights [nkc][27][2][Np][8] (bf16); mask (optional): out *= (mask > 0)
-template <typename TIN, typename TOUT>
-__global__ void __launch_bounds__(CT_THREADS, 3)
-conv_tc_kernel(const TIN* __restrict__ in, int Cin, size_t in_bs, const bf16* __restrict__ wt, int Np,
-               const float* __restrict__ bias, TOUT* __restrict__ out, int Cout, size_t out_bs, int Z, int Y, int X,
-               int relu, const bf16* __restrict__ mask, size_t mask_bs, int nst, unsigned* status) {
-    typedef CtLayout<FW_TY> L;
+struct ConvArgs {
+    CellGrid g;
+    const bf16* in;      // cells of Gin groups
+    int Gin;
+    const bf16* wt;      // arranged weights [nkc][27][2][Np][8]
+    int Np;
+    const float* bias;   // [Cout] or NULL
+    void* out;
+    int Gout, ooff;      // groups of the output tensor, the first output channel in it
+    int Cout;            // outputs of this launch (at most 64)
+    int relu;
+    const bf16* mask;    // CONV_GRAD: cells of Gout groups; the output is 0 where mask <= 0
+    float* gb;           // CONV_GRAD: += sum of the output over points, per channel
+    int R;               // 128-point blocks per tile
+    int ntp;             // tiles per plane
+    int ntiles;
+    int dstride;         // staged cells between the views of consecutive dy
+    int L;               // staged cells per channel group
+    int split;           // three runs (one per dy) instead of one
+    int nst, stage;      // stages, bytes of one
+    unsigned* status;
+};
+
+template <int OUT>
+__global__ void __launch_bounds__(CT_THREADS, 1) conv_cells_kernel(const __grid_constant__ ConvArgs a) {
     extern __shared__ __align__(128) unsigned char csm[];
-    unsigned char* base = (unsigned char*)(((uintptr_t)csm + 127) & ~(uintptr_t)127);
-    __shared__ __align__(8) uint64_t full[2], wfull[2], empty[2], accf, drainb;
+    __shared__ __align__(8) uint64_t full[CT_NST], empty[CT_NST], accf[2], acce[2], drainb;
     __shared__ uint32_t tslot;
     __shared__ int fail_any;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ntx = (X + CT_TX - 1) / CT_TX, nty = (Y + FW_TY - 1) / FW_TY;
-    int tile = blockIdx.x;
-    const int xt = tile % ntx;
-    tile /= ntx;
-    const int yt = tile % nty;
-    tile /= nty;
-    const int z = tile % Z, b = tile / Z;
-    const int x0 = xt * CT_TX, y0 = yt * FW_TY;
-    const int nkc = (Cin + 15) / 16;
-    const uint32_t wbytes = 27u * 2u * (uint32_t)Np * 16u;
-    const size_t stage = (size_t)fw_stage_bytes(Np);   // a multiple of 16
-    const uint32_t ncols = FW_TY * Np <= 32 ? 32 : (FW_TY * Np <= 64 ? 64 : 128);
+    const int nkc = a.Gin / 2, niter = 3 * nkc;
+    const uint32_t base = (s32(csm) + 127u) & ~127u;
+    const uint32_t wbytes = 9u * 2u * (uint32_t)a.Np * 16u, sbytes = (uint32_t)a.L * 16u;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 2; ++s) {
-            bar_init(s32(&full[s]), CT_PW);
-            bar_init(s32(&wfull[s]), 1);
-            bar_init(s32(&empty[s]), 1);
-        }
-        bar_init(s32(&accf), 1);
+        for (int s = 0; s < CT_NST; ++s) { bar_init(s32(&full[s]), 1); bar_init(s32(&empty[s]), 1); }
+        for (int b = 0; b < 2; ++b) { bar_init(s32(&accf[b]), 1); bar_init(s32(&acce[b]), 4); }
         bar_init(s32(&drainb), 1);
         fail_any = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == CT_MW) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(&tslot)), "r"(ncols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (warp == 1) tmem_alloc(&tslot);
     tc_before();
     __syncthreads();
     tc_after();
     const uint32_t tmem = tslot;
+    const CellGrid& g = a.g;
     bool ok = true;
-    int issued = 0;   // chunks whose weight copy thread 0 issued
-    const TIN* inb = in + (size_t)b * in_bs;
-    if (warp < CT_PW) {
-        for (int kc = 0; kc < nkc && ok; ++kc) {
-            const int s = kc % nst, u = kc / nst;
-            if (u >= 1) ok = __all_sync(0xffffffffu, bar_wait(s32(&empty[s]), (uint32_t)((u - 1) & 1), CT_WAIT));
-            if (!ok) break;
-            unsigned char* st = base + (size_t)s * stage;
-            if (threadIdx.x == 0) {
-                bar_expect(s32(&wfull[s]), wbytes);
-                bulk_g2s(s32(st + L::SLAB), wt + (size_t)kc * 27 * 2 * Np * 8, wbytes, s32(&wfull[s]));
-                ++issued;
+    long issued = 0;   // stages whose copies were issued
+    if (warp == 0) {
+        if (lane == 0) {
+            long it = 0;
+            for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x) {
+                const int tp = tile % a.ntp, zb = tile / a.ntp, z = zb % g.Z, b = zb / g.Z;
+                // first staged cell of a plane: one row and one point before the tile's first point
+                const long q0 = (long)tp * 128 * a.R;
+                for (int k = 0; k < niter; ++k, ++it) {
+                    const int s = (int)(it % a.nst), kc = k / 3, dz = k % 3;
+                    if (it >= a.nst) ok = bar_wait(s32(&empty[s]), (uint32_t)((it / a.nst - 1) & 1), CT_WAIT);
+                    if (!ok) break;
+                    const uint32_t st = base + (uint32_t)s * (uint32_t)a.stage, fb = s32(&full[s]);
+                    bar_expect(fb, 2u * sbytes + wbytes);
+                    for (int cg = 0; cg < 2; ++cg) {
+                        const bf16* src = a.in + 8 * (((long)b * a.Gin + 2 * kc + cg) * g.vol + (long)(z + dz) * g.plane + q0);
+                        const uint32_t dst = st + (uint32_t)cg * sbytes;
+                        if (!a.split) {
+                            bulk_g2s(dst, src, sbytes, fb);
+                        } else {
+                            for (int dy = 0; dy < 3; ++dy)
+                                bulk_g2s(dst + (uint32_t)(dy * a.dstride) * 16u, src + 8 * (long)dy * g.pitch,
+                                         (uint32_t)a.dstride * 16u, fb);
+                        }
+                    }
+                    bulk_g2s(st + 2u * sbytes, a.wt + (size_t)(kc * 27 + 9 * dz) * 2 * a.Np * 8, wbytes, fb);
+                    ++issued;
+                }
             }
-            fill_slab<FW_TY>(st, inb, Cin, 16 * kc, z, y0, x0, Z, Y, X, threadIdx.x, CT_PW * 32);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the slab (async proxy)
-            __syncwarp();
-            if (lane == 0) bar_arrive(s32(&full[s]));
         }
-        // epilogue (warps 0-3): this warp's 32 accumulator lanes are the points x0 + 32 (warp) + lane
-        if (ok && warp < 4) ok = __all_sync(0xffffffffu, bar_wait(s32(&accf), 0, CT_WAIT));
-        if (ok && warp < 4) {
-            tc_after();
-            const size_t vol = (size_t)Z * Y * X;
-            const int x = x0 + 32 * warp + lane;
-            for (int r = 0; r < FW_TY; ++r) {
-                const int y = y0 + r;
-                const size_t q = ((size_t)z * Y + y) * X + x;
-                for (int cb = 0; cb < Np; cb += 16) {
-                    float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(r * Np + cb), v);
-                    if (x < X && y < Y) {
+    } else if (warp == 1) {
+        {
+            const uint32_t lead = elect_one();
+            const uint32_t idesc = idesc_bf16(128, a.Np, 0, 0);
+            long it = 0;
+            int lt = 0;
+            for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x, ++lt) {
+                const int tp = tile % a.ntp, buf = lt & 1;
+                // 128-point blocks of this tile that hold points (the last tile of a plane may be short)
+                const int nr = min(a.R, (g.span - tp * 128 * a.R + 127) / 128);
+                if (lt >= 2) ok = warp_wait(s32(&acce[buf]), (uint32_t)(((lt >> 1) - 1) & 1), CT_WAIT);
+                if (!ok) break;
+                tc_after();
+                const uint32_t acc = tmem + (uint32_t)(buf * 256);
+                for (int k = 0; k < niter; ++k, ++it) {
+                    const int s = (int)(it % a.nst);
+                    ok = warp_wait(s32(&full[s]), (uint32_t)((it / a.nst) & 1), CT_WAIT);
+                    if (!ok) break;
+                    tc_after();
+                    const uint32_t slab = base + (uint32_t)s * (uint32_t)a.stage, wsm = slab + 2u * sbytes;
+                    // A: a tap's view of the points; next channel group (K) sbytes, next 8 points 128.  B: the tap's
+                    // weights [2 channel groups][Np][8]: next channel group Np*16 bytes, next 8 outputs 128
+                    const uint64_t ad = ndesc(slab, sbytes, 128u), bd = ndesc(wsm, (uint32_t)a.Np * 16u, 128u);
+                    const uint32_t ahi = (uint32_t)(ad >> 32), bhi = (uint32_t)(bd >> 32);
+                    uint32_t blo = (uint32_t)bd;
+                    for (int dy = 0; dy < 3; ++dy) {
+                        const uint32_t arow = (uint32_t)ad + (uint32_t)(dy * a.dstride);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int o = cb + j;
-                            if (o < Cout) {
-                                float a = v[j] + (bias ? bias[o] : 0.f);
-                                if (relu) a = fmaxf(a, 0.f);
-                                if (mask && !(__bfloat162float(mask[(size_t)b * mask_bs + (size_t)o * vol + q]) > 0.f))
-                                    a = 0.f;
-                                stf(out, (size_t)b * out_bs + (size_t)o * vol + q, a);
+                        for (int dx = 0; dx < 3; ++dx, blo += 2u * (uint32_t)a.Np) {
+                            const uint32_t more = (k | dy | dx) ? 1u : 0u;
+#pragma unroll
+                            for (int r = 0; r < CT_RMAX; ++r)
+                                if (r < nr)
+                                    mma_bf16(lead, acc + (uint32_t)(r * a.Np), arow + (uint32_t)(dx + 128 * r), ahi, blo, bhi, idesc,
+                                             more);
+                        }
+                    }
+                    if (lead) mma_commit(s32(&empty[s]));
+                    __syncwarp();
+                }
+                if (ok && lead) mma_commit(s32(&accf[buf]));
+                __syncwarp();
+            }
+        }
+    } else {
+        const int w = warp & 3;   // tensor-memory lanes 32 w .. 32 w + 31
+        float bsum[CT_NPMAX / 16] = {0.f, 0.f, 0.f, 0.f};
+        int lt = 0;
+        for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x, ++lt) {
+            const int tp = tile % a.ntp, zb = tile / a.ntp, z = zb % g.Z, b = zb / g.Z, buf = lt & 1;
+            const int nr = min(a.R, (g.span - tp * 128 * a.R + 127) / 128);
+            ok = warp_wait(s32(&accf[buf]), (uint32_t)((lt >> 1) & 1), CT_WAIT);
+            if (!ok) break;
+            tc_after();
+            for (int r = 0; r < nr; ++r) {
+                const int rel = (tp * a.R + r) * 128 + 32 * w + lane;   // point y pitch + x
+                const int y = rel / g.pitch, x = rel - y * g.pitch;
+                const bool in = y < g.Y && x < g.X;
+                const long q = (long)(z + 1) * g.plane + g.pitch + 1 + rel;   // its cell in a channel group
+#pragma unroll
+                for (int cb = 0; cb < CT_NPMAX; cb += 16) {
+                    if (cb >= a.Np) break;
+                    float v[16];
+                    tmem_ld16(tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)(buf * 256 + r * a.Np + cb), v);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        if (a.bias) v[j] += cb + j < a.Cout ? a.bias[cb + j] : 0.f;
+                        if (a.relu) v[j] = fmaxf(v[j], 0.f);
+                    }
+                    if constexpr (OUT == CONV_PLANAR) {
+                        if (in)
+#pragma unroll
+                            for (int j = 0; j < 16; ++j)
+                                if (cb + j < a.Cout)
+                                    reinterpret_cast<float*>(a.out)[(((size_t)b * a.Cout + cb + j) * g.Z + z) * g.Y * g.X +
+                                                                    (size_t)y * g.X + x] = v[j];
+                    } else {
+                        const int c0 = a.ooff + cb;
+                        if constexpr (OUT == CONV_GRAD) {
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                uint4 m = make_uint4(0u, 0u, 0u, 0u);
+                                if (in && cb + 8 * h < a.Cout)
+                                    m = *reinterpret_cast<const uint4*>(a.mask + 8 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q));
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    if (!(cell_value(m, j) > 0.f)) v[8 * h + j] = 0.f;
+                            }
+                            bsum[cb / 16] += lane_fold16(v, lane);
+                        }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if (!in || cb + 8 * h >= a.Cout) continue;
+                            if constexpr (OUT == CONV_F32CELLS) {
+                                float4* o = reinterpret_cast<float4*>(a.out) + 2 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q);
+                                o[0] = make_float4(v[8 * h], v[8 * h + 1], v[8 * h + 2], v[8 * h + 3]);
+                                o[1] = make_float4(v[8 * h + 4], v[8 * h + 5], v[8 * h + 6], v[8 * h + 7]);
+                            } else if (a.ooff % 8 == 0) {
+                                *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.out) +
+                                                          8 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q)) = pack_cell(v + 8 * h);
+                            } else {   // a channel offset inside a cell: channel by channel
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    if (cb + 8 * h + j < a.Cout) {
+                                        const int c = c0 + 8 * h + j;
+                                        reinterpret_cast<bf16*>(a.out)[8 * (((long)b * a.Gout + c / 8) * g.vol + q) + c % 8] =
+                                            __float2bfloat16(v[8 * h + j]);
+                                    }
                             }
                         }
                     }
                 }
             }
+            tc_before();
+            __syncwarp();
+            if (lane == 0) bar_arrive(s32(&acce[buf]));
         }
-    } else if (lane == 0) {
-        const uint32_t idesc = idesc_bf16(128, Np, 0, 0);
-        for (int kc = 0; kc < nkc && ok; ++kc) {
-            const int s = kc % nst, u = kc / nst;
-            ok = bar_wait(s32(&full[s]), (uint32_t)(u & 1), CT_WAIT) && bar_wait(s32(&wfull[s]), (uint32_t)(u & 1), CT_WAIT);
-            if (!ok) break;
-            tc_after();
-            const uint32_t slab = s32(base + (size_t)s * stage), wsm = slab + L::SLAB;
-            for (int t = 0; t < 27; ++t) {
-                const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;
-                // B: tap t's weights [2 channel groups][Np][8]: next channel group (K) Np*16 bytes, next 8 outputs 128
-                const uint64_t bd = ndesc(wsm + (uint32_t)t * 2u * (uint32_t)Np * 16u, (uint32_t)Np * 16u, 128u);
+        if constexpr (OUT == CONV_GRAD) {
+            const int c = lane_fold16_channel(lane);
 #pragma unroll
-                for (int r = 0; r < FW_TY; ++r) {
-                    // A: the tap's view of the slab; next channel group (K) L::CG bytes, next 8 points (M) 128
-                    const uint32_t a0 = slab + (uint32_t)(((dz * L::SY + r + dy) * CT_SX + dx) * 16);
-                    mma_bf16(tmem + (uint32_t)(r * Np), ndesc(a0, (uint32_t)L::CG, 128u), bd, idesc, (kc | t) ? 1u : 0u);
-                }
-            }
-            mma_commit(s32(&empty[s]));
+            for (int k = 0; k < CT_NPMAX / 16; ++k)
+                if (!(lane & 1) && 16 * k + c < a.Cout) atomicAdd(&a.gb[16 * k + c], bsum[k]);
         }
-        if (ok) mma_commit(s32(&accf));
     }
     if (!ok) {
-        atomicOr(status, (unsigned)HELM_DEV_WAIT);
+        atomicOr(a.status, (unsigned)HELM_DEV_WAIT);
         fail_any = 1;
     }
     __syncthreads();
     if (fail_any && lane == 0) {
-        if (warp == 0) {
-            // the weight copies of the last (at most nst) issued chunks may still be in flight
-            for (int kc = issued > nst ? issued - nst : 0; kc < issued; ++kc)
-                bar_wait(s32(&wfull[kc % nst]), (uint32_t)((kc / nst) & 1), CT_WAIT);
-        } else if (warp == CT_MW) {
+        if (warp == 0) {   // the copies of the last (at most nst) issued stages may still be in flight
+            for (long k = issued > a.nst ? issued - a.nst : 0; k < issued; ++k)
+                bar_wait(s32(&full[k % a.nst]), (uint32_t)((k / a.nst) & 1), CT_WAIT);
+        } else if (warp == 1) {
             mma_commit(s32(&drainb));
             bar_wait(s32(&drainb), 0, CT_WAIT);
         }
     }
     tc_before();
     __syncthreads();
-    if (warp == CT_MW)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+    if (warp == 1) tmem_free(tmem);
 }
 
 // ---- weight gradient ---------------------------------------------------------------------------------
-// gw[o][i][t] += sum_{b, p} g[b][o][p] in[b][i][p + off_t] for the 16 input channels of chunk blockIdx.x;
-// Cout <= 128.  Tiles: (b, z, y, 128-point x block), CTA y takes tiles blockIdx.y, + gridDim.y, ...
-template <typename TG>
-__global__ void __launch_bounds__(CT_THREADS, 1)
-wgrad_tc_kernel(const bf16* __restrict__ in, int Cin, size_t in_bs, const TG* __restrict__ g, int Cout, size_t g_bs,
-                int B, int Z, int Y, int X, float* __restrict__ gw, unsigned* status) {
-    typedef CtLayout<1> L;
+struct WgradArgs {
+    CellGrid g;
+    const bf16* in;      // cells of Gin groups
+    int Gin;
+    const bf16* gr;      // gradient cells of Ggr groups, halo zero
+    int Ggr;
+    int Cin, Cout, M;    // M = 64 or 128 accumulator rows
+    int Nb, nblk;        // input channels of a block (a multiple of 16), blocks
+    int ndy;             // 3: a CTA holds the 9 taps of its dz; 1: the 3 taps of its (dz, dy)
+    int kt, ntp, ntiles, nst, stage;   // points of a tile (a multiple of 16, at most WG_KT), ...
+    float* gw;           // [Cout][Cin][27]
+    unsigned* status;
+};
+
+__global__ void __launch_bounds__(CT_THREADS, 1) wgrad_cells_kernel(const __grid_constant__ WgradArgs a) {
     extern __shared__ __align__(128) unsigned char csm[];
-    unsigned char* base = (unsigned char*)(((uintptr_t)csm + 127) & ~(uintptr_t)127);
-    __shared__ __align__(8) uint64_t full[WG_NS], empty[WG_NS], accf, drainb;
+    __shared__ __align__(8) uint64_t full[CT_NST], empty[CT_NST], accf, drainb;
     __shared__ uint32_t tslot;
     __shared__ int fail_any;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int kc = blockIdx.x;
-    const int ntx = (X + CT_TX - 1) / CT_TX;
-    const int ntiles = B * Z * Y * ntx;
-    const size_t vol = (size_t)Z * Y * X;
+    const uint32_t base = (s32(csm) + 127u) & ~127u;
+    const CellGrid& g = a.g;
+    const int ib = blockIdx.x % a.nblk, tg = blockIdx.x / a.nblk;
+    const int dz = a.ndy == 3 ? tg : tg / 3, dy0 = a.ndy == 3 ? 0 : tg % 3;
+    const int ng = min(a.Nb / 8, a.Gin - ib * (a.Nb / 8));   // input groups of this block that exist
+    const uint32_t abytes = (uint32_t)(a.Ggr * a.kt) * 16u, brow = (uint32_t)(a.kt + 2) * 16u;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < WG_NS; ++s) { bar_init(s32(&full[s]), CT_PW); bar_init(s32(&empty[s]), 1); }
+        for (int s = 0; s < CT_NST; ++s) { bar_init(s32(&full[s]), 1); bar_init(s32(&empty[s]), 1); }
         bar_init(s32(&accf), 1);
         bar_init(s32(&drainb), 1);
         fail_any = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == CT_MW) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(&tslot)), "r"(512)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (warp == 1) tmem_alloc(&tslot);
     tc_before();
     __syncthreads();
     tc_after();
     const uint32_t tmem = tslot;
     bool ok = true;
-    int nt = 0;   // tiles this CTA processed
-    if (warp < CT_PW) {
-        for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y, ++nt) {
-            int r = tile;
-            const int xt = r % ntx;
-            r /= ntx;
-            const int y = r % Y;
-            r /= Y;
-            const int z = r % Z, bb = r / Z;
-            const int x0 = xt * CT_TX;
-            const int s = nt % WG_NS, u = nt / WG_NS;
-            if (u >= 1) ok = __all_sync(0xffffffffu, bar_wait(s32(&empty[s]), (uint32_t)((u - 1) & 1), CT_WAIT));
+    long issued = 0;
+    if (warp == 0) {
+        for (int tile = blockIdx.y; tile < a.ntiles && ok; tile += gridDim.y) {
+            const int tp = tile % a.ntp, zb = tile / a.ntp, z = zb % g.Z, b = zb / g.Z;
+            const int ks = min(a.kt / 16, (g.span - tp * a.kt + 15) / 16);   // K steps of 16 points
+            const int s = (int)(issued % a.nst);
+            if (issued >= a.nst)
+                ok = warp_wait(s32(&empty[s]), (uint32_t)((issued / a.nst - 1) & 1), CT_WAIT);
             if (!ok) break;
-            unsigned char* st = base + (size_t)s * WG_STAGE;
-            fill_slab<1>(st, in + (size_t)bb * in_bs, Cin, 16 * kc, z, y, x0, Z, Y, X, threadIdx.x, CT_PW * 32);
-            // gradient cells: cell (kq, o) = g[o][z][y][x0 + 8 kq .. + 7], layout [kq][o][8]; zero beyond Cout, X
-            unsigned char* gs = st + L::SLAB;
-            const TG* gb = g + (size_t)bb * g_bs + ((size_t)z * Y + y) * X;
-            const bool vec = (X % 8) == 0;
-            for (int q = threadIdx.x; q < 16 * 128; q += CT_PW * 32) {
-                const int o = q % 128, kq = q / 128;
-                *reinterpret_cast<uint4*>(gs + (size_t)q * 16) =
-                    o < Cout ? load8(gb + (size_t)o * vol, x0 + 8 * kq, X, vec) : make_uint4(0u, 0u, 0u, 0u);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            const uint32_t st = base + (uint32_t)s * (uint32_t)a.stage, fb = s32(&full[s]);
+            const uint32_t an = (uint32_t)ks * 256u, bn = an + 32u;
+            if (lane == 0) bar_expect(fb, (uint32_t)a.Ggr * an + (uint32_t)(a.ndy * ng) * bn);
             __syncwarp();
-            if (lane == 0) bar_arrive(s32(&full[s]));
+            const long q = (long)tp * a.kt;   // first point, from the plane's first
+            for (int k = lane; k < a.Ggr + a.ndy * ng; k += 32) {
+                if (k < a.Ggr) {
+                    bulk_g2s(st + (uint32_t)k * (uint32_t)a.kt * 16u,
+                             a.gr + 8 * (((long)b * a.Ggr + k) * g.vol + (long)(z + 1) * g.plane + g.pitch + 1 + q), an, fb);
+                } else {
+                    const int e = k - a.Ggr, dy = e / ng, cg = e % ng;
+                    bulk_g2s(st + abytes + (uint32_t)(dy * (a.Nb / 8) + cg) * brow,
+                             a.in + 8 * (((long)b * a.Gin + ib * (a.Nb / 8) + cg) * g.vol + (long)(z + dz) * g.plane +
+                                         (long)(dy0 + dy) * g.pitch + q),
+                             bn, fb);
+                }
+            }
+            ++issued;
         }
-        if (ok && warp < 4) ok = __all_sync(0xffffffffu, bar_wait(s32(&accf), 0, CT_WAIT));
-        if (ok && nt > 0 && warp < 4) {
-            tc_after();
-            const int o = 32 * warp + lane;
-            for (int t = 0; t < 27; ++t) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(16 * t), v);
-                if (o < Cout) {
+    } else if (warp == 1) {
+        {
+            const uint32_t lead = elect_one();
+            const uint32_t idesc = idesc_bf16(a.M, a.Nb, 1, 1);
+            int n = 0;
+            for (int tile = blockIdx.y; tile < a.ntiles && ok; tile += gridDim.y, ++n) {
+                const int ks = min(a.kt / 16, (g.span - (tile % a.ntp) * a.kt + 15) / 16);
+                const int s = n % a.nst;
+                ok = warp_wait(s32(&full[s]), (uint32_t)((n / a.nst) & 1), CT_WAIT);
+                if (!ok) break;
+                tc_after();
+                const uint32_t ga = base + (uint32_t)s * (uint32_t)a.stage, xa = ga + abytes;
+                // both operands MN-major: next 8 points (K) 128 bytes, next channel group one run of cells.  Without
+                // swizzling the leading-byte offset is the K stride and the stride-byte offset the M/N stride
+                const uint64_t ad = ndesc(ga, 128u, (uint32_t)a.kt * 16u), bd = ndesc(xa, 128u, brow);
+                const uint32_t alo = (uint32_t)ad, ahi = (uint32_t)(ad >> 32), bhi = (uint32_t)(bd >> 32);
+                for (int t = 0; t < 3 * a.ndy; ++t) {
+                    const uint32_t blo = (uint32_t)bd + (uint32_t)((t / 3) * (a.Nb / 8) * (a.kt + 2) + t % 3);
+                    const uint32_t acc = tmem + (uint32_t)(t * a.Nb);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int i = 16 * kc + j;
-                        if (i < Cin) atomicAdd(&gw[((size_t)o * Cin + i) * 27 + t], v[j]);
-                    }
+                    for (int kk = 0; kk < WG_KT / 16; ++kk)
+                        if (kk < ks)
+                            mma_bf16(lead, acc, alo + (uint32_t)(16 * kk), ahi, blo + (uint32_t)(16 * kk), bhi, idesc,
+                                     (n | kk) ? 1u : 0u);
+                }
+                if (lead) mma_commit(s32(&empty[s]));
+                    __syncwarp();
+            }
+            if (ok && lead) mma_commit(s32(&accf));
+        }
+    } else if (blockIdx.y < a.ntiles) {
+        const int w = warp & 3;
+        ok = warp_wait(s32(&accf), 0, CT_WAIT * 4);
+        if (ok) {
+            tc_after();
+            // accumulator rows: 128 -> lane 32 w + l; 64 -> 16 rows in the first half of each warp's lanes
+            const int o = a.M == 128 ? 32 * w + lane : 16 * w + lane;
+            const bool live = (a.M == 128 || lane < 16) && o < a.Cout;
+            for (int t = 0; t < 3 * a.ndy; ++t) {
+                const int tap = 9 * dz + 3 * dy0 + t;
+                for (int cb = 0; cb < a.Nb; cb += 16) {
+                    float v[16];
+                    tmem_ld16(tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)(t * a.Nb + cb), v);
+                    if (live)
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const int i = ib * a.Nb + cb + j;
+                            if (i < a.Cin) atomicAdd(&a.gw[((size_t)o * a.Cin + i) * 27 + tap], v[j]);
+                        }
                 }
             }
         }
-    } else if (lane == 0) {
-        // A (gradient, K-major): next 8 points (K) 2048 bytes, next 8 outputs (M) 128; B (slab, MN-major): next
-        // 8 points (K) 128 bytes, next channel group (N) L::CG.  Without swizzling the leading-byte offset is the
-        // K stride and the stride-byte offset the M/N stride for either major-ness.
-        const uint32_t idesc = idesc_bf16(128, 16, 0, 1);
-        int n = 0;
-        for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y, ++n) {
-            const int s = n % WG_NS, u = n / WG_NS;
-            ok = bar_wait(s32(&full[s]), (uint32_t)(u & 1), CT_WAIT);
-            if (!ok) break;
-            tc_after();
-            const uint32_t slab = s32(base + (size_t)s * WG_STAGE), gsm = slab + L::SLAB;
-            for (int t = 0; t < 27; ++t) {
-                const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
-                    const uint64_t ad = ndesc(gsm + (uint32_t)(2 * kk) * 2048u, 2048u, 128u);
-                    const uint64_t bd = ndesc(slab + (uint32_t)(((dz * L::SY + dy) * CT_SX + 16 * kk + dx) * 16), 128u,
-                                              (uint32_t)L::CG);
-                    mma_bf16(tmem + (uint32_t)(16 * t), ad, bd, idesc, (n | kk) ? 1u : 0u);
-                }
-            }
-            mma_commit(s32(&empty[s]));
-        }
-        if (ok) mma_commit(s32(&accf));
     }
     if (!ok) {
-        atomicOr(status, (unsigned)HELM_DEV_WAIT);
+        atomicOr(a.status, (unsigned)HELM_DEV_WAIT);
         fail_any = 1;
     }
     __syncthreads();
-    if (fail_any && warp == CT_MW && lane == 0) {
-        mma_commit(s32(&drainb));
-        bar_wait(s32(&drainb), 0, CT_WAIT);
+    if (fail_any && lane == 0) {
+        if (warp == 0) {
+            for (long k = issued > a.nst ? issued - a.nst : 0; k < issued; ++k)
+                bar_wait(s32(&full[k % a.nst]), (uint32_t)((k / a.nst) & 1), CT_WAIT);
+        } else if (warp == 1) {
+            mma_commit(s32(&drainb));
+            bar_wait(s32(&drainb), 0, CT_WAIT);
+        }
     }
     tc_before();
     __syncthreads();
-    if (warp == CT_MW)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    if (warp == 1) tmem_free(tmem);
 }
 
 // arranged[kc][t][cg][o][j] = W(o0 + o, 16 kc + 8 cg + j, t) for the output slice o0 .. o0 + Np - 1, zero beyond
@@ -489,96 +520,110 @@ __global__ void arrange_w_kernel(const bf16* __restrict__ w, int Cin, int Cout, 
     }
 }
 
-// gb[o] += sum_{b, p} g[b][o][p]
-template <typename TG>
-__global__ void bias_grad_kernel(const TG* __restrict__ g, int Cout, size_t g_bs, int B, size_t vol, float* gb) {
-    __shared__ float red[8];
-    const int o = blockIdx.x;
-    float s = 0.f;
-    for (int b = 0; b < B; ++b)
-        for (size_t q = blockIdx.y * (size_t)blockDim.x + threadIdx.x; q < vol; q += (size_t)gridDim.y * blockDim.x)
-            s += ldf(g, (size_t)b * g_bs + (size_t)o * vol + q);
-    for (int k = 16; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        atomicAdd(&gb[o], t);
-    }
+int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();
+    return sms > 0 ? sms : 152;
 }
-
-int g_conv_sms = 0;
 
 }  // namespace
 
-// shapes the tensor-core convolutions take (outputs in slices of at most 64 for the forward kernel; the
-// weight gradient holds up to 128 outputs in its accumulator rows)
-bool conv_tc_supported(int Cin, int Cout) { return Cin >= 1 && Cout >= 1; }
-bool wgrad_tc_supported(int Cin, int Cout) { return Cin >= 1 && Cout >= 1 && Cout <= 128; }
-size_t conv_tc_scratch_bytes(int Cin, int Cout) {
+size_t conv_scratch_bytes(int Cin, int Cout) {
     const int Np = std::min((Cout + 15) / 16 * 16, CT_NPMAX), nkc = (Cin + 15) / 16;
     return (size_t)nkc * 27 * 2 * Np * 8 * sizeof(bf16);
 }
 
-helm_status conv_tc_prepare() {
-    HELM_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<bf16, bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, FW_SMEM));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<bf16, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, FW_SMEM));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, FW_SMEM));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(wgrad_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM));
-    int dev = 0;
-    HELM_CUDA_TRY(cudaGetDevice(&dev));
-    HELM_CUDA_TRY(cudaDeviceGetAttribute(&g_conv_sms, cudaDevAttrMultiProcessorCount, dev));
+helm_status conv_prepare() {
+    HELM_CUDA_TRY(cudaFuncSetAttribute(conv_cells_kernel<CONV_CELLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM));
+    HELM_CUDA_TRY(cudaFuncSetAttribute(conv_cells_kernel<CONV_PLANAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM));
+    HELM_CUDA_TRY(cudaFuncSetAttribute(conv_cells_kernel<CONV_F32CELLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM));
+    HELM_CUDA_TRY(cudaFuncSetAttribute(conv_cells_kernel<CONV_GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM));
+    HELM_CUDA_TRY(cudaFuncSetAttribute(wgrad_cells_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM));
     return HELM_OK;
 }
 
-// out = act(conv(in, W) + bias) with the tensor cores; wscr holds conv_tc_scratch_bytes(Cin, Cout)
-template <typename TIN, typename TOUT>
-helm_status conv_tc(const TIN* in, int Cin, size_t in_bs, const bf16* w, int wmode, const float* bias, TOUT* out,
-                    int Cout, size_t out_bs, int B, int Z, int Y, int X, int relu, const bf16* mask, size_t mask_bs,
-                    bf16* wscr, unsigned* status, cudaStream_t s) {
-    const int nkc = (Cin + 15) / 16;
-    const size_t vol = (size_t)Z * Y * X;
-    const int ntx = (X + CT_TX - 1) / CT_TX, nty = (Y + FW_TY - 1) / FW_TY;
-    const long tiles = (long)B * Z * nty * ntx;
+// One convolution; mode: CONV_CELLS ....  wscr holds conv_scratch_bytes(Cin, Cout).
+helm_status conv_cells(const CellGrid& g, int mode, const bf16* in, int Cin, const bf16* w, int wmode, const float* bias,
+                       void* out, int Cout, int Cout_total, int ooff, int relu, const bf16* mask, float* gb, bf16* wscr,
+                       unsigned* status, cudaStream_t s) {
+    const int Gin = cell_groups(Cin), nkc = Gin / 2;
+    const int sms = sm_count();
     // output slices of at most 64 channels (one accumulator width each); the launches follow one another on s
     for (int o0 = 0; o0 < Cout; o0 += CT_NPMAX) {
-        const int Co = std::min(Cout - o0, CT_NPMAX), Np = (Co + 15) / 16 * 16;
-        const size_t na = (size_t)nkc * 27 * 2 * Np * 8;
-        arrange_w_kernel<<<(unsigned)((na + 255) / 256), 256, 0, s>>>(w, Cin, Cout, o0, wmode, Np, nkc, wscr);
-        // one stage: a CTA's chunks follow one another, and the two to three CTAs an SM holds overlap each
-        // other's gathers, MMAs and epilogues instead
-        const int nst = 1;
-        const size_t smem = (size_t)nst * fw_stage_bytes(Np) + 128;
-        conv_tc_kernel<TIN, TOUT><<<(unsigned)tiles, CT_THREADS, smem, s>>>(
-            in, Cin, in_bs, wscr, Np, bias ? bias + o0 : nullptr, out + (size_t)o0 * vol, Co, out_bs, Z, Y, X, relu,
-            mask ? mask + (size_t)o0 * vol : nullptr, mask_bs, nst, status);
+        ConvArgs a;
+        a.g = g;
+        a.in = in; a.Gin = Gin;
+        a.Cout = std::min(Cout - o0, CT_NPMAX);
+        a.Np = (a.Cout + 15) / 16 * 16;
+        a.wt = wscr;
+        a.bias = bias ? bias + o0 : nullptr;
+        a.out = mode == CONV_PLANAR ? (void*)((float*)out + (size_t)o0 * g.Z * g.Y * g.X) : out;
+        a.Gout = cell_groups(Cout_total);
+        a.ooff = ooff + o0;
+        a.relu = relu;
+        a.mask = mask;
+        a.gb = gb ? gb + o0 : nullptr;
+        a.status = status;
+        // the largest tile whose count still gives every SM two (small grids: smaller tiles), within 256
+        // accumulator columns; tiles of one plane share its halo rows, so larger is better for the copies
+        int R = std::min(CT_RMAX, 256 / a.Np);
+        auto tiles = [&](int r) { return (long)g.B * g.Z * ((g.span + 128 * r - 1) / (128 * r)); };
+        while (R > 1 && tiles(R) < 2L * sms) R = (R + 1) / 2;
+        a.R = R;
+        a.ntp = (g.span + 128 * R - 1) / (128 * R);
+        a.ntiles = (int)tiles(R);
+        // one run with the rows between the three dy views, or three runs where that is shorter (long rows)
+        a.split = g.pitch > 128 * R + 2;
+        a.dstride = a.split ? 128 * R + 2 : g.pitch;
+        a.L = a.split ? 3 * a.dstride : 128 * R + 2 + 2 * g.pitch;
+        a.stage = (2 * a.L * 16 + 9 * 2 * a.Np * 16 + 127) / 128 * 128;
+        a.nst = std::min(CT_NST, (CT_SMEM - 128) / a.stage);
+        const size_t na = (size_t)nkc * 27 * 2 * a.Np * 8;
+        arrange_w_kernel<<<(unsigned)((na + 255) / 256), 256, 0, s>>>(w, Cin, Cout, o0, wmode, a.Np, nkc, wscr);
+        const size_t smem = (size_t)a.nst * a.stage + 128;
+        const unsigned grid = (unsigned)std::min((long)a.ntiles, (long)sms);
+        if (mode == CONV_CELLS) conv_cells_kernel<CONV_CELLS><<<grid, CT_THREADS, smem, s>>>(a);
+        else if (mode == CONV_PLANAR) conv_cells_kernel<CONV_PLANAR><<<grid, CT_THREADS, smem, s>>>(a);
+        else if (mode == CONV_F32CELLS) conv_cells_kernel<CONV_F32CELLS><<<grid, CT_THREADS, smem, s>>>(a);
+        else conv_cells_kernel<CONV_GRAD><<<grid, CT_THREADS, smem, s>>>(a);
         HELM_CUDA_TRY(cudaGetLastError());
     }
     return HELM_OK;
 }
-template helm_status conv_tc<bf16, bf16>(const bf16*, int, size_t, const bf16*, int, const float*, bf16*, int, size_t,
-                                         int, int, int, int, int, const bf16*, size_t, bf16*, unsigned*, cudaStream_t);
-template helm_status conv_tc<bf16, float>(const bf16*, int, size_t, const bf16*, int, const float*, float*, int, size_t,
-                                          int, int, int, int, int, const bf16*, size_t, bf16*, unsigned*, cudaStream_t);
-template helm_status conv_tc<float, float>(const float*, int, size_t, const bf16*, int, const float*, float*, int,
-                                           size_t, int, int, int, int, int, const bf16*, size_t, bf16*, unsigned*,
-                                           cudaStream_t);
 
-// gw += d loss/d W and gb += d loss/d bias for the gradient g of the layer output (FP32, [B][Cout][vol])
-helm_status wgrad_tc(const bf16* in, int Cin, size_t in_bs, const float* g, int Cout, size_t g_bs, int B, int Z, int Y,
-                     int X, float* gw, float* gb, unsigned* status, cudaStream_t s) {
-    const int nkc = (Cin + 15) / 16;
-    const int ntx = (X + CT_TX - 1) / CT_TX;
-    const long ntiles = (long)B * Z * Y * ntx;
-    const int sms = g_conv_sms > 0 ? g_conv_sms : 148;
-    long per = (2L * sms + nkc - 1) / nkc;   // CTAs per chunk: about two waves over the SMs in all
-    if (per > ntiles) per = ntiles;
-    if (per < 1) per = 1;
-    wgrad_tc_kernel<float><<<dim3((unsigned)nkc, (unsigned)per), CT_THREADS, WG_SMEM, s>>>(in, Cin, in_bs, g, Cout, g_bs, B, Z,
-                                                                                      Y, X, gw, status);
-    const size_t vol = (size_t)Z * Y * X;
-    bias_grad_kernel<float><<<dim3((unsigned)Cout, 64), 256, 0, s>>>(g, Cout, g_bs, B, vol, gb);
+// gw += d loss/d W for the gradient cells gr of the layer output (Cout <= 128)
+helm_status wgrad_cells(const CellGrid& g, const bf16* in, int Cin, const bf16* gr, int Cout, float* gw, unsigned* status,
+                        cudaStream_t s) {
+    WgradArgs a;
+    a.g = g;
+    a.in = in; a.Gin = cell_groups(Cin);
+    a.gr = gr; a.Ggr = cell_groups(Cout);
+    a.Cin = Cin; a.Cout = Cout;
+    a.M = Cout <= 64 ? 64 : 128;
+    a.gw = gw;
+    a.status = status;
+    // accumulators in tensor memory (512 columns): the 9 taps of a dz up to 48 inputs, else 3 taps of up to 160
+    const int Nin = 8 * a.Gin;
+    a.ndy = Nin <= 48 ? 3 : 1;
+    a.nblk = (Nin + 159) / 160;
+    a.Nb = (Nin / 16 + a.nblk - 1) / a.nblk * 16;
+    // the MMAs read M / 8 groups of gradient rows; those beyond Ggr fall into the staged inputs (their accumulator
+    // rows are not used), so a stage is at least as long as all of them
+    auto stage = [&](int kt) {
+        return (std::max(a.M / 8 * kt * 16, a.Ggr * kt * 16 + a.ndy * (a.Nb / 8) * (kt + 2) * 16) + 127) / 128 * 128;
+    };
+    a.kt = 3 * stage(WG_KT) + 128 <= CT_SMEM ? WG_KT : WG_KT / 2;   // at least three stages
+    a.stage = stage(a.kt);
+    a.nst = std::min(CT_NST, (CT_SMEM - 128) / a.stage);
+    a.ntp = (g.span + a.kt - 1) / a.kt;
+    a.ntiles = (int)((long)g.B * g.Z * a.ntp);
+    // whole waves of CTAs (one per SM), each with at most WG_TILES tiles
+    const int groups = (a.ndy == 3 ? 3 : 9) * a.nblk, sms = sm_count();
+    const int one = std::max(1, sms / groups), per = WG_POINTS / a.kt;
+    const int waves = (a.ntiles + per * one - 1) / (per * one);
+    const int split = std::min(a.ntiles, std::max(1, waves * sms / groups));
+    wgrad_cells_kernel<<<dim3((unsigned)groups, (unsigned)split), CT_THREADS, (size_t)a.nst * a.stage + 128, s>>>(a);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
 }

@@ -10,22 +10,29 @@
 // b1 = relu(conv(p, c->2c)), b2 = relu(conv(b1, 2c->2c)), u = [upsample2(b2), a2],
 // d1 = relu(conv(u, 3c->c)), y = conv(d1, c->2).  3x3x3 convolutions, zero padding, stride 1.
 // Activations and weights are stored in BF16, every product is accumulated in FP32; training keeps FP32
-// master weights, FP32 activation gradients and Adam moments.  Layout [B][C][Z][Y][X].
+// master weights and Adam moments.  The caller's tensors are channel-first [B][C][Z][Y][X]; inside, activations
+// are cells of 8 channels on halo grids (cells.cuh).  The gradient of a layer's output is an MMA operand twice
+// (data and weight gradient), which rounds it to BF16, so it is stored that way; whatever is summed from it in
+// FP32 (the bias gradient) is summed before the rounding, by the kernel that produces it, and the gradients that
+// are summed further (those of u and p) stay FP32.
 //
 // Kernels: the 3x3x3 convolutions run on the tcgen05 tensor cores as implicit GEMMs (conv_tc.cu: forward
 // and data gradient through flipped/transposed weights with the ReLU mask fused, weight gradient with the
-// taps' accumulators in tensor memory) whenever a layer has at most 64 outputs (widths up to 32); wider
-// layers take the direct kernels written here (a shared-memory halo tile per input channel, and the
-// weight gradient as a tiled reduction with one atomic per CTA and tap).  Also here: pooling/upsampling and
-// their adjoints, MSE, Adam, feature assembly and the correction step.
-#include "common.cuh"
-#include <cuda_bf16.h>
+// taps' accumulators in tensor memory).  Here: packing of the caller's tensors into cells, pooling/upsampling
+// and their adjoints, MSE, Adam, feature assembly and the correction step.
+#include "cells.cuh"
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
-typedef __nv_bfloat16 bf16;
+namespace {
+// a device buffer that grows on demand
+struct Buf {
+    void* p = nullptr;
+    size_t cap = 0;
+};
+}  // namespace
 
 struct helm_net {
     int c = 0;
@@ -34,14 +41,16 @@ struct helm_net {
     bf16* Wb = nullptr;                                                 // bf16 copy
     size_t woff[6], boff[6];
     int co[6], ci[6];
-    // activation workspace for B x Z x Y x X
-    size_t cap = 0;   // inference capacity in (B * vol) points
-    size_t gcap = 0;  // gradient-buffer capacity
+    // workspace of the last forward's shape (full-resolution and half-resolution grids); grown on demand, never
+    // shrunk.  `fresh`: the cells have to be zeroed before use (new shape or new memory)
     int B = 0, Z = 0, Y = 0, X = 0;
-    bf16 *x = nullptr, *a1 = nullptr, *u = nullptr, *d1 = nullptr;      // full resolution (u holds [up(b2), a2])
-    bf16 *p = nullptr, *b1 = nullptr, *b2 = nullptr;                    // half resolution
-    float* y = nullptr;
-    float *gA = nullptr, *gB = nullptr, *gU = nullptr, *gH1 = nullptr, *gH2 = nullptr;   // gradient buffers
+    CellGrid gf, gh;
+    bool fresh = false, gfresh = false;
+    int gB_ = 0, gZ_ = 0, gY_ = 0, gX_ = 0;                 // shape of the gradient workspace
+    Buf xp, y;                                              // channel-first features (BF16) and output (FP32)
+    Buf x, a1, u, d1, p, b1, b2;                            // BF16 cells; u holds [up(b2), a2]; p, b1, b2 half resolution
+    Buf gy, gC, gD, gH1, gH2;                                   // gradients, BF16 cells (gH1, gH2 half resolution)
+    Buf gU, gP;                                             // gradients of u and p, FP32 cells
     // statistics and reduction scratch (16 doubles): 0 sum|v|^2, 1 sum|M^-1 v|^2, 2 |alpha| of the last
     // correction, 3 corrections dropped, 4 corrections applied, 5 sum over applied corrections of
     // |v - A z|^2/|v - A M^-1 v|^2, 6-7 <Ac, rho>, 8 |Ac|^2, 9 |rho|^2, 15 scratch of helm_net_target
@@ -53,223 +62,183 @@ struct helm_net {
     unsigned* status = nullptr;    // device status word of the network's own calls (bounded waits)
 };
 
-// conv_tc.cu
-bool conv_tc_supported(int Cin, int Cout);
-bool wgrad_tc_supported(int Cin, int Cout);
-size_t conv_tc_scratch_bytes(int Cin, int Cout);
-helm_status conv_tc_prepare();
-template <typename TIN, typename TOUT>
-helm_status conv_tc(const TIN* in, int Cin, size_t in_bs, const __nv_bfloat16* w, int wmode, const float* bias,
-                    TOUT* out, int Cout, size_t out_bs, int B, int Z, int Y, int X, int relu,
-                    const __nv_bfloat16* mask, size_t mask_bs, __nv_bfloat16* wscr, unsigned* status, cudaStream_t s);
-helm_status wgrad_tc(const __nv_bfloat16* in, int Cin, size_t in_bs, const float* g, int Cout, size_t g_bs, int B, int Z,
-                     int Y, int X, float* gw, float* gb, unsigned* status, cudaStream_t s);
-
 namespace {
 
-constexpr int TXC = 8, TYC = 8, TZC = 4;      // output tile of the convolution (256 threads)
-constexpr int COT = 8;                        // output channels per CTA
+bf16* cells(const Buf& b) { return reinterpret_cast<bf16*>(b.p); }
+float* floats(const Buf& b) { return reinterpret_cast<float*>(b.p); }
 
-__device__ __forceinline__ float ld(const bf16* p, size_t i) { return __bfloat162float(p[i]); }
-__device__ __forceinline__ float ld(const float* p, size_t i) { return p[i]; }
-__device__ __forceinline__ void st(bf16* p, size_t i, float v) { p[i] = __float2bfloat16(v); }
-__device__ __forceinline__ void st(float* p, size_t i, float v) { p[i] = v; }
-
-// out[b][o][q] = act( bias[o] + sum_{i,t} W(o,i,t) in[b][i][q + off_t] ),  zero padding.
-// W(o,i,t) = w[(o*Cin + i)*27 + t] (wmode 0) or w[(i*Cout + o)*27 + 26 - t] (wmode 1: data gradient).
-// mask (optional): out *= (mask[b][o][q] > 0), for the ReLU of the layer whose gradient this is.
-template <typename TIN, typename TOUT>
-__global__ void __launch_bounds__(256) conv3_kernel(const TIN* __restrict__ in, int Cin, size_t in_bs,
-                                                    const bf16* __restrict__ w, int wmode,
-                                                    const float* __restrict__ bias, TOUT* __restrict__ out, int Cout,
-                                                    size_t out_bs, int Z, int Y, int X, int relu,
-                                                    const bf16* __restrict__ mask, size_t mask_bs) {
-    __shared__ float tile[(TZC + 2) * (TYC + 2) * (TXC + 2)];
-    __shared__ float wsm[COT * 27];
-    const int tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7, tz = threadIdx.x >> 6;
-    const int ntx = (X + TXC - 1) / TXC;
-    const int bx = blockIdx.x % ntx, by = blockIdx.x / ntx;
-    const int x0 = bx * TXC, y0 = by * TYC, z0 = blockIdx.y * TZC;
-    const int nco = (Cout + COT - 1) / COT;
-    const int b = blockIdx.z / nco, o0 = (blockIdx.z % nco) * COT;
-    const size_t vol = (size_t)Z * Y * X;
-    const int gx = x0 + tx, gy = y0 + ty, gz = z0 + tz;
-    float acc[COT];
+// ---- element kernels on cells: one thread per point (of the coarse grid where there are two) and group of 8
+// channels, 16-byte cells; blockIdx.y = batch * groups + group.  The channels of a2 start at channel 2c of u: where
+// that is inside a cell (width not a multiple of 4), cells are assembled channel by channel. ----
+struct Pt { int z, y, x; };
+__device__ __forceinline__ Pt point_of(long id, const CellGrid& g) {
+    const int x = (int)(id % g.X);
+    const long r = id / g.X;
+    return {(int)(r / g.Y), (int)(r % g.Y), x};
+}
+__device__ __forceinline__ long cell_of(const CellGrid& g, int z, int y, int x) {
+    return (long)(z + 1) * g.plane + (long)(y + 1) * g.pitch + x + 1;
+}
+// channels c0 .. c0 + 7 (below C) of a BF16 tensor of G groups at cell q
+__device__ __forceinline__ uint4 read_cell(const bf16* t, int G, int b, long vol, long q, int c0, int C) {
+    if (c0 % 8 == 0) return *reinterpret_cast<const uint4*>(t + 8 * (((long)b * G + c0 / 8) * vol + q));
+    float v[8];
 #pragma unroll
-    for (int o = 0; o < COT; ++o) acc[o] = 0.f;
-    const TIN* inb = in + (size_t)b * in_bs;
-    for (int i = 0; i < Cin; ++i) {
-        __syncthreads();
-        const TIN* ch = inb + (size_t)i * vol;
-        for (int q = threadIdx.x; q < (TZC + 2) * (TYC + 2) * (TXC + 2); q += 256) {
-            const int lx = q % (TXC + 2), ly = (q / (TXC + 2)) % (TYC + 2), lz = q / ((TXC + 2) * (TYC + 2));
-            const int X_ = x0 + lx - 1, Y_ = y0 + ly - 1, Z_ = z0 + lz - 1;
-            float v = 0.f;
-            if (X_ >= 0 && X_ < X && Y_ >= 0 && Y_ < Y && Z_ >= 0 && Z_ < Z) v = ld(ch, ((size_t)Z_ * Y + Y_) * X + X_);
-            tile[q] = v;
-        }
-        for (int q = threadIdx.x; q < COT * 27; q += 256) {
-            const int o = q / 27, t = q - o * 27;
-            float v = 0.f;
-            if (o0 + o < Cout)
-                v = __bfloat162float(wmode ? w[((size_t)i * Cout + o0 + o) * 27 + 26 - t] : w[((size_t)(o0 + o) * Cin + i) * 27 + t]);
-            wsm[q] = v;
-        }
-        __syncthreads();
+    for (int j = 0; j < 8; ++j)
+        v[j] = c0 + j < C ? __bfloat162float(t[8 * (((long)b * G + (c0 + j) / 8) * vol + q) + (c0 + j) % 8]) : 0.f;
+    return pack_cell(v);
+}
+__device__ __forceinline__ void read_cell_f32(const float* t, int G, int b, long vol, long q, int c0, int C, float* v) {
+    if (c0 % 8 == 0) {
+        const float4* p = reinterpret_cast<const float4*>(t) + 2 * (((long)b * G + c0 / 8) * vol + q);
+        const float4 lo = p[0], hi = p[1];
+        v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w;
+        v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
+        return;
+    }
 #pragma unroll
-        for (int t = 0; t < 27; ++t) {
-            const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;
-            const float v = tile[((tz + dz) * (TYC + 2) + ty + dy) * (TXC + 2) + tx + dx];
+    for (int j = 0; j < 8; ++j) v[j] = c0 + j < C ? t[8 * (((long)b * G + (c0 + j) / 8) * vol + q) + (c0 + j) % 8] : 0.f;
+}
+// gb[c0 + k] += the block's sums of s[k] (channels below C)
+__device__ __forceinline__ void add_channel_sums(const float* s, float* gb, int c0, int C) {
+    __shared__ float red[8];
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 8) red[threadIdx.x] = 0.f;
+    __syncthreads();
+    const float f = lane_fold8(s, lane);
+    if (!(lane & 3)) atomicAdd(&red[lane_fold8_channel(lane)], f);
+    __syncthreads();
+    if (threadIdx.x < 8 && c0 + threadIdx.x < C) atomicAdd(&gb[c0 + threadIdx.x], red[threadIdx.x]);
+}
+
+// channel-first features (5 channels) -> cells of group 0 (channels 5-7 zero)
+__global__ void pack_x_kernel(CellGrid g, const bf16* __restrict__ in, int G, bf16* __restrict__ out) {
+    const long n = (long)g.Z * g.Y * g.X;
+    const int b = blockIdx.y;
+    const uint16_t* s = reinterpret_cast<const uint16_t*>(in) + (size_t)b * 5 * n;
+    for (long id = blockIdx.x * (long)blockDim.x + threadIdx.x; id < n; id += (long)gridDim.x * blockDim.x) {
+        const Pt p = point_of(id, g);
+        const uint32_t c0 = s[id], c1 = s[id + n], c2 = s[id + 2 * n], c3 = s[id + 3 * n], c4 = s[id + 4 * n];
+        *reinterpret_cast<uint4*>(out + 8 * ((long)b * G * g.vol + cell_of(g, p.z, p.y, p.x))) =
+            make_uint4(c0 | c1 << 16, c2 | c3 << 16, c4, 0u);
+    }
+}
+
+// channel-first gradient of the output (2 channels, FP32) -> cells of group 0; gb += its sums
+__global__ void __launch_bounds__(256) pack_gy_kernel(CellGrid g, const float* __restrict__ in, int G, bf16* __restrict__ out,
+                                                      float* __restrict__ gb) {
+    const long n = (long)g.Z * g.Y * g.X;
+    const int b = blockIdx.y;
+    const float* s = in + (size_t)b * 2 * n;
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (long id = blockIdx.x * (long)blockDim.x + threadIdx.x; id < n; id += (long)gridDim.x * blockDim.x) {
+        const Pt p = point_of(id, g);
+        const float c0 = s[id], c1 = s[id + n];
+        sum[0] += c0;
+        sum[1] += c1;
+        *reinterpret_cast<uint4*>(out + 8 * ((long)b * G * g.vol + cell_of(g, p.z, p.y, p.x))) =
+            make_uint4(pack2(c0, c1), 0u, 0u, 0u);
+    }
+    add_channel_sums(sum, gb, 0, 2);
+}
+
+// out (coarse, C channels) = mean of the 8 children of a2 (channels ca .. ca + C - 1 of u)
+__global__ void avgpool2_kernel(CellGrid gf, CellGrid gh, const bf16* __restrict__ u, int Gu, int ca, int C,
+                                bf16* __restrict__ out, int G) {
+    const long n = (long)gh.Z * gh.Y * gh.X;
+    const int ng = (C + 7) / 8, b = blockIdx.y / ng, cg = blockIdx.y % ng;
+    for (long id = blockIdx.x * (long)blockDim.x + threadIdx.x; id < n; id += (long)gridDim.x * blockDim.x) {
+        const Pt p = point_of(id, gh);
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int o = 0; o < COT; ++o) acc[o] = fmaf(wsm[o * 27 + t], v, acc[o]);
-        }
-    }
-    if (gx >= X || gy >= Y || gz >= Z) return;
-    const size_t q = ((size_t)gz * Y + gy) * X + gx;
+        for (int k = 0; k < 8; ++k) {
+            const uint4 v = read_cell(u, Gu, b, gf.vol, cell_of(gf, 2 * p.z + (k >> 2), 2 * p.y + ((k >> 1) & 1), 2 * p.x + (k & 1)),
+                                      ca + 8 * cg, ca + C);
 #pragma unroll
-    for (int o = 0; o < COT; ++o) {
-        if (o0 + o >= Cout) break;
-        float v = acc[o] + (bias ? bias[o0 + o] : 0.f);
-        if (relu) v = fmaxf(v, 0.f);
-        if (mask && !(__bfloat162float(mask[(size_t)b * mask_bs + (size_t)(o0 + o) * vol + q]) > 0.f)) v = 0.f;
-        st(out, (size_t)b * out_bs + (size_t)(o0 + o) * vol + q, v);
+            for (int j = 0; j < 8; ++j) acc[j] += cell_value(v, j);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] *= 0.125f;
+        *reinterpret_cast<uint4*>(out + 8 * (((long)b * G + cg) * gh.vol + cell_of(gh, p.z, p.y, p.x))) = pack_cell(acc);
     }
 }
 
-// gw[o][i][t] += sum_{b,q} g[b][o][q] in[b][i][q + off_t];  gb[o] += sum g  (one atomic per CTA and tap)
-__global__ void __launch_bounds__(256) conv3_wgrad_kernel(const bf16* __restrict__ in, int Cin, size_t in_bs,
-                                                          const float* __restrict__ g, int Cout, size_t g_bs, int B,
-                                                          int Z, int Y, int X, float* __restrict__ gw,
-                                                          float* __restrict__ gb) {
-    __shared__ float tile[(TZC + 2) * (TYC + 2) * (TXC + 2)];
-    __shared__ float gt[COT][TZC * TYC * TXC];
-    const int i = blockIdx.x;
-    const int o0 = blockIdx.y * COT;
-    const int ntx = (X + TXC - 1) / TXC, nty = (Y + TYC - 1) / TYC, ntz = (Z + TZC - 1) / TZC;
-    const int ntiles = B * ntx * nty * ntz;
-    const size_t vol = (size_t)Z * Y * X;
-    // thread -> (o, t) pair; 8 x 27 = 216 active
-    const int o = threadIdx.x / 27, t = threadIdx.x - o * 27;
-    const bool act = threadIdx.x < COT * 27 && o0 + o < Cout;
-    const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;
-    float acc = 0.f, accb = 0.f;
-    for (int tile_id = blockIdx.z; tile_id < ntiles; tile_id += gridDim.z) {
-        int r = tile_id;
-        const int bx = r % ntx; r /= ntx;
-        const int by = r % nty; r /= nty;
-        const int bz = r % ntz; r /= ntz;
-        const int b = r;
-        const int x0 = bx * TXC, y0 = by * TYC, z0 = bz * TZC;
-        __syncthreads();
-        const bf16* ch = in + (size_t)b * in_bs + (size_t)i * vol;
-        for (int q = threadIdx.x; q < (TZC + 2) * (TYC + 2) * (TXC + 2); q += 256) {
-            const int lx = q % (TXC + 2), ly = (q / (TXC + 2)) % (TYC + 2), lz = q / ((TXC + 2) * (TYC + 2));
-            const int X_ = x0 + lx - 1, Y_ = y0 + ly - 1, Z_ = z0 + lz - 1;
-            float v = 0.f;
-            if (X_ >= 0 && X_ < X && Y_ >= 0 && Y_ < Y && Z_ >= 0 && Z_ < Z) v = ld(ch, ((size_t)Z_ * Y + Y_) * X + X_);
-            tile[q] = v;
-        }
-        for (int q = threadIdx.x; q < COT * TZC * TYC * TXC; q += 256) {
-            const int oo = q / (TZC * TYC * TXC), pp = q - oo * (TZC * TYC * TXC);
-            const int lx = pp % TXC, ly = (pp / TXC) % TYC, lz = pp / (TXC * TYC);
-            const int X_ = x0 + lx, Y_ = y0 + ly, Z_ = z0 + lz;
-            float v = 0.f;
-            if (o0 + oo < Cout && X_ < X && Y_ < Y && Z_ < Z)
-                v = g[(size_t)b * g_bs + (size_t)(o0 + oo) * vol + ((size_t)Z_ * Y + Y_) * X + X_];
-            gt[oo][pp] = v;
-        }
-        __syncthreads();
-        if (act) {
-            for (int pp = 0; pp < TZC * TYC * TXC; ++pp) {
-                const int lx = pp % TXC, ly = (pp / TXC) % TYC, lz = pp / (TXC * TYC);
-                const float gv = gt[o][pp];
-                acc = fmaf(gv, tile[((lz + dz) * (TYC + 2) + ly + dy) * (TXC + 2) + lx + dx], acc);
-                if (t == 0 && i == 0) accb += gv;
-            }
+// channels 0 .. C - 1 of u (fine) = upsample2(in) (coarse): a thread writes the 8 children of a cell
+__global__ void upsample2_kernel(CellGrid gf, CellGrid gh, const bf16* __restrict__ in, int G, int C, bf16* __restrict__ u,
+                                 int Gu) {
+    const long n = (long)gh.Z * gh.Y * gh.X;
+    const int ng = (C + 7) / 8, b = blockIdx.y / ng, cg = blockIdx.y % ng;
+    const bool whole = 8 * cg + 8 <= C;   // else a2's channels follow in the same cell
+    for (long id = blockIdx.x * (long)blockDim.x + threadIdx.x; id < n; id += (long)gridDim.x * blockDim.x) {
+        const Pt p = point_of(id, gh);
+        const uint4 v = *reinterpret_cast<const uint4*>(in + 8 * (((long)b * G + cg) * gh.vol + cell_of(gh, p.z, p.y, p.x)));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            bf16* o = u + 8 * (((long)b * Gu + cg) * gf.vol +
+                               cell_of(gf, 2 * p.z + (k >> 2), 2 * p.y + ((k >> 1) & 1), 2 * p.x + (k & 1)));
+            if (whole) *reinterpret_cast<uint4*>(o) = v;
+            else
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (8 * cg + j < C) o[j] = __float2bfloat16(cell_value(v, j));
         }
     }
-    if (act) {
-        atomicAdd(&gw[((size_t)(o0 + o) * Cin + i) * 27 + t], acc);
-        if (t == 0 && i == 0) atomicAdd(&gb[o0 + o], accb);
-    }
 }
 
-__global__ void avgpool2_kernel(const bf16* __restrict__ in, size_t in_bs, bf16* __restrict__ out, int C, int B,
-                                int Z, int Y, int X) {
-    const int Zh = Z / 2, Yh = Y / 2, Xh = X / 2;
-    const size_t n = (size_t)B * C * Zh * Yh * Xh;
-    for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < n; id += (size_t)gridDim.x * blockDim.x) {
-        size_t r = id;
-        const int x = r % Xh; r /= Xh;
-        const int y = r % Yh; r /= Yh;
-        const int z = r % Zh; r /= Zh;
-        const int c = r % C; const int b = (int)(r / C);
-        const bf16* s = in + (size_t)b * in_bs + (size_t)c * Z * Y * X;
-        float acc = 0.f;
-        for (int k = 0; k < 8; ++k)
-            acc += ld(s, ((size_t)(2 * z + (k >> 2)) * Y + 2 * y + ((k >> 1) & 1)) * X + 2 * x + (k & 1));
-        out[id] = __float2bfloat16(0.125f * acc);
+// gh (coarse cells, C channels) = mask(b2 > 0) * sum of the 8 children of gu (adjoint of upsample2); gb += its sums
+__global__ void __launch_bounds__(256) upsample2_adj_kernel(CellGrid gf, CellGrid gh, const float* __restrict__ gu, int Gu,
+                                                            const bf16* __restrict__ mask, bf16* __restrict__ out, int G, int C,
+                                                            float* __restrict__ gb) {
+    const long n = (long)gh.Z * gh.Y * gh.X;
+    const int ng = (C + 7) / 8, b = blockIdx.y / ng, cg = blockIdx.y % ng;
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (long id = blockIdx.x * (long)blockDim.x + threadIdx.x; id < n; id += (long)gridDim.x * blockDim.x) {
+        const Pt p = point_of(id, gh);
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            float v[8];
+            read_cell_f32(gu, Gu, b, gf.vol, cell_of(gf, 2 * p.z + (k >> 2), 2 * p.y + ((k >> 1) & 1), 2 * p.x + (k & 1)), 8 * cg,
+                          C, v);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] += v[j];
+        }
+        const long q = ((long)b * G + cg) * gh.vol + cell_of(gh, p.z, p.y, p.x);
+        const uint4 m = *reinterpret_cast<const uint4*>(mask + 8 * q);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (!(cell_value(m, j) > 0.f)) acc[j] = 0.f;
+            sum[j] += acc[j];
+        }
+        *reinterpret_cast<uint4*>(out + 8 * q) = pack_cell(acc);
     }
+    add_channel_sums(sum, gb, 8 * cg, C);
 }
 
-// out (full res, channels 0..C-1 of a [B][Cu] buffer) = upsample2(in): one thread per pair of output points
-// (x even, x + 1) of a row, which share their source value; grid.x = (x block, y, z), grid.y = (b, c)
-__global__ void upsample2_kernel(const bf16* __restrict__ in, bf16* __restrict__ out, size_t out_bs, int C, int B,
-                                 int Z, int Y, int X) {
-    const int Zh = Z / 2, Yh = Y / 2, Xh = X / 2;
-    const int nxb = (Xh + blockDim.x - 1) / blockDim.x;
-    int r = blockIdx.x;
-    const int xh = (r % nxb) * blockDim.x + threadIdx.x;
-    r /= nxb;
-    const int y = r % Y, z = r / Y;
-    if (xh >= Xh) return;
-    const int c = blockIdx.y % C, b = blockIdx.y / C;
-    const bf16 v = in[(((size_t)b * C + c) * Zh + z / 2) * ((size_t)Yh * Xh) + (size_t)(y / 2) * Xh + xh];
-    __nv_bfloat162 two;
-    two.x = v;
-    two.y = v;
-    bf16* o = out + (size_t)b * out_bs + (size_t)c * Z * Y * X + ((size_t)z * Y + y) * X + 2 * xh;
-    *reinterpret_cast<__nv_bfloat162*>(o) = two;
-}
-
-// g_half[b][c] = mask(b2 > 0) * sum of the 8 children of gu[b][c] (adjoint of upsample2)
-__global__ void upsample2_adj_kernel(const float* __restrict__ gu, size_t gu_bs, const bf16* __restrict__ mask,
-                                     float* __restrict__ gh, int C, int B, int Z, int Y, int X) {
-    const int Zh = Z / 2, Yh = Y / 2, Xh = X / 2;
-    const size_t n = (size_t)B * C * Zh * Yh * Xh;
-    for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < n; id += (size_t)gridDim.x * blockDim.x) {
-        size_t r = id;
-        const int x = r % Xh; r /= Xh;
-        const int y = r % Yh; r /= Yh;
-        const int z = r % Zh; r /= Zh;
-        const int c = r % C; const int b = (int)(r / C);
-        const float* s = gu + (size_t)b * gu_bs + (size_t)c * Z * Y * X;
-        float acc = 0.f;
-        for (int k = 0; k < 8; ++k)
-            acc += s[((size_t)(2 * z + (k >> 2)) * Y + 2 * y + ((k >> 1) & 1)) * X + 2 * x + (k & 1)];
-        gh[id] = (__bfloat162float(mask[id]) > 0.f) ? acc : 0.f;
+// ga2 (cells, C channels) = mask(a2 > 0) * (gu_a2 + upsample2(gp)/8) (adjoint of avgpool2 added to the skip
+// gradient; a2 and its gradient are channels ca .. ca + C - 1 of u and gu); gb += its sums
+__global__ void __launch_bounds__(256) skip_grad_kernel(CellGrid gf, CellGrid gh, const float* __restrict__ gu,
+                                                        const float* __restrict__ gp, int Gp, const bf16* __restrict__ u, int Gu,
+                                                        int ca, int C, bf16* __restrict__ out, int G, float* __restrict__ gb) {
+    const long n = (long)gf.Z * gf.Y * gf.X;
+    const int ng = (C + 7) / 8, b = blockIdx.y / ng, cg = blockIdx.y % ng;
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (long id = blockIdx.x * (long)blockDim.x + threadIdx.x; id < n; id += (long)gridDim.x * blockDim.x) {
+        const Pt p = point_of(id, gf);
+        const long q = cell_of(gf, p.z, p.y, p.x);
+        float v[8], c[8];
+        read_cell_f32(gu, Gu, b, gf.vol, q, ca + 8 * cg, ca + C, v);
+        read_cell_f32(gp, Gp, b, gh.vol, cell_of(gh, p.z / 2, p.y / 2, p.x / 2), 8 * cg, C, c);
+        const uint4 m = read_cell(u, Gu, b, gf.vol, q, ca + 8 * cg, ca + C);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            v[j] += 0.125f * c[j];
+            if (8 * cg + j >= C || !(cell_value(m, j) > 0.f)) v[j] = 0.f;
+            sum[j] += v[j];
+        }
+        *reinterpret_cast<uint4*>(out + 8 * (((long)b * G + cg) * gf.vol + q)) = pack_cell(v);
     }
-}
-
-// ga2 = mask(a2 > 0) * (gu_a2 + upsample2(gp)/8)   (adjoint of avgpool2 added to the skip gradient)
-__global__ void skip_grad_kernel(const float* __restrict__ gu_a2, size_t gu_bs, const float* __restrict__ gp,
-                                 const bf16* __restrict__ a2, size_t a2_bs, float* __restrict__ ga2, int C, int B,
-                                 int Z, int Y, int X) {
-    const size_t vol = (size_t)Z * Y * X;
-    const size_t n = (size_t)B * C * vol;
-    const int Zh = Z / 2, Yh = Y / 2, Xh = X / 2;
-    for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < n; id += (size_t)gridDim.x * blockDim.x) {
-        size_t r = id;
-        const int x = r % X; r /= X;
-        const int y = r % Y; r /= Y;
-        const int z = r % Z; r /= Z;
-        const int c = r % C; const int b = (int)(r / C);
-        const size_t q = ((size_t)z * Y + y) * X + x;
-        float v = gu_a2[(size_t)b * gu_bs + (size_t)c * vol + q] +
-                  0.125f * gp[(((size_t)b * C + c) * Zh + z / 2) * Yh * Xh + (size_t)(y / 2) * Xh + x / 2];
-        if (!(__bfloat162float(a2[(size_t)b * a2_bs + (size_t)c * vol + q]) > 0.f)) v = 0.f;
-        ga2[id] = v;
-    }
+    add_channel_sums(sum, gb, 8 * cg, C);
 }
 
 __global__ void mse_kernel(const float* __restrict__ y, const float* __restrict__ t, float* __restrict__ g, size_t n,
@@ -439,95 +408,84 @@ __global__ void target_kernel(const double2* __restrict__ xs, const double2* __r
 
 unsigned nblk(size_t n) { const size_t b = (n + 255) / 256; return (unsigned)(b > 4096 ? 4096 : b); }
 
-// the convolution of a layer: tensor cores where the shape allows, else the direct kernel
-template <typename TIN, typename TOUT>
-void conv(helm_net* n, const TIN* in, int Cin, size_t in_bs, const bf16* w, int wmode, const float* bias, TOUT* out,
-          int Cout, size_t out_bs, int B, int Z, int Y, int X, int relu, const bf16* mask, size_t mask_bs,
-          unsigned* status, cudaStream_t s) {
-    if (conv_tc_supported(Cin, Cout)) {
-        conv_tc<TIN, TOUT>(in, Cin, in_bs, w, wmode, bias, out, Cout, out_bs, B, Z, Y, X, relu, mask, mask_bs, n->wscr,
-                           status, s);
-        return;
-    }
-    const int ntx = (X + TXC - 1) / TXC, nty = (Y + TYC - 1) / TYC, ntz = (Z + TZC - 1) / TZC;
-    dim3 grid(ntx * nty, ntz, B * ((Cout + COT - 1) / COT));
-    conv3_kernel<TIN, TOUT><<<grid, 256, 0, s>>>(in, Cin, in_bs, w, wmode, bias, out, Cout, out_bs, Z, Y, X, relu, mask,
-                                                mask_bs);
-}
-
-void wgrad(helm_net* n, const bf16* in, int Cin, size_t in_bs, const float* g, int Cout, size_t g_bs, int B, int Z,
-           int Y, int X, float* gw, float* gb, cudaStream_t s) {
-    if (wgrad_tc_supported(Cin, Cout)) {
-        wgrad_tc(in, Cin, in_bs, g, Cout, g_bs, B, Z, Y, X, gw, gb, n->status, s);
-        return;
-    }
-    dim3 grid(Cin, (Cout + COT - 1) / COT, 16);
-    conv3_wgrad_kernel<<<grid, 256, 0, s>>>(in, Cin, in_bs, g, Cout, g_bs, B, Z, Y, X, gw, gb);
-}
-
 void free_bufs(void** ps, int n) {
     for (int i = 0; i < n; ++i) {
         if (ps[i]) cudaFree(ps[i]);
     }
 }
+bool grow(Buf& b, size_t bytes) {
+    if (bytes <= b.cap) return true;
+    cudaFree(b.p);
+    b = Buf();
+    if (cudaMalloc(&b.p, bytes) != cudaSuccess) { cudaGetLastError(); return false; }
+    b.cap = bytes;
+    return true;
+}
 
-// inference workspace for B x Z x Y x X (grown on demand, never shrunk)
+// inference workspace for B x Z x Y x X (grown on demand, never shrunk); the cells are zeroed by the next
+// forward when the shape or the memory is new
 helm_status ensure_ws(helm_net* n, int B, int Z, int Y, int X) {
     if (B < 1 || Z < 2 || Y < 2 || X < 2 || Z % 2 || Y % 2 || X % 2) return HELM_ERR_ARG;
+    if (B == n->B && Z == n->Z && Y == n->Y && X == n->X) return HELM_OK;
+    n->B = 0;
+    n->gf = cell_grid(B, Z, Y, X);
+    n->gh = cell_grid(B, Z / 2, Y / 2, X / 2);
+    const int c = n->c;
     const size_t pts = (size_t)B * Z * Y * X;
+    if (!grow(n->xp, 5 * pts * 2) || !grow(n->y, 2 * pts * 4) || !grow(n->x, cell_bytes(n->gf, 5)) ||
+        !grow(n->a1, cell_bytes(n->gf, c)) || !grow(n->u, cell_bytes(n->gf, 3 * c)) || !grow(n->d1, cell_bytes(n->gf, c)) ||
+        !grow(n->p, cell_bytes(n->gh, c)) || !grow(n->b1, cell_bytes(n->gh, 2 * c)) || !grow(n->b2, cell_bytes(n->gh, 2 * c)))
+        return HELM_ERR_NOMEM;
+    n->fresh = true;
     n->B = B; n->Z = Z; n->Y = Y; n->X = X;
-    if (pts <= n->cap) return HELM_OK;
-    void* ps[] = {n->x, n->a1, n->u, n->d1, n->p, n->b1, n->b2, n->y};
-    free_bufs(ps, 8);
-    n->x = n->a1 = n->u = n->d1 = n->p = n->b1 = n->b2 = nullptr;
-    n->y = nullptr;
-    n->cap = 0;
-    const size_t c = n->c, h = pts / 8;
-    auto A = [&](void** p, size_t bytes) { return cudaMalloc(p, bytes) == cudaSuccess; };
-    const bool ok = A((void**)&n->x, 5 * pts * 2) && A((void**)&n->a1, c * pts * 2) && A((void**)&n->u, 3 * c * pts * 2) &&
-                    A((void**)&n->d1, c * pts * 2) && A((void**)&n->p, c * h * 2) && A((void**)&n->b1, 2 * c * h * 2) &&
-                    A((void**)&n->b2, 2 * c * h * 2) && A((void**)&n->y, 2 * pts * 4);
-    if (!ok) { cudaGetLastError(); return HELM_ERR_NOMEM; }
-    n->cap = pts;
     return HELM_OK;
 }
 
 // gradient workspace for the current B x Z x Y x X (training only)
 helm_status ensure_grad_ws(helm_net* n) {
-    const size_t pts = (size_t)n->B * n->Z * n->Y * n->X;
-    if (pts <= n->gcap) return HELM_OK;
-    void* ps[] = {n->gA, n->gB, n->gU, n->gH1, n->gH2};
-    free_bufs(ps, 5);
-    n->gA = n->gB = n->gU = n->gH1 = n->gH2 = nullptr;
-    n->gcap = 0;
-    const size_t c = n->c, h = pts / 8;
-    auto A = [&](void** p, size_t bytes) { return cudaMalloc(p, bytes) == cudaSuccess; };
-    const bool ok = A((void**)&n->gA, c * pts * 4) && A((void**)&n->gB, c * pts * 4) && A((void**)&n->gU, 3 * c * pts * 4) &&
-                    A((void**)&n->gH1, 2 * c * h * 4) && A((void**)&n->gH2, 2 * c * h * 4);
-    if (!ok) { cudaGetLastError(); return HELM_ERR_NOMEM; }
-    n->gcap = pts;
+    if (n->B == n->gB_ && n->Z == n->gZ_ && n->Y == n->gY_ && n->X == n->gX_) return HELM_OK;
+    n->gB_ = 0;
+    const int c = n->c;
+    if (!grow(n->gy, cell_bytes(n->gf, 2)) || !grow(n->gC, cell_bytes(n->gf, c)) || !grow(n->gD, cell_bytes(n->gf, c)) || !grow(n->gU, cell_bytes(n->gf, 3 * c, 4)) ||
+        !grow(n->gP, cell_bytes(n->gh, c, 4)) || !grow(n->gH1, cell_bytes(n->gh, 2 * c)) || !grow(n->gH2, cell_bytes(n->gh, 2 * c)))
+        return HELM_ERR_NOMEM;
+    n->gfresh = true;
+    n->gB_ = n->B; n->gZ_ = n->Z; n->gY_ = n->Y; n->gX_ = n->X;
     return HELM_OK;
 }
 
-// forward of the workspace input n->x into n->y (bounded-wait failures OR-ed into *status)
-void forward(helm_net* n, unsigned* status, cudaStream_t s) {
-    const int c = n->c, B = n->B, Z = n->Z, Y = n->Y, X = n->X;
-    const size_t vol = (size_t)Z * Y * X, hv = vol / 8;
+dim3 cell_blocks(const CellGrid& g, int C) {
+    const long pts = (long)g.Z * g.Y * g.X, b = (pts + 255) / 256;
+    return dim3((unsigned)(b > 1024 ? 1024 : b), (unsigned)(g.B * ((C + 7) / 8)));
+}
+
+// forward of channel-first features xp into y (channel-first FP32); bounded-wait failures OR-ed into *status
+helm_status forward(helm_net* n, const bf16* xp, float* y, unsigned* status, cudaStream_t s) {
+    const int c = n->c;
+    const CellGrid &gf = n->gf, &gh = n->gh;
     const bf16* W = n->Wb;
     const float* F = n->W;
-    bf16* a2 = n->u + 2 * c * vol;   // skip channels live inside u
-    conv<bf16, bf16>(n, n->x, 5, 5 * vol, W + n->woff[0], 0, F + n->boff[0], n->a1, c, c * vol, B, Z, Y, X, 1, nullptr, 0, status, s);
-    conv<bf16, bf16>(n, n->a1, c, c * vol, W + n->woff[1], 0, F + n->boff[1], a2, c, 3 * c * vol, B, Z, Y, X, 1, nullptr, 0, status, s);
-    avgpool2_kernel<<<nblk(B * c * hv), 256, 0, s>>>(a2, 3 * c * vol, n->p, c, B, Z, Y, X);
-    conv<bf16, bf16>(n, n->p, c, c * hv, W + n->woff[2], 0, F + n->boff[2], n->b1, 2 * c, 2 * c * hv, B, Z / 2, Y / 2, X / 2, 1,
-                     nullptr, 0, status, s);
-    conv<bf16, bf16>(n, n->b1, 2 * c, 2 * c * hv, W + n->woff[3], 0, F + n->boff[3], n->b2, 2 * c, 2 * c * hv, B, Z / 2, Y / 2,
-                     X / 2, 1, nullptr, 0, status, s);
-    upsample2_kernel<<<dim3((unsigned)((X / 2 + 127) / 128 * Y * Z), (unsigned)(B * 2 * c)), 128, 0, s>>>(
-        n->b2, n->u, 3 * c * vol, 2 * c, B, Z, Y, X);
-    conv<bf16, bf16>(n, n->u, 3 * c, 3 * c * vol, W + n->woff[4], 0, F + n->boff[4], n->d1, c, c * vol, B, Z, Y, X, 1, nullptr,
-                     0, status, s);
-    conv<bf16, float>(n, n->d1, c, c * vol, W + n->woff[5], 0, F + n->boff[5], n->y, 2, 2 * vol, B, Z, Y, X, 0, nullptr, 0, status, s);
+    helm_status st;
+    if (n->fresh) {
+        for (const Buf* b : {&n->x, &n->a1, &n->u, &n->d1, &n->p, &n->b1, &n->b2})
+            HELM_CUDA_TRY(cudaMemsetAsync(b->p, 0, b->cap, s));
+        n->fresh = false;
+    }
+    auto conv = [&](const CellGrid& g, int mode, int l, const Buf& in, void* out, int Cout_total, int ooff, int relu) {
+        return conv_cells(g, mode, cells(in), n->ci[l], W + n->woff[l], 0, F + n->boff[l], out, n->co[l], Cout_total, ooff, relu,
+                          nullptr, nullptr, n->wscr, status, s);
+    };
+    pack_x_kernel<<<cell_blocks(gf, 8), 256, 0, s>>>(gf, xp, cell_groups(5), cells(n->x));
+    if ((st = conv(gf, CONV_CELLS, 0, n->x, cells(n->a1), c, 0, 1)) != HELM_OK) return st;
+    if ((st = conv(gf, CONV_CELLS, 1, n->a1, cells(n->u), 3 * c, 2 * c, 1)) != HELM_OK) return st;   // a2 lives in u
+    avgpool2_kernel<<<cell_blocks(gh, c), 256, 0, s>>>(gf, gh, cells(n->u), cell_groups(3 * c), 2 * c, c, cells(n->p),
+                                                       cell_groups(c));
+    if ((st = conv(gh, CONV_CELLS, 2, n->p, cells(n->b1), 2 * c, 0, 1)) != HELM_OK) return st;
+    if ((st = conv(gh, CONV_CELLS, 3, n->b1, cells(n->b2), 2 * c, 0, 1)) != HELM_OK) return st;
+    upsample2_kernel<<<cell_blocks(gh, 2 * c), 256, 0, s>>>(gf, gh, cells(n->b2), cell_groups(2 * c), 2 * c, cells(n->u),
+                                                            cell_groups(3 * c));
+    if ((st = conv(gf, CONV_CELLS, 4, n->u, cells(n->d1), c, 0, 1)) != HELM_OK) return st;
+    return conv(gf, CONV_PLANAR, 5, n->d1, y, 2, 0, 0);
 }
 
 }  // namespace
@@ -572,8 +530,8 @@ helm_status helm_net_create(int width, unsigned long long seed, helm_net** out) 
     }
     size_t scr = 0;   // arranged weights of the largest layer, in either direction
     for (int l = 0; l < 6; ++l) {
-        scr = std::max(scr, conv_tc_scratch_bytes(ci[l], co[l]));
-        scr = std::max(scr, conv_tc_scratch_bytes(co[l], ci[l]));
+        scr = std::max(scr, conv_scratch_bytes(ci[l], co[l]));
+        scr = std::max(scr, conv_scratch_bytes(co[l], ci[l]));
     }
     bool ok = cudaMalloc(&n->W, off * 4) == cudaSuccess && cudaMalloc(&n->G, off * 4) == cudaSuccess &&
               cudaMalloc(&n->Mom, off * 4) == cudaSuccess && cudaMalloc(&n->Vel, off * 4) == cudaSuccess &&
@@ -586,7 +544,7 @@ helm_status helm_net_create(int width, unsigned long long seed, helm_net** out) 
     cudaMemset(n->Vel, 0, off * 4);
     cudaMemset(n->stats, 0, 16 * sizeof(double));
     cudaMemset(n->status, 0, sizeof(unsigned));
-    if (conv_tc_prepare() != HELM_OK) { cudaGetLastError(); helm_net_destroy(n); return HELM_ERR_CUDA; }
+    if (conv_prepare() != HELM_OK) { cudaGetLastError(); helm_net_destroy(n); return HELM_ERR_CUDA; }
     to_bf16_kernel<<<(unsigned)((off + 255) / 256), 256>>>(n->W, n->Wb, off);
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaGetLastError(); helm_net_destroy(n); return HELM_ERR_CUDA; }
     *out = n;
@@ -595,8 +553,9 @@ helm_status helm_net_create(int width, unsigned long long seed, helm_net** out) 
 
 void helm_net_destroy(helm_net* n) {
     if (!n) return;
-    void* ps[] = {n->W, n->G, n->Mom, n->Vel, n->Wb, n->stats, n->x, n->a1, n->u, n->d1, n->p, n->b1, n->b2, n->y,
-                  n->gA, n->gB, n->gU, n->gH1, n->gH2, n->vbuf, n->cbuf, n->az0, n->ac, n->wscr, n->status};
+    void* ps[] = {n->W, n->G, n->Mom, n->Vel, n->Wb, n->stats, n->vbuf, n->cbuf, n->az0, n->ac, n->wscr, n->status,
+                  n->xp.p, n->y.p, n->x.p, n->a1.p, n->u.p, n->d1.p, n->p.p, n->b1.p, n->b2.p, n->gy.p, n->gC.p, n->gD.p, n->gH1.p,
+                  n->gH2.p, n->gU.p, n->gP.p};
     for (void* p : ps) if (p) cudaFree(p);
     delete n;
 }
@@ -635,48 +594,58 @@ helm_status helm_net_forward(helm_net* n, const void* x, float* y, int B, int Z,
     helm_status st = ensure_ws(n, B, Z, Y, X);
     if (st != HELM_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t pts = (size_t)B * Z * Y * X;
-    HELM_CUDA_TRY(cudaMemcpyAsync(n->x, x, 5 * pts * 2, cudaMemcpyDeviceToDevice, s));
-    forward(n, n->status, s);
-    HELM_CUDA_TRY(cudaMemcpyAsync(y, n->y, 2 * pts * 4, cudaMemcpyDeviceToDevice, s));
+    if ((st = forward(n, (const bf16*)x, y, n->status, s)) != HELM_OK) return st;
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
 }
 
 helm_status helm_net_backward(helm_net* n, const float* gy, void* stream) {
-    if (!n || !gy || !n->cap) return HELM_ERR_ARG;
+    if (!n || !gy || !n->B) return HELM_ERR_ARG;
     helm_status st = ensure_grad_ws(n);
     if (st != HELM_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const int c = n->c, B = n->B, Z = n->Z, Y = n->Y, X = n->X;
-    const size_t vol = (size_t)Z * Y * X, hv = vol / 8;
+    const int c = n->c;
+    const CellGrid &gf = n->gf, &gh = n->gh;
     const bf16* W = n->Wb;
     float* G = n->G;
-    const bf16* a2 = n->u + 2 * c * vol;
+    if (n->gfresh) {
+        for (const Buf* b : {&n->gy, &n->gC, &n->gD, &n->gH1, &n->gH2}) HELM_CUDA_TRY(cudaMemsetAsync(b->p, 0, b->cap, s));
+        n->gfresh = false;
+    }
+    auto wgrad = [&](const CellGrid& g, int l, const Buf& in, const Buf& gr) {
+        return wgrad_cells(g, cells(in), n->ci[l], cells(gr), n->co[l], G + n->woff[l], n->status, s);
+    };
+    // data gradient of layer l (flipped, transposed weights): CONV_GRAD masks by the layer input's ReLU and sums
+    // the bias gradient of the layer that produced it, bl
+    auto dgrad = [&](const CellGrid& g, int mode, int l, const Buf& gr, const Buf& out, const Buf* mask, int bl) {
+        return conv_cells(g, mode, cells(gr), n->co[l], W + n->woff[l], 1, nullptr, out.p, n->ci[l], n->ci[l], 0, 0,
+                          mask ? cells(*mask) : nullptr, mask ? G + n->boff[bl] : nullptr, n->wscr, n->status, s);
+    };
     // layer 6 (linear): d1 gradient with the ReLU mask of d1
-    wgrad(n, n->d1, c, c * vol, gy, 2, 2 * vol, B, Z, Y, X, G + n->woff[5], G + n->boff[5], s);
-    conv<float, float>(n, gy, 2, 2 * vol, W + n->woff[5], 1, nullptr, n->gB, c, c * vol, B, Z, Y, X, 0, n->d1, c * vol, n->status, s);
+    pack_gy_kernel<<<cell_blocks(gf, 2), 256, 0, s>>>(gf, gy, cell_groups(2), cells(n->gy), G + n->boff[5]);
+    if ((st = wgrad(gf, 5, n->d1, n->gy)) != HELM_OK) return st;
+    if ((st = dgrad(gf, CONV_GRAD, 5, n->gy, n->gC, &n->d1, 4)) != HELM_OK) return st;
     // layer 5: u gradient (no mask: u mixes up(b2) and a2, masks applied below)
-    wgrad(n, n->u, 3 * c, 3 * c * vol, n->gB, c, c * vol, B, Z, Y, X, G + n->woff[4], G + n->boff[4], s);
-    conv<float, float>(n, n->gB, c, c * vol, W + n->woff[4], 1, nullptr, n->gU, 3 * c, 3 * c * vol, B, Z, Y, X, 0, nullptr, 0, n->status, s);
+    if ((st = wgrad(gf, 4, n->u, n->gC)) != HELM_OK) return st;
+    if ((st = dgrad(gf, CONV_F32CELLS, 4, n->gC, n->gU, nullptr, 0)) != HELM_OK) return st;
     // up branch: adjoint of upsample2 with the ReLU mask of b2
-    upsample2_adj_kernel<<<nblk(B * 2 * c * hv), 256, 0, s>>>(n->gU, 3 * c * vol, n->b2, n->gH1, 2 * c, B, Z, Y, X);
+    upsample2_adj_kernel<<<cell_blocks(gh, 2 * c), 256, 0, s>>>(gf, gh, floats(n->gU), cell_groups(3 * c), cells(n->b2),
+                                                                cells(n->gH1), cell_groups(2 * c), 2 * c, G + n->boff[3]);
     // layer 4: b1 gradient with mask(b1)
-    wgrad(n, n->b1, 2 * c, 2 * c * hv, n->gH1, 2 * c, 2 * c * hv, B, Z / 2, Y / 2, X / 2, G + n->woff[3], G + n->boff[3], s);
-    conv<float, float>(n, n->gH1, 2 * c, 2 * c * hv, W + n->woff[3], 1, nullptr, n->gH2, 2 * c, 2 * c * hv, B, Z / 2, Y / 2,
-                       X / 2, 0, n->b1, 2 * c * hv, n->status, s);
-    // layer 3: p gradient (no ReLU on p) into gH1 (c channels)
-    wgrad(n, n->p, c, c * hv, n->gH2, 2 * c, 2 * c * hv, B, Z / 2, Y / 2, X / 2, G + n->woff[2], G + n->boff[2], s);
-    conv<float, float>(n, n->gH2, 2 * c, 2 * c * hv, W + n->woff[2], 1, nullptr, n->gH1, c, c * hv, B, Z / 2, Y / 2, X / 2, 0,
-                       nullptr, 0, n->status, s);
+    if ((st = wgrad(gh, 3, n->b1, n->gH1)) != HELM_OK) return st;
+    if ((st = dgrad(gh, CONV_GRAD, 3, n->gH1, n->gH2, &n->b1, 2)) != HELM_OK) return st;
+    // layer 3: p gradient (no ReLU on p)
+    if ((st = wgrad(gh, 2, n->p, n->gH2)) != HELM_OK) return st;
+    if ((st = dgrad(gh, CONV_F32CELLS, 2, n->gH2, n->gP, nullptr, 0)) != HELM_OK) return st;
     // a2 gradient: skip part + adjoint of avgpool2, masked by a2
-    skip_grad_kernel<<<nblk(B * c * vol), 256, 0, s>>>(n->gU + 2 * c * vol, 3 * c * vol, n->gH1, a2, 3 * c * vol, n->gA, c,
-                                                       B, Z, Y, X);
+    skip_grad_kernel<<<cell_blocks(gf, c), 256, 0, s>>>(gf, gh, floats(n->gU), floats(n->gP), cell_groups(c), cells(n->u),
+                                                        cell_groups(3 * c), 2 * c, c, cells(n->gC), cell_groups(c),
+                                                        G + n->boff[1]);
     // layer 2: a1 gradient with mask(a1)
-    wgrad(n, n->a1, c, c * vol, n->gA, c, c * vol, B, Z, Y, X, G + n->woff[1], G + n->boff[1], s);
-    conv<float, float>(n, n->gA, c, c * vol, W + n->woff[1], 1, nullptr, n->gB, c, c * vol, B, Z, Y, X, 0, n->a1, c * vol, n->status, s);
+    if ((st = wgrad(gf, 1, n->a1, n->gC)) != HELM_OK) return st;
+    if ((st = dgrad(gf, CONV_GRAD, 1, n->gC, n->gD, &n->a1, 0)) != HELM_OK) return st;
     // layer 1
-    wgrad(n, n->x, 5, 5 * vol, n->gB, c, c * vol, B, Z, Y, X, G + n->woff[0], G + n->boff[0], s);
+    if ((st = wgrad(gf, 0, n->x, n->gD)) != HELM_OK) return st;
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
 }
@@ -774,8 +743,8 @@ helm_status learned_pre(helm_ctx* c, const float2* r, const double* sigma, int s
     HELM_CUDA_TRY(cudaMemsetAsync(acc, 0, 2 * sizeof(double), s));
     HELM_CUDA_TRY(cudaMemsetAsync(acc + 6, 0, 4 * sizeof(double), s));
     sumsq_kernel<<<nblk(N), 256, 0, s>>>(r, N, acc);
-    feat_v_kernel<<<nblk(N), 256, 0, s>>>(r, acc, N, n->x, n->x + N, sigma, sidx, n->vbuf);
-    feat_contrast_kernel<<<nblk(N), 256, 0, s>>>(c->k2_f, (float)(1.0 / (c->k0 * c->k0)), N, n->x + 4 * N);
+    feat_v_kernel<<<nblk(N), 256, 0, s>>>(r, acc, N, cells(n->xp), cells(n->xp) + N, sigma, sidx, n->vbuf);
+    feat_contrast_kernel<<<nblk(N), 256, 0, s>>>(c->k2_f, (float)(1.0 / (c->k0 * c->k0)), N, cells(n->xp) + 4 * N);
     prof_end(c, s);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
@@ -789,9 +758,9 @@ helm_status learned_post(helm_ctx* c, float2* z, cudaStream_t s) {
     helm_status st;
     prof_begin(c, s, PROF_LEARNED);
     sumsq_kernel<<<nblk(N), 256, 0, s>>>(z, N, acc + 1);
-    feat_pair_kernel<<<nblk(N), 256, 0, s>>>(z, acc + 1, N, n->x + 2 * N, n->x + 3 * N);
-    forward(n, c->status_d, s);
-    make_c_kernel<<<nblk(N), 256, 0, s>>>(n->y, acc, N, n->cbuf);
+    feat_pair_kernel<<<nblk(N), 256, 0, s>>>(z, acc + 1, N, cells(n->xp) + 2 * N, cells(n->xp) + 3 * N);
+    if ((st = forward(n, cells(n->xp), floats(n->y), c->status_d, s)) != HELM_OK) return st;
+    make_c_kernel<<<nblk(N), 256, 0, s>>>(floats(n->y), acc, N, n->cbuf);
     prof_end(c, s);
     if ((st = launch_stencil_f32_cls(c, z, n->az0, nullptr, 0, PROF_LEARNED, s)) != HELM_OK) return st;
     if ((st = launch_stencil_f32_cls(c, n->cbuf, n->ac, nullptr, 0, PROF_LEARNED, s)) != HELM_OK) return st;
