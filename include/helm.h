@@ -386,11 +386,11 @@ helm_status helm_attach_net(helm_ctx* ctx, helm_net* net);
 helm_status helm_set_wait_limit(helm_ctx* ctx, long long polls);
 
 /* helm_set_matvec_variant - pin the kernel of the context's complex64 matvec (staggered grids of order 4
- * or 6; other contexts use the general stencil kernel whatever is set):
+ * or 6; other contexts use one kernel whatever is set):
  *   0  cp.async plane ring, one output per thread, four CTAs per SM
  *   1  TMA plane ring (even N_x; else as 0)
- *   2  cp.async plane ring, three CTAs per SM (the default for complex k^2)
- *   3  two outputs per thread, k^2 U in registers (real k^2; the default for a real medium; else as 2)
+ *   2  cp.async plane ring, three CTAs per SM
+ *   3  two outputs per thread (the default)
  *   4  as 3 with the sixth-order fields formed from a two-point-halo k^2 ring (real k^2, order 6; else as 3)
  * All compute the same operator (Eqs. scheme4/scheme6) in complex64; they differ in speed and bytes moved.
  * helm_autotune overrides the choice with the fastest.  Errors: HELM_ERR_ARG (NULL, out of range). */

@@ -12,19 +12,74 @@
 // it, so edge and corner ghosts come from the rule applied along an already-filled ghost line.
 // The closure's f part (U-independent) belongs to the right-hand side the caller supplies.
 //
-// Layout: the operand is copied into a padded array (nx+2) x (ny+2) x (nz+2), x fastest; the general
-// stencil kernels then read it with no ghost logic.  Per face two launches: V1 = L U_B into a scratch
-// face, then the ghost from U_I, U_B, V1 and L V1 (formed on the fly).  The arithmetic is FP64 whatever
-// the storage (complex64, complex128 or double-float): the faces are O(N^2) work.
+// Layout: the ghosts go into a padded array (nx+2) x (ny+2) x (nz+2), x fastest.  The complex64 matvec reads the
+// interior from the operand itself and only the shell from there; for the general kernels (complex128,
+// double-float) the operand is copied into the interior too.  Per face two launches: V1 = L U_B into a scratch face,
+// then the ghost from U_I, U_B, V1 and L V1 (formed on the fly).  The arithmetic is FP64 for complex128 and
+// double-float operands and double-float (about 44 bits) for complex64 ones, whose ghosts are rounded to FP32: the
+// faces are O(N^2) work, so a launch is a chain of latencies, and on GB300 the 34 conversions and 32 products of a
+// point in FP64 were the longest part of it.  The loads of a point are independent (eight per direction).
+// Measured at 100^3, complex64: 8 and 7 us per launch in FP64 with loops over the rows -> 5.1-5.8 us; the whole
+// matvec (its stencil kernel in stencil_fast.cu) 142 -> 64 us.
 #include "common.cuh"
+#include "dfloat.cuh"
 #include <cmath>
 #include <cstring>
 
 namespace {
 
+constexpr int HO_NT = 64;   // small blocks: a face has tens of thousands of points for 152 SMs
+
+// ---- arithmetic of the faces: FP64, or double-float for complex64 operands -------------------------------
+struct A64 {
+    typedef double2 V;    // value
+    typedef double S;     // real scalar
+    typedef double2 St;   // stored value (scratch faces)
+    static S cst(double v) { return v; }
+    static __device__ __forceinline__ S minus_one() { return -1.0; }
+    static __device__ __forceinline__ V zero() { return make_double2(0.0, 0.0); }
+    static __device__ __forceinline__ V add(V a, V b) { return make_double2(a.x + b.x, a.y + b.y); }
+    static __device__ __forceinline__ V mul(V a, S s) { return make_double2(a.x * s, a.y * s); }
+    static __device__ __forceinline__ V times_i(V a) { return make_double2(-a.y, a.x); }
+    static __device__ __forceinline__ V ld(const double2* p, long long i) { return p[i]; }
+    static __device__ __forceinline__ V ld(const float4* p, long long i) {
+        const float4 v = p[i];
+        return make_double2((double)v.x + (double)v.z, (double)v.y + (double)v.w);
+    }
+    static __device__ __forceinline__ void st(double2* p, long long i, V v) { p[i] = v; }
+    static __device__ __forceinline__ void st(float4* p, long long i, V v) {
+        const float rh = (float)v.x, ih = (float)v.y;
+        p[i] = make_float4(rh, ih, (float)(v.x - (double)rh), (float)(v.y - (double)ih));
+    }
+};
+struct ADF {
+    typedef cdf V;
+    typedef df S;
+    typedef float4 St;
+    static S cst(double v) {
+        const float h = (float)v;
+        return df{h, (float)(v - (double)h)};
+    }
+    static __device__ __forceinline__ S minus_one() { return df{-1.f, 0.f}; }
+    static __device__ __forceinline__ V zero() { return cdf_zero(); }
+    static __device__ __forceinline__ V add(V a, V b) { return cdf_add(a, b); }
+    static __device__ __forceinline__ V mul(V a, S s) { return cdf_scale(a, s); }
+    static __device__ __forceinline__ V times_i(V a) {
+        return cdf{make_float2(-a.hi.y, a.hi.x), make_float2(-a.lo.y, a.lo.x)};
+    }
+    static __device__ __forceinline__ V ld(const float2* p, long long i) { return cdf_from_f2(p[i]); }
+    static __device__ __forceinline__ V ld(const float4* p, long long i) { return cdf_from4(p[i]); }
+    static __device__ __forceinline__ void st(float2* p, long long i, V v) { p[i] = cdf_round(v); }
+    static __device__ __forceinline__ void st(float4* p, long long i, V v) { p[i] = cdf_to4(v); }
+};
+template <class M> struct ArithOf { typedef A64 T; };
+template <> struct ArithOf<float2> { typedef ADF T; };
+
+// Rows of the second-derivative stencils (times h^2) over eight consecutive nodes: nodes 0, 1, 2 of a line
+// (one-sided), inner nodes (seven centred weights and a zero), node n - 4 (a zero and the seven), nodes n - 3 .. n - 1
+template <class A>
 struct Wts {
-    double wl[3][8];     // rows 0, 1, 2 of the one-sided stencils (second derivative, times 1/h^2)
-    double wc[7];        // centred seven-point stencil
+    typename A::S w[8][8];
 };
 
 struct Face {
@@ -33,71 +88,60 @@ struct Face {
     int sa0, sb0;        // first padded coordinate along ta, tb
     long long sn, sa, sb;  // padded strides along the normal and the tangential axes
     int nb_lo, nb_hi;    // padded normal index of the two boundary planes (1 and n)
-    double iha2, ihb2;   // 1/h_ta^2, 1/h_tb^2
-    double c0, c1, c2;   // Taylor weights of the normal step
-    double k0;
+};
+template <class A>
+struct FaceC {
+    typename A::S iha2, ihb2;      // 1/h_ta^2, 1/h_tb^2
+    typename A::S c0, mc1, c2;     // Taylor weights of the normal step (c_1 negated)
+    typename A::S c1, k0, kk, mkk; // c_1, k0, k0^2, -k0^2
 };
 
-__device__ __forceinline__ double2 ld2(const float2* p, long long i) { const float2 v = p[i]; return make_double2(v.x, v.y); }
-__device__ __forceinline__ double2 ld2(const double2* p, long long i) { return p[i]; }
-__device__ __forceinline__ double2 ld2(const float4* p, long long i) {
-    const float4 v = p[i];
-    return make_double2((double)v.x + (double)v.z, (double)v.y + (double)v.w);
-}
-__device__ __forceinline__ void st2(float2* p, long long i, double2 v) { p[i] = make_float2((float)v.x, (float)v.y); }
-__device__ __forceinline__ void st2(double2* p, long long i, double2 v) { p[i] = v; }
-__device__ __forceinline__ void st2(float4* p, long long i, double2 v) {
-    const float rh = (float)v.x, ih = (float)v.y;
-    p[i] = make_float4(rh, ih, (float)(v.x - (double)rh), (float)(v.y - (double)ih));
+// the row of node i on a line of n nodes, and its first node
+__device__ __forceinline__ int lap_row(int i, int n, int& first) {
+    first = min(max(i - 3, 0), n - 8);
+    return i < 3 ? i : (i <= n - 5 ? 3 : i - (n - 8));
 }
 
-// Stencil row of node i on a line of n nodes: fills idx/w, returns the count (7 centred or 8 one-sided).
-__device__ __forceinline__ int lap_row(const Wts& W, int i, int n, int* idx, double* w) {
-    if (i >= 3 && i <= n - 4) {
+// L V at face point (ia, ib): at(ia, ib) gives V
+template <class A, class At>
+__device__ __forceinline__ typename A::V apply_L(const Face& f, const FaceC<A>& k, const Wts<A>& W, const At& at, int ia, int ib) {
+    int sa, sb;
+    const int ra = lap_row(ia, f.la, sa), rb = lap_row(ib, f.lb, sb);
+    typename A::V ua[8], ub[8];
+    const typename A::V v = at(ia, ib);
 #pragma unroll
-        for (int k = 0; k < 7; ++k) { idx[k] = i - 3 + k; w[k] = W.wc[k]; }
-        return 7;
+    for (int q = 0; q < 8; ++q) {
+        ua[q] = at(sa + q, ib);
+        ub[q] = at(ia, sb + q);
     }
-    if (i < 3) {
+    typename A::V s = A::zero(), t = s;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) { idx[k] = k; w[k] = W.wl[i][k]; }
-        return 8;
+    for (int q = 0; q < 8; ++q) {
+        s = A::add(s, A::mul(ua[q], W.w[ra][q]));
+        t = A::add(t, A::mul(ub[q], W.w[rb][q]));
     }
-    // mirror image of the left rows
-    const int r = n - 1 - i;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) { idx[k] = n - 1 - k; w[k] = W.wl[r][k]; }
-    return 8;
+    return A::add(A::mul(v, k.kk), A::add(A::mul(s, k.iha2), A::mul(t, k.ihb2)));
 }
 
-// L V at face point (ia, ib) for a face stored with strides (fa, fb) from base p
+// The operand with its ghosts: the interior from U (from P where U is NULL), the shell from the padded P
 template <class M>
-__device__ __forceinline__ double2 apply_L(const Face& f, const Wts& W, const M* p, long long base, long long fa,
-                                           long long fb, int ia, int ib) {
-    int idx[8];
-    double w[8];
-    double2 v = ld2(p, base + ia * fa + ib * fb);
-    double2 acc = make_double2(f.k0 * f.k0 * v.x, f.k0 * f.k0 * v.y);
-    int n = lap_row(W, ia, f.la, idx, w);
-    double2 s = make_double2(0.0, 0.0);
-    for (int k = 0; k < n; ++k) {
-        const double2 u = ld2(p, base + idx[k] * fa + ib * fb);
-        s.x += w[k] * u.x; s.y += w[k] * u.y;
+struct Operand {
+    const M* U;
+    const M* P;
+    int nx, ny, nz;
+    typedef typename ArithOf<M>::T A;
+    // padded coordinates
+    __device__ __forceinline__ typename A::V at(int X, int Y, int Z) const {
+        if (U && X >= 1 && X <= nx && Y >= 1 && Y <= ny && Z >= 1 && Z <= nz)
+            return A::ld(U, ((long long)(Z - 1) * ny + (Y - 1)) * nx + (X - 1));
+        return A::ld(P, ((long long)Z * (ny + 2) + Y) * (nx + 2) + X);
     }
-    acc.x += s.x * f.iha2; acc.y += s.y * f.iha2;
-    n = lap_row(W, ib, f.lb, idx, w);
-    s = make_double2(0.0, 0.0);
-    for (int k = 0; k < n; ++k) {
-        const double2 u = ld2(p, base + ia * fa + idx[k] * fb);
-        s.x += w[k] * u.x; s.y += w[k] * u.y;
+    // point (ia, ib) of the face's plane with normal index n
+    __device__ __forceinline__ typename A::V face(const Face& f, int n, int ia, int ib) const {
+        const int a = ia + f.sa0, b = ib + f.sb0;
+        return f.axis == 0 ? at(n, b, a) : (f.axis == 1 ? at(b, n, a) : at(b, a, n));
     }
-    acc.x += s.x * f.ihb2; acc.y += s.y * f.ihb2;
-    return acc;
-}
-
-__device__ __forceinline__ long long plane_base(const Face& f, int plane) {
-    return plane * f.sn + f.sa0 * f.sa + f.sb0 * f.sb;
-}
+};
 
 // copy the operand into the interior of the padded array
 template <class M>
@@ -112,49 +156,50 @@ __global__ void ho_copy_kernel(int nx, int ny, int nz, const M* __restrict__ U, 
 }
 
 // S[side][ia][ib] = L U_B on both boundary planes of one direction
-template <class M>
-__global__ void ho_lap_kernel(Face f, Wts W, const M* __restrict__ P, double2* __restrict__ S) {
-    const long long per = (long long)f.la * f.lb;
-    const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+template <class M, class A>
+__global__ void __launch_bounds__(HO_NT) ho_lap_kernel(const __grid_constant__ Face f, const __grid_constant__ FaceC<A> k,
+                                                       const __grid_constant__ Wts<A> W, const Operand<M> op,
+                                                       typename A::St* __restrict__ S) {
+    const int per = f.la * f.lb;
+    const int id = blockIdx.x * HO_NT + threadIdx.x;
     if (id >= 2 * per) return;
-    const int side = (int)(id / per);
-    const long long q = id - side * per;
-    const int ia = (int)(q / f.lb), ib = (int)(q % f.lb);
-    const long long base = plane_base(f, side ? f.nb_hi : f.nb_lo);
-    S[id] = apply_L(f, W, P, base, f.sa, f.sb, ia, ib);
+    const int side = id >= per, q = id - side * per;
+    const int n = side ? f.nb_hi : f.nb_lo;
+    A::st(S, id, apply_L<A>(f, k, W, [&](int ia, int ib) { return op.face(f, n, ia, ib); }, q / f.lb, q % f.lb));
 }
 
 // U_G = U_I + i k0 (c0 U_B - c1 L U_B + c2 L^2 U_B) on both ghost planes of one direction, plus (when fd
-// is given) the f part s [c1 f_n + c2 (f_nnn - k0^2 f_n - lap_T f_n)], s = -1 near face, +1 far face;
+// is given; FP64 only) the f part s [c1 f_n + c2 (f_nnn - k0^2 f_n - lap_T f_n)], s = -1 near face, +1 far face;
 // fd holds [side][field][ia][ib] with the fields f_n, f_nnn, lap_T f_n (derivatives along the axis).
-template <class M>
-__global__ void ho_ghost_kernel(Face f, Wts W, M* __restrict__ P, const double2* __restrict__ S,
-                                const double2* __restrict__ fd) {
-    const long long per = (long long)f.la * f.lb;
-    const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+template <class M, class A>
+__global__ void __launch_bounds__(HO_NT) ho_ghost_kernel(const __grid_constant__ Face f, const __grid_constant__ FaceC<A> k,
+                                                         const __grid_constant__ Wts<A> W, const Operand<M> op, M* P,
+                                                         const typename A::St* __restrict__ S,
+                                                         const double2* __restrict__ fd) {
+    typedef typename A::V V;
+    const int per = f.la * f.lb;
+    const int id = blockIdx.x * HO_NT + threadIdx.x;
     if (id >= 2 * per) return;
-    const int side = (int)(id / per);
-    const long long q = id - side * per;
-    const int ia = (int)(q / f.lb), ib = (int)(q % f.lb);
+    const int side = id >= per, q = id - side * per;
+    const int ia = q / f.lb, ib = q % f.lb;
     const int pb = side ? f.nb_hi : f.nb_lo;
     const int pi = side ? pb - 1 : pb + 1;
     const int pg = side ? pb + 1 : pb - 1;
-    const long long off = ia * f.sa + ib * f.sb;
-    const double2 ub = ld2(P, plane_base(f, pb) + off);
-    const double2 ui = ld2(P, plane_base(f, pi) + off);
-    const double2 v1 = S[id];
-    const double2 v2 = apply_L(f, W, S, side * per, (long long)f.lb, 1LL, ia, ib);
-    const double2 t = make_double2(f.c0 * ub.x - f.c1 * v1.x + f.c2 * v2.x, f.c0 * ub.y - f.c1 * v1.y + f.c2 * v2.y);
-    // i k0 t
-    double2 g = make_double2(ui.x - f.k0 * t.y, ui.y + f.k0 * t.x);
-    if (fd) {
-        const long long fb = (long long)side * 3 * per + q;
-        const double2 fn = fd[fb], fnnn = fd[fb + per], flt = fd[fb + 2 * per];
-        const double sg = side ? 1.0 : -1.0, kk = f.k0 * f.k0;
-        g.x += sg * (f.c1 * fn.x + f.c2 * (fnnn.x - kk * fn.x - flt.x));
-        g.y += sg * (f.c1 * fn.y + f.c2 * (fnnn.y - kk * fn.y - flt.y));
+    const typename A::St* __restrict__ L1 = S + (long long)side * per;
+    const V ub = op.face(f, pb, ia, ib), ui = op.face(f, pi, ia, ib);
+    const V v1 = A::ld(L1, q);
+    const V v2 = apply_L<A>(f, k, W, [&](int a, int b) { return A::ld(L1, a * f.lb + b); }, ia, ib);
+    const V t = A::add(A::mul(ub, k.c0), A::add(A::mul(v1, k.mc1), A::mul(v2, k.c2)));
+    V g = A::add(ui, A::times_i(A::mul(t, k.k0)));
+    if constexpr (sizeof(typename A::S) == sizeof(double) && sizeof(M) == sizeof(double2)) {
+        if (fd) {
+            const long long fb = (long long)side * 3 * per + q;
+            const V fn = A::ld(fd, fb), fnnn = A::ld(fd, fb + per), flt = A::ld(fd, fb + 2 * per);
+            const V part = A::add(A::mul(fn, k.c1), A::mul(A::add(fnnn, A::add(A::mul(fn, k.mkk), A::mul(flt, A::minus_one()))), k.c2));
+            g = A::add(g, side ? part : A::mul(part, A::minus_one()));
+        }
     }
-    st2(P, plane_base(f, pg) + off, g);
+    A::st(P, pg * f.sn + (ia + f.sa0) * f.sa + (ib + f.sb0) * f.sb, g);
 }
 
 // Second-derivative weights on offsets o_k (Taylor conditions sum_k w_k o_k^q / q! = [q == 2]), FP64
@@ -183,16 +228,39 @@ void fd_weights(const double* o, int n, double* w) {
     }
 }
 
-Wts make_weights() {
-    Wts W;
-    double o[8];
+template <class A>
+Wts<A> make_weights() {
+    Wts<A> W;
+    double o[8], wc[7], w[8][8] = {};
     for (int k = 0; k < 7; ++k) o[k] = k - 3;
-    fd_weights(o, 7, W.wc);
+    fd_weights(o, 7, wc);
+    for (int k = 0; k < 7; ++k) w[3][k] = w[4][k + 1] = wc[k];
     for (int i = 0; i < 3; ++i) {
+        double wl[8];
         for (int k = 0; k < 8; ++k) o[k] = k - i;
-        fd_weights(o, 8, W.wl[i]);
+        fd_weights(o, 8, wl);
+        for (int k = 0; k < 8; ++k) w[i][k] = w[7 - i][7 - k] = wl[k];   // the right rows mirror the left ones
     }
+    for (int r = 0; r < 8; ++r)
+        for (int k = 0; k < 8; ++k) W.w[r][k] = A::cst(w[r][k]);
     return W;
+}
+
+template <class A>
+FaceC<A> make_face_consts(const helm_ctx* c, int axis) {
+    const int ta = axis == 2 ? 1 : 2, tb = axis == 0 ? 1 : 0;
+    const double h = c->h[axis], c1 = 2.0 * h * h * h / 6.0;
+    FaceC<A> k;
+    k.iha2 = A::cst(1.0 / (c->h[ta] * c->h[ta]));
+    k.ihb2 = A::cst(1.0 / (c->h[tb] * c->h[tb]));
+    k.c0 = A::cst(2.0 * h);
+    k.c1 = A::cst(c1);
+    k.mc1 = A::cst(-c1);
+    k.c2 = A::cst(2.0 * h * h * h * h * h / 120.0);
+    k.k0 = A::cst(c->k0);
+    k.kk = A::cst(c->k0 * c->k0);
+    k.mkk = A::cst(-c->k0 * c->k0);
+    return k;
 }
 
 Face make_face(const helm_ctx* c, int axis) {
@@ -209,36 +277,34 @@ Face make_face(const helm_ctx* c, int axis) {
     f.sb0 = tb < axis ? 0 : 1;
     f.sn = st[axis]; f.sa = st[ta]; f.sb = st[tb];
     f.nb_lo = 1; f.nb_hi = n[axis];
-    f.iha2 = 1.0 / (c->h[ta] * c->h[ta]);
-    f.ihb2 = 1.0 / (c->h[tb] * c->h[tb]);
-    const double h = c->h[axis];
-    f.c0 = 2.0 * h;
-    f.c1 = 2.0 * h * h * h / 6.0;
-    f.c2 = 2.0 * h * h * h * h * h / 120.0;
-    f.k0 = c->k0;
     return f;
 }
 
-// U = nullptr: the interior is zero (the f part of the closure alone); faces = nullptr: no f part.
+// The ghost shell of P.  copy: also U into the interior of P (which then holds the whole operand); U = nullptr: the
+// interior is zero (the f part of the closure alone); faces = nullptr: no f part.
 template <class M>
-helm_status fill(helm_ctx* c, const M* U, M* P, const double2* faces, cudaStream_t s) {
-    if (U) {
+helm_status fill(helm_ctx* c, const M* U, M* P, const double2* faces, bool copy, cudaStream_t s) {
+    if (!U) {
+        HELM_CUDA_TRY(cudaMemsetAsync(P, 0, (size_t)(c->nx + 2) * (c->ny + 2) * (c->nz + 2) * sizeof(M), s));
+    } else if (copy) {
         ho_copy_kernel<M><<<1024, 256, 0, s>>>(c->nx, c->ny, c->nz, U, P);
         HELM_CUDA_TRY(cudaGetLastError());
-    } else {
-        HELM_CUDA_TRY(cudaMemsetAsync(P, 0, (size_t)(c->nx + 2) * (c->ny + 2) * (c->nz + 2) * sizeof(M), s));
     }
-    static const Wts W = make_weights();   // the same for every grid (weights times 1/h^2 per face)
+    typedef typename ArithOf<M>::T A;
+    static const Wts<A> W = make_weights<A>();   // the same for every grid (weights times 1/h^2 per face)
+    typename A::St* S = reinterpret_cast<typename A::St*>(c->ho_S);   // 16 bytes a value either way
+    const Operand<M> op = {U, P, c->nx, c->ny, c->nz};
     long long foff = 0;
     for (int axis = 0; axis < 3; ++axis) {
         const Face f = make_face(c, axis);
-        const long long tot = 2LL * f.la * f.lb;
-        const unsigned blocks = (unsigned)((tot + 255) / 256);
-        ho_lap_kernel<M><<<blocks, 256, 0, s>>>(f, W, P, c->ho_S);
+        const int tot = 2 * f.la * f.lb;
+        const unsigned blocks = (unsigned)((tot + HO_NT - 1) / HO_NT);
+        const FaceC<A> k = make_face_consts<A>(c, axis);
+        ho_lap_kernel<M, A><<<blocks, HO_NT, 0, s>>>(f, k, W, op, S);
         HELM_CUDA_TRY(cudaGetLastError());
-        ho_ghost_kernel<M><<<blocks, 256, 0, s>>>(f, W, P, c->ho_S, faces ? faces + foff : nullptr);
+        ho_ghost_kernel<M, A><<<blocks, HO_NT, 0, s>>>(f, k, W, op, P, S, faces ? faces + foff : nullptr);
         HELM_CUDA_TRY(cudaGetLastError());
-        foff += 3 * tot;
+        foff += 3LL * tot;
     }
     return HELM_OK;
 }
@@ -260,15 +326,15 @@ size_t closure_face_points(const helm_ctx* c) {
     return tot;
 }
 
-helm_status closure_fill_f32(helm_ctx* c, const float2* U, cudaStream_t s) { return fill(c, U, c->ho_P32, nullptr, s); }
-helm_status closure_fill_f64(helm_ctx* c, const double2* U, cudaStream_t s) { return fill(c, U, c->ho_P64, nullptr, s); }
-helm_status closure_fill_df(helm_ctx* c, const float4* U, cudaStream_t s) { return fill(c, U, c->ho_Pdf, nullptr, s); }
+helm_status closure_fill_f32(helm_ctx* c, const float2* U, bool copy, cudaStream_t s) { return fill(c, U, c->ho_P32, nullptr, copy, s); }
+helm_status closure_fill_f64(helm_ctx* c, const double2* U, cudaStream_t s) { return fill(c, U, c->ho_P64, nullptr, true, s); }
+helm_status closure_fill_df(helm_ctx* c, const float4* U, cudaStream_t s) { return fill(c, U, c->ho_Pdf, nullptr, true, s); }
 
 // F_out = F_in - A(G_f), G_f the ghosts of the closure's f part with a zero interior (FP64)
 helm_status closure_rhs(helm_ctx* c, const double2* faces, const double2* Fin, double2* Fout, cudaStream_t s) {
     double2* y = nullptr;
     if (cudaMalloc(&y, c->npts * sizeof(double2)) != cudaSuccess) { cudaGetLastError(); return HELM_ERR_NOMEM; }
-    helm_status st = fill<double2>(c, nullptr, c->ho_P64, faces, s);
+    helm_status st = fill<double2>(c, nullptr, c->ho_P64, faces, false, s);
     if (st == HELM_OK) st = launch_stencil_f64_padded(c, c->ho_P64, y, s);
     if (st == HELM_OK) {
         sub_kernel<<<1024, 256, 0, s>>>(Fin, y, Fout, c->npts);

@@ -169,7 +169,8 @@ struct helm_ctx {
 // stencil.cu
 helm_status launch_derived_fields(helm_ctx* c, cudaStream_t s);
 // closure.cu: padded operand with the high-order collocated closure ghosts
-helm_status closure_fill_f32(helm_ctx* c, const float2* U, cudaStream_t s);
+// (complex64: the ghost shell, and with `copy` the operand in the interior too)
+helm_status closure_fill_f32(helm_ctx* c, const float2* U, bool copy, cudaStream_t s);
 helm_status closure_fill_f64(helm_ctx* c, const double2* U, cudaStream_t s);
 helm_status closure_fill_df(helm_ctx* c, const float4* U, cudaStream_t s);
 void closure_release(helm_ctx* c);
@@ -198,6 +199,9 @@ helm_status launch_residual_fast(helm_ctx* c, const float4* x, const float4* F, 
 bool stencil_fast_supported(const helm_ctx* c);
 helm_status launch_stencil_fast(helm_ctx* c, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s,
                                 int nb = 1);
+// collocated grids with the high-order closure, orders 4 and 6: the operand x with its ghosts in the shell of the
+// context's padded array (x = NULL: the whole operand is there)
+helm_status launch_stencil_padded(helm_ctx* c, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s);
 // eig.cu
 helm_status run_eig_setup(helm_ctx* c, cudaStream_t s);
 // gemm_simt.cu

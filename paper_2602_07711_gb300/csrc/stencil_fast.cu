@@ -67,8 +67,10 @@ struct FParams {
     float h2_20, h_20, hh6;       // order 6: h^2/20, h/20, h^2/6
     const float2* k2;
     const float2* fld[4];         // G, g_x, g_y, g_z (order 6)
+    const float2* pad = nullptr;  // padded operand (PAD)
     const float* k2r;             // real k^2 (real-medium kernels)
     const float4* fr;             // real (G, g_x, g_y, g_z) per point (real-medium kernels, order 6)
+    int zch = FZCH;               // planes per CTA
     int nb = 1;                   // vectors in one launch (the right-hand sides of a batch group), npts apart;
                                   // blockIdx.z = z chunk * nb + vector
     float i12h[3], i12h2[3];      // 1/(12 h_d), 1/(12 h_d^2): the in-kernel sixth-order fields
@@ -99,7 +101,8 @@ __device__ __forceinline__ float2 f2mul(float2 a, float2 b) {
     return fma2(make_float2(-a.y, a.y), swap2(b), mul2(bc2(a.x), b));
 }
 
-template <int ORDER, int MINB, bool RK = false>
+// RT: chunks of p.zch planes (small grids, fast_chunk), else FZCH.
+template <int ORDER, int MINB, bool RK = false, bool RT = false>
 __global__ void __launch_bounds__(FNT, MINB)
 stencil_fast_kernel(FParams p, const float2* __restrict__ U, float2* __restrict__ Y, const double* __restrict__ sigma,
                     int sidx) {
@@ -109,8 +112,9 @@ stencil_fast_kernel(FParams p, const float2* __restrict__ U, float2* __restrict_
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * FTX + tx;
     const int x0 = blockIdx.x * FTX, y0 = blockIdx.y * FTY;
     const int vb = blockIdx.z % p.nb;   // the vector of the batch this CTA works on
-    const int z0 = (blockIdx.z / p.nb) * FZCH;
-    const int z1 = min(z0 + FZCH, p.nz);
+    const int zch = RT ? p.zch : FZCH;
+    const int z0 = (blockIdx.z / p.nb) * zch;
+    const int z1 = min(z0 + zch, p.nz);
     const int gx = x0 + tx, gy = y0 + ty;
     const bool active = gx < p.nx && gy < p.ny;
     const float sg = sigma ? (float)sigma[sidx] : 1.f;
@@ -276,34 +280,66 @@ stencil_fast_kernel(FParams p, const float2* __restrict__ U, float2* __restrict_
     }
 }
 
-// Two rows per thread (real media): the kernel above is bound by shared-memory traffic (each point reads a
+// Two rows per thread: the kernel above is bound by shared-memory traffic (each point reads a
 // 3 x 3 patch of U and of KU per plane, and KU is written once per staged point).  Here a thread computes
-// the points (x, 2 t) and (x, 2 t + 1) of the same 32 x 8 tile from one 4 x 3 patch of U and of the real
+// the points (x, 2 t) and (x, 2 t + 1) of the same 32 x 8 tile from one 4 x 3 patch of U and of
 // k^2 (a third fewer reads per point) and forms k^2 U itself, so no KU plane is written; the ghost factors
 // are applied in shared memory only by tiles that touch the boundary (and on the ghost planes), so interior
 // tiles take one barrier per plane.  128 threads per CTA, each staging three halo points.
-template <int ORDER>
+// The sixth-order fields of a point serve its own thread alone, so they stay out of shared memory: each thread
+// loads those of plane P + 1 into registers while it works on plane P (139 -> 136 us at 256^3, order 6, real).
+// RK: real k^2 and fields; without (a medium with attenuation) k^2 and the fields are complex, and the complex
+// products k^2 U (with their register moves, six per point here) are formed once per staged point in a pass of their
+// own: 200^3, order 6, 120 us against 135 us for the kernel above (three CTAs per SM: at four the registers spill,
+// 243 us).
+// PAD (collocated grids, high-order closure): the ghosts are read from the shell of the padded array p.pad
+// ((nx+2)(ny+2)(nz+2) points; closure.cu), the interior from U (from p.pad where U is NULL), and k^2 is reflected
+// about the boundary nodes, so no ghost factors apply: 100^3, order 6, 26 us (caches cold) against 82 us for the
+// general kernel and 7 us for the copy of the operand it needs.  The fourth-order form then sums second differences of neighbours
+// ((lo - mid) + (hi - mid)) instead of the planes' separate contributions: fine grids (60 points per wavelength)
+// cancel so much that the latter lost a digit against the general kernel.
+template <bool RK = true>
 struct F2Stage {
     float2 u[FHALO];
     float kr[FHALO];
-    float4 f4[ORDER == 6 ? FNT : 1];   // G, g_x, g_y, g_z at the tile's points
+};
+template <>
+struct F2Stage<false> {
+    float2 u[FHALO];
+    float2 k[FHALO];
+};
+// (G, g_x, g_y, g_z) of a point, real or complex
+template <bool RK>
+struct Fields {
+    float4 f;
+    __device__ __forceinline__ void load(const FParams& p, size_t g) { f = p.fr[g]; }
+};
+template <>
+struct Fields<false> {
+    float2 f[4];
+    __device__ __forceinline__ void load(const FParams& p, size_t g) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) f[q] = p.fld[q][g];
+    }
 };
 constexpr int F2T = FNT / 2;
-template <int ORDER>
-size_t fast2_smem() { return FNS * sizeof(F2Stage<ORDER>); }
+template <bool RK = true>
+size_t fast2_smem() { return FNS * sizeof(F2Stage<RK>); }
+constexpr int fast2_minb(int order, bool rk) { return order == 6 && !rk ? 3 : 4; }
 
-template <int ORDER, int MINB>
-__global__ void __launch_bounds__(F2T, MINB)
+template <int ORDER, bool RK = true, bool PAD = false, bool RT = false>
+__global__ void __launch_bounds__(F2T, fast2_minb(ORDER, RK))
 stencil_fast2_kernel(FParams p, const float2* __restrict__ U, float2* __restrict__ Y, const double* __restrict__ sigma,
                      int sidx) {
     extern __shared__ __align__(16) unsigned char fsm[];
-    using Stage = F2Stage<ORDER>;
+    using Stage = F2Stage<RK>;
     Stage* ring = reinterpret_cast<Stage*>(fsm);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * FTX + tx;   // ty = 0 .. 3
     const int x0 = blockIdx.x * FTX, y0 = blockIdx.y * FTY;
     const int vb = blockIdx.z % p.nb;
-    const int z0 = (blockIdx.z / p.nb) * FZCH;
-    const int z1 = min(z0 + FZCH, p.nz);
+    const int zch = RT ? p.zch : FZCH;
+    const int z0 = (blockIdx.z / p.nb) * zch;
+    const int z1 = min(z0 + zch, p.nz);
     const int gx = x0 + tx, gy0 = y0 + 2 * ty;
     const bool act[2] = {gx < p.nx && gy0 < p.ny, gx < p.nx && gy0 + 1 < p.ny};
     // the tile's halo reaches a ghost point in x or y (its interior points never need a ghost factor)
@@ -314,38 +350,44 @@ stencil_fast2_kernel(FParams p, const float2* __restrict__ U, float2* __restrict
         U += off;
         Y += off;
     }
-    unsigned sl[3] = {0u, 0u, 0u};
+    // PAD: sl = the offset in a plane of k^2 and of U, ul that in a padded plane, bit 31 = U is read there
+    unsigned sl[3] = {0u, 0u, 0u}, ul[3] = {0u, 0u, 0u};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const int q = tid + k * F2T;
         if (q < FHALO) {
             const int ly = q / FPX, lx = q - ly * FPX;
             const int Xg = x0 + lx - 1, Yg = y0 + ly - 1;
+            if (PAD) {
+                // points beyond the far ghosts are staged for nobody: any address inside will do
+                const int Xk = Xg < 0 ? 1 : (Xg >= p.nx ? p.nx - 2 : Xg), Yk = Yg < 0 ? 1 : (Yg >= p.ny ? p.ny - 2 : Yg);
+                sl[k] = (unsigned)(Yk * p.nx + Xk);
+                ul[k] = (unsigned)((min(Yg, p.ny) + 1) * (p.nx + 2) + min(Xg, p.nx) + 1) |
+                        (!U || Xg < 0 || Xg >= p.nx || Yg < 0 || Yg >= p.ny ? 1u << 31 : 0u);
+                continue;
+            }
             const int Xc = min(max(Xg, 0), p.nx - 1), Yc = min(max(Yg, 0), p.ny - 1);
             sl[k] = (unsigned)(Yc * p.nx + Xc) | (Xc != Xg ? 1u << 30 : 0u) | (Yc != Yg ? 1u << 31 : 0u);
         }
     }
     const size_t plane = (size_t)p.nx * p.ny;
     const int poff = gy0 * p.nx + gx;
-    const int fi = (2 * ty) * FTX + tx;   // the fields of point r at f4[fi + r FTX]
 
     auto issue = [&](int P) {
         if (P <= z1) {
             Stage& S = ring[(P + FNS) % FNS];
-            const int Pc = min(max(P, 0), p.nz - 1);
+            const int Pc = PAD ? (P < 0 ? 1 : (P >= p.nz ? p.nz - 2 : P)) : min(max(P, 0), p.nz - 1);
             const float2* Ub = U + (size_t)Pc * plane;
-            const float* Kb = p.k2r + (size_t)Pc * plane;
+            const float2* Pb = PAD ? p.pad + (size_t)(P + 1) * (p.nx + 2) * (p.ny + 2) : nullptr;
+            const bool shell = PAD && (P < 0 || P >= p.nz);
 #pragma unroll
             for (int k = 0; k < 3; ++k)
                 if (tid + k * F2T < FHALO) {
-                    cp8(&S.u[tid + k * F2T], Ub + (sl[k] & 0x3FFFFFFFu));
-                    cp4(&S.kr[tid + k * F2T], Kb + (sl[k] & 0x3FFFFFFFu));
+                    const unsigned o = sl[k] & 0x3FFFFFFFu;
+                    cp8(&S.u[tid + k * F2T], PAD && (shell || ul[k] >> 31) ? Pb + (ul[k] & 0x7FFFFFFFu) : Ub + o);
+                    if constexpr (RK) cp4(&S.kr[tid + k * F2T], p.k2r + (size_t)Pc * plane + o);
+                    else cp8(&S.k[tid + k * F2T], p.k2 + (size_t)Pc * plane + o);
                 }
-            if (ORDER == 6 && P >= z0 && P < z1) {
-                const size_t g = (size_t)P * plane + poff;
-                if (act[0]) cp16f(&S.f4[fi], p.fr + g);
-                if (act[1]) cp16f(&S.f4[fi + FTX], p.fr + g + p.nx);
-            }
         }
         cp_commit();
     };
@@ -356,23 +398,40 @@ stencil_fast2_kernel(FParams p, const float2* __restrict__ U, float2* __restrict
         cA[r] = cX[r] = cY[r] = cZ[r] = make_float2(0, 0);
         nA[r] = nX[r] = nY[r] = nZ[r] = make_float2(0, 0);
     }
+    Fields<RK> fn[2], fm[2], fp[2];   // order 6: the fields of planes P + 1, P and P - 1
     issue(z0 - 1);
     issue(z0);
     for (int P = z0 - 1; P <= z1; ++P) {
         Stage& S = ring[(P + FNS) % FNS];
+        if (ORDER == 6) {
+            const size_t g = (size_t)(P + 1) * plane + poff;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                fp[r] = fm[r];
+                fm[r] = fn[r];
+                if (P + 1 < z1 && act[r]) fn[r].load(p, g + r * p.nx);
+            }
+        }
         cp_wait1();
         __syncthreads();          // plane P landed for everyone; everyone is done with planes P-1 and P-2
         const bool zghost = P < 0 || P >= p.nz;
-        if (edge || zghost) {     // uniform per CTA and plane
+        if (!RK || (!PAD && (edge || zghost))) {     // uniform per CTA and plane
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const int q = tid + k * F2T;
-                if (q < FHALO && ((sl[k] >> 30) || zghost)) {
+                if (q < FHALO) {
+                    const bool ghost = !PAD && ((sl[k] >> 30) || zghost);
+                    if constexpr (RK) {
+                        if (!ghost) continue;
+                    }
                     float2 u = S.u[q];
-                    if (sl[k] & (1u << 30)) u = f2mul(u, p.gx);
-                    if (sl[k] & (1u << 31)) u = f2mul(u, p.gy);
-                    if (zghost) u = f2mul(u, p.gz);
-                    S.u[q] = u;
+                    if (ghost) {
+                        if (sl[k] & (1u << 30)) u = f2mul(u, p.gx);
+                        if (sl[k] & (1u << 31)) u = f2mul(u, p.gy);
+                        if (zghost) u = f2mul(u, p.gz);
+                        S.u[q] = u;
+                    }
+                    if constexpr (!RK) S.k[q] = f2mul(S.k[q], u);
                 }
             }
             __syncthreads();
@@ -385,11 +444,12 @@ stencil_fast2_kernel(FParams p, const float2* __restrict__ U, float2* __restrict
             for (int a = 0; a < 3; ++a) {
                 const int i = (2 * ty + b) * FPX + tx + a;
                 u[b][a] = S.u[i];
-                kv[b][a] = f2scl(u[b][a], S.kr[i]);   // KU = k^2 U (k^2 at a ghost point is the mirror value)
+                // KU = k^2 U (k^2 at a ghost point is the mirror value)
+                if constexpr (RK) kv[b][a] = f2scl(u[b][a], S.kr[i]);
+                else kv[b][a] = S.k[i];
             }
         const bool out_prev = P - 1 >= z0 && P - 1 < z1;
         const bool do_mid = P >= z0 && P < z1;
-        const Stage& Sp = ring[(P - 1 + FNS) % FNS];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const float2 c = u[r + 1][1];
@@ -408,10 +468,17 @@ stencil_fast2_kernel(FParams p, const float2* __restrict__ U, float2* __restrict
                 const float2 Zs = f2add(f2fma(p.hh6, kc, c), f2scl(f2fma(-4.f, c, f2add(fx, fy)), 1.f / 6.f));
                 if (out_prev) {
                     const float2 A = f2add(cA[r], As);
-                    const float4 fv = Sp.f4[fi + r * FTX];
-                    float2 g = f2scl(f2add(cX[r], Xs), fv.y);
-                    g = f2fma(fv.z, f2add(cY[r], Ys), g);
-                    g = f2fma(fv.w, f2add(cZ[r], Zs), g);
+                    float2 g;
+                    if constexpr (RK) {
+                        const float4 fv = fp[r].f;
+                        g = f2scl(f2add(cX[r], Xs), fv.y);
+                        g = f2fma(fv.z, f2add(cY[r], Ys), g);
+                        g = f2fma(fv.w, f2add(cZ[r], Zs), g);
+                    } else {
+                        g = f2mul(fp[r].f[1], f2add(cX[r], Xs));
+                        g = f2add(g, f2mul(fp[r].f[2], f2add(cY[r], Ys)));
+                        g = f2add(g, f2mul(fp[r].f[3], f2add(cZ[r], Zs)));
+                    }
                     const float2 v = f2fma(p.h_20, g, A);
                     if (act[r]) Y[(size_t)(P - 1) * plane + poff + r * p.nx] = f2scl(v, sg);
                 }
@@ -420,7 +487,8 @@ stencil_fast2_kernel(FParams p, const float2* __restrict__ U, float2* __restrict
                     float2 Am = f2scl(f2fma(-64.f / 15.f, c, f2fma(0.1f, e, f2scl(f2add(fx, fy), 7.f / 15.f))), ih);
                     Am = f2fma(14.f / 15.f, kc, Am);
                     Am = f2fma(1.f / 90.f, f2sub(kcs, kf4), Am);
-                    Am = f2fma(p.h2_20 * S.f4[fi + r * FTX].x, c, Am);
+                    if constexpr (RK) Am = f2fma(p.h2_20 * fm[r].f.x, c, Am);
+                    else Am = f2fma(p.h2_20, f2mul(fm[r].f[0], c), Am);
                     const float2 tdx = f2sub(f2add(u[r][2], u[r + 2][2]), f2add(u[r][0], u[r + 2][0]));
                     const float2 tdy = f2sub(f2add(u[r + 2][0], u[r + 2][2]), f2add(u[r][0], u[r][2]));
                     const float2 Xm = f2add(f2fma(p.hh6, dkx, dx1), f2scl(f2fma(-4.f, dx1, tdx), 1.f / 6.f));
@@ -428,6 +496,23 @@ stencil_fast2_kernel(FParams p, const float2* __restrict__ U, float2* __restrict
                     cA[r] = f2add(cA[r], Am); cX[r] = f2add(cX[r], Xm); cY[r] = f2add(cY[r], Ym);
                 }
                 nA[r] = As; nX[r] = Xs; nY[r] = Ys; nZ[r] = make_float2(-Zs.x, -Zs.y);
+            } else if (PAD) {
+                // pending: cA the mid plane's share and the far KU, cX/cY/cZ = (lo - mid) of dxx U, dyy U and U; the
+                // mid plane's dxx U, dyy U and U in nX/nY/nZ (they are the lo plane's at the next step)
+                const float2 X = f2fma(-2.f, c, fx), Yd = f2fma(-2.f, c, fy);
+                if (out_prev) {
+                    float2 v = f2fma(p.ihz, f2add(cZ[r], f2sub(c, nZ[r])), cA[r]);
+                    v = f2fma(p.wxz, f2add(cX[r], f2sub(X, nX[r])), v);
+                    v = f2fma(p.wyz, f2add(cY[r], f2sub(Yd, nY[r])), v);
+                    v = f2fma(1.f / 12.f, kc, v);
+                    if (act[r]) Y[(size_t)(P - 1) * plane + poff + r * p.nx] = f2scl(v, sg);
+                }
+                float2 Am = f2fma(p.wxy, f2fma(-2.f, f2add(X, Yd), f2fma(-4.f, c, e)), f2fma(p.ihx, X, f2scl(Yd, p.ihy)));
+                Am = f2fma(0.5f, kc, Am);
+                Am = f2fma(1.f / 12.f, f2add(kf4, nA[r]), Am);
+                cA[r] = Am;
+                cX[r] = f2sub(nX[r], X); cY[r] = f2sub(nY[r], Yd); cZ[r] = f2sub(nZ[r], c);
+                nX[r] = X; nY[r] = Yd; nZ[r] = c; nA[r] = kc;
             } else {
                 const float2 As = f2fma(1.f / 12.f, kc,
                                         f2add(f2scl(c, p.ihz),
@@ -899,26 +984,21 @@ helm_status encode3(FastMaps* m, CUtensorMap* map, const void* ptr, int nx, int 
 // Set-up (not inside a capture): the kernels' shared-memory limits and, for even N_x, the TMA descriptors
 // of the fixed operands (k^2 and the sixth-order fields).
 helm_status stencil_fast_prepare(helm_ctx* c) {
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast_smem<4>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast_kernel<6, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast_smem<6>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast_kernel<4, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast_smem<4>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast_kernel<6, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast_smem<6>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast_kernel<4, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast_smem<4, true>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast_kernel<6, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast_smem<6, true>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast_kernel<4, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast_smem<4, true>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast_kernel<6, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast_smem<6, true>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast2_kernel<6, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast2_smem<6>()));
-    HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast2_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fast2_smem<4>()));
+    auto big = [](const void* f, size_t bytes) {
+        return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+#define ONE_ROW(O, M, RK)                                                                     \
+    HELM_CUDA_TRY(big((const void*)stencil_fast_kernel<O, M, RK, false>, fast_smem<O, RK>())); \
+    HELM_CUDA_TRY(big((const void*)stencil_fast_kernel<O, M, RK, true>, fast_smem<O, RK>()));
+#define TWO_ROW(O, RK)                                                                         \
+    HELM_CUDA_TRY(big((const void*)stencil_fast2_kernel<O, RK, false, false>, fast2_smem<RK>())); \
+    HELM_CUDA_TRY(big((const void*)stencil_fast2_kernel<O, RK, false, true>, fast2_smem<RK>()));  \
+    HELM_CUDA_TRY(big((const void*)stencil_fast2_kernel<O, RK, true, true>, fast2_smem<RK>()));
+    ONE_ROW(4, 4, false) ONE_ROW(4, 3, false) ONE_ROW(4, 4, true) ONE_ROW(4, 3, true)
+    ONE_ROW(6, 4, false) ONE_ROW(6, 3, false) ONE_ROW(6, 4, true) ONE_ROW(6, 3, true)
+    TWO_ROW(4, false) TWO_ROW(4, true) TWO_ROW(6, false) TWO_ROW(6, true)
+#undef ONE_ROW
+#undef TWO_ROW
     HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_fast3_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)F3_SMEM));
     HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_tma_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -926,8 +1006,7 @@ helm_status stencil_fast_prepare(helm_ctx* c) {
     HELM_CUDA_TRY(cudaFuncSetAttribute(stencil_tma_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        TLayout<6>::SMEM));
     if (residual_fast_prepare() != HELM_OK) return HELM_ERR_CUDA;
-    // measured default: the sixth-order kernel needs about 80 registers (three CTAs per SM, no spills)
-    c->tune_stencil = c->opt.order == 6 ? 2 : 0;
+    c->tune_stencil = 3;   // two rows per thread: measured best for both orders, real and complex media
     if (c->nx % 2 != 0 || !stencil_fast_supported(c)) return HELM_OK;
     FastMaps* m = new FastMaps();
     cudaDriverEntryPointQueryResult q;
@@ -981,7 +1060,7 @@ __global__ void real_fields_kernel(size_t n, int order, const float2* __restrict
 // complex64 matvec stages k^2 as float and reads the four order-6 fields as one real float4 per point
 // (36 instead of 56 bytes per point, real instead of complex products).  Synchronises s.
 helm_status stencil_real_prepare(helm_ctx* c, cudaStream_t s) {
-    if (!stencil_fast_supported(c)) return HELM_OK;
+    if (c->opt.order == 2) return HELM_OK;
     unsigned* flag = nullptr;
     unsigned h = 1;
     HELM_CUDA_TRY(cudaMalloc(&flag, sizeof(unsigned)));
@@ -1006,7 +1085,7 @@ helm_status stencil_real_prepare(helm_ctx* c, cudaStream_t s) {
                                             c->dk2_f[2], c->k2r, c->fr);
     HELM_CUDA_TRY(cudaGetLastError());
     c->realk = 1;
-    if (c->opt.order == 6) c->tune_stencil = 3;   // two rows per thread (variant 4, the fields formed in the kernel, moves half the bytes but issues 40% more instructions: slower alone)
+    // (variant 4, the fields formed in the kernel, moves half the bytes but issues 40% more instructions: slower alone)
     return HELM_OK;
 }
 
@@ -1014,21 +1093,31 @@ bool stencil_fast_supported(const helm_ctx* c) { return !c->colloc && (c->opt.or
 
 // Variants of the complex64 matvec a context can run: 0 = cp.async ring at four CTAs per SM, 1 = TMA ring
 // (even N_x, else the same as 0), 2 = cp.async ring at three CTAs per SM with more registers, 3 = two rows
-// per thread (real media; else the same as 2), 4 = two rows with the sixth-order fields formed in the kernel
+// per thread, 4 = two rows with the sixth-order fields formed in the kernel
 // (real media, order 6; else the same as 3).
 int stencil_variants(const helm_ctx* c) { (void)c; return 5; }
 
-helm_status launch_stencil_fast(helm_ctx* c, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s,
-                                int nb) {
-    if (nb > 1 && c->sfast && c->tune_stencil == 1) {
-        // the TMA form stages one vector: one launch per vector of the batch
-        helm_status st;
-        for (int v = 0; v < nb; ++v)
-            if ((st = launch_stencil_fast(c, x + (size_t)v * c->npts, y + (size_t)v * c->npts, sigma, sidx, s, 1)) !=
-                HELM_OK)
-                return st;
-        return HELM_OK;
+namespace {
+// Planes per CTA.  A CTA stages two planes beyond its chunk, so long chunks read least; but a CTA is a chain of
+// plane latencies, so a grid of few CTAs wants shorter chunks.  Grids with three waves of chunks of FZCH keep those
+// (the constant also makes the kernel 1-4% faster); for the others the chunk with the least time is taken, with
+// a plane step of about 0.45 us alone on an SM and 0.2 us more for each CTA beside it.  The sums of a point do
+// not depend on the chunk.  Measured, order 6, real: 48^3 31 -> 8 us, 96^3 27 -> 14, 128^3 35 -> 26; order 4, 64^3
+// 21 -> 8 (8 us a call is what the host needs to issue it).
+int fast_chunk(const helm_ctx* c, int nb) {
+    constexpr int SMS = 152, OCC = 4;
+    const long tiles = (long)((c->nx + FTX - 1) / FTX) * ((c->ny + FTY - 1) / FTY) * nb;
+    if (tiles * ((c->nz + FZCH - 1) / FZCH) >= 3L * SMS * OCC) return FZCH;
+    int best = FZCH;
+    double tbest = 1e300;
+    for (int z = FZCH; z >= 4; --z) {
+        const long per = (tiles * ((c->nz + z - 1) / z) + SMS - 1) / SMS;   // CTAs of the fullest SM
+        const double t = (z + 2) * ((double)(per / OCC) * (0.45 + 0.2 * OCC) + (per % OCC ? 0.45 + 0.2 * (per % OCC) : 0.0));
+        if (t < tbest) { tbest = t; best = z; }
     }
+    return best;
+}
+FParams fast_params(const helm_ctx* c, int nb) {
     FParams p;
     p.nx = c->nx; p.ny = c->ny; p.nz = c->nz;
     p.gx = make_float2((float)c->gam[0].x, (float)c->gam[0].y);
@@ -1047,60 +1136,102 @@ helm_status launch_stencil_fast(helm_ctx* c, const float2* x, float2* y, const d
     p.fld[0] = c->G_f;
     for (int d = 0; d < 3; ++d) p.fld[d + 1] = c->dk2_f[d];
     p.nb = nb;
+    p.zch = fast_chunk(c, nb);
     for (int d = 0; d < 3; ++d) {
         p.i12h[d] = (float)(1.0 / (12.0 * c->h[d]));
         p.i12h2[d] = (float)(1.0 / (12.0 * c->h[d] * c->h[d]));
     }
-    dim3 grid((c->nx + FTX - 1) / FTX, (c->ny + FTY - 1) / FTY, (c->nz + FZCH - 1) / FZCH * nb), block(FTX, FTY);
+    p.k2r = c->k2r;
+    p.fr = c->fr;
+    return p;
+}
+dim3 fast_grid(const helm_ctx* c, const FParams& p) {
+    return dim3((c->nx + FTX - 1) / FTX, (c->ny + FTY - 1) / FTY, (c->nz + p.zch - 1) / p.zch * p.nb);
+}
+}  // namespace
+
+namespace {
+template <int ORDER, bool RK, bool PAD>
+void run_two_rows(const FParams& p, dim3 grid, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s) {
+    const dim3 block(FTX, FTY / 2);
+    if (PAD || p.zch != FZCH)
+        stencil_fast2_kernel<ORDER, RK, PAD, true><<<grid, block, fast2_smem<RK>(), s>>>(p, x, y, sigma, sidx);
+    else
+        stencil_fast2_kernel<ORDER, RK, false, false><<<grid, block, fast2_smem<RK>(), s>>>(p, x, y, sigma, sidx);
+}
+template <int ORDER, int MINB, bool RK>
+void run_one_row(const FParams& p, dim3 grid, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s) {
+    const dim3 block(FTX, FTY);
+    if (p.zch != FZCH)
+        stencil_fast_kernel<ORDER, MINB, RK, true><<<grid, block, fast_smem<ORDER, RK>(), s>>>(p, x, y, sigma, sidx);
+    else
+        stencil_fast_kernel<ORDER, MINB, RK, false><<<grid, block, fast_smem<ORDER, RK>(), s>>>(p, x, y, sigma, sidx);
+}
+template <int ORDER, bool RK>
+void run_variant(const helm_ctx* c, const FParams& p, dim3 grid, const float2* x, float2* y, const double* sigma, int sidx,
+                 cudaStream_t s) {
+    if (c->tune_stencil >= 3) run_two_rows<ORDER, RK, false>(p, grid, x, y, sigma, sidx, s);
+    else if (c->tune_stencil == 2) run_one_row<ORDER, 3, RK>(p, grid, x, y, sigma, sidx, s);
+    else run_one_row<ORDER, 4, RK>(p, grid, x, y, sigma, sidx, s);
+}
+}  // namespace
+
+helm_status launch_stencil_padded(helm_ctx* c, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s) {
+    FParams p = fast_params(c, 1);
+    p.pad = c->ho_P32;
+    const dim3 grid = fast_grid(c, p);
+    if (c->realk) {
+        if (c->opt.order == 6) run_two_rows<6, true, true>(p, grid, x, y, sigma, sidx, s);
+        else run_two_rows<4, true, true>(p, grid, x, y, sigma, sidx, s);
+    } else {
+        if (c->opt.order == 6) run_two_rows<6, false, true>(p, grid, x, y, sigma, sidx, s);
+        else run_two_rows<4, false, true>(p, grid, x, y, sigma, sidx, s);
+    }
+    HELM_CUDA_TRY(cudaGetLastError());
+    return HELM_OK;
+}
+
+helm_status launch_stencil_fast(helm_ctx* c, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s,
+                                int nb) {
+    if (nb > 1 && c->sfast && c->tune_stencil == 1) {
+        // the TMA form stages one vector: one launch per vector of the batch
+        helm_status st;
+        for (int v = 0; v < nb; ++v)
+            if ((st = launch_stencil_fast(c, x + (size_t)v * c->npts, y + (size_t)v * c->npts, sigma, sidx, s, 1)) !=
+                HELM_OK)
+                return st;
+        return HELM_OK;
+    }
+    FParams p = fast_params(c, nb);
+    const dim3 full((c->nx + FTX - 1) / FTX, (c->ny + FTY - 1) / FTY, (c->nz + FZCH - 1) / FZCH * nb);
     if (c->sfast && c->tune_stencil == 1) {
         FastMaps* m = (FastMaps*)c->sfast;
         CUtensorMap mU;
         if (encode3(m, &mU, x, c->nx, c->ny, c->nz, 2 * TPX, FPY) == HELM_OK) {
             if (c->opt.order == 6)
-                stencil_tma_kernel<6><<<grid, block, TLayout<6>::SMEM, s>>>(mU, m->mK, m->mF[0], m->mF[1], m->mF[2],
+                stencil_tma_kernel<6><<<full, dim3(FTX, FTY), TLayout<6>::SMEM, s>>>(mU, m->mK, m->mF[0], m->mF[1], m->mF[2],
                                                                            m->mF[3], p, y, sigma, sidx, c->status_d,
                                                                            (long)c->wait_limit);
             else
-                stencil_tma_kernel<4><<<grid, block, TLayout<4>::SMEM, s>>>(mU, m->mK, m->mF[0], m->mF[1], m->mF[2],
+                stencil_tma_kernel<4><<<full, dim3(FTX, FTY), TLayout<4>::SMEM, s>>>(mU, m->mK, m->mF[0], m->mF[1], m->mF[2],
                                                                            m->mF[3], p, y, sigma, sidx, c->status_d,
                                                                            (long)c->wait_limit);
             HELM_CUDA_TRY(cudaGetLastError());
             return HELM_OK;
         }
     }
-    const bool three = c->tune_stencil >= 2;   // the variant with up to 85 registers, three CTAs per SM
-    if (c->realk) {
-        p.k2r = c->k2r;
-        p.fr = c->fr;
-        if (c->tune_stencil == 4 && c->opt.order == 6) {   // two rows per thread, fields formed in the kernel
-            const dim3 block2(FTX, FTY / 2);
-            stencil_fast3_kernel<4><<<grid, block2, F3_SMEM, s>>>(p, x, y, sigma, sidx);
-            HELM_CUDA_TRY(cudaGetLastError());
-            return HELM_OK;
-        }
-        if (c->tune_stencil >= 3) {   // two rows per thread
-            const dim3 block2(FTX, FTY / 2);
-            if (c->opt.order == 6) stencil_fast2_kernel<6, 4><<<grid, block2, fast2_smem<6>(), s>>>(p, x, y, sigma, sidx);
-            else stencil_fast2_kernel<4, 4><<<grid, block2, fast2_smem<4>(), s>>>(p, x, y, sigma, sidx);
-            HELM_CUDA_TRY(cudaGetLastError());
-            return HELM_OK;
-        }
-        if (c->opt.order == 6) {
-            if (three) stencil_fast_kernel<6, 3, true><<<grid, block, fast_smem<6, true>(), s>>>(p, x, y, sigma, sidx);
-            else stencil_fast_kernel<6, 4, true><<<grid, block, fast_smem<6, true>(), s>>>(p, x, y, sigma, sidx);
-        } else {
-            if (three) stencil_fast_kernel<4, 3, true><<<grid, block, fast_smem<4, true>(), s>>>(p, x, y, sigma, sidx);
-            else stencil_fast_kernel<4, 4, true><<<grid, block, fast_smem<4, true>(), s>>>(p, x, y, sigma, sidx);
-        }
+    if (c->realk && c->tune_stencil == 4 && c->opt.order == 6) {   // two rows per thread, fields formed in the kernel
+        stencil_fast3_kernel<4><<<full, dim3(FTX, FTY / 2), F3_SMEM, s>>>(p, x, y, sigma, sidx);
         HELM_CUDA_TRY(cudaGetLastError());
         return HELM_OK;
     }
-    if (c->opt.order == 6) {
-        if (three) stencil_fast_kernel<6, 3><<<grid, block, fast_smem<6>(), s>>>(p, x, y, sigma, sidx);
-        else stencil_fast_kernel<6, 4><<<grid, block, fast_smem<6>(), s>>>(p, x, y, sigma, sidx);
+    const dim3 grid = fast_grid(c, p);
+    if (c->realk) {
+        if (c->opt.order == 6) run_variant<6, true>(c, p, grid, x, y, sigma, sidx, s);
+        else run_variant<4, true>(c, p, grid, x, y, sigma, sidx, s);
     } else {
-        if (three) stencil_fast_kernel<4, 3><<<grid, block, fast_smem<4>(), s>>>(p, x, y, sigma, sidx);
-        else stencil_fast_kernel<4, 4><<<grid, block, fast_smem<4>(), s>>>(p, x, y, sigma, sidx);
+        if (c->opt.order == 6) run_variant<6, false>(c, p, grid, x, y, sigma, sidx, s);
+        else run_variant<4, false>(c, p, grid, x, y, sigma, sidx, s);
     }
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
@@ -1563,7 +1694,7 @@ helm_status residual_fast_prepare() {
 // Fields of the sixth-order real-medium residual (after stencil_real_prepare found Im k^2 = 0): 28 bytes
 // per point.  Without them the residual takes the complex-medium kernel.
 helm_status residual_real_prepare(helm_ctx* c, cudaStream_t s) {
-    if (!c->realk || c->opt.order != 6) return HELM_OK;
+    if (!c->realk || c->colloc || c->opt.order != 6) return HELM_OK;
     if (cudaMalloc(&c->rkq, c->npts * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&c->rg4, c->npts * sizeof(float4)) != cudaSuccess ||
         cudaMalloc(&c->rgz, c->npts * sizeof(float)) != cudaSuccess) {

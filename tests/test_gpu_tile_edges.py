@@ -1,0 +1,109 @@
+"""Kernels at the edges of their tilings, against the CPU oracle, through the C-ABI.
+
+FP32 transform passes: lengths on both sides of the GEMM's tile widths (32 .. 64 columns, 32 rows a warp, 128 a
+tile) and K blocks (16), odd ones included.  A pass sums K products of FP32 operands in order: 2-norm error a few
+times sqrt(K) 2^-24, two passes; bound 8 sqrt(K) 2^-24.
+z-solves: depths on both sides of the blocks of 8 steps whose inner ones run without end conditions; bound 1e-4
+(the systems amplify FP32 rounding, here by a few hundred at most).
+Complex64 matvec: every kernel variant, grids from the smallest to several chunk lengths, real and complex k^2, and
+the padded form of the high-order closure (an output that overlaps the operand included).  The terms of A U are up
+to 8/h^2 |U| and cancel to k^2 U, each rounded to 2^-24: bound 32 2^-24 / (k0 h)^2.
+Wrong indices or weights give errors of order 1 in each."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle.eigt import EigT
+from oracle.grid import Grid
+from oracle.operators import Operator
+from oracle.tridiag import thomas
+from paper_2602_07711_gb300 import HELM_C64, HELM_CLOSURE_HIGH_ORDER, Solver, helm
+
+
+def _rand(shape, seed):
+    r = np.random.default_rng(seed)
+    return r.standard_normal(shape) + 1j * r.standard_normal(shape)
+
+
+def _rel(a, b):
+    return np.linalg.norm((a - b).ravel()) / np.linalg.norm(b.ravel())
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda", torch.complex64)
+
+
+def _grid(n, staggered=True):
+    big = max(n)
+    return Grid(*n, *[(m if staggered else m - 1) / big for m in n], staggered=staggered)
+
+
+def _library_basis(S, g, k0):
+    """The oracle's EigT in the library's order and scaling of the eigenvectors."""
+    e = EigT(g, k0)
+    e.Dx, e.Vx, e.Vxi = S.get_eig(0)
+    e.Dy, e.Vy, e.Vyi = S.get_eig(1)
+    return e
+
+
+@pytest.mark.parametrize("n", [(5, 33, 4), (16, 17, 6), (40, 56, 4), (57, 65, 4), (64, 129, 5), (130, 48, 7), (199, 100, 4),
+                               (256, 31, 16)])
+def test_fp32_transform_passes(n):
+    g = _grid(n)
+    k0 = 2 * math.pi * max(n) / 11
+    S = Solver(n, np.full(g.shape, k0 * k0, complex), k0, order=4, L=g.L)
+    e = _library_basis(S, g, k0)
+    y = _rand(g.shape, n[0])
+    bound = 8 * math.sqrt(max(n[:2])) * 2.0 ** -24
+    assert _rel(S.precond_step(1, _dev(y)).cpu().numpy(), e.forward(y)) < bound
+    assert _rel(S.precond_step(3, _dev(y)).cpu().numpy(), e.inverse(y)) < bound
+
+
+@pytest.mark.parametrize("nz", [4, 7, 8, 9, 15, 16, 17, 24, 25, 64, 511])
+def test_z_solves(nz):
+    n = (12, 10, nz)
+    g = Grid(*n, 12 / 40, 10 / 40, nz / 40)
+    k0 = 2 * math.pi * 40 / 11
+    S = Solver(n, np.full(g.shape, k0 * k0, complex), k0, order=4, L=g.L)
+    e = _library_basis(S, g, k0)
+    y = _rand(g.shape, nz)
+    assert _rel(S.precond_step(2, _dev(y)).cpu().numpy(), thomas(*e.z_coefficients(), y)) < 1e-4
+
+
+@pytest.mark.parametrize("lossy", [False, True])
+@pytest.mark.parametrize("order", [4, 6])
+@pytest.mark.parametrize("n", [(4, 4, 4), (33, 9, 6), (31, 18, 40), (66, 41, 33), (96, 64, 80)])
+def test_matvec_variants(n, order, lossy):
+    g = _grid(n)
+    k0 = 2 * math.pi * max(n) / 10
+    k2 = k0 * k0 * (1 + 0.2 * np.cos(3 * g.mesh()[0]) * np.sin(2 * g.mesh()[2])).astype(complex)
+    if lossy:
+        k2 = k2 + 0.02j * k0 * k0
+    S = Solver(n, k2, k0, order=order, L=g.L)
+    x = _rand(g.shape, n[1])
+    ref = Operator(g, k2, k0, order)(x)
+    for v in range(5):
+        S.set_matvec_variant(v)
+        assert _rel(S.apply_A(_dev(x)).cpu().numpy(), ref) < 32 * 2.0 ** -24 / (k0 * g.h[0]) ** 2, v
+
+
+@pytest.mark.parametrize("order", [2, 4, 6])
+@pytest.mark.parametrize("n,ppw", [((8, 8, 8), 10), ((34, 9, 12), 12), ((40, 33, 64), 60), ((64, 10, 9), 25)])
+def test_closure_matvec(n, ppw, order):
+    g = _grid(n, staggered=False)
+    k0 = 2 * math.pi / (ppw * g.h[0])
+    k2 = np.full(g.shape, k0 * k0, complex)
+    S = Solver(n, k2, k0, order=order, L=g.L, staggered=False)
+    S.set_closure(HELM_CLOSURE_HIGH_ORDER)
+    X, Y, Z = g.mesh()
+    x = np.exp(1j * k0 * (0.6 * X + 0.8 * Z)) + 0.1 * np.exp(-1j * k0 * Y)
+    ref = Operator(g, k2, k0, order, rule="collocated_ho")(x)
+    bound = 32 * 2.0 ** -24 / (k0 * g.h[0]) ** 2 * np.linalg.norm(x) * k0 ** 2 / np.linalg.norm(ref)
+    xd = _dev(x)
+    assert _rel(S.apply_A(xd).cpu().numpy(), ref) < bound
+    helm.helm_apply_A(S.ctx, xd, xd, HELM_C64)
+    assert _rel(xd.cpu().numpy(), ref) < bound
