@@ -11,17 +11,23 @@
 //
 // Forward and data gradient (the same convolution with flipped, transposed weights):
 //   out[o][p] = act(bias[o] + sum_{t, i} W(o, i, t) in[i][p + off_t])
-//   A tile is R x 128 consecutive points of a padded plane, taken along the flattened (y, x) index: rows follow
-//   one another across the halo, so the waste is the two halo points per row and not the remainder of a row to
-//   128.  Per 128 points one accumulator of 128 x Np (Np: outputs padded to 16) in tensor memory, R Np <= 256
-//   columns, two buffers.  The K dimension runs over 16-channel chunks, then the taps in order; a stage is one
-//   chunk and one dz: the points of plane z + dz - 1 (128 R plus a row and a point on both sides, or three runs
-//   for the three dy where rows are longer than a tile) and the 9 taps' weights.
-//   Persistent, one CTA per SM: warp 0 issues the bulk copies, one thread of warp 1 the MMAs (M = 128, N = Np,
-//   K = 16), warps 2-5 run the epilogue of the previous tile.
-//   The tensor unit bounds it (84% busy at 160^3): it takes about 64 cycles for an MMA of M = 128, K = 16 however
-//   small N is, so 28 outputs use an eighth of its rate.  The order of the sums is chunk, tap, 16 channels.
-//   Measured at 160^3, width 28: the 84 -> 28 layer 4.14 -> 1.38 ms, the forward pass 9.2 -> 3.2 ms.
+//   A tile is R x 128 consecutive points of a padded plane, taken along the flattened (y, x) index, in S consecutive
+//   planes: rows follow one another across the halo, so the waste is the two halo points per row and not the
+//   remainder of a row to 128.  Per 128 points and plane one accumulator of 128 x Np (Np: outputs padded to 16) in
+//   tensor memory, R S Np <= 256 columns, two buffers.
+//   The tensor unit bounds it: it takes 64 cycles for an MMA of M = 128, K = 16 with any N up to 128, so N = Np = 32
+//   outputs alone used an eighth of its rate (84% busy).  So an MMA takes one view of the points (one input plane,
+//   dy, dx) for up to three output planes at once: their accumulators are adjacent columns, and the weights of
+//   the three dz are adjacent rows, stored from dz = 2 down.  9 (S + 2) MMAs serve S planes instead of 27 S.
+//   The K dimension runs over 16-channel chunks, then the input planes, then dy, dx: every output sums chunk, tap, 16
+//   channels in that order whatever R and S are.  A stage is one chunk of one input plane: the points of the tile
+//   plus a row and a point on both sides (or three runs for the three dy where rows are longer than a tile); the
+//   27 taps' weights of a chunk have two buffers of their own.
+//   Persistent, one CTA per SM: warp 0 issues the bulk copies, warps 1 and 10 the MMAs (M = 128, K = 16) of one
+//   128-point block each (one warp alone could not issue them fast enough: 118 cycles an MMA), warps 2-9 run the epilogue
+//   of the previous tile.
+//   Measured at 160^3, width 28: the 84 -> 28 layer 4.14 ms before cells, 1.38 with one output plane per MMA, 1.05 with
+//   one MMA warp and four epilogue warps, 0.90 now; the forward pass 9.2, 3.17, 2.46, 2.09 ms.
 // Weight gradient:  gW[o][i][t] = sum_p g[o][p] in[i][p + off_t].
 //   Both operands are read as MN-major cells (channels x points): M = output channels (64, or 128), N = all
 //   input channels of a block (up to 160), K = 256 points of a flattened plane (the gradient's halo is zero, so
@@ -29,7 +35,7 @@
 //   one dy in tensor memory for its whole share of the points and adds them to gW (FP32 atomics) at the end.
 //   The copies bound it: one warp issues a 4 KiB copy per channel group and tile.  Measured on two 96^3 fields, 84 ->
 //   28 layer: 0.65 ms with tiles of 256 points, 1.19 ms with 128; 7.6 ms with M = 128 rows of which 28 were used, N =
-//   16 inputs at a time and a gathered slab per input chunk.  A training pass: 24.2 -> 5.0 ms.
+//   16 inputs at a time and a gathered slab per input chunk.  A training pass: 24.2 -> 4.1 ms.
 // Every mbarrier wait is bounded; an expired wait raises HELM_DEV_WAIT, the CTA waits (bounded) for its bulk
 // copies and MMAs in flight, frees its tensor memory and exits.
 #include "cells.cuh"
@@ -39,9 +45,13 @@ namespace {
 
 constexpr long CT_WAIT = 1L << 22;                 // bound of every mbarrier wait (polls)
 constexpr int CT_NPMAX = 64;                       // largest padded output-channel count of a launch
-constexpr int CT_RMAX = 8;                         // largest tile: 8 x 128 points
+constexpr int CT_RMAX = 2;                         // 128-point blocks of a tile at most
+constexpr int CT_PLANES = 128;                     // S Np at most: output planes of a tile times outputs
 constexpr int CT_THREADS = 192;                    // producer warp, MMA warp, four epilogue warps
-constexpr int CT_NST = 6;                          // most stages
+constexpr int CV_THREADS = CT_THREADS + 5 * 32;    // convolutions: eight epilogue warps (2 .. 9), one MMA warp per 128-point
+                                                   // block (warps 1 and 10)
+constexpr int CT_NST = 8;                          // most stages
+constexpr int CT_CHUNK = 128;                      // cells of a bulk copy at most (whole runs measured the same)
 constexpr int CT_SMEM = 229376;                    // dynamic shared memory of a CTA at most (224 KiB)
 constexpr int WG_KT = 256;                         // points of a weight-gradient tile at most
 // Points a CTA sums in tensor memory before it adds to gW.  The accumulators of the tensor cores are FP32 with
@@ -105,7 +115,9 @@ __device__ __forceinline__ void mma_bf16(uint32_t lead, uint32_t d, uint32_t alo
         "setp.ne.b32 q, %7, 0;\n@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d), "r"(alo), "r"(ahi),
         "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(lead));
 }
-// 1 in one lane of the (converged) warp
+// 1 in one lane of the (converged) warp.  The MMA instructions are predicated on this value directly: the compiler
+// then issues them back to back; predicated on lane == 0, or on a copy of this in a variable that other code sets too,
+// an MMA took twice as long (weight gradient of 28 -> 28 channels on two 96^3 fields 341 against 781 us)
 __device__ __forceinline__ uint32_t elect_one() {
     uint32_t r;
     asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
@@ -140,7 +152,7 @@ struct ConvArgs {
     CellGrid g;
     const bf16* in;      // cells of Gin groups
     int Gin;
-    const bf16* wt;      // arranged weights [nkc][27][2][Np][8]
+    const bf16* wt;      // arranged weights [nkc][9][2][3][Np][8]
     int Np;
     const float* bias;   // [Cout] or NULL
     void* out;
@@ -149,8 +161,8 @@ struct ConvArgs {
     int relu;
     const bf16* mask;    // CONV_GRAD: cells of Gout groups; the output is 0 where mask <= 0
     float* gb;           // CONV_GRAD: += sum of the output over points, per channel
-    int R;               // 128-point blocks per tile
-    int ntp;             // tiles per plane
+    int R, S;            // 128-point blocks and planes per tile
+    int ntp, nzg;        // tiles per plane, groups of S planes
     int ntiles;
     int dstride;         // staged cells between the views of consecutive dy
     int L;               // staged cells per channel group
@@ -160,22 +172,30 @@ struct ConvArgs {
 };
 
 template <int OUT>
-__global__ void __launch_bounds__(CT_THREADS, 1) conv_cells_kernel(const __grid_constant__ ConvArgs a) {
+__global__ void __launch_bounds__(CV_THREADS, 1) conv_cells_kernel(const __grid_constant__ ConvArgs a) {
     extern __shared__ __align__(128) unsigned char csm[];
-    __shared__ __align__(8) uint64_t full[CT_NST], empty[CT_NST], accf[2], acce[2], drainb;
+    __shared__ __align__(8) uint64_t full[CT_NST], empty[CT_NST], wfull[2], wempty[2], accf[2], acce[2], drainb;
     __shared__ uint32_t tslot;
     __shared__ int fail_any;
+    __shared__ float sbias[CT_NPMAX];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nkc = a.Gin / 2, niter = 3 * nkc;
+    const int nkc = a.Gin / 2;
     const uint32_t base = (s32(csm) + 127u) & ~127u;
-    const uint32_t wbytes = 9u * 2u * (uint32_t)a.Np * 16u, sbytes = (uint32_t)a.L * 16u;
+    const uint32_t wbytes = 27u * 2u * (uint32_t)a.Np * 16u, sbytes = (uint32_t)a.L * 16u;
+    const uint32_t ring = base + 2u * wbytes;   // (wbytes is a multiple of 128)
     if (threadIdx.x == 0) {
-        for (int s = 0; s < CT_NST; ++s) { bar_init(s32(&full[s]), 1); bar_init(s32(&empty[s]), 1); }
-        for (int b = 0; b < 2; ++b) { bar_init(s32(&accf[b]), 1); bar_init(s32(&acce[b]), 4); }
-        bar_init(s32(&drainb), 1);
+        for (int s = 0; s < CT_NST; ++s) { bar_init(s32(&full[s]), 1); bar_init(s32(&empty[s]), CT_RMAX); }
+        for (int b = 0; b < 2; ++b) {
+            bar_init(s32(&wfull[b]), 1);
+            bar_init(s32(&wempty[b]), CT_RMAX);
+            bar_init(s32(&accf[b]), CT_RMAX);
+            bar_init(s32(&acce[b]), 8);
+        }
+        bar_init(s32(&drainb), CT_RMAX);
         fail_any = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (threadIdx.x < CT_NPMAX) sbias[threadIdx.x] = a.bias && threadIdx.x < a.Cout ? a.bias[threadIdx.x] : 0.f;
     if (warp == 1) tmem_alloc(&tslot);
     tc_before();
     __syncthreads();
@@ -183,87 +203,107 @@ __global__ void __launch_bounds__(CT_THREADS, 1) conv_cells_kernel(const __grid_
     const uint32_t tmem = tslot;
     const CellGrid& g = a.g;
     bool ok = true;
-    long issued = 0;   // stages whose copies were issued
+    long issued = 0, wissued = 0;   // stages and weight chunks whose copies were issued
     if (warp == 0) {
-        if (lane == 0) {
-            long it = 0;
-            for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x) {
-                const int tp = tile % a.ntp, zb = tile / a.ntp, z = zb % g.Z, b = zb / g.Z;
-                // first staged cell of a plane: one row and one point before the tile's first point
-                const long q0 = (long)tp * 128 * a.R;
-                for (int k = 0; k < niter; ++k, ++it) {
-                    const int s = (int)(it % a.nst), kc = k / 3, dz = k % 3;
-                    if (it >= a.nst) ok = bar_wait(s32(&empty[s]), (uint32_t)((it / a.nst - 1) & 1), CT_WAIT);
+        // a stage's pieces: runs (two channel groups, times three dy in the split form) in chunks of CT_CHUNK cells
+        const int nrun = a.split ? 6 : 2, run = a.split ? a.dstride : a.L, nch = (run + CT_CHUNK - 1) / CT_CHUNK;
+        for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x) {
+            const int tp = tile % a.ntp, zg = tile / a.ntp, z0 = zg % a.nzg * a.S, b = zg / a.nzg;
+            const int planes = min(a.S, g.Z - z0) + 2;   // input planes
+            // first staged cell of a plane: one row and one point before the tile's first point
+            const long q0 = (long)tp * 128 * a.R;
+            for (int kc = 0; kc < nkc && ok; ++kc) {
+                const int wb = (int)(wissued & 1);
+                if (wissued >= 2) ok = warp_wait(s32(&wempty[wb]), (uint32_t)((wissued / 2 - 1) & 1), CT_WAIT);
+                if (!ok) break;
+                if (lane == 0) bar_expect(s32(&wfull[wb]), wbytes);
+                __syncwarp();
+                for (uint32_t o = (uint32_t)lane * (CT_CHUNK * 16u); o < wbytes; o += 32u * CT_CHUNK * 16u)
+                    bulk_g2s(base + (uint32_t)wb * wbytes + o, reinterpret_cast<const unsigned char*>(a.wt) + (size_t)kc * wbytes + o,
+                             min(CT_CHUNK * 16u, wbytes - o), s32(&wfull[wb]));
+                ++wissued;
+                for (int zp = 0; zp < planes; ++zp, ++issued) {
+                    const int s = (int)(issued % a.nst);
+                    if (issued >= a.nst) ok = warp_wait(s32(&empty[s]), (uint32_t)((issued / a.nst - 1) & 1), CT_WAIT);
                     if (!ok) break;
-                    const uint32_t st = base + (uint32_t)s * (uint32_t)a.stage, fb = s32(&full[s]);
-                    bar_expect(fb, 2u * sbytes + wbytes);
-                    for (int cg = 0; cg < 2; ++cg) {
-                        const bf16* src = a.in + 8 * (((long)b * a.Gin + 2 * kc + cg) * g.vol + (long)(z + dz) * g.plane + q0);
-                        const uint32_t dst = st + (uint32_t)cg * sbytes;
-                        if (!a.split) {
-                            bulk_g2s(dst, src, sbytes, fb);
-                        } else {
-                            for (int dy = 0; dy < 3; ++dy)
-                                bulk_g2s(dst + (uint32_t)(dy * a.dstride) * 16u, src + 8 * (long)dy * g.pitch,
-                                         (uint32_t)a.dstride * 16u, fb);
-                        }
+                    const uint32_t st = ring + (uint32_t)s * (uint32_t)a.stage, fb = s32(&full[s]);
+                    if (lane == 0) bar_expect(fb, 2u * sbytes);
+                    __syncwarp();
+                    const bf16* plane = a.in + 8 * (((long)b * a.Gin + 2 * kc) * g.vol + (long)(z0 + zp) * g.plane + q0);
+                    for (int k = lane; k < nrun * nch; k += 32) {
+                        const int rn = k / nch, c = (k - rn * nch) * CT_CHUNK, cg = rn & 1, dy = rn >> 1;
+                        bulk_g2s(st + (uint32_t)cg * sbytes + (uint32_t)(dy * a.dstride + c) * 16u,
+                                 plane + 8 * (cg * g.vol + (long)dy * g.pitch + c), (uint32_t)min(CT_CHUNK, run - c) * 16u, fb);
                     }
-                    bulk_g2s(st + 2u * sbytes, a.wt + (size_t)(kc * 27 + 9 * dz) * 2 * a.Np * 8, wbytes, fb);
-                    ++issued;
                 }
             }
         }
-    } else if (warp == 1) {
-        {
-            const uint32_t lead = elect_one();
-            const uint32_t idesc = idesc_bf16(128, a.Np, 0, 0);
-            long it = 0;
-            int lt = 0;
-            for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x, ++lt) {
-                const int tp = tile % a.ntp, buf = lt & 1;
-                // 128-point blocks of this tile that hold points (the last tile of a plane may be short)
-                const int nr = min(a.R, (g.span - tp * 128 * a.R + 127) / 128);
-                if (lt >= 2) ok = warp_wait(s32(&acce[buf]), (uint32_t)(((lt >> 1) - 1) & 1), CT_WAIT);
+    } else if (warp == 1 || warp >= 10) {
+        const int r = warp == 1 ? 0 : warp - 9;   // this warp's 128-point block of every tile
+        const uint32_t lead = elect_one();
+        long it = 0, wit = 0;
+        int lt = 0;
+        for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x, ++lt) {
+            const int tp = tile % a.ntp, z0 = tile / a.ntp % a.nzg * a.S, buf = lt & 1;
+            const int S = min(a.S, g.Z - z0);
+            // (the last tile of a plane may be short)
+            const bool mine = r < a.R && (tp * a.R + r) * 128 < g.span;
+            if (lt >= 2) ok = warp_wait(s32(&acce[buf]), (uint32_t)(((lt >> 1) - 1) & 1), CT_WAIT);
+            if (!ok) break;
+            tc_after();
+            const uint32_t Np = (uint32_t)a.Np, acc = tmem + (uint32_t)(buf * 256) + (uint32_t)(r * a.S) * Np;
+            for (int kc = 0; kc < nkc && ok; ++kc, ++wit) {
+                const int wb = (int)(wit & 1);
+                ok = warp_wait(s32(&wfull[wb]), (uint32_t)((wit >> 1) & 1), CT_WAIT);
                 if (!ok) break;
-                tc_after();
-                const uint32_t acc = tmem + (uint32_t)(buf * 256);
-                for (int k = 0; k < niter; ++k, ++it) {
+                // B: a view's weights [2 channel groups][dz = 2, 1, 0][Np][8]: next channel group 3 Np*16 bytes, next 8
+                // rows 128
+                const uint64_t bd = ndesc(base + (uint32_t)wb * wbytes, 3u * Np * 16u, 128u);
+                const uint32_t bhi = (uint32_t)(bd >> 32);
+                for (int zp = 0; zp < S + 2; ++zp, ++it) {
                     const int s = (int)(it % a.nst);
                     ok = warp_wait(s32(&full[s]), (uint32_t)((it / a.nst) & 1), CT_WAIT);
                     if (!ok) break;
                     tc_after();
-                    const uint32_t slab = base + (uint32_t)s * (uint32_t)a.stage, wsm = slab + 2u * sbytes;
-                    // A: a tap's view of the points; next channel group (K) sbytes, next 8 points 128.  B: the tap's
-                    // weights [2 channel groups][Np][8]: next channel group Np*16 bytes, next 8 outputs 128
-                    const uint64_t ad = ndesc(slab, sbytes, 128u), bd = ndesc(wsm, (uint32_t)a.Np * 16u, 128u);
-                    const uint32_t ahi = (uint32_t)(ad >> 32), bhi = (uint32_t)(bd >> 32);
-                    uint32_t blo = (uint32_t)bd;
-                    for (int dy = 0; dy < 3; ++dy) {
-                        const uint32_t arow = (uint32_t)ad + (uint32_t)(dy * a.dstride);
+                    // A: a tap's view of the points; next channel group sbytes, next 8 points 128
+                    const uint64_t ad = ndesc(ring + (uint32_t)s * (uint32_t)a.stage + (uint32_t)r * 2048u, sbytes, 128u);
+                    const uint32_t ahi = (uint32_t)(ad >> 32);
+                    // input plane zp serves the output planes s0 .. s1 (dz = zp - s0 .. zp - s1)
+                    const int s0 = max(0, zp - 2), s1 = min(S - 1, zp);
+                    const uint32_t row0 = (uint32_t)(2 - zp + s0) * Np;
+                    const uint32_t id = idesc_bf16(128, (s1 - s0 + 1) * a.Np, 0, 0);
+                    uint32_t blo = (uint32_t)bd + row0;
+                    const bool opens = kc == 0 && zp < S;   // plane zp's first tap: its accumulator starts here
+                    const uint32_t d = acc + (uint32_t)s0 * Np;
+                    if (mine) {
 #pragma unroll
-                        for (int dx = 0; dx < 3; ++dx, blo += 2u * (uint32_t)a.Np) {
-                            const uint32_t more = (k | dy | dx) ? 1u : 0u;
-#pragma unroll
-                            for (int r = 0; r < CT_RMAX; ++r)
-                                if (r < nr)
-                                    mma_bf16(lead, acc + (uint32_t)(r * a.Np), arow + (uint32_t)(dx + 128 * r), ahi, blo, bhi, idesc,
-                                             more);
+                        for (int t = 0; t < 9; ++t, blo += 6u * Np) {
+                            const uint32_t al = (uint32_t)ad + (uint32_t)((t / 3) * a.dstride + t % 3);
+                            if (t == 0 && opens) {
+                                if (zp > s0) mma_bf16(lead, d, al, ahi, blo, bhi, idesc_bf16(128, (zp - s0) * a.Np, 0, 0), 1u);
+                                mma_bf16(lead, acc + (uint32_t)zp * Np, al, ahi, (uint32_t)bd + 2u * Np, bhi,
+                                         idesc_bf16(128, a.Np, 0, 0), 0u);
+                            } else {
+                                mma_bf16(lead, d, al, ahi, blo, bhi, id, 1u);
+                            }
                         }
                     }
                     if (lead) mma_commit(s32(&empty[s]));
                     __syncwarp();
                 }
-                if (ok && lead) mma_commit(s32(&accf[buf]));
+                if (ok && lead) mma_commit(s32(&wempty[wb]));
                 __syncwarp();
             }
+            if (ok && lead) mma_commit(s32(&accf[buf]));
+            __syncwarp();
         }
     } else {
-        const int w = warp & 3;   // tensor-memory lanes 32 w .. 32 w + 31
+        const int w = warp & 3, half = (warp - 2) >> 2;   // tensor-memory lanes 32 w .. 32 w + 31; every second plane
         float bsum[CT_NPMAX / 16] = {0.f, 0.f, 0.f, 0.f};
         int lt = 0;
         for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x, ++lt) {
-            const int tp = tile % a.ntp, zb = tile / a.ntp, z = zb % g.Z, b = zb / g.Z, buf = lt & 1;
-            const int nr = min(a.R, (g.span - tp * 128 * a.R + 127) / 128);
+            const int tp = tile % a.ntp, zg = tile / a.ntp, z0 = zg % a.nzg * a.S, b = zg / a.nzg, buf = lt & 1;
+            const int nr = min(a.R, (g.span - tp * 128 * a.R + 127) / 128), S = min(a.S, g.Z - z0);
             ok = warp_wait(s32(&accf[buf]), (uint32_t)((lt >> 1) & 1), CT_WAIT);
             if (!ok) break;
             tc_after();
@@ -271,56 +311,59 @@ __global__ void __launch_bounds__(CT_THREADS, 1) conv_cells_kernel(const __grid_
                 const int rel = (tp * a.R + r) * 128 + 32 * w + lane;   // point y pitch + x
                 const int y = rel / g.pitch, x = rel - y * g.pitch;
                 const bool in = y < g.Y && x < g.X;
-                const long q = (long)(z + 1) * g.plane + g.pitch + 1 + rel;   // its cell in a channel group
+                for (int sp = half; sp < S; sp += 2) {
+                    const int z = z0 + sp;
+                    const long q = (long)(z + 1) * g.plane + g.pitch + 1 + rel;   // its cell in a channel group
 #pragma unroll
-                for (int cb = 0; cb < CT_NPMAX; cb += 16) {
-                    if (cb >= a.Np) break;
-                    float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)(buf * 256 + r * a.Np + cb), v);
+                    for (int cb = 0; cb < CT_NPMAX; cb += 16) {
+                        if (cb >= a.Np) break;
+                        float v[16];
+                        tmem_ld16(tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)(buf * 256 + (r * a.S + sp) * a.Np + cb), v);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        if (a.bias) v[j] += cb + j < a.Cout ? a.bias[cb + j] : 0.f;
-                        if (a.relu) v[j] = fmaxf(v[j], 0.f);
-                    }
-                    if constexpr (OUT == CONV_PLANAR) {
-                        if (in)
+                        for (int j = 0; j < 16; ++j) {
+                            v[j] += sbias[cb + j];
+                            if (a.relu) v[j] = fmaxf(v[j], 0.f);
+                        }
+                        if constexpr (OUT == CONV_PLANAR) {
+                            if (in)
 #pragma unroll
-                            for (int j = 0; j < 16; ++j)
-                                if (cb + j < a.Cout)
-                                    reinterpret_cast<float*>(a.out)[(((size_t)b * a.Cout + cb + j) * g.Z + z) * g.Y * g.X +
-                                                                    (size_t)y * g.X + x] = v[j];
-                    } else {
-                        const int c0 = a.ooff + cb;
-                        if constexpr (OUT == CONV_GRAD) {
+                                for (int j = 0; j < 16; ++j)
+                                    if (cb + j < a.Cout)
+                                        reinterpret_cast<float*>(a.out)[(((size_t)b * a.Cout + cb + j) * g.Z + z) * g.Y * g.X +
+                                                                        (size_t)y * g.X + x] = v[j];
+                        } else {
+                            const int c0 = a.ooff + cb;
+                            if constexpr (OUT == CONV_GRAD) {
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) {
+                                    uint4 m = make_uint4(0u, 0u, 0u, 0u);
+                                    if (in && cb + 8 * h < a.Cout)
+                                        m = *reinterpret_cast<const uint4*>(a.mask + 8 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q));
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j)
+                                        if (!(cell_value(m, j) > 0.f)) v[8 * h + j] = 0.f;
+                                }
+                                bsum[cb / 16] += lane_fold16(v, lane);
+                            }
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
-                                uint4 m = make_uint4(0u, 0u, 0u, 0u);
-                                if (in && cb + 8 * h < a.Cout)
-                                    m = *reinterpret_cast<const uint4*>(a.mask + 8 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q));
+                                if (!in || cb + 8 * h >= a.Cout) continue;
+                                if constexpr (OUT == CONV_F32CELLS) {
+                                    float4* o = reinterpret_cast<float4*>(a.out) + 2 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q);
+                                    o[0] = make_float4(v[8 * h], v[8 * h + 1], v[8 * h + 2], v[8 * h + 3]);
+                                    o[1] = make_float4(v[8 * h + 4], v[8 * h + 5], v[8 * h + 6], v[8 * h + 7]);
+                                } else if (a.ooff % 8 == 0) {
+                                    *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.out) +
+                                                              8 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q)) = pack_cell(v + 8 * h);
+                                } else {   // a channel offset inside a cell: channel by channel
 #pragma unroll
-                                for (int j = 0; j < 8; ++j)
-                                    if (!(cell_value(m, j) > 0.f)) v[8 * h + j] = 0.f;
-                            }
-                            bsum[cb / 16] += lane_fold16(v, lane);
-                        }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            if (!in || cb + 8 * h >= a.Cout) continue;
-                            if constexpr (OUT == CONV_F32CELLS) {
-                                float4* o = reinterpret_cast<float4*>(a.out) + 2 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q);
-                                o[0] = make_float4(v[8 * h], v[8 * h + 1], v[8 * h + 2], v[8 * h + 3]);
-                                o[1] = make_float4(v[8 * h + 4], v[8 * h + 5], v[8 * h + 6], v[8 * h + 7]);
-                            } else if (a.ooff % 8 == 0) {
-                                *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.out) +
-                                                          8 * (((long)b * a.Gout + c0 / 8 + h) * g.vol + q)) = pack_cell(v + 8 * h);
-                            } else {   // a channel offset inside a cell: channel by channel
-#pragma unroll
-                                for (int j = 0; j < 8; ++j)
-                                    if (cb + 8 * h + j < a.Cout) {
-                                        const int c = c0 + 8 * h + j;
-                                        reinterpret_cast<bf16*>(a.out)[8 * (((long)b * a.Gout + c / 8) * g.vol + q) + c % 8] =
-                                            __float2bfloat16(v[8 * h + j]);
-                                    }
+                                    for (int j = 0; j < 8; ++j)
+                                        if (cb + 8 * h + j < a.Cout) {
+                                            const int c = c0 + 8 * h + j;
+                                            reinterpret_cast<bf16*>(a.out)[8 * (((long)b * a.Gout + c / 8) * g.vol + q) + c % 8] =
+                                                __float2bfloat16(v[8 * h + j]);
+                                        }
+                                }
                             }
                         }
                     }
@@ -342,11 +385,13 @@ __global__ void __launch_bounds__(CT_THREADS, 1) conv_cells_kernel(const __grid_
         fail_any = 1;
     }
     __syncthreads();
-    if (fail_any && lane == 0) {
-        if (warp == 0) {   // the copies of the last (at most nst) issued stages may still be in flight
+    if (fail_any) {
+        if (warp == 0 && lane == 0) {   // the copies of the last (at most nst, two) issued stages and chunks may still be in flight
             for (long k = issued > a.nst ? issued - a.nst : 0; k < issued; ++k)
                 bar_wait(s32(&full[k % a.nst]), (uint32_t)((k / a.nst) & 1), CT_WAIT);
-        } else if (warp == 1) {
+            for (long k = wissued > 2 ? wissued - 2 : 0; k < wissued; ++k)
+                bar_wait(s32(&wfull[k & 1]), (uint32_t)((k >> 1) & 1), CT_WAIT);
+        } else if ((warp == 1 || warp >= 10) && elect_one()) {   // the lane that issued (the election is deterministic)
             mma_commit(s32(&drainb));
             bar_wait(s32(&drainb), 0, CT_WAIT);
         }
@@ -482,11 +527,11 @@ __global__ void __launch_bounds__(CT_THREADS, 1) wgrad_cells_kernel(const __grid
         fail_any = 1;
     }
     __syncthreads();
-    if (fail_any && lane == 0) {
-        if (warp == 0) {
+    if (fail_any) {
+        if (warp == 0 && lane == 0) {
             for (long k = issued > a.nst ? issued - a.nst : 0; k < issued; ++k)
                 bar_wait(s32(&full[k % a.nst]), (uint32_t)((k / a.nst) & 1), CT_WAIT);
-        } else if (warp == 1) {
+        } else if (warp == 1 && elect_one()) {
             mma_commit(s32(&drainb));
             bar_wait(s32(&drainb), 0, CT_WAIT);
         }
@@ -496,9 +541,9 @@ __global__ void __launch_bounds__(CT_THREADS, 1) wgrad_cells_kernel(const __grid
     if (warp == 1) tmem_free(tmem);
 }
 
-// arranged[kc][t][cg][o][j] = W(o0 + o, 16 kc + 8 cg + j, t) for the output slice o0 .. o0 + Np - 1, zero beyond
-// Cout / Cin; W(o, i, t) = w[(o Cin + i) 27 + t] (wmode 0) or w[(i Cout + o) 27 + 26 - t] (wmode 1: the data
-// gradient's flipped, transposed weights)
+// arranged[kc][3 dy + dx][cg][2 - dz][o][j] = W(o0 + o, 16 kc + 8 cg + j, t), t = 9 dz + 3 dy + dx, for the output slice
+// o0 .. o0 + Np - 1, zero beyond Cout / Cin; W(o, i, t) = w[(o Cin + i) 27 + t] (wmode 0) or
+// w[(i Cout + o) 27 + 26 - t] (wmode 1: the data gradient's flipped, transposed weights)
 __global__ void arrange_w_kernel(const bf16* __restrict__ w, int Cin, int Cout, int o0, int wmode, int Np, int nkc,
                                  bf16* __restrict__ dst) {
     const size_t n = (size_t)nkc * 27 * 2 * Np * 8;
@@ -508,10 +553,12 @@ __global__ void arrange_w_kernel(const bf16* __restrict__ w, int Cin, int Cout, 
         r /= 8;
         const int o = (int)(r % Np);
         r /= Np;
+        const int dz = 2 - (int)(r % 3);
+        r /= 3;
         const int cg = (int)(r % 2);
         r /= 2;
-        const int t = (int)(r % 27);
-        const int kc = (int)(r / 27);
+        const int t = 9 * dz + (int)(r % 9);
+        const int kc = (int)(r / 9);
         const int i = 16 * kc + 8 * cg + j, oo = o0 + o;
         bf16 v = __float2bfloat16(0.f);
         if (oo < Cout && i < Cin)
@@ -565,28 +612,32 @@ helm_status conv_cells(const CellGrid& g, int mode, const bf16* in, int Cin, con
         a.mask = mask;
         a.gb = gb ? gb + o0 : nullptr;
         a.status = status;
-        // the largest tile whose count still gives every SM two (small grids: smaller tiles), within 256
-        // accumulator columns; tiles of one plane share its halo rows, so larger is better for the copies
-        int R = std::min(CT_RMAX, 256 / a.Np);
-        auto tiles = [&](int r) { return (long)g.B * g.Z * ((g.span + 128 * r - 1) / (128 * r)); };
-        while (R > 1 && tiles(R) < 2L * sms) R = (R + 1) / 2;
+        // the largest tile whose count still gives every SM two (small grids: shorter runs, then fewer planes), within
+        // 256 accumulator columns: more planes save MMAs, longer runs share their halo rows
+        int R = CT_RMAX, S = std::max(1, CT_PLANES / a.Np);
+        auto tiles = [&](int r, int sp) { return (long)g.B * ((g.Z + sp - 1) / sp) * ((g.span + 128 * r - 1) / (128 * r)); };
+        while (R > 1 && tiles(R, S) < 2L * sms) R /= 2;
+        while (S > 1 && tiles(R, S) < 2L * sms) S = (S + 1) / 2;
         a.R = R;
+        a.S = S;
         a.ntp = (g.span + 128 * R - 1) / (128 * R);
-        a.ntiles = (int)tiles(R);
+        a.nzg = (g.Z + S - 1) / S;
+        a.ntiles = (int)tiles(R, S);
         // one run with the rows between the three dy views, or three runs where that is shorter (long rows)
         a.split = g.pitch > 128 * R + 2;
         a.dstride = a.split ? 128 * R + 2 : g.pitch;
         a.L = a.split ? 3 * a.dstride : 128 * R + 2 + 2 * g.pitch;
-        a.stage = (2 * a.L * 16 + 9 * 2 * a.Np * 16 + 127) / 128 * 128;
-        a.nst = std::min(CT_NST, (CT_SMEM - 128) / a.stage);
+        a.stage = (2 * a.L * 16 + 127) / 128 * 128;
+        const int wbytes = 27 * 2 * a.Np * 16;
+        a.nst = std::min(CT_NST, (CT_SMEM - 128 - 2 * wbytes) / a.stage);
         const size_t na = (size_t)nkc * 27 * 2 * a.Np * 8;
         arrange_w_kernel<<<(unsigned)((na + 255) / 256), 256, 0, s>>>(w, Cin, Cout, o0, wmode, a.Np, nkc, wscr);
-        const size_t smem = (size_t)a.nst * a.stage + 128;
+        const size_t smem = (size_t)a.nst * a.stage + 2 * wbytes + 128;
         const unsigned grid = (unsigned)std::min((long)a.ntiles, (long)sms);
-        if (mode == CONV_CELLS) conv_cells_kernel<CONV_CELLS><<<grid, CT_THREADS, smem, s>>>(a);
-        else if (mode == CONV_PLANAR) conv_cells_kernel<CONV_PLANAR><<<grid, CT_THREADS, smem, s>>>(a);
-        else if (mode == CONV_F32CELLS) conv_cells_kernel<CONV_F32CELLS><<<grid, CT_THREADS, smem, s>>>(a);
-        else conv_cells_kernel<CONV_GRAD><<<grid, CT_THREADS, smem, s>>>(a);
+        if (mode == CONV_CELLS) conv_cells_kernel<CONV_CELLS><<<grid, CV_THREADS, smem, s>>>(a);
+        else if (mode == CONV_PLANAR) conv_cells_kernel<CONV_PLANAR><<<grid, CV_THREADS, smem, s>>>(a);
+        else if (mode == CONV_F32CELLS) conv_cells_kernel<CONV_F32CELLS><<<grid, CV_THREADS, smem, s>>>(a);
+        else conv_cells_kernel<CONV_GRAD><<<grid, CV_THREADS, smem, s>>>(a);
         HELM_CUDA_TRY(cudaGetLastError());
     }
     return HELM_OK;
