@@ -152,7 +152,7 @@ struct helm_ctx {
     int tune_stencil = 0;                   // complex64 matvec variant chosen by helm_autotune (0 = cp.async ring)
     int zring_sms = 0;                      // SM count, set with the ring kernel's attributes at set-up
     int zpiv_ready = 0;                     // shared-memory attribute of the pivot-recomputing z-solve set
-    void* zck = nullptr;                    // pivot checkpoints of that z-solve ([block][line pair] float4)
+    void* zck = nullptr;                    // checkpoints of that z-solve ([block][state][line pair] float4)
     int zpiv_off = 0;                       // set while capturing launches that may run concurrently (batch lanes)
     int zck_slot = 0;                       // first checkpoint slot of the z-solve launches being captured (batch plans)
     size_t zck_bytes = 0;
@@ -223,7 +223,7 @@ helm_status tc_ypass_h16(helm_ctx* c, int inverse, const void* in, void* out, fl
 helm_status h16_scales(helm_ctx* c, cudaStream_t s);
 helm_status precond_h16_basis(helm_ctx* c, const uint16_t* V16, float2* z, const double* cs, int cidx, cudaStream_t s);
 helm_status to_h16_basis(helm_ctx* c, const float2* r, uint16_t* V16, const double* sigma, int sidx, cudaStream_t s);
-helm_status launch_zsolve_h16(helm_ctx* c, const void* in, void* out, float4* dscr, float oscale, cudaStream_t s,
+helm_status launch_zsolve_h16(helm_ctx* c, const void* in, void* out, float oscale, cudaStream_t s,
                               int nb = 1, double* h16d = nullptr, float gain = 1.f);
 // operand sets of tc_xpass/tc_ypass (`inverse`): 0/1 EigT forward/inverse, 2/3 PFFT sine forward/inverse
 helm_status tc_prepare_sine(helm_ctx* c, const double2* Sx, const double2* Sy, const double2* SxT, const double2* SyT,

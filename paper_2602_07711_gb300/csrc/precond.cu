@@ -161,7 +161,7 @@ helm_status h16_chain(helm_ctx* c, const uint16_t* In, uint16_t* T1, float2* z, 
     st = tc_ypass_h16(c, 0, T1, T0, sc[2], s, nb, d, c->h16g[0]);
     prof_end(c, s);
     if (st != HELM_OK) return st;
-    if ((st = launch_zsolve_h16(c, T0, T0, reinterpret_cast<float4*>(z), sc[3], s, nb, d, c->h16g[1])) != HELM_OK) return st;
+    if ((st = launch_zsolve_h16(c, T0, T0, sc[3], s, nb, d, c->h16g[1])) != HELM_OK) return st;
     prof_begin(c, s, PROF_YPASS);
     st = tc_ypass_h16(c, 1, T0, T1, sc[4], s, nb, d, c->h16g[2]);
     prof_end(c, s);
@@ -176,8 +176,8 @@ helm_status h16_chain(helm_ctx* c, const uint16_t* In, uint16_t* T1, float2* z, 
 // EigT with 16-bit intermediate grids (HELM_PREC_BF16, HELM_PREC_FP16): r (complex64) -> 16 bits ->
 // x-pass -> y-pass -> z-solve -> y-pass -> x-pass -> z (complex64), every stored grid times its power-of-two
 // stage scale c->h16s (FP16; all 1 for BF16, whose range is FP32's), the last pass undoing them.  The two
-// 16-bit grids live in the halves of the context's scratch vector (T0, T1); the z-solve keeps its FP32
-// forward values in z, which is free until the last pass, so r may alias z.
+// 16-bit grids live in the halves of the context's scratch vector (T0, T1); z is written by the last pass alone, so r
+// may alias z.
 helm_status precond_h16(helm_ctx* c, const float2* r, float2* z, const double* sigma, int sidx, cudaStream_t s) {
     const size_t n = c->npts;
     const int H = c->opt.precision == HELM_PREC_FP16 ? 2 : 1;

@@ -466,23 +466,29 @@ __global__ void __launch_bounds__(ZRT) zsolve_ring_kernel(int nx, int ny, int nz
 }
 
 // EigT form without the factor stream: the pivots depend only on the line's lateral shift
-// s_ij = alpha_x d_{x,i} + alpha_y d_{y,j} and the plane, so the forward sweep recomputes them step by step
-// (the same operations as zfactor_kernel, one reciprocal per step) and saves the recurrence's state
-// c'_{l-1} at the start of every block of ZU2 steps to a small scratch (2 bytes per point, [block][pair]
-// so that a warp's saves are one contiguous row); the backward sweep recomputes the ZU2 factors of a block
-// forward from its checkpoint into registers and then runs the block backwards.  HBM sees y read, the
-// forward values written over the output and read back (mostly from L2), and x written: the 8 bytes per
-// point of factors and their L2 footprint are gone.  A grid is one thread per pair of lines (32k threads
-// at 256^3, three to four 64-thread CTAs per SM), so latency is hidden by prefetch depth: a six-block ring
-// per thread (48 steps ahead, 48 KiB per CTA), and each backward block's checkpoint is loaded one block
-// ahead of its use.  The recurrence is the bound where the grid is small (one reciprocal and six dependent operations
-// a step), and everything else is kept off it: cz comes from shared memory, and the blocks without an end row run
-// without per-step conditions, behind which each step's loads used to wait.  Measured: 256^3, FP16 chain 105 -> 74
-// us; 200^3 FP32 63 -> 41; 150 x 100 x 75 25 -> 15; 32^3 10.6 -> 8.9.
+// s_ij = alpha_x d_{x,i} + alpha_y d_{y,j} and the plane, so the sweeps recompute them step by step (the same
+// operations as zfactor_kernel, one reciprocal per step).  The forward sweep writes no forward values either: it only
+// saves the recurrences' state (c'_{l-1}, d_{l-1}) at the start of every block of ZU2 steps to a small scratch (4
+// bytes per point, [block][pair] so that a warp's saves are contiguous rows), and the backward sweep recomputes a
+// block's factors and forward values from its checkpoint and from y, read a second time.  HBM and L2 see y read twice
+// and x written: for 16-bit grids 12 bytes a point where forward values in FP32 took 28.
+// A grid is one thread per pair of lines (32k threads at 256^3, three to four 64-thread CTAs per SM), so latency is
+// hidden by prefetch depth: a six-block ring per thread (48 steps ahead).  Block b lives in slot b mod 6 in both
+// sweeps, so the last six blocks need no second read.  ALL: grids of few CTAs hold every block of their lines
+// (and the checkpoints) in shared memory: one read, all loads in flight at once.
+// The recurrence is the bound where the grid is small (one reciprocal and six dependent operations a step), and
+// everything else is kept off it: cz comes from shared memory, and the blocks without an end row run without
+// per-step conditions, behind which each step's loads used to wait.
+// CTAs of 32 threads, for a fuller last wave, gain nothing.
+// Measured (with per-step conditions; without; without forward values): 256^3, FP16 chain 105, 74, 59 us; 200^3 FP32
+// 63, 41, 40; 150 x 100 x 75 25, 15, 13; 32^3 10.6, 8.9, 7.5.
 constexpr int ZPB = 6;   // ring depth (blocks) of the pivot-recomputing kernel
-// the ring (48 KiB) and cz
-constexpr size_t zpiv_smem(int nz) { return (size_t)ZPB * ZU2 * ZRT * sizeof(float4) + (size_t)nz * sizeof(float2); }
-constexpr int ZPIV_SMEM_MAX = (int)zpiv_smem(512);
+// a step of a line pair: FP32 16 bytes, 16-bit 8; then cz, and for ALL the checkpoints
+constexpr size_t zpiv_smem(int nz, bool h16, bool all) {
+    return (size_t)(all ? (nz + ZU2 - 1) / ZU2 : ZPB) * ZU2 * ZRT * (h16 ? 8 : 16) + (size_t)(nz + 1) / 2 * sizeof(float4) +
+           (all ? (size_t)((nz + ZU2 - 1) / ZU2) * 2 * ZRT * sizeof(float4) : 0);
+}
+constexpr size_t ZPIV_ALL_MAX = 112 * 1024;   // two CTAs per SM
 template <bool B>
 struct BoolC {
     constexpr operator bool() const { return B; }
@@ -505,6 +511,13 @@ __device__ __forceinline__ float4 h4_to_f4(uint2 w) {
     return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
                        __uint_as_float(w.y & 0xFFFF0000u));
 }
+// a step's input values of a line pair as stored, and widened
+template <bool BF> struct ZPairOf { typedef float4 T; };
+template <> struct ZPairOf<true> { typedef uint2 T; };
+template <int H>
+__device__ __forceinline__ float4 zwiden(float4 v) { return v; }
+template <int H>
+__device__ __forceinline__ float4 zwiden(uint2 v) { return h4_to_f4<H>(v); }
 template <int H>
 __device__ __forceinline__ uint32_t zpack16(float lo, float hi) {
     if (H == 2) {
@@ -515,17 +528,16 @@ __device__ __forceinline__ uint32_t zpack16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// H (1 BF16, 2 FP16): y read and x written (times oscale) in 16 bits (uint2 per line pair), the forward
-// values d kept in FP32 in dscr (a complex64-sized grid of the caller); H = 0: float4 in and out and
-// dscr = out (d over the output).
-template <int H>
-__global__ void __launch_bounds__(ZRT, 4) zsolve_piv_kernel(int nx, int ny, int nz, float zz, float2 gz,
-                                                           const float2* __restrict__ dxs,
-                                                           const float2* __restrict__ dys,
-                                                           const float2* __restrict__ cz, const void* inv, void* outv,
-                                                           float4* dscr, float4* __restrict__ ck, int nb,
-                                                           float oscale = 1.f, double* __restrict__ h16d = nullptr,
-                                                           float gain = 1.f) {
+// H (1 BF16, 2 FP16): y read and x written (times oscale) in 16 bits (uint2 per line pair); H = 0: float4.  in may
+// equal out.
+template <int H, bool ALL>
+__global__ void __launch_bounds__(ZRT, ALL ? 2 : 4) zsolve_piv_kernel(int nx, int ny, int nz, float zz, float2 gz,
+                                                                      const float2* __restrict__ dxs,
+                                                                      const float2* __restrict__ dys,
+                                                                      const float2* __restrict__ cz, const void* inv,
+                                                                      void* outv, float4* __restrict__ ck, int nb,
+                                                                      float oscale = 1.f, double* __restrict__ h16d = nullptr,
+                                                                      float gain = 1.f) {
     constexpr bool BF = H != 0;
     // FP16 chain with dynamic stage scales (h16d): the output scale from the bound of ||T2|| (h16d[1]),
     // recorded in h16d[5]; the squared norm of what is stored accumulates into h16d[2]
@@ -541,125 +553,133 @@ __global__ void __launch_bounds__(ZRT, 4) zsolve_piv_kernel(int nx, int ny, int 
         oscale *= sc;
         if (blockIdx.x == 0 && threadIdx.x == 0) h16d[5] = sc;
     }
-    extern __shared__ float4 zsm[];   // [ZPB * ZU2][ZRT], then cz [nz]
-    const float4* in = reinterpret_cast<const float4*>(inv);
-    const uint2* inb = reinterpret_cast<const uint2*>(inv);
-    float4* out = BF ? dscr : reinterpret_cast<float4*>(outv);   // where d goes (and comes back from)
-    uint2* outb = reinterpret_cast<uint2*>(outv);
+    typedef typename ZPairOf<BF>::T Y;   // a step's input values of a line pair
+    extern __shared__ float4 zsm[];      // ring [depth * ZU2][ZRT], cz [nz], ALL: checkpoints [block][2][ZRT]
+    const Y* in = reinterpret_cast<const Y*>(inv);
+    Y* out = reinterpret_cast<Y*>(outv);
     const int tid = threadIdx.x;
     const int hx = nx / 2, npairs = hx * ny, nall = npairs * nb;
-    const int nblk = (nz + ZU2 - 1) / ZU2;
-    const size_t plane = (size_t)hx * ny;   // in float4 (two lines) units
-    float2* scz = reinterpret_cast<float2*>(zsm + (size_t)ZPB * ZU2 * ZRT);
+    const int nblk = (nz + ZU2 - 1) / ZU2, depth = ALL ? nblk : ZPB;
+    const size_t plane = (size_t)hx * ny;   // in line pairs
+    Y* ring = reinterpret_cast<Y*>(zsm);
+    float4* after = zsm + (size_t)depth * ZU2 * ZRT * sizeof(Y) / sizeof(float4);
+    float2* scz = reinterpret_cast<float2*>(after);
+    float4* sck = after + (nz + 1) / 2;
     for (int l = tid; l < nz; l += ZRT) scz[l] = cz[l];
     __syncthreads();
-    auto slot = [&](int st) -> float4* { return &zsm[(size_t)st * ZRT + tid]; };
+    auto slot = [&](int blk, int u) -> Y* { return ring + (size_t)((ALL ? blk : blk % ZPB) * ZU2 + u) * ZRT + tid; };
     for (int prb = blockIdx.x * ZRT + tid; prb < nall; prb += gridDim.x * ZRT) {
         const int pr = prb % npairs, vb = prb / npairs;
         const int j = pr / hx, i0 = 2 * (pr - j * hx);
-        const float2 s0 = make_float2(__fadd_rn(dxs[i0].x, dys[j].x), __fadd_rn(dxs[i0].y, dys[j].y));
-        const float2 s1 = make_float2(__fadd_rn(dxs[i0 + 1].x, dys[j].x), __fadd_rn(dxs[i0 + 1].y, dys[j].y));
         const size_t base = (size_t)vb * plane * nz + (size_t)pr;
-        // block blk (steps l = blk ZU2 + u) of the input (BF: 8 bytes per step into the first half of a slot) or of
-        // the forward values into ring position pos
-        auto fetch = [&](bool input, int blk, int pos) {
+        // the input of block blk (steps l = blk ZU2 + u) into its slot; one group per call, empty ones included
+        auto fetch = [&](int blk) {
             if (blk >= 0 && blk < nblk) {
-                const size_t o = base + (size_t)(blk * ZU2) * plane;
+                const Y* src = in + base + (size_t)(blk * ZU2) * plane;
                 const int n = min(ZU2, nz - blk * ZU2);
 #pragma unroll
-                for (int u = 0; u < ZU2; ++u) {
-                    float4* d = slot((pos % ZPB) * ZU2 + u);
+                for (int u = 0; u < ZU2; ++u)
                     if (u < n) {
-                        if (BF && input) zcp8(d, inb + o + (size_t)u * plane);
-                        else zcp16(d, (input ? in : out) + o + (size_t)u * plane);
+                        if (BF) zcp8(slot(blk, u), src + (size_t)u * plane);
+                        else zcp16(slot(blk, u), src + (size_t)u * plane);
                     }
-                }
             }
             zcommit();
         };
+        for (int b = 0; b < depth - (ALL ? 0 : 1); ++b) fetch(b);
+        const float2 s0 = make_float2(__fadd_rn(dxs[i0].x, dys[j].x), __fadd_rn(dxs[i0].y, dys[j].y));
+        const float2 s1 = make_float2(__fadd_rn(dxs[i0 + 1].x, dys[j].x), __fadd_rn(dxs[i0 + 1].y, dys[j].y));
         // blocks whose steps are all interior (off-diagonals 1, no corner) run without per-step conditions: with
         // them, every step's loads waited inside the recurrence
         auto interior = [&](int blk) { return blk > 0 && blk * ZU2 + ZU2 < nz; };
-        // one pivot step of both lines: m_l and the new c'_l from c'_{l-1}
-        auto pivots = [&](auto edge, int l, float2& c0, float2& c1, float2& m0, float2& m1) {
-            const bool end = edge && (l == 0 || l == nz - 1);
-            const float a = !edge ? 1.f : (l == 0 ? 0.f : (l == nz - 1 ? zz : 1.f));
-            const float sup = !edge ? 1.f : (l == nz - 1 ? 0.f : (l == 0 ? zz : 1.f));
-            const float2 czl = scz[l];
-            m0 = zpivot(s0, czl, end, gz, a, sup, c0);
-            m1 = zpivot(s1, czl, end, gz, a, sup, c1);
-        };
-        // ---- forward: d_l = (y_l - a_l d_{l-1}) m_l
-        for (int b = 0; b < ZPB - 1; ++b) fetch(true, b, b);
-        float2 d0 = f2(0.f, 0.f), d1 = d0, c0 = d0, c1 = d0;
-        auto fwd = [&](auto edge, int b) {
+        // block blk forward from the state c0, c1 (c'_{l-1}) and d0, d1 (d_{l-1}): its factors m and values
+        // d_l = (y_l - a_l d_{l-1}) m_l go to keep(u, m0, m1, d0, d1)
+        auto forward = [&](auto edge, int blk, float2& c0, float2& c1, float2& d0, float2& d1, auto keep) {
             float4 y[ZU2];
 #pragma unroll
-            for (int u = 0; u < ZU2; ++u)
-                y[u] = BF ? h4_to_f4<H>(*reinterpret_cast<const uint2*>(slot((b % ZPB) * ZU2 + u)))
-                          : *slot((b % ZPB) * ZU2 + u);
-            float4* o = out + base + (size_t)(b * ZU2) * plane;
-#pragma unroll
-            for (int u = 0; u < ZU2; ++u) {
-                const int l = b * ZU2 + u;
-                if (!edge || l < nz) {
-                    const float a = !edge ? 1.f : (l == 0 ? 0.f : (l == nz - 1 ? zz : 1.f));
-                    float2 m0, m1;
-                    pivots(edge, l, c0, c1, m0, m1);
-                    d0 = zfwd(f2(y[u].x, y[u].y), d0, a, m0);
-                    d1 = zfwd(f2(y[u].z, y[u].w), d1, a, m1);
-                    o[(size_t)u * plane] = make_float4(d0.x, d0.y, d1.x, d1.y);
-                }
-            }
-        };
-        for (int b = 0; b < nblk; ++b) {
-            fetch(true, b + ZPB - 1, b + ZPB - 1);
-            zwait_piv();   // block b has landed
-            ck[(size_t)b * nall + prb] = make_float4(c0.x, c0.y, c1.x, c1.y);
-            if (interior(b)) fwd(BoolC<false>(), b);
-            else fwd(BoolC<true>(), b);
-        }
-        zwait_all();
-        __threadfence_block();
-        // ---- backward: x_l = d_l - sup_l m_l x_{l+1}, blocks in decreasing order
-        for (int b = 0; b < ZPB - 1; ++b) fetch(false, nblk - 1 - b, b);
-        float2 x0 = f2(0.f, 0.f), x1 = x0;
-        float4 cnext = ck[(size_t)(nblk - 1) * nall + prb];
-        auto bwd = [&](auto edge, int b, int blk, const float4& cv) {
-            float2 cc0 = f2(cv.x, cv.y), cc1 = f2(cv.z, cv.w);
-            float2 m0[ZU2], m1[ZU2];
+            for (int u = 0; u < ZU2; ++u) y[u] = zwiden<H>(*slot(blk, u));
 #pragma unroll
             for (int u = 0; u < ZU2; ++u) {
                 const int l = blk * ZU2 + u;
-                m0[u] = m1[u] = f2(0.f, 0.f);
-                if (!edge || l < nz) pivots(edge, l, cc0, cc1, m0[u], m1[u]);
+                if (!edge || l < nz) {
+                    const bool end = edge && (l == 0 || l == nz - 1);
+                    const float a = !edge ? 1.f : (l == 0 ? 0.f : (l == nz - 1 ? zz : 1.f));
+                    const float sup = !edge ? 1.f : (l == nz - 1 ? 0.f : (l == 0 ? zz : 1.f));
+                    const float2 czl = scz[l];
+                    const float2 m0 = zpivot(s0, czl, end, gz, a, sup, c0), m1 = zpivot(s1, czl, end, gz, a, sup, c1);
+                    d0 = zfwd(f2(y[u].x, y[u].y), d0, a, m0);
+                    d1 = zfwd(f2(y[u].z, y[u].w), d1, a, m1);
+                    keep(u, m0, m1, d0, d1);
+                }
             }
-            zwait_piv();
-            const size_t o = base + (size_t)(blk * ZU2) * plane;
+        };
+        auto save = [&](int b, const float4& c, const float4& d) {
+            float4* o = ALL ? sck + (size_t)(2 * b) * ZRT + tid : ck + (size_t)(2 * b) * nall + prb;
+            o[0] = c;
+            o[ALL ? ZRT : nall] = d;
+        };
+        auto state = [&](int b, float4& c, float4& d) {
+            const float4* o = ALL ? sck + (size_t)(2 * b) * ZRT + tid : ck + (size_t)(2 * b) * nall + prb;
+            c = o[0];
+            d = o[ALL ? ZRT : nall];
+        };
+        // ---- forward: the checkpoints (the last block's values are formed by the backward sweep alone)
+        float2 d0 = f2(0.f, 0.f), d1 = d0, c0 = d0, c1 = d0;
+        if (ALL) zwait_all();
+        for (int b = 0; b < nblk; ++b) {
+            if (!ALL) {
+                fetch(b + ZPB - 1);
+                zwait_piv();   // block b has landed
+            }
+            save(b, make_float4(c0.x, c0.y, c1.x, c1.y), make_float4(d0.x, d0.y, d1.x, d1.y));
+            if (b == nblk - 1) break;
+            auto none = [](int, float2, float2, float2, float2) {};
+            if (interior(b)) forward(BoolC<false>(), b, c0, c1, d0, d1, none);
+            else forward(BoolC<true>(), b, c0, c1, d0, d1, none);
+        }
+        // ---- backward: x_l = d_l - sup_l m_l x_{l+1}, blocks in decreasing order
+        float2 x0 = f2(0.f, 0.f), x1 = x0;
+        float4 cn, dn;
+        state(nblk - 1, cn, dn);
+        auto bwd = [&](auto edge, int blk, const float4& cv, const float4& dv) {
+            float2 e0 = f2(cv.x, cv.y), e1 = f2(cv.z, cv.w), g0 = f2(dv.x, dv.y), g1 = f2(dv.z, dv.w);
+            float2 m0[ZU2], m1[ZU2], v0[ZU2], v1[ZU2];
+            forward(edge, blk, e0, e1, g0, g1, [&](int u, float2 a, float2 b, float2 p, float2 q) {
+                m0[u] = a;
+                m1[u] = b;
+                v0[u] = p;
+                v1[u] = q;
+            });
+            Y* o = out + base + (size_t)(blk * ZU2) * plane;
 #pragma unroll
             for (int uu = 0; uu < ZU2; ++uu) {
                 const int u = ZU2 - 1 - uu, l = blk * ZU2 + u;
                 if (!edge || l < nz) {
-                    const float4 dv = *slot((b % ZPB) * ZU2 + u);
                     const float sup = !edge ? 1.f : (l == nz - 1 ? 0.f : (l == 0 ? zz : 1.f));
-                    x0 = zbwd(f2(dv.x, dv.y), m0[u], x0, sup);
-                    x1 = zbwd(f2(dv.z, dv.w), m1[u], x1, sup);
-                    if (BF) {
+                    x0 = zbwd(v0[u], m0[u], x0, sup);
+                    x1 = zbwd(v1[u], m1[u], x1, sup);
+                    if constexpr (BF) {
                         const float a = oscale * x0.x, b2 = oscale * x0.y, c2 = oscale * x1.x, d2 = oscale * x1.y;
-                        outb[o + (size_t)u * plane] = make_uint2(zpack16<H>(a, b2), zpack16<H>(c2, d2));
+                        o[(size_t)u * plane] = make_uint2(zpack16<H>(a, b2), zpack16<H>(c2, d2));
                         nacc = fmaf(a, a, fmaf(b2, b2, fmaf(c2, c2, fmaf(d2, d2, nacc))));
+                    } else {
+                        o[(size_t)u * plane] = make_float4(x0.x, x0.y, x1.x, x1.y);
                     }
-                    else out[o + (size_t)u * plane] = make_float4(x0.x, x0.y, x1.x, x1.y);
                 }
             }
         };
         for (int b = 0; b < nblk; ++b) {
-            fetch(false, nblk - 1 - (b + ZPB - 1), b + ZPB - 1);
             const int blk = nblk - 1 - b;
-            const float4 cv = cnext;
-            if (blk > 0) cnext = ck[(size_t)(blk - 1) * nall + prb];   // the next block's checkpoint, early
-            if (interior(blk)) bwd(BoolC<false>(), b, blk, cv);
-            else bwd(BoolC<true>(), b, blk, cv);
+            if (!ALL) {
+                // the last ZPB blocks are still in their slots; slot of block blk + 1 is free for blk - (ZPB - 1)
+                if (b > 0) fetch(blk - (ZPB - 1));
+                else zcommit();
+                zwait_piv();   // block blk has landed
+            }
+            const float4 cv = cn, dv = dn;
+            if (blk > 0) state(blk - 1, cn, dn);   // the next block's checkpoint, early
+            if (interior(blk)) bwd(BoolC<false>(), blk, cv, dv);
+            else bwd(BoolC<true>(), blk, cv, dv);
         }
         zwait_all();
     }
@@ -766,7 +786,7 @@ static helm_status launch_zsolve_part(helm_ctx* c, const float2* in, float2* out
 }
 
 size_t zsolve_ck_bytes(const helm_ctx* c, int nb) {
-    return (size_t)((c->nz + ZU2 - 1) / ZU2) * (size_t)(c->nx / 2) * c->ny * nb * sizeof(float4);
+    return (size_t)((c->nz + ZU2 - 1) / ZU2) * 2 * (size_t)(c->nx / 2) * c->ny * nb * sizeof(float4);
 }
 
 // the pivot checkpoints of nb right-hand sides per z-solve launch (device memory of the context)
@@ -778,6 +798,35 @@ helm_status zsolve_reserve(helm_ctx* c, int nb) {
     c->zck_bytes = 0;
     if (cudaMalloc(&c->zck, bytes) != cudaSuccess) { cudaGetLastError(); return HELM_ERR_NOMEM; }
     c->zck_bytes = bytes;
+    return HELM_OK;
+}
+
+// the pivot-recomputing kernel on checkpoint slots slot .. slot + nb - 1
+template <int H>
+static helm_status run_zpiv(helm_ctx* c, const void* in, void* out, int slot, int nb, float oscale, double* h16d, float gain,
+                            cudaStream_t s) {
+    const int need = (c->nx / 2 * c->ny * nb + ZRT - 1) / ZRT;
+    const int cap = c->zring_sms * 2 * (c->tune_zring > 0 ? c->tune_zring : 1);   // tune_zring 1..3: 2, 4 or 6 CTAs per SM
+    // lines held whole where all CTAs fit the SMs that way, two on each
+    const size_t all = zpiv_smem(c->nz, H != 0, true), ring = zpiv_smem(c->nz, H != 0, false);
+    const bool whole = all <= ZPIV_ALL_MAX && need <= 2 * c->zring_sms;
+    float4* ck = reinterpret_cast<float4*>(c->zck) + (size_t)slot * zsolve_ck_bytes(c, 1) / sizeof(float4);
+    const float2 gz = make_float2((float)c->gam[2].x, (float)c->gam[2].y);
+    if (!(c->zpiv_ready & (1 << H))) {
+        HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_piv_kernel<H, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)zpiv_smem(512, H != 0, false)));
+        HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_piv_kernel<H, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)ZPIV_ALL_MAX));
+        c->zpiv_ready |= 1 << H;
+    }
+    if (whole)
+        zsolve_piv_kernel<H, true><<<need, ZRT, all, s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2], gz, c->dxs, c->dys, c->cz, in,
+                                                          out, ck, nb, oscale, h16d, gain);
+    else
+        zsolve_piv_kernel<H, false><<<need < cap ? need : cap, ZRT, ring, s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2], gz,
+                                                                               c->dxs, c->dys, c->cz, in, out, ck, nb, oscale,
+                                                                               h16d, gain);
+    HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
 }
 
@@ -793,7 +842,6 @@ helm_status launch_zsolve(helm_ctx* c, const float2* in, float2* out, cudaStream
         // of the context (grown here outside stream capture; a capturing caller reserves it beforehand)
         // (c->zck_slot: the first checkpoint slot of this launch; concurrent solves of one context in a batch
         // plan each capture with their own slots)
-        const int npairs = c->nx / 2 * c->ny * nb;
         const int slot = c->zck_slot;
         if (zsolve_ck_bytes(c, slot + nb) > c->zck_bytes) {
             cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -802,33 +850,18 @@ helm_status launch_zsolve(helm_ctx* c, const float2* in, float2* out, cudaStream
             helm_status st;
             if ((st = zsolve_reserve(c, slot + nb)) != HELM_OK) return st;
         }
-        if (!(c->zpiv_ready & 1)) {
-            HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_piv_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               ZPIV_SMEM_MAX));
-            c->zpiv_ready |= 1;
-        }
         prof_begin(c, s, PROF_ZSOLVE);
-        const int sms = c->zring_sms;
-        const int need = (npairs + ZRT - 1) / ZRT;
-        const int cap = sms * 2 * c->tune_zring;   // tune_zring 1..3: 2, 4 or 6 CTAs per SM (at most 4 resident)
-        const int grid = need < cap ? need : cap;
-        zsolve_piv_kernel<0><<<grid, ZRT, zpiv_smem(c->nz), s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2],
-                                                               make_float2((float)c->gam[2].x, (float)c->gam[2].y), c->dxs,
-                                                               c->dys, c->cz, in, out, reinterpret_cast<float4*>(out),
-                                                               reinterpret_cast<float4*>(c->zck) + (size_t)slot * zsolve_ck_bytes(c, 1) / sizeof(float4),
-                                                               nb);
+        const helm_status st = run_zpiv<0>(c, in, out, slot, nb, 1.f, nullptr, 1.f, s);
         prof_end(c, s);
-        HELM_CUDA_TRY(cudaGetLastError());
-        return HELM_OK;
+        return st;
     }
     return launch_zsolve_fact(c, c->zfac, in, out, s, nb);
 }
 
 // The z-solves of the 16-bit transform chain (HELM_PREC_BF16, HELM_PREC_FP16): the pivot-recomputing kernel
-// with 16-bit y and x (in may equal out; x scaled by oscale) and the FP32 forward values in dscr (npts * nb
-// complex64 of the caller).  No fallback: a launch under stream capture without reserved checkpoints
-// returns HELM_ERR_UNSUPPORTED.
-helm_status launch_zsolve_h16(helm_ctx* c, const void* in, void* out, float4* dscr, float oscale, cudaStream_t s, int nb,
+// with 16-bit y and x (in may equal out; x scaled by oscale).  No fallback: a launch under stream capture without
+// reserved checkpoints returns HELM_ERR_UNSUPPORTED.
+helm_status launch_zsolve_h16(helm_ctx* c, const void* in, void* out, float oscale, cudaStream_t s, int nb,
                               double* h16d, float gain) {
     const int H = c->opt.precision == HELM_PREC_FP16 ? 2 : 1;
     if (c->nx % 2 != 0 || c->zring_sms <= 0) return HELM_ERR_UNSUPPORTED;
@@ -840,27 +873,9 @@ helm_status launch_zsolve_h16(helm_ctx* c, const void* in, void* out, float4* ds
         helm_status st;
         if ((st = zsolve_reserve(c, slot + nb)) != HELM_OK) return st;
     }
-    if (!(c->zpiv_ready & (2 << (H - 1)))) {
-        if (H == 2)
-            HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_piv_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, ZPIV_SMEM_MAX));
-        else
-            HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_piv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, ZPIV_SMEM_MAX));
-        c->zpiv_ready |= 2 << (H - 1);
-    }
     prof_begin(c, s, PROF_ZSOLVE);
-    const int npairs = c->nx / 2 * c->ny * nb;
-    const int need = (npairs + ZRT - 1) / ZRT;
-    const int cap = c->zring_sms * 2 * (c->tune_zring > 0 ? c->tune_zring : 1);
-    const int grid = need < cap ? need : cap;
-    float4* ck = reinterpret_cast<float4*>(c->zck) + (size_t)slot * zsolve_ck_bytes(c, 1) / sizeof(float4);
-    const float2 gz = make_float2((float)c->gam[2].x, (float)c->gam[2].y);
-    if (H == 2)
-        zsolve_piv_kernel<2><<<grid, ZRT, zpiv_smem(c->nz), s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2], gz, c->dxs, c->dys, c->cz,
-                                                           in, out, dscr, ck, nb, oscale, h16d, gain);
-    else
-        zsolve_piv_kernel<1><<<grid, ZRT, zpiv_smem(c->nz), s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2], gz, c->dxs, c->dys, c->cz,
-                                                           in, out, dscr, ck, nb, oscale);
+    const helm_status st = H == 2 ? run_zpiv<2>(c, in, out, slot, nb, oscale, h16d, gain, s)
+                                  : run_zpiv<1>(c, in, out, slot, nb, oscale, nullptr, 1.f, s);
     prof_end(c, s);
-    HELM_CUDA_TRY(cudaGetLastError());
-    return HELM_OK;
+    return st;
 }

@@ -4,7 +4,9 @@ FP32 transform passes: lengths on both sides of the GEMM's tile widths (32 .. 64
 tile) and K blocks (16), odd ones included.  A pass sums K products of FP32 operands in order: 2-norm error a few
 times sqrt(K) 2^-24, two passes; bound 8 sqrt(K) 2^-24.
 z-solves: depths on both sides of the blocks of 8 steps whose inner ones run without end conditions; bound 1e-4
-(the systems amplify FP32 rounding, here by a few hundred at most).
+(the systems amplify FP32 rounding, here by a few hundred at most).  Wide grids: the same where the lines do not fit
+the SMs whole and pass through the ring of 6 blocks, and the whole FP16 chain there against FP32 within a few hundred
+2^-11.
 Complex64 matvec: every kernel variant, grids from the smallest to several chunk lengths, real and complex k^2, and
 the padded form of the high-order closure (an output that overlaps the operand included).  The terms of A U are up
 to 8/h^2 |U| and cancel to k^2 U, each rounded to 2^-24: bound 32 2^-24 / (k0 h)^2.
@@ -21,7 +23,7 @@ from oracle.eigt import EigT
 from oracle.grid import Grid
 from oracle.operators import Operator
 from oracle.tridiag import thomas
-from paper_2602_07711_gb300 import HELM_C64, HELM_CLOSURE_HIGH_ORDER, Solver, helm
+from paper_2602_07711_gb300 import HELM_C64, HELM_CLOSURE_HIGH_ORDER, HELM_PREC_FP16, Solver, helm
 
 
 def _rand(shape, seed):
@@ -72,6 +74,20 @@ def test_z_solves(nz):
     e = _library_basis(S, g, k0)
     y = _rand(g.shape, nz)
     assert _rel(S.precond_step(2, _dev(y)).cpu().numpy(), thomas(*e.z_coefficients(), y)) < 1e-4
+
+
+@pytest.mark.parametrize("nz", [4, 9, 40, 41, 48, 49, 57])
+def test_z_solves_wide(nz):
+    n = (208, 192, nz)
+    L = [m / 208 for m in n]
+    k0 = 2 * math.pi * 208 / 11
+    k2 = np.full((nz, 192, 208), k0 * k0, complex)
+    S = Solver(n, k2, k0, order=4, L=L)
+    e = _library_basis(S, Grid(*n, *L), k0)
+    y = _rand(k2.shape, nz)
+    assert _rel(S.precond_step(2, _dev(y)).cpu().numpy(), thomas(*e.z_coefficients(), y)) < 1e-4
+    H = Solver(n, k2, k0, order=4, L=L, precision=HELM_PREC_FP16, flexible=True)
+    assert _rel(H.apply_precond(_dev(y)).cpu().numpy(), S.apply_precond(_dev(y)).cpu().numpy()) < 0.1
 
 
 @pytest.mark.parametrize("lossy", [False, True])
