@@ -20,7 +20,7 @@
 // Every mbarrier wait is bounded by the context's wait limit (a kernel argument); on expiry the CTA raises
 // HELM_DEV_WAIT and skips its remaining work.  Before it frees its tensor memory and exits, it drains what
 // it still has in flight under a separate fixed bound: the producer waits for the TMA loads it issued, the
-// MMA thread commits once more and waits for its MMAs.  No cluster multicast is used.
+// MMA thread commits once more and waits for its MMAs.  No TMA multicast is used.
 #include "common.cuh"
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -57,6 +57,7 @@ struct TcState {
     uint16_t* Bxb[2] = {nullptr, nullptr};
     uint16_t* Wyb[2] = {nullptr, nullptr};
     CUtensorMap mapBxb[2], mapBxb256[2], mapWyb[2];
+    int pairs_x = 0, pairs_y = 0;   // CTA pairs of the pair kernels that fit the GPU at once
 };
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -145,11 +146,19 @@ __device__ __forceinline__ float stage_scale(double gain, double nsq) {
 template <int H>
 __device__ __forceinline__ uint32_t pack16(float lo, float hi) {
     if (H == 2) {
-        const __half2 v = __floats2half2_rn(fminf(fmaxf(lo, -65504.f), 65504.f), fminf(fmaxf(hi, -65504.f), 65504.f));
+        // clamped after the rounding, two values at once: infinities from the rounding become the largest value too
+        const __half2 lim = __half2half2(__ushort_as_half(0x7BFF));
+        const __half2 v = __hmin2(__hmax2(__floats2half2_rn(lo, hi), __hneg2(lim)), lim);
         return *reinterpret_cast<const uint32_t*>(&v);
     }
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
+}
+// 32 bytes to a 32-byte aligned address: a whole sector per thread
+__device__ __forceinline__ void store32(void* dst, const uint32_t* w) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                 "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -444,6 +453,130 @@ ypass_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
 }
 
+// ---- epilogue pieces of 32 accumulator columns (gc0 .. gc0 + 31 of the output), one row per thread -------
+// wide: the output rows start on 32-byte boundaries, and each thread writes its row's 64 or 128 bytes as whole sectors
+// straight from its registers.  Else the columns go through the warp's staging rows (stride XEPI_LD words,
+// conflict-free both ways) and out as 64-byte row segments.  The staging shares the shared-memory bandwidth with the
+// MMAs' operand reads: at 256^3 the 16-bit x-pass took 34 us with it and 32 without, the
+// y-pass 37 and 34.5.
+__host__ __device__ __forceinline__ bool rows_aligned(const void* out, int N2, int elem) {
+    return ((reinterpret_cast<uintptr_t>(out) | (uintptr_t)((size_t)N2 * elem)) & 31) == 0;
+}
+// 16 16-bit pairs w of row rbase + lane
+__device__ __forceinline__ void store_pairs(const uint32_t (&w)[16], bool wide, float* stg, int lane, uint16_t* ob, int rbase,
+                                            int gc0, int rows, int N2) {
+    if (wide) {
+        if (rbase + lane < rows) {
+            uint16_t* dst = ob + (size_t)(rbase + lane) * N2 + gc0;
+            if (gc0 < N2) store32(dst, w);
+            if (gc0 + 16 < N2) store32(dst + 16, w + 8);
+        }
+        return;
+    }
+    uint32_t* su = reinterpret_cast<uint32_t*>(stg);
+#pragma unroll
+    for (int v = 0; v < 16; v += 4)
+        *reinterpret_cast<uint4*>(su + lane * XEPI_LD + v) = make_uint4(w[v], w[v + 1], w[v + 2], w[v + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int rr = 8 * i + (lane >> 2), cc = 4 * (lane & 3);
+        const int grow = rbase + rr, gcol = gc0 + 2 * cc;
+        const uint4 v = *reinterpret_cast<const uint4*>(su + rr * XEPI_LD + cc);
+        if (grow < rows && gcol < N2) {
+            uint16_t* dst = ob + (size_t)grow * N2 + gcol;
+            if (gcol + 8 <= N2) *reinterpret_cast<uint4*>(dst) = v;
+            else {
+                const uint32_t e4[4] = {v.x, v.y, v.z, v.w};
+                for (int e = 0; e < 4 && gcol + 2 * e < N2; ++e) reinterpret_cast<uint32_t*>(dst)[e] = e4[e];
+            }
+        }
+    }
+    __syncwarp();
+}
+// squared norm of 16 complex values (columns beyond N2 left out), in two chains
+__device__ __forceinline__ float norm32(const float (&x)[32], int gc0, int N2) {
+    float n0 = 0.f, n1 = 0.f;
+#pragma unroll
+    for (int v = 0; v < 32; v += 2)
+        if (gc0 + 32 <= N2 || gc0 + v < N2) {
+            n0 = fmaf(x[v], x[v], n0);
+            n1 = fmaf(x[v + 1], x[v + 1], n1);
+        }
+    return n0 + n1;
+}
+// x-pass to a 16-bit grid of M rows
+template <int H>
+__device__ __forceinline__ void x_store_h16(const uint32_t (&r)[32], float al, bool wide, float* stg, int lane, void* outv,
+                                            int rbase, int gc0, int M, int N2, bool nsq, float& nacc) {
+    float x[32];
+    uint32_t w[16];
+#pragma unroll
+    for (int v = 0; v < 32; ++v) x[v] = al * __uint_as_float(r[v]);
+#pragma unroll
+    for (int v = 0; v < 16; ++v) w[v] = pack16<H>(x[2 * v], x[2 * v + 1]);
+    if (nsq && rbase + lane < M) nacc += norm32(x, gc0, N2);
+    store_pairs(w, wide, stg, lane, reinterpret_cast<uint16_t*>(outv), rbase, gc0, M, N2);
+}
+// x-pass to an FP32 grid of M rows
+__device__ __forceinline__ void x_store_f32(const uint32_t (&r)[32], float al, bool wide, float* stg, int lane, float* out,
+                                            int rbase, int gc0, int M, int N2) {
+    if (wide) {
+        if (rbase + lane < M) {
+            float* dst = out + (size_t)(rbase + lane) * N2 + gc0;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                uint32_t w[8];
+#pragma unroll
+                for (int v = 0; v < 8; ++v) w[v] = __float_as_uint(al * __uint_as_float(r[8 * h + v]));
+                if (gc0 + 8 * h < N2) store32(dst + 8 * h, w);
+            }
+        }
+        return;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int v = 0; v < 16; v += 4)
+            *reinterpret_cast<float4*>(stg + lane * XEPI_LD + v) =
+                make_float4(al * __uint_as_float(r[16 * h + v]), al * __uint_as_float(r[16 * h + v + 1]),
+                            al * __uint_as_float(r[16 * h + v + 2]), al * __uint_as_float(r[16 * h + v + 3]));
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int rr = 8 * i + (lane >> 2), cc = 4 * (lane & 3);
+            const int grow = rbase + rr, gcol = gc0 + 16 * h + cc;
+            const float4 v = *reinterpret_cast<const float4*>(stg + rr * XEPI_LD + cc);
+            if (grow < M && gcol < N2) {
+                float* dst = out + (size_t)grow * N2 + gcol;
+                if (gcol + 4 <= N2) *reinterpret_cast<float4*>(dst) = v;
+                else {
+                    dst[0] = v.x;
+                    if (gcol + 1 < N2) dst[1] = v.y;
+                    if (gcol + 2 < N2) dst[2] = v.z;
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+// y-pass to slice l of a 16-bit grid: 16 complex values re = P_re - Q_im, im = P_im + Q_re
+template <int H>
+__device__ __forceinline__ void y_store_h16(const uint32_t (&p)[32], const uint32_t (&qq)[32], float alpha, bool wide, float* stg,
+                                            int lane, void* outv, int l, int rbase, int gc0, int ny, int N2, bool nsq,
+                                            float& nacc) {
+    float x[32];
+    uint32_t w[16];
+#pragma unroll
+    for (int k = 0; k < 32; k += 2) {
+        x[k] = alpha * (__uint_as_float(p[k]) - __uint_as_float(qq[k + 1]));
+        x[k + 1] = alpha * (__uint_as_float(p[k + 1]) + __uint_as_float(qq[k]));
+        w[k / 2] = pack16<H>(x[k], x[k + 1]);
+    }
+    if (nsq && rbase + lane < ny) nacc += norm32(x, gc0, N2);
+    store_pairs(w, wide, stg, lane, reinterpret_cast<uint16_t*>(outv) + (size_t)l * ny * N2, rbase, gc0, ny, N2);
+}
+
 // stage counts of the persistent x-pass: 128-wide tiles two CTAs per SM, 256-wide tiles one CTA per SM
 // (2 x 256 accumulator columns fill the tensor memory); 1024 bytes of slack align the ring
 // the split (3xTF32) form holds the data tile, its remainder and both halves of the basis tile per stage
@@ -568,6 +701,7 @@ xpass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         int lt = 0;
         float nacc = 0.f;   // squared norm of what this thread stored (OBF, nsq_out)
         const float al2 = alpha_dev2 ? (float)alpha_dev2[0] : 1.f;
+        const bool wide = rows_aligned(outv, N2, OBF ? 2 : 4);
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++lt) {
             const int b = lt & 1;
             const int n0 = (t % ntn) * BNT, m0 = (t / ntn) * BM;
@@ -577,8 +711,6 @@ xpass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             ok = __all_sync(0xffffffffu, mbar_wait(su32(&accf[b]), (uint32_t)((lt >> 1) & 1), wlim));
             if (!ok) break;
             fence_after();
-            // each thread holds one row of the accumulator; 16-column halves go through this warp's staging
-            // rows (stride XEPI_LD floats, conflict-free both ways) so that the stores are 64-byte row segments
             float* stg = epi + q * 32 * XEPI_LD;
             const int rbase = m0 + 32 * q;
 #pragma unroll 1
@@ -586,67 +718,8 @@ xpass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 uint32_t r[32];
                 TMEM_LD32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * BNT + c), r);
                 tmem_wait_ld();
-                if (OBF) {
-                    // the thread's 32 columns as 16 16-bit pairs (64 bytes) into its staging row, then 16-byte
-                    // pieces of four rows per instruction: 64-byte row segments in global memory
-                    uint32_t* su = reinterpret_cast<uint32_t*>(stg);
-                    if (nsq_out && m0 + 32 * q + lane < M)
-#pragma unroll
-                        for (int v = 0; v < 32; ++v) {
-                            const float x = al * __uint_as_float(r[v]);
-                            if (n0 + c + v < N2) nacc = fmaf(x, x, nacc);
-                        }
-#pragma unroll
-                    for (int v = 0; v < 16; v += 4)
-                        *reinterpret_cast<uint4*>(su + lane * XEPI_LD + v) =
-                            make_uint4(pack16<H>(al * __uint_as_float(r[2 * v]), al * __uint_as_float(r[2 * v + 1])),
-                                       pack16<H>(al * __uint_as_float(r[2 * v + 2]), al * __uint_as_float(r[2 * v + 3])),
-                                       pack16<H>(al * __uint_as_float(r[2 * v + 4]), al * __uint_as_float(r[2 * v + 5])),
-                                       pack16<H>(al * __uint_as_float(r[2 * v + 6]), al * __uint_as_float(r[2 * v + 7])));
-                    __syncwarp();
-                    uint16_t* ob = reinterpret_cast<uint16_t*>(outv);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int rr = 8 * i + (lane >> 2), cc = 4 * (lane & 3);
-                        const int grow = rbase + rr, gcol = n0 + c + 2 * cc;
-                        const uint4 v = *reinterpret_cast<const uint4*>(su + rr * XEPI_LD + cc);
-                        if (grow < M && gcol < N2) {
-                            uint16_t* dst = ob + (size_t)grow * N2 + gcol;
-                            if (gcol + 8 <= N2) *reinterpret_cast<uint4*>(dst) = v;
-                            else {
-                                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-                                for (int e = 0; e < 4 && gcol + 2 * e < N2; ++e) reinterpret_cast<uint32_t*>(dst)[e] = w[e];
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    continue;
-                }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                    for (int v = 0; v < 16; v += 4)
-                        *reinterpret_cast<float4*>(stg + lane * XEPI_LD + v) =
-                            make_float4(al * __uint_as_float(r[16 * h + v]), al * __uint_as_float(r[16 * h + v + 1]),
-                                        al * __uint_as_float(r[16 * h + v + 2]), al * __uint_as_float(r[16 * h + v + 3]));
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int rr = 8 * i + (lane >> 2), cc = 4 * (lane & 3);
-                        const int grow = rbase + rr, gcol = n0 + c + 16 * h + cc;
-                        const float4 v = *reinterpret_cast<const float4*>(stg + rr * XEPI_LD + cc);
-                        if (grow < M && gcol < N2) {
-                            float* dst = out + (size_t)grow * N2 + gcol;
-                            if (gcol + 4 <= N2) *reinterpret_cast<float4*>(dst) = v;
-                            else {
-                                dst[0] = v.x;
-                                if (gcol + 1 < N2) dst[1] = v.y;
-                                if (gcol + 2 < N2) dst[2] = v.z;
-                            }
-                        }
-                    }
-                    __syncwarp();
-                }
+                if (OBF) x_store_h16<H>(r, al, wide, stg, lane, outv, rbase, n0 + c, M, N2, nsq_out != nullptr, nacc);
+                else x_store_f32(r, al, wide, stg, lane, out, rbase, n0 + c, M, N2);
             }
             fence_before();
             __syncwarp();
@@ -841,6 +914,7 @@ ypass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
             }
             alpha *= sc;
         }
+        const bool wide = H && rows_aligned(outv, N2, 2);
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++lt) {
             const int b = lt & 1;
             const int mb = t % ntm, nb = (t / ntm) % ntn, l = t / (ntm * ntn);
@@ -856,38 +930,7 @@ ypass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
                 TMEM_LD32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * 2 * BN + BN + c), qq);
                 tmem_wait_ld();
                 if (H) {
-                    // 16 complex values (re = P_re - Q_im, im = P_im + Q_re) as 16-bit pairs: 64 bytes per row
-                    uint32_t* su = reinterpret_cast<uint32_t*>(stg);
-#pragma unroll
-                    for (int v = 0; v < 16; v += 4) {
-                        uint32_t w[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int k = 2 * (v + e);
-                            const float re = alpha * (__uint_as_float(p[k]) - __uint_as_float(qq[k + 1]));
-                            const float im = alpha * (__uint_as_float(p[k + 1]) + __uint_as_float(qq[k]));
-                            w[e] = pack16<H>(re, im);
-                            if (h16d && role == 0 && rbase + lane < ny && n0 + c + k < N2) nacc = fmaf(re, re, fmaf(im, im, nacc));
-                        }
-                        *reinterpret_cast<uint4*>(su + lane * XEPI_LD + v) = make_uint4(w[0], w[1], w[2], w[3]);
-                    }
-                    __syncwarp();
-                    uint16_t* ob = reinterpret_cast<uint16_t*>(outv);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int rr = 8 * i + (lane >> 2), cc = 4 * (lane & 3);
-                        const int grow = rbase + rr, gcol = n0 + c + 2 * cc;
-                        const uint4 v = *reinterpret_cast<const uint4*>(su + rr * XEPI_LD + cc);
-                        if (grow < ny && gcol < N2) {
-                            uint16_t* dst = ob + ((size_t)l * ny + grow) * N2 + gcol;
-                            if (gcol + 8 <= N2) *reinterpret_cast<uint4*>(dst) = v;
-                            else {
-                                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-                                for (int e = 0; e < 4 && gcol + 2 * e < N2; ++e) reinterpret_cast<uint32_t*>(dst)[e] = w[e];
-                            }
-                        }
-                    }
-                    __syncwarp();
+                    y_store_h16<H>(p, qq, alpha, wide, stg, lane, outv, l, rbase, n0 + c, ny, N2, h16d && role == 0, nacc);
                     continue;
                 }
 #pragma unroll
@@ -952,6 +995,289 @@ ypass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     __syncthreads();
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(4 * BN) : "memory");
+}
+
+// ---- 16-bit passes on CTA pairs with the basis resident in shared memory -----------------------------
+// The tiles of the persistent kernels above re-read their basis operand from L2 for every output tile: at 256^3 a pass
+// moved 403 MB through L2 for a 67 MB grid and was bound by that.  Here the two CTAs of a cluster work as one
+// (cta_group::2, M = 256: each CTA holds 128 rows of A and half of B's columns, and the accumulator rows of its A), which
+// halves every operand, so that the whole basis operand of a CTA (at most 128 KiB) stays in shared memory from the
+// first tile to the last and only the grid streams, once (y-pass) or once per half of the output columns (x-pass).
+//   y-pass  A = [Wr | Wi], rows 128 rank .. of W (N_y <= 256, K = N_y <= 256); B = 64 + 64 columns of a slice
+//   x-pass  A = 128 + 128 grid rows; B = BN / 2 + BN / 2 rows of the embedding (K = 2 N_x <= 512), BN <= 256 output
+//           columns: a pair keeps to one of the ntn column blocks
+// Barriers: full[s] (own TMA loads), empty[s] and accf[b] (commits of the leader, CTA 0, to both CTAs), and in the leader
+// pfull[s] (the peer's stage has landed: its warp 1 waits for that and arrives), acce[b] (eight arrivals, the
+// epilogue warps of both); resf[kb]: a chunk of the resident operand (the peer's warp 1 waits for its own).  Waits and drains as above; both CTAs
+// meet in a cluster barrier before either frees its tensor memory or exits, and every thread reaches it, because each
+// wait before it is bounded.
+// The streamed operand is bound by the ring's depth (latency of load, relay and commit: six stages of 16 KiB against four,
+// x-pass 32 -> 29 us), the rest by the epilogue: eight warps, as four took 41 us.
+// Measured at 256^3: y-pass 39 -> 30 us, x-pass 40 -> 29 (FP16 out) and 43 -> 42 (FP32 out, 134 MB written on top of a
+// 67 MB grid that is still dirty in L2).
+// Above 128 points a side (x-pass: 256 real columns): one 128-row tile or one column block leaves a pair half idle and
+// its cluster start costs more than the basis reads.  Whole FP16 preconditioner, persistent kernels against pairs:
+// 96^3 72 and 82 us, 128^3 81 and 94, 160^3 122 and 121, 192^3 150 and 149, 224^3 235 and 218, 256^3 298 and 270.
+constexpr int PAIR_MIN_N2 = 2 * BM;
+constexpr int PAIR_THREADS = 320;    // loads, MMAs, eight epilogue warps
+constexpr int PAIR_RES = 8 * TILE;   // the resident operand: 8 chunks of 16 KiB
+template <bool X>
+struct Pair {
+    static constexpr int STAGE = X ? TILE : TILE / 2;   // 64 K elements of this CTA's half of the streamed operand
+    // stages: the staging rows' space holds two or three more where the epilogue needs none
+    static constexpr int NS = X ? 6 : 12, NS_STAGED = X ? 4 : 9;
+    static constexpr size_t SMEM = (size_t)PAIR_RES + NS * STAGE + 1024;
+    static_assert((NS - NS_STAGED) * STAGE >= 2 * XEPI_BYTES, "staging rows");
+};
+__device__ __forceinline__ uint32_t cta_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// arrive on the barrier at the same offset in CTA 0 of the cluster.  What it orders are accesses of the asynchronous
+// proxy and of tensor memory (a landed TMA load before an MMA, tcgen05.ld behind its fence before the next MMA), no
+// generic ones; with cluster-scope release and acquire on these barriers a stage took 1.2 us instead of 0.7.
+__device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
+    asm volatile(
+        "{\n.reg .b32 ra;\nmapa.shared::cluster.u32 ra, %0, 0;\n"
+        "mbarrier.arrive.shared::cluster.b64 _, [ra];\n}\n" ::"r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r;
+}
+// the warp runs the issuing loop and the elected lane's value predicates the instruction itself, which keeps its
+// operands in uniform registers
+__device__ __forceinline__ void mma_pair(uint32_t lead, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(lead));
+}
+// commit to the barrier at this offset in both CTAs
+__device__ __forceinline__ void commit_pair(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+                 "h"((uint16_t)3)
+                 : "memory");
+}
+
+// X: the x-pass, dim = M rows, OBF as above; else the y-pass, dim = N_y, nz slices.  tmR the resident operand, tmS the
+// streamed one; nk chunks of 64 K elements; scales and norms as in the kernels above.
+struct PairArgs {
+    void* out;
+    int dim, N2, nz, nk, BNT;        // BNT: output columns of a tile (x-pass), a multiple of 32
+    int wide, ns;                    // direct stores; stages of the ring
+    float alpha;
+    const double* alpha_dev;         // x-pass
+    int aidx, rows_per, astride;
+    const double* alpha_dev2;
+    double* nsq_out;
+    double* h16d;                    // y-pass
+    float gain;
+    int role;
+    unsigned* status;
+    long wlim;
+};
+template <bool X, int H, bool OBF>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 1)
+pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmS, const PairArgs a) {
+    extern __shared__ uint8_t dsm[];
+    constexpr int STAGE = Pair<X>::STAGE;
+    __shared__ __align__(8) uint64_t full[Pair<X>::NS], pfull[Pair<X>::NS], empty[Pair<X>::NS], accf[2], acce[2], resf[8], drainb;
+    __shared__ int fail_any;
+    __shared__ uint32_t tslot;
+    const uint32_t raw = su32(dsm);
+    const uint32_t base = (raw + 1023u) & ~1023u;   // the same offset in both CTAs
+    const uint32_t ring = base + PAIR_RES;
+    const int NS = a.ns;
+    float* epi = reinterpret_cast<float*>(dsm + (base - raw) + PAIR_RES + NS * STAGE);   // staging rows (not wide)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)cta_rank(), pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+    // tiles of this pair: x-pass column block pair % ntn and 256-row blocks; y-pass (slice, 128-column block)
+    const int ntn = X ? (a.N2 + a.BNT - 1) / a.BNT : (a.N2 + BN - 1) / BN;
+    const int ntiles = X ? (a.dim + 2 * BM - 1) / (2 * BM) : ntn * a.nz;
+    const int t0 = X ? pair / ntn : pair, dt = X ? npairs / ntn : npairs;
+    const int nfix = X ? (pair % ntn) * a.BNT : 0;
+    const int nk = a.nk;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(su32(&full[s]), 1);
+            mbar_init(su32(&pfull[s]), 1);
+            mbar_init(su32(&empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) { mbar_init(su32(&accf[b]), 1); mbar_init(su32(&acce[b]), 16); }
+        for (int kb = 0; kb < 8; ++kb) mbar_init(su32(&resf[kb]), 1);
+        mbar_init(su32(&drainb), 1);
+        fail_any = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    cluster_sync();   // the peer's barriers are initialised
+    fence_after();
+    const uint32_t tmem = tslot;
+    bool ok = true;
+    long issued = 0;      // pipeline iterations whose TMA loads the producer issued
+    int rissued = 0;      // resident chunks it issued
+    if (warp == 0) {
+        if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 0;
+            for (int t = t0; t < ntiles && ok; t += dt)
+                for (int kb = 0; kb < nk; ++kb) {
+                    // the resident chunks go out between the first tile's stages, all before the first wait
+                    for (; rissued < nk && (rissued <= kb || issued == NS); ++rissued) {
+                        const uint32_t bar = su32(&resf[rissued]);
+                        mbar_expect_tx(bar, (X ? 1 : 2) * TILE);
+                        if (X) tma_2d(base + rissued * TILE, &tmR, bar, rissued * 64, nfix + rank * (a.BNT / 2));
+                        else {
+                            tma_3d(base + 2 * rissued * TILE, &tmR, bar, rissued * 64, rank * BM, 0);
+                            tma_3d(base + (2 * rissued + 1) * TILE, &tmR, bar, rissued * 64, rank * BM, 1);
+                        }
+                    }
+                    if (issued >= NS && !(ok = mbar_wait(su32(&empty[s]), ph ^ 1, a.wlim))) break;
+                    mbar_expect_tx(su32(&full[s]), STAGE);
+                    if (X) tma_2d(ring + s * STAGE, &tmS, su32(&full[s]), kb * 64, t * 2 * BM + rank * BM);
+                    else tma_3d(ring + s * STAGE, &tmS, su32(&full[s]), (t % ntn) * BN + rank * (BN / 2), kb * 64, t / ntn);
+                    ++issued;
+                    if (++s == NS) { s = 0; ph ^= 1; }
+                }
+            // the last stages' MMAs: no commit is on its way to this CTA when it leaves
+            for (long it = issued > NS ? issued - NS : 0; it < issued && ok; ++it)
+                ok = mbar_wait(su32(&empty[it % NS]), (uint32_t)((it / NS) & 1), a.wlim);
+        }
+    } else if (warp == 1 && rank == 0) {
+        const uint32_t lead = elect_one();
+        const uint32_t idesc = X ? idesc_h16(H, 2 * BM, a.BNT, 0, 0) : idesc_h16(H, 2 * BM, BN, 0, 1);
+        int s = 0, lt = 0;
+        uint32_t ph = 0;
+        for (int t = t0; t < ntiles && ok; t += dt, ++lt) {
+            const int b = lt & 1;
+            if (lt >= 2) ok = __all_sync(0xffffffffu, mbar_wait(su32(&acce[b]), (uint32_t)(((lt >> 1) - 1) & 1), a.wlim));
+            if (!ok) break;
+            fence_after();
+            const uint32_t acc_t = tmem + (uint32_t)(b * 256);
+            for (int kb = 0; kb < nk; ++kb) {
+                ok = __all_sync(0xffffffffu, (lt > 0 || mbar_wait(su32(&resf[kb]), 0, a.wlim)) &&
+                                                 mbar_wait(su32(&full[s]), ph, a.wlim) && mbar_wait(su32(&pfull[s]), ph, a.wlim));
+                if (!ok) break;
+                fence_after();
+                const uint32_t st = ring + s * STAGE;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const uint32_t acc = (kb | kk) ? 1u : 0u;
+                    if (X) {
+                        mma_pair(lead, acc_t, sdesc(st + kk * 32, 16, 1024), sdesc(base + kb * TILE + kk * 32, 16, 1024), idesc, acc);
+                    } else {
+                        const uint64_t bd = sdesc(st + kk * 2048, 8192, 1024);
+                        mma_pair(lead, acc_t, sdesc(base + 2 * kb * TILE + kk * 32, 16, 1024), bd, idesc, acc);
+                        mma_pair(lead, acc_t + BN, sdesc(base + (2 * kb + 1) * TILE + kk * 32, 16, 1024), bd, idesc, acc);
+                    }
+                }
+                if (lead) commit_pair(su32(&empty[s]));
+                if (++s == NS) { s = 0; ph ^= 1; }
+            }
+            if (ok && lead) commit_pair(su32(&accf[b]));
+        }
+    } else if (warp == 1) {
+        // the peer: tell the leader which of this CTA's loads have landed
+        if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 0;
+            for (int t = t0; t < ntiles && ok; t += dt)
+                for (int kb = 0; kb < nk; ++kb) {
+                    ok = (t > t0 || mbar_wait(su32(&resf[kb]), 0, a.wlim)) && mbar_wait(su32(&full[s]), ph, a.wlim);
+                    if (!ok) break;
+                    mbar_arrive_leader(su32(&pfull[s]));
+                    if (++s == NS) { s = 0; ph ^= 1; }
+                }
+        }
+    } else {
+        // two warps per 32 accumulator rows, which take its 32-column chunks in turn
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        float* stg = epi + (warp - 2) * 32 * XEPI_LD;
+        const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
+        int lt = 0;
+        float nacc = 0.f;   // squared norm of what this thread stored
+        const bool wide = a.wide;
+        float al2 = a.alpha;
+        if (X) {
+            if (a.alpha_dev2) al2 = (float)a.alpha_dev2[0];
+            else al2 = 1.f;
+        } else if (a.h16d) {
+            const float sc = stage_scale((double)a.gain, a.h16d[a.role == 0 ? 0 : 2]);
+            if (blockIdx.x == 0 && threadIdx.x == 64) {
+                a.h16d[a.role == 0 ? 4 : 6] = sc;
+                if (a.role == 1) a.h16d[7] = 1.0 / (a.h16d[4] * a.h16d[5] * (double)sc);
+            }
+            al2 *= sc;
+        }
+        for (int t = t0; t < ntiles && ok; t += dt, ++lt) {
+            const int b = lt & 1;
+            const int n0 = X ? nfix : (t % ntn) * BN, l = X ? 0 : t / ntn;
+            const int rbase = (X ? t * 2 * BM : 0) + rank * BM + 32 * q;
+            float al = al2;
+            if (X) {
+                const int arow = min(rbase + lane, a.dim - 1);
+                al = a.alpha * al2 * (a.alpha_dev ? (float)a.alpha_dev[a.aidx + (arow / a.rows_per) * a.astride] : 1.f);
+            }
+            ok = __all_sync(0xffffffffu, mbar_wait(su32(&accf[b]), (uint32_t)((lt >> 1) & 1), a.wlim));
+            if (!ok) break;
+            fence_after();
+            const int nc = X ? a.BNT : BN;
+#pragma unroll 1
+            for (int c = 32 * half; c < nc; c += 64) {
+                uint32_t r[32];
+                TMEM_LD32(trow + (uint32_t)(b * 256 + c), r);
+                if constexpr (X) {
+                    tmem_wait_ld();
+                    if (OBF) x_store_h16<H>(r, al, wide, stg, lane, a.out, rbase, n0 + c, a.dim, a.N2, a.nsq_out != nullptr, nacc);
+                    else x_store_f32(r, al, wide, stg, lane, reinterpret_cast<float*>(a.out), rbase, n0 + c, a.dim, a.N2);
+                } else {
+                    uint32_t qq[32];
+                    TMEM_LD32(trow + (uint32_t)(b * 256 + BN + c), qq);
+                    tmem_wait_ld();
+                    y_store_h16<H>(r, qq, al, wide, stg, lane, a.out, l, rbase, n0 + c, a.dim, a.N2, a.h16d && a.role == 0, nacc);
+                }
+            }
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_leader(su32(&acce[b]));
+        }
+        double* nsq = X ? a.nsq_out : (a.h16d && a.role == 0 ? a.h16d + 1 : nullptr);
+        if (nsq) {
+            double d = (double)nacc;
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+            if (lane == 0) atomicAdd(nsq, d);
+        }
+    }
+    if (!ok) {
+        atomicOr(a.status, (unsigned)HELM_DEV_WAIT);
+        fail_any = 1;
+    }
+    __syncthreads();
+    if (fail_any) {
+        if (warp == 0 && lane == 0) {
+            drain_tma(full, NS, issued);
+            for (int kb = 0; kb < rissued; ++kb) mbar_wait(su32(&resf[kb]), 0, DRAIN_LIMIT);
+        } else if (warp == 1 && rank == 0 && elect_one()) {   // the lane that issued (the election is deterministic)
+            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&drainb)) : "memory");
+            mbar_wait(su32(&drainb), 0, DRAIN_LIMIT);
+        }
+    }
+    fence_before();
+    __syncthreads();
+    cluster_sync();
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 
 // ---- operand preparation (set-up) ----------------------------------------------------------------
@@ -1032,6 +1358,24 @@ helm_status encode(TcState* t, CUtensorMap* map, int rank, void* ptr, const cuui
 size_t xsmem() { return (size_t)XSTAGES * 2 * TILE + 1024; }
 size_t ysmem() { return (size_t)YSTAGES * 3 * TILE + 1024; }
 int g_sms = 0;
+
+// clusters of two CTAs of a pair kernel that the GPU holds at once (its shared-memory attribute set first)
+template <typename K>
+cudaError_t pair_count(K kernel, size_t bytes, int* n) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2);
+    cfg.blockDim = dim3(PAIR_THREADS);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(n, kernel, &cfg);
+}
 
 template <typename K>
 cudaError_t smem_attr(K kernel, size_t bytes) {
@@ -1135,6 +1479,12 @@ helm_status tc_prepare(helm_ctx* c, cudaStream_t s) {
         HELM_CUDA_TRY(smem_attr(xpass_tc_pers_kernel<256, false, 2, false>, PersX<256, false>::SMEM));
         HELM_CUDA_TRY(smem_attr(ypass_tc_pers_kernel<false, 1>, PersY<false>::SMEM));
         HELM_CUDA_TRY(smem_attr(ypass_tc_pers_kernel<false, 2>, PersY<false>::SMEM));
+        HELM_CUDA_TRY(pair_count(pair_pass_kernel<true, 1, true>, Pair<true>::SMEM, &t->pairs_x));
+        HELM_CUDA_TRY(pair_count(pair_pass_kernel<true, 1, false>, Pair<true>::SMEM, &t->pairs_x));
+        HELM_CUDA_TRY(pair_count(pair_pass_kernel<true, 2, true>, Pair<true>::SMEM, &t->pairs_x));
+        HELM_CUDA_TRY(pair_count(pair_pass_kernel<true, 2, false>, Pair<true>::SMEM, &t->pairs_x));
+        HELM_CUDA_TRY(pair_count(pair_pass_kernel<false, 1, true>, Pair<false>::SMEM, &t->pairs_y));
+        HELM_CUDA_TRY(pair_count(pair_pass_kernel<false, 2, true>, Pair<false>::SMEM, &t->pairs_y));
     }
     HELM_CUDA_TRY(smem_attr(xpass_tc_kernel, xsmem()));
     HELM_CUDA_TRY(smem_attr(ypass_tc_kernel, ysmem()));
@@ -1268,7 +1618,16 @@ void xpass_h16_launch(TcState* t, helm_ctx* c, int inverse, const CUtensorMap& m
                       const double* alpha_dev2, double* nsq_out) {
     const long wl = (long)c->wait_limit;
     const int mt = (M + BM - 1) / BM;
-    if (N2 % 256 == 0) {
+    // column blocks of the pair kernel: even shares of at most 256 columns, rounded up to 32
+    const int ntn = (N2 + 255) / 256, bn = ((N2 + ntn - 1) / ntn + 31) / 32 * 32;
+    if (N2 > PAIR_MIN_N2 && N2 <= 512 && t->pairs_x >= ntn) {
+        const int want = ntn * ((M + 2 * BM - 1) / (2 * BM));
+        const int np = (want < t->pairs_x ? want : t->pairs_x) / ntn * ntn;
+        const bool wide = rows_aligned(out, N2, OBF ? 2 : 4);
+        const PairArgs a = {out, M, N2, 1, (N2 + 63) / 64, bn, wide, wide ? Pair<true>::NS : Pair<true>::NS_STAGED, alpha, alpha_dev, aidx, rp, astride, alpha_dev2, nsq_out,
+                            nullptr, 1.f, 0, c->status_d, wl};
+        pair_pass_kernel<true, H, OBF><<<2 * np, PAIR_THREADS, Pair<true>::SMEM, s>>>(t->mapBxb[inverse], mapA, a);
+    } else if (N2 % 256 == 0) {
         const int ntiles = (N2 / 256) * mt, pg = ntiles < g_sms ? ntiles : g_sms;
         xpass_tc_pers_kernel<256, false, H, OBF><<<pg, 192, PersX<256, false>::SMEM, s>>>(
             mapA, t->mapBxb256[inverse], t->mapBxb256[inverse], out, M, N2, N2, alpha, alpha_dev, aidx, rp, astride,
@@ -1318,6 +1677,16 @@ helm_status tc_ypass_h16(helm_ctx* c, int inverse, const void* in, void* out, fl
     const CUtensorMapDataType dt = t->h16 == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     if (encode(t, &mapY, 3, (void*)in, d, st, box, CU_TENSOR_MAP_SWIZZLE_128B, dt) != HELM_OK) return HELM_ERR_CUDA;
     const long wl = (long)c->wait_limit;
+    if (ny > BM && ny <= 2 * BM && t->pairs_y > 0) {
+        const int tiles = ((N2 + BN - 1) / BN) * nzb, np = tiles < t->pairs_y ? tiles : t->pairs_y;
+        const bool wide = rows_aligned(out, N2, 2);
+        const PairArgs a = {out, ny, N2, nzb, (ny + 63) / 64, BN, wide, wide ? Pair<false>::NS : Pair<false>::NS_STAGED, alpha, nullptr, 0, 1, 0, nullptr, nullptr,
+                            t->h16 == 2 ? h16d : nullptr, gain, inverse, c->status_d, wl};
+        if (t->h16 == 2) pair_pass_kernel<false, 2, true><<<2 * np, PAIR_THREADS, Pair<false>::SMEM, s>>>(t->mapWyb[inverse], mapY, a);
+        else pair_pass_kernel<false, 1, true><<<2 * np, PAIR_THREADS, Pair<false>::SMEM, s>>>(t->mapWyb[inverse], mapY, a);
+        HELM_CUDA_TRY(cudaGetLastError());
+        return HELM_OK;
+    }
     const int ntiles = ((N2 + BN - 1) / BN) * ((ny + BM - 1) / BM) * nzb;
     const int pg = ntiles > g_sms ? g_sms : ntiles;
     if (t->h16 == 2)

@@ -7,6 +7,9 @@ z-solves: depths on both sides of the blocks of 8 steps whose inner ones run wit
 (the systems amplify FP32 rounding, here by a few hundred at most).  Wide grids: the same where the lines do not fit
 the SMs whole and pass through the ring of 6 blocks, and the whole FP16 chain there against FP32 within a few hundred
 2^-11.
+16-bit transform chain: sides below, at and above the 128 rows and 256 columns at which the passes go to CTA pairs,
+ragged blocks, several vectors' worth of rows.  Input, basis entries and the grids between the stages carry one rounding u
+(2^-11, 2^-8) each, white like the input, so each adds about u relative to the result: bound 16 u against FP32.
 Complex64 matvec: every kernel variant, grids from the smallest to several chunk lengths, real and complex k^2, and
 the padded form of the high-order closure (an output that overlaps the operand included).  The terms of A U are up
 to 8/h^2 |U| and cancel to k^2 U, each rounded to 2^-24: bound 32 2^-24 / (k0 h)^2.
@@ -23,7 +26,7 @@ from oracle.eigt import EigT
 from oracle.grid import Grid
 from oracle.operators import Operator
 from oracle.tridiag import thomas
-from paper_2602_07711_gb300 import HELM_C64, HELM_CLOSURE_HIGH_ORDER, HELM_PREC_FP16, Solver, helm
+from paper_2602_07711_gb300 import HELM_C64, HELM_CLOSURE_HIGH_ORDER, HELM_PREC_BF16, HELM_PREC_FP16, Solver, helm
 
 
 def _rand(shape, seed):
@@ -88,6 +91,39 @@ def test_z_solves_wide(nz):
     assert _rel(S.precond_step(2, _dev(y)).cpu().numpy(), thomas(*e.z_coefficients(), y)) < 1e-4
     H = Solver(n, k2, k0, order=4, L=L, precision=HELM_PREC_FP16, flexible=True)
     assert _rel(H.apply_precond(_dev(y)).cpu().numpy(), S.apply_precond(_dev(y)).cpu().numpy()) < 0.1
+
+
+PAIR_SIZES = [(128, 128, 5), (132, 129, 4), (160, 250, 7), (148, 200, 33), (256, 256, 9), (260, 257, 4), (64, 192, 20)]
+
+
+@pytest.mark.parametrize("precision, u", [(HELM_PREC_FP16, 2.0 ** -11), (HELM_PREC_BF16, 2.0 ** -8)])
+@pytest.mark.parametrize("n", PAIR_SIZES)
+def test_16_bit_passes(n, precision, u):
+    big = max(n)
+    k0 = 2 * math.pi * big / 11
+    k2 = np.full(n[::-1], k0 * k0, complex)
+    L = [m / big for m in n]
+    y = _dev(_rand(k2.shape, n[2]))
+    S = Solver(n, k2, k0, order=4, L=L)
+    H = Solver(n, k2, k0, order=4, L=L, precision=precision, flexible=True)
+    ref = S.apply_precond(y).cpu().numpy()
+    assert _rel(H.apply_precond(y).cpu().numpy(), ref) < 16 * u
+
+
+def test_expired_waits_of_the_pair_passes_leave_the_context_usable():
+    n = (144, 144, 40)
+    k0 = 2 * math.pi * 144 / 11
+    k2 = np.full(n[::-1], k0 * k0, complex)
+    S = Solver(n, k2, k0, order=4, L=(1, 1, 40 / 144), precision=HELM_PREC_FP16, flexible=True)
+    y = _dev(_rand(k2.shape, 3))
+    ref = S.apply_precond(y)
+    S.set_wait_limit(1)      # one poll a wait
+    try:
+        S.apply_precond(y)
+    except RuntimeError:
+        pass
+    S.set_wait_limit(0)
+    assert torch.equal(S.apply_precond(y), ref)
 
 
 @pytest.mark.parametrize("lossy", [False, True])
