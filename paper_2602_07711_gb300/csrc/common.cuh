@@ -67,6 +67,30 @@ struct StencilParams {
     const typename cplx<R>::t* G;        // lap(k^2) - k^4             (order 6)
 };
 
+// ---- programmatic dependent launch -------------------------------------------------------------
+// A kernel launched with follows = 1 may start while the kernel before it in its stream still runs; grid_wait() returns
+// once that one has completed and its writes are visible, and every kernel launched this way runs it in all threads before it
+// touches memory that any kernel of the chain writes.  grid_trigger() after it lets the next kernel start: a kernel is
+// then at most one ahead, and tensor memory is allocated before, so that a waiting kernel never holds what the running
+// one still needs.  Both are no-ops in a kernel launched with follows = 0, which waits for its predecessor as usual.
+// It hides the launch latency between the five passes of a preconditioner (Chain in precond.cu sets helm_ctx::follows).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_after(int follows, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = follows ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- the context -----------------------------------------------------------------------------
 struct KrylovWork;
 struct helm_net;
@@ -150,6 +174,7 @@ struct helm_ctx {
     helm_net* net = nullptr;                // attached learned correction (not owned)
     int tune_nb = 0;                        // CTAs of the Arnoldi kernels chosen by helm_autotune (0 = default)
     int tune_stencil = 0;                   // complex64 matvec variant chosen by helm_autotune (0 = cp.async ring)
+    int follows = 0;                        // the next launch of a preconditioner chain may start early (launch_after)
     int zring_sms = 0;                      // SM count, set with the ring kernel's attributes at set-up
     int zpiv_ready = 0;                     // shared-memory attribute of the pivot-recomputing z-solve set
     void* zck = nullptr;                    // checkpoints of that z-solve ([block][state][line pair] float4)
@@ -208,7 +233,7 @@ helm_status run_eig_setup(helm_ctx* c, cudaStream_t s);
 // rows of C: row r scales by alpha_dev[aidx + (r / rows_per) astride] (rows_per = 0: alpha_dev[aidx] for all)
 void launch_cgemm_simt(int M, int N, int K, const float2* A, long lda, long sA, const float2* B, long ldb, long sB,
                        float2* C, long ldc, long sC, int batch, float alpha, const double* alpha_dev, int aidx,
-                       cudaStream_t s, int rows_per = 0, int astride = 0);
+                       cudaStream_t s, int rows_per = 0, int astride = 0, int follows = 0);
 // gemm_tc.cu
 helm_status tc_prepare(helm_ctx* c, cudaStream_t s);
 // nb > 1: nb grid vectors back to back (a batch group); the x-pass scales vector v by alpha_dev[aidx + v astride]

@@ -103,6 +103,8 @@ cgemm_kernel(int M, int N, int K, const float2* __restrict__ A, long lda, long s
     for (int i = 0; i < TM / 2; ++i)
 #pragma unroll
         for (int j = 0; j < TN; ++j) re[i][j] = im[i][j] = make_float2(0.f, 0.f);
+    grid_wait();
+    grid_trigger();
     for (int b = 0; b < GST - 1; ++b) fetch(b);
     for (int kb = 0; kb < nk; ++kb) {
         asm volatile("cp.async.wait_group %0;\n" ::"n"(GST - 2) : "memory");
@@ -157,7 +159,7 @@ struct Args {
     int batch;
     float alpha;
     const double* alpha_dev;
-    int aidx, rows_per, astride;
+    int aidx, rows_per, astride, follows;
 };
 template <int TM, int TN, int NW>
 void run(const Args& a, cudaStream_t s) {
@@ -165,8 +167,8 @@ void run(const Args& a, cudaStream_t s) {
     const dim3 grid((a.N + T::BN - 1) / T::BN, (a.M + T::BM - 1) / T::BM, a.batch);
     if (T::SMEM > 48 * 1024)
         cudaFuncSetAttribute(cgemm_kernel<TM, TN, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM);
-    cgemm_kernel<TM, TN, NW><<<grid, T::NT, T::SMEM, s>>>(a.M, a.N, a.K, a.A, a.lda, a.sA, a.B, a.ldb, a.sB, a.C, a.ldc, a.sC,
-                                                         a.alpha, a.alpha_dev, a.aidx, a.rows_per, a.astride);
+    launch_after(a.follows, cgemm_kernel<TM, TN, NW>, grid, T::NT, T::SMEM, s, a.M, a.N, a.K, a.A, a.lda, a.sA, a.B, a.ldb,
+                 a.sB, a.C, a.ldc, a.sC, a.alpha, a.alpha_dev, a.aidx, a.rows_per, a.astride);
 }
 template <int TM, int NW>
 void run_n(const Args& a, int tn, cudaStream_t s) {
@@ -182,7 +184,7 @@ void run_n(const Args& a, int tn, cudaStream_t s) {
 
 void launch_cgemm_simt(int M, int N, int K, const float2* A, long lda, long sA, const float2* B, long ldb, long sB,
                        float2* C, long ldc, long sC, int batch, float alpha, const double* alpha_dev, int aidx,
-                       cudaStream_t s, int rows_per, int astride) {
+                       cudaStream_t s, int rows_per, int astride, int follows) {
     // The tile with the least time for the whole grid of tiles: an SM works through its share of them at a rate
     // proportional to their area, padding included (of the rows, that of a warp: 32), but no faster than one warp
     // per scheduler; a tile's fixed cost (the first loads, the epilogue) is worth about 1500 outputs.  Widths 64, 56,
@@ -199,7 +201,7 @@ void launch_cgemm_simt(int M, int N, int K, const float2* A, long lda, long sA, 
     };
     for (int n = 8; n >= 4; --n) consider(128, n);
     consider(32, 4);
-    const Args a = {M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, alpha, alpha_dev, aidx, rows_per, astride};
+    const Args a = {M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, alpha, alpha_dev, aidx, rows_per, astride, follows};
     if (bm == 128) run_n<8, 4>(a, tn, s);
     else run<2, 4, 4>(a, s);
 }

@@ -640,6 +640,8 @@ xpass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     __syncthreads();
     fence_after();
     const uint32_t tmem = tslot;
+    grid_wait();
+    grid_trigger();
     bool ok = true;
     long issued = 0;   // pipeline iterations whose TMA loads the producer issued
     if (warp == 0) {
@@ -700,7 +702,8 @@ xpass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const int q = warp & 3;
         int lt = 0;
         float nacc = 0.f;   // squared norm of what this thread stored (OBF, nsq_out)
-        const float al2 = alpha_dev2 ? (float)alpha_dev2[0] : 1.f;
+        // written by the kernel before this one: not to be read ahead of grid_wait
+        const float al2 = alpha_dev2 ? (float)*(const volatile double*)alpha_dev2 : 1.f;
         const bool wide = rows_aligned(outv, N2, OBF ? 2 : 4);
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++lt) {
             const int b = lt & 1;
@@ -822,6 +825,8 @@ ypass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
     __syncthreads();
     fence_after();
     const uint32_t tmem = tslot;
+    grid_wait();
+    grid_trigger();
     bool ok = true;
     long issued = 0;   // pipeline iterations whose TMA loads the producer issued
     if (warp == 0) {
@@ -1125,6 +1130,8 @@ pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant_
     cluster_sync();   // the peer's barriers are initialised
     fence_after();
     const uint32_t tmem = tslot;
+    grid_wait();
+    grid_trigger();
     bool ok = true;
     long issued = 0;      // pipeline iterations whose TMA loads the producer issued
     int rissued = 0;      // resident chunks it issued
@@ -1555,26 +1562,30 @@ helm_status tc_xpass(helm_ctx* c, int inverse, const float2* in, float2* out, fl
         if (N2 % 256 == 0) {
             const int ntiles = (N2 / 256) * (int)grid.y;
             const int pg = ntiles < g_sms ? ntiles : g_sms;
-            xpass_tc_pers_kernel<256, true><<<pg, 320, PersX<256, true>::SMEM, s>>>(
-                mapA, t->mapBx256[inverse], t->mapBx256l[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as, c->status_d, wl);
+            launch_after(c->follows, xpass_tc_pers_kernel<256, true>, pg, 320, PersX<256, true>::SMEM, s, mapA,
+                         t->mapBx256[inverse], t->mapBx256l[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as,
+                         c->status_d, wl, nullptr, nullptr);
         } else {
             const int ntiles = (int)(grid.x * grid.y);
             const int pg = ntiles < g_sms ? ntiles : g_sms;
-            xpass_tc_pers_kernel<128, true><<<pg, 320, PersX<128, true>::SMEM, s>>>(
-                mapA, t->mapBx[inverse], t->mapBxl[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as, c->status_d, wl);
+            launch_after(c->follows, xpass_tc_pers_kernel<128, true>, pg, 320, PersX<128, true>::SMEM, s, mapA,
+                         t->mapBx[inverse], t->mapBxl[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as,
+                         c->status_d, wl, nullptr, nullptr);
         }
     } else if (c->tune_tc == 1 && g_sms > 0) {
         if (N2 % 256 == 0) {
             // 256-wide tiles, one CTA per SM
             const int ntiles = (N2 / 256) * (int)grid.y;
             const int pg = ntiles < g_sms ? ntiles : g_sms;
-            xpass_tc_pers_kernel<256, false><<<pg, 192, PersX<256, false>::SMEM, s>>>(
-                mapA, t->mapBx256[inverse], t->mapBx256[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as, c->status_d, wl);
+            launch_after(c->follows, xpass_tc_pers_kernel<256, false>, pg, 192, PersX<256, false>::SMEM, s, mapA,
+                         t->mapBx256[inverse], t->mapBx256[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as,
+                         c->status_d, wl, nullptr, nullptr);
         } else {
             const int ntiles = (int)(grid.x * grid.y);
             const int pg = ntiles < 2 * g_sms ? ntiles : 2 * g_sms;
-            xpass_tc_pers_kernel<128, false><<<pg, 192, PersX<128, false>::SMEM, s>>>(
-                mapA, t->mapBx[inverse], t->mapBx[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as, c->status_d, wl);
+            launch_after(c->follows, xpass_tc_pers_kernel<128, false>, pg, 192, PersX<128, false>::SMEM, s, mapA,
+                         t->mapBx[inverse], t->mapBx[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as,
+                         c->status_d, wl, nullptr, nullptr);
         }
     } else {
         xpass_tc_kernel<<<grid, 192, xsmem(), s>>>(mapA, t->mapBx[inverse], o, M, N2, N2, alpha, alpha_dev, aidx, rp, as,
@@ -1598,11 +1609,11 @@ helm_status tc_ypass(helm_ctx* c, int inverse, const float2* in, float2* out, cu
     const int ntiles = (int)(grid.x * grid.y * grid.z);
     const int pg = g_sms > 0 && ntiles > g_sms ? g_sms : ntiles;
     if (t->split && g_sms > 0) {
-        ypass_tc_pers_kernel<true><<<pg, 320, PersY<true>::SMEM, s>>>(t->mapWy[inverse], mapY, t->mapWyl[inverse],
-                                                                     (float*)out, ny, N2, nzb, c->status_d, wl);
+        launch_after(c->follows, ypass_tc_pers_kernel<true>, pg, 320, PersY<true>::SMEM, s, t->mapWy[inverse], mapY,
+                     t->mapWyl[inverse], (float*)out, ny, N2, nzb, c->status_d, wl, 1.f, nullptr, 1.f, 0);
     } else if (c->tune_ypers && g_sms > 0) {
-        ypass_tc_pers_kernel<false><<<pg, 192, PersY<false>::SMEM, s>>>(t->mapWy[inverse], mapY, t->mapWy[inverse],
-                                                                       (float*)out, ny, N2, nzb, c->status_d, wl);
+        launch_after(c->follows, ypass_tc_pers_kernel<false>, pg, 192, PersY<false>::SMEM, s, t->mapWy[inverse], mapY,
+                     t->mapWy[inverse], (float*)out, ny, N2, nzb, c->status_d, wl, 1.f, nullptr, 1.f, 0);
     } else {
         ypass_tc_kernel<<<grid, 192, ysmem(), s>>>(t->mapWy[inverse], mapY, (float*)out, ny, N2, c->status_d, wl);
     }
@@ -1626,17 +1637,18 @@ void xpass_h16_launch(TcState* t, helm_ctx* c, int inverse, const CUtensorMap& m
         const bool wide = rows_aligned(out, N2, OBF ? 2 : 4);
         const PairArgs a = {out, M, N2, 1, (N2 + 63) / 64, bn, wide, wide ? Pair<true>::NS : Pair<true>::NS_STAGED, alpha, alpha_dev, aidx, rp, astride, alpha_dev2, nsq_out,
                             nullptr, 1.f, 0, c->status_d, wl};
-        pair_pass_kernel<true, H, OBF><<<2 * np, PAIR_THREADS, Pair<true>::SMEM, s>>>(t->mapBxb[inverse], mapA, a);
+        launch_after(c->follows, pair_pass_kernel<true, H, OBF>, 2 * np, PAIR_THREADS, Pair<true>::SMEM, s,
+                     t->mapBxb[inverse], mapA, a);
     } else if (N2 % 256 == 0) {
         const int ntiles = (N2 / 256) * mt, pg = ntiles < g_sms ? ntiles : g_sms;
-        xpass_tc_pers_kernel<256, false, H, OBF><<<pg, 192, PersX<256, false>::SMEM, s>>>(
-            mapA, t->mapBxb256[inverse], t->mapBxb256[inverse], out, M, N2, N2, alpha, alpha_dev, aidx, rp, astride,
-            c->status_d, wl, alpha_dev2, nsq_out);
+        launch_after(c->follows, xpass_tc_pers_kernel<256, false, H, OBF>, pg, 192, PersX<256, false>::SMEM, s, mapA,
+                     t->mapBxb256[inverse], t->mapBxb256[inverse], out, M, N2, N2, alpha, alpha_dev, aidx, rp, astride,
+                     c->status_d, wl, alpha_dev2, nsq_out);
     } else {
         const int ntiles = ((N2 + BN - 1) / BN) * mt, pg = ntiles < 2 * g_sms ? ntiles : 2 * g_sms;
-        xpass_tc_pers_kernel<128, false, H, OBF><<<pg, 192, PersX<128, false>::SMEM, s>>>(
-            mapA, t->mapBxb[inverse], t->mapBxb[inverse], out, M, N2, N2, alpha, alpha_dev, aidx, rp, astride,
-            c->status_d, wl, alpha_dev2, nsq_out);
+        launch_after(c->follows, xpass_tc_pers_kernel<128, false, H, OBF>, pg, 192, PersX<128, false>::SMEM, s, mapA,
+                     t->mapBxb[inverse], t->mapBxb[inverse], out, M, N2, N2, alpha, alpha_dev, aidx, rp, astride,
+                     c->status_d, wl, alpha_dev2, nsq_out);
     }
 }
 
@@ -1682,20 +1694,21 @@ helm_status tc_ypass_h16(helm_ctx* c, int inverse, const void* in, void* out, fl
         const bool wide = rows_aligned(out, N2, 2);
         const PairArgs a = {out, ny, N2, nzb, (ny + 63) / 64, BN, wide, wide ? Pair<false>::NS : Pair<false>::NS_STAGED, alpha, nullptr, 0, 1, 0, nullptr, nullptr,
                             t->h16 == 2 ? h16d : nullptr, gain, inverse, c->status_d, wl};
-        if (t->h16 == 2) pair_pass_kernel<false, 2, true><<<2 * np, PAIR_THREADS, Pair<false>::SMEM, s>>>(t->mapWyb[inverse], mapY, a);
-        else pair_pass_kernel<false, 1, true><<<2 * np, PAIR_THREADS, Pair<false>::SMEM, s>>>(t->mapWyb[inverse], mapY, a);
+        if (t->h16 == 2) launch_after(c->follows, pair_pass_kernel<false, 2, true>, 2 * np, PAIR_THREADS,
+                                      Pair<false>::SMEM, s, t->mapWyb[inverse], mapY, a);
+        else launch_after(c->follows, pair_pass_kernel<false, 1, true>, 2 * np, PAIR_THREADS, Pair<false>::SMEM, s,
+                          t->mapWyb[inverse], mapY, a);
         HELM_CUDA_TRY(cudaGetLastError());
         return HELM_OK;
     }
     const int ntiles = ((N2 + BN - 1) / BN) * ((ny + BM - 1) / BM) * nzb;
     const int pg = ntiles > g_sms ? g_sms : ntiles;
     if (t->h16 == 2)
-        ypass_tc_pers_kernel<false, 2><<<pg, 192, PersY<false>::SMEM, s>>>(t->mapWyb[inverse], mapY, t->mapWyb[inverse],
-                                                                          out, ny, N2, nzb, c->status_d, wl, alpha, h16d,
-                                                                          gain, inverse);
+        launch_after(c->follows, ypass_tc_pers_kernel<false, 2>, pg, 192, PersY<false>::SMEM, s, t->mapWyb[inverse],
+                     mapY, t->mapWyb[inverse], out, ny, N2, nzb, c->status_d, wl, alpha, h16d, gain, inverse);
     else
-        ypass_tc_pers_kernel<false, 1><<<pg, 192, PersY<false>::SMEM, s>>>(t->mapWyb[inverse], mapY, t->mapWyb[inverse],
-                                                                          out, ny, N2, nzb, c->status_d, wl, alpha);
+        launch_after(c->follows, ypass_tc_pers_kernel<false, 1>, pg, 192, PersY<false>::SMEM, s, t->mapWyb[inverse],
+                     mapY, t->mapWyb[inverse], out, ny, N2, nzb, c->status_d, wl, alpha, nullptr, 1.f, 0);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
 }

@@ -142,6 +142,23 @@ __global__ void __launch_bounds__(256) normed_to_h16_kernel(const float4* __rest
     }
 }
 
+// The launches of a preconditioner chain after its first may start early (launch_after): their predecessor in the stream
+// is the chain's own kernel before them.  Not under capture (the conditional bodies that hold the batch plans' chains take
+// plain edges) and not while the passes are timed by events.
+// Measured (without, with): 32^3 FP32 24.6, 23 us; 150 x 100 x 75 TF32 68, 60; 256^3 FP16 270, 260.
+struct Chain {
+    helm_ctx* c;
+    bool allowed = false;
+    Chain(helm_ctx* ctx, cudaStream_t s) : c(ctx) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        allowed = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+                  !(c->prof && c->prof->enabled);
+    }
+    void first_done() { c->follows = allowed; }
+    void plain() { c->follows = 0; }
+    ~Chain() { c->follows = 0; }
+};
+
 // The passes of the 16-bit chain from the 16-bit input In to the complex64 z (T0, T1: the halves of the
 // context's scratch vector; In may be T0).  BF16: the static factors of c->h16s (all 1 but the last).  FP16:
 // the x-pass forward scales statically (its input's norm is bounded by h16s[0]), every later stage by the
@@ -153,10 +170,12 @@ helm_status h16_chain(helm_ctx* c, const uint16_t* In, uint16_t* T1, float2* z, 
     const float* sc = c->h16s;
     double* d = c->opt.precision == HELM_PREC_FP16 ? c->h16d : nullptr;
     if (d) HELM_CUDA_TRY(cudaMemsetAsync(d, 0, 3 * sizeof(double), s));
+    Chain chain(c, s);
     prof_begin(c, s, PROF_XPASS);
     st = tc_xpass_h16(c, 0, In, T1, 1, sc[1], nullptr, 0, s, nb, 0, nullptr, d);
     prof_end(c, s);
     if (st != HELM_OK) return st;
+    chain.first_done();
     prof_begin(c, s, PROF_YPASS);
     st = tc_ypass_h16(c, 0, T1, T0, sc[2], s, nb, d, c->h16g[0]);
     prof_end(c, s);
@@ -167,7 +186,10 @@ helm_status h16_chain(helm_ctx* c, const uint16_t* In, uint16_t* T1, float2* z, 
     prof_end(c, s);
     if (st != HELM_OK) return st;
     prof_begin(c, s, PROF_XPASS);
-    if (c->h16_join) HELM_CUDA_TRY(cudaStreamWaitEvent(s, c->h16_join, 0));
+    if (c->h16_join) {
+        chain.plain();
+        HELM_CUDA_TRY(cudaStreamWaitEvent(s, c->h16_join, 0));
+    }
     st = tc_xpass_h16(c, 1, T1, z, 0, alpha_last, adev, aidx, s, nb, 0, d ? d + 7 : nullptr, nullptr);
     prof_end(c, s);
     return st;
@@ -213,7 +235,7 @@ helm_status xpass(helm_ctx* c, int inverse, const float2* in, float2* out, float
     }
     const int rows = c->ny * c->nz, M = rows * nb, N = c->nx;
     launch_cgemm_simt(M, N, N, in, N, 0, inverse ? c->XI : c->XF, N, 0, out, N, 0, 1, alpha, sigma, sidx, s, rows,
-                      sstride);
+                      sstride, c->follows);
     prof_end(c, s);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
@@ -229,7 +251,7 @@ helm_status ypass(helm_ctx* c, int inverse, const float2* in, float2* out, cudaS
     const int nx = c->nx, ny = c->ny;
     const long slice = (long)nx * ny;
     launch_cgemm_simt(ny, nx, ny, inverse ? c->YI : c->YF, ny, 0, in, nx, slice, out, nx, slice, c->nz * nb, 1.f,
-                      nullptr, 0, s);
+                      nullptr, 0, s, 0, 0, c->follows);
     prof_end(c, s);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
@@ -269,7 +291,9 @@ static helm_status precond_base(helm_ctx* c, const float2* r, float2* z, const d
     }
     if (c->opt.precision == HELM_PREC_BF16 || c->opt.precision == HELM_PREC_FP16) return precond_h16(c, r, z, sigma, sidx, s);
     const float hz2 = (float)(c->h[2] * c->h[2]);
+    Chain chain(c, s);
     if ((st = xpass(c, 0, r, c->tmp, 1.f, sigma, sidx, s)) != HELM_OK) return st;
+    chain.first_done();
     if ((st = ypass(c, 0, c->tmp, z, s)) != HELM_OK) return st;
     if ((st = launch_zsolve(c, z, z, s)) != HELM_OK) return st;
     if ((st = ypass(c, 1, z, c->tmp, s)) != HELM_OK) return st;
@@ -330,7 +354,9 @@ helm_status precond_apply_nb(helm_ctx* c, const float2* r, float2* z, int nb, co
         return h16_chain(c, T0, T1, z, c->h16s[5], nullptr, 0, s, nb);
     }
     const float hz2 = (float)(c->h[2] * c->h[2]);
+    Chain chain(c, s);
     if ((st = xpass(c, 0, r, c->tmp, 1.f, sigma, sidx, s, nb, sstride)) != HELM_OK) return st;
+    chain.first_done();
     if ((st = ypass(c, 0, c->tmp, z, s, nb)) != HELM_OK) return st;
     if ((st = launch_zsolve(c, z, z, s, nb)) != HELM_OK) return st;
     if ((st = ypass(c, 1, z, c->tmp, s, nb)) != HELM_OK) return st;

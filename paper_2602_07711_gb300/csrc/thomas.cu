@@ -539,20 +539,6 @@ __global__ void __launch_bounds__(ZRT, ALL ? 2 : 4) zsolve_piv_kernel(int nx, in
                                                                       float oscale = 1.f, double* __restrict__ h16d = nullptr,
                                                                       float gain = 1.f) {
     constexpr bool BF = H != 0;
-    // FP16 chain with dynamic stage scales (h16d): the output scale from the bound of ||T2|| (h16d[1]),
-    // recorded in h16d[5]; the squared norm of what is stored accumulates into h16d[2]
-    float nacc = 0.f;
-    if (BF && h16d) {
-        const double n2 = h16d[1];
-        float sc = 1.f;
-        if (n2 > 0.0) {
-            int e = 15 - (int)ceil(log2((double)gain * sqrt(n2)));
-            e = e < -100 ? -100 : (e > 100 ? 100 : e);
-            sc = ldexpf(1.f, e);
-        }
-        oscale *= sc;
-        if (blockIdx.x == 0 && threadIdx.x == 0) h16d[5] = sc;
-    }
     typedef typename ZPairOf<BF>::T Y;   // a step's input values of a line pair
     extern __shared__ float4 zsm[];      // ring [depth * ZU2][ZRT], cz [nz], ALL: checkpoints [block][2][ZRT]
     const Y* in = reinterpret_cast<const Y*>(inv);
@@ -567,6 +553,22 @@ __global__ void __launch_bounds__(ZRT, ALL ? 2 : 4) zsolve_piv_kernel(int nx, in
     float4* sck = after + (nz + 1) / 2;
     for (int l = tid; l < nz; l += ZRT) scz[l] = cz[l];
     __syncthreads();
+    grid_wait();
+    grid_trigger();
+    // FP16 chain with dynamic stage scales (h16d): the output scale from the bound of ||T2|| (h16d[1]),
+    // recorded in h16d[5]; the squared norm of what is stored accumulates into h16d[2]
+    float nacc = 0.f;
+    if (BF && h16d) {
+        const double n2 = h16d[1];
+        float sc = 1.f;
+        if (n2 > 0.0) {
+            int e = 15 - (int)ceil(log2((double)gain * sqrt(n2)));
+            e = e < -100 ? -100 : (e > 100 ? 100 : e);
+            sc = ldexpf(1.f, e);
+        }
+        oscale *= sc;
+        if (blockIdx.x == 0 && threadIdx.x == 0) h16d[5] = sc;
+    }
     auto slot = [&](int blk, int u) -> Y* { return ring + (size_t)((ALL ? blk : blk % ZPB) * ZU2 + u) * ZRT + tid; };
     for (int prb = blockIdx.x * ZRT + tid; prb < nall; prb += gridDim.x * ZRT) {
         const int pr = prb % npairs, vb = prb / npairs;
@@ -820,12 +822,11 @@ static helm_status run_zpiv(helm_ctx* c, const void* in, void* out, int slot, in
         c->zpiv_ready |= 1 << H;
     }
     if (whole)
-        zsolve_piv_kernel<H, true><<<need, ZRT, all, s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2], gz, c->dxs, c->dys, c->cz, in,
-                                                          out, ck, nb, oscale, h16d, gain);
+        launch_after(c->follows, zsolve_piv_kernel<H, true>, need, ZRT, all, s, c->nx, c->ny, c->nz, (float)c->zeta[2], gz, c->dxs,
+                     c->dys, c->cz, in, out, ck, nb, oscale, h16d, gain);
     else
-        zsolve_piv_kernel<H, false><<<need < cap ? need : cap, ZRT, ring, s>>>(c->nx, c->ny, c->nz, (float)c->zeta[2], gz,
-                                                                               c->dxs, c->dys, c->cz, in, out, ck, nb, oscale,
-                                                                               h16d, gain);
+        launch_after(c->follows, zsolve_piv_kernel<H, false>, need < cap ? need : cap, ZRT, ring, s, c->nx, c->ny, c->nz,
+                     (float)c->zeta[2], gz, c->dxs, c->dys, c->cz, in, out, ck, nb, oscale, h16d, gain);
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
 }

@@ -159,3 +159,32 @@ def test_closure_matvec(n, ppw, order):
     assert _rel(S.apply_A(xd).cpu().numpy(), ref) < bound
     helm.helm_apply_A(S.ctx, xd, xd, HELM_C64)
     assert _rel(xd.cpu().numpy(), ref) < bound
+
+
+@pytest.mark.parametrize("precision", [helm.HELM_PREC_FP32, helm.HELM_PREC_TF32, helm.HELM_PREC_TF32X3, HELM_PREC_FP16])
+@pytest.mark.parametrize("n", [(16, 10, 7), (100, 64, 40), (160, 144, 24)])
+def test_passes_started_early_see_their_predecessors_results(n, precision):
+    """Back-to-back preconditioners, in place too, against the same with every launch in plain stream order (as it is
+    while the passes are timed): the kernels are the same, so the results are."""
+    big = max(n)
+    k0 = 2 * math.pi * big / 10
+    k2 = np.full(n[::-1], k0 * k0, complex)
+    S = Solver(n, k2, k0, order=4, L=[m / big for m in n], precision=precision, flexible=True)
+    x = [_dev(_rand(k2.shape, v)) for v in range(6)]
+
+    def run():
+        r = []
+        for _ in range(4):
+            r = [S.apply_precond(v) for v in x]
+        z = x[0].clone()
+        for _ in range(3):
+            helm.helm_apply_precond(S.ctx, z, z)
+        return r + [z]
+
+    early = run()
+    L = helm.lib()
+    assert L.helm_profile(S.ctx, 1) == 0
+    plain = run()
+    assert L.helm_profile(S.ctx, 0) == 0
+    for a, b in zip(early, plain):
+        assert torch.equal(a, b)
