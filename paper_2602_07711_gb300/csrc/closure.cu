@@ -159,7 +159,9 @@ __global__ void ho_copy_kernel(int nx, int ny, int nz, const M* __restrict__ U, 
 template <class M, class A>
 __global__ void __launch_bounds__(HO_NT) ho_lap_kernel(const __grid_constant__ Face f, const __grid_constant__ FaceC<A> k,
                                                        const __grid_constant__ Wts<A> W, const Operand<M> op,
-                                                       typename A::St* __restrict__ S) {
+                                                       typename A::St* S) {
+    grid_wait();
+    grid_trigger();
     const int per = f.la * f.lb;
     const int id = blockIdx.x * HO_NT + threadIdx.x;
     if (id >= 2 * per) return;
@@ -174,9 +176,10 @@ __global__ void __launch_bounds__(HO_NT) ho_lap_kernel(const __grid_constant__ F
 template <class M, class A>
 __global__ void __launch_bounds__(HO_NT) ho_ghost_kernel(const __grid_constant__ Face f, const __grid_constant__ FaceC<A> k,
                                                          const __grid_constant__ Wts<A> W, const Operand<M> op, M* P,
-                                                         const typename A::St* __restrict__ S,
-                                                         const double2* __restrict__ fd) {
+                                                         const typename A::St* S, const double2* __restrict__ fd) {
     typedef typename A::V V;
+    grid_wait();
+    grid_trigger();
     const int per = f.la * f.lb;
     const int id = blockIdx.x * HO_NT + threadIdx.x;
     if (id >= 2 * per) return;
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(HO_NT) ho_ghost_kernel(const __grid_constant__
     const int pb = side ? f.nb_hi : f.nb_lo;
     const int pi = side ? pb - 1 : pb + 1;
     const int pg = side ? pb + 1 : pb - 1;
-    const typename A::St* __restrict__ L1 = S + (long long)side * per;
+    const typename A::St* L1 = S + (long long)side * per;
     const V ub = op.face(f, pb, ia, ib), ui = op.face(f, pi, ia, ib);
     const V v1 = A::ld(L1, q);
     const V v2 = apply_L<A>(f, k, W, [&](int a, int b) { return A::ld(L1, a * f.lb + b); }, ia, ib);
@@ -295,14 +298,16 @@ helm_status fill(helm_ctx* c, const M* U, M* P, const double2* faces, bool copy,
     typename A::St* S = reinterpret_cast<typename A::St*>(c->ho_S);   // 16 bytes a value either way
     const Operand<M> op = {U, P, c->nx, c->ny, c->nz};
     long long foff = 0;
+    LaunchChain chain(c, s);
     for (int axis = 0; axis < 3; ++axis) {
         const Face f = make_face(c, axis);
         const int tot = 2 * f.la * f.lb;
         const unsigned blocks = (unsigned)((tot + HO_NT - 1) / HO_NT);
         const FaceC<A> k = make_face_consts<A>(c, axis);
-        ho_lap_kernel<M, A><<<blocks, HO_NT, 0, s>>>(f, k, W, op, S);
+        launch_after(c->follows, ho_lap_kernel<M, A>, blocks, HO_NT, 0, s, f, k, W, op, S);
+        chain.first_done();
         HELM_CUDA_TRY(cudaGetLastError());
-        ho_ghost_kernel<M, A><<<blocks, HO_NT, 0, s>>>(f, k, W, op, P, S, faces ? faces + foff : nullptr);
+        launch_after(c->follows, ho_ghost_kernel<M, A>, blocks, HO_NT, 0, s, f, k, W, op, P, S, faces ? faces + foff : nullptr);
         HELM_CUDA_TRY(cudaGetLastError());
         foff += 3LL * tot;
     }

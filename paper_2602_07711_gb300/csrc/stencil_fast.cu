@@ -372,6 +372,7 @@ stencil_fast2_kernel(FParams p, const float2* __restrict__ U, float2* __restrict
     }
     const size_t plane = (size_t)p.nx * p.ny;
     const int poff = gy0 * p.nx + gx;
+    if (PAD) grid_wait();   // the ghosts
 
     auto issue = [&](int P) {
         if (P <= z1) {
@@ -1152,10 +1153,13 @@ dim3 fast_grid(const helm_ctx* c, const FParams& p) {
 
 namespace {
 template <int ORDER, bool RK, bool PAD>
-void run_two_rows(const FParams& p, dim3 grid, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s) {
+void run_two_rows(const FParams& p, dim3 grid, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s,
+                  int follows = 0) {
     const dim3 block(FTX, FTY / 2);
-    if (PAD || p.zch != FZCH)
-        stencil_fast2_kernel<ORDER, RK, PAD, true><<<grid, block, fast2_smem<RK>(), s>>>(p, x, y, sigma, sidx);
+    if (PAD)
+        launch_after(follows, stencil_fast2_kernel<ORDER, RK, PAD, true>, grid, block, fast2_smem<RK>(), s, p, x, y, sigma, sidx);
+    else if (p.zch != FZCH)
+        stencil_fast2_kernel<ORDER, RK, false, true><<<grid, block, fast2_smem<RK>(), s>>>(p, x, y, sigma, sidx);
     else
         stencil_fast2_kernel<ORDER, RK, false, false><<<grid, block, fast2_smem<RK>(), s>>>(p, x, y, sigma, sidx);
 }
@@ -1181,11 +1185,11 @@ helm_status launch_stencil_padded(helm_ctx* c, const float2* x, float2* y, const
     p.pad = c->ho_P32;
     const dim3 grid = fast_grid(c, p);
     if (c->realk) {
-        if (c->opt.order == 6) run_two_rows<6, true, true>(p, grid, x, y, sigma, sidx, s);
-        else run_two_rows<4, true, true>(p, grid, x, y, sigma, sidx, s);
+        if (c->opt.order == 6) run_two_rows<6, true, true>(p, grid, x, y, sigma, sidx, s, c->follows);
+        else run_two_rows<4, true, true>(p, grid, x, y, sigma, sidx, s, c->follows);
     } else {
-        if (c->opt.order == 6) run_two_rows<6, false, true>(p, grid, x, y, sigma, sidx, s);
-        else run_two_rows<4, false, true>(p, grid, x, y, sigma, sidx, s);
+        if (c->opt.order == 6) run_two_rows<6, false, true>(p, grid, x, y, sigma, sidx, s, c->follows);
+        else run_two_rows<4, false, true>(p, grid, x, y, sigma, sidx, s, c->follows);
     }
     HELM_CUDA_TRY(cudaGetLastError());
     return HELM_OK;
