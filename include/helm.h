@@ -53,7 +53,8 @@ typedef enum {
  *   the three-point second-order closure of the ABC, U_0 = U_2 + 2 i k0 h U_1 per direction (edge and
  *   corner ghosts: the one-dimensional rules applied in turn), and the preconditioner is EigT3 (Lbar with
  *   gamma = 2 i k0 h, zeta = 2; Sec. 4.1).  k^2 and f are reflected about the boundary node.  The matvec
- *   and the residual run on the general stencil kernels (the fast ones are staggered).  EigT (EigT3),
+ *   and the residual run on the general stencil kernels (the fast ones are staggered), except the complex64 matvec with
+ *   the high-order closure (helm_set_closure).  EigT (EigT3),
  *   PFFT (PFFT3: the boundary correction spans the two outer layers, since zeta = 2) and FFT2; the 1D
  *   eigensetup needs k0 h <= 1 (HELM_ERR_EIG beyond). */
 typedef struct {
@@ -154,7 +155,8 @@ enum { HELM_CLOSURE_THREE_POINT = 0, HELM_CLOSURE_HIGH_ORDER = 1 };
  *     closure's f part (s sum_m c_m sum_{j<m} (-L)^j d_n^(2(m-j)-1) f, s = +-1 on the far/near face) does
  *     not involve U and belongs to the right-hand side the caller passes to helm_gmres_solve, which
  *     helm_build_rhs does not form.
- * Each matvec first copies its operand into a padded array and fills the ghosts (seven small launches).
+ * Each matvec first fills the ghosts in a padded array (six small launches); a complex64 operand of order 4 or 6 is
+ * read in place unless the output overlaps it, others are copied into that array.
  * Memory: three padded copies ((N_x+2)(N_y+2)(N_z+2) points as complex64, complex128 and double-float)
  * and two scratch faces, allocated here and freed by helm_destroy or by HELM_CLOSURE_THREE_POINT.  The
  * scratch is shared by every operator call of the context: issue them on one stream (or order them), and
