@@ -298,7 +298,7 @@ helm_status fill(helm_ctx* c, const M* U, M* P, const double2* faces, bool copy,
     typename A::St* S = reinterpret_cast<typename A::St*>(c->ho_S);   // 16 bytes a value either way
     const Operand<M> op = {U, P, c->nx, c->ny, c->nz};
     long long foff = 0;
-    LaunchChain chain(c, s);
+    LaunchChain chain(c, s, 0);   // timed as one launch, if at all
     for (int axis = 0; axis < 3; ++axis) {
         const Face f = make_face(c, axis);
         const int tot = 2 * f.la * f.lb;

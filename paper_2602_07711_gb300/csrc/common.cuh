@@ -232,17 +232,21 @@ helm_status launch_stencil_padded(helm_ctx* c, const float2* x, float2* y, const
 helm_status run_eig_setup(helm_ctx* c, cudaStream_t s);
 // The launches of a chain after its first may start early (launch_after): their predecessor in the stream is the chain's
 // own kernel before them.  Not under capture (the conditional bodies that hold the batch plans' chains take plain
-// edges) and not while launches are timed by events.
+// edges) and not while one of the chain's classes (a mask of 1 << ProfClass) is timed, whose events lie between the launches.
 // Measured (without, with): preconditioner 32^3 FP32 24.6, 23 us; 150 x 100 x 75 TF32 68, 60; 256^3 FP16 270, 260;
 // order-6 matvec of the high-order closure at 100^3 64, 51.
 struct LaunchChain {
     helm_ctx* c;
     bool allowed = false;
-    LaunchChain(helm_ctx* ctx, cudaStream_t s) : c(ctx) {
+    LaunchChain(helm_ctx* ctx, cudaStream_t s, unsigned classes) : c(ctx) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        allowed = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-                  !(c->prof && c->prof->enabled);
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        allowed = cap == cudaStreamCaptureStatusNone && !(c->prof && c->prof->enabled && (c->prof->mask & classes));
     }
+    LaunchChain(const LaunchChain&) = delete;
     void first_done() { c->follows = allowed; }
     void plain() { c->follows = 0; }
     ~LaunchChain() { c->follows = 0; }

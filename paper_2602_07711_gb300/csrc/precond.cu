@@ -142,6 +142,8 @@ __global__ void __launch_bounds__(256) normed_to_h16_kernel(const float4* __rest
     }
 }
 
+constexpr unsigned PASS_CLASSES = 1u << PROF_XPASS | 1u << PROF_YPASS | 1u << PROF_ZSOLVE;
+
 // The passes of the 16-bit chain from the 16-bit input In to the complex64 z (T0, T1: the halves of the
 // context's scratch vector; In may be T0).  BF16: the static factors of c->h16s (all 1 but the last).  FP16:
 // the x-pass forward scales statically (its input's norm is bounded by h16s[0]), every later stage by the
@@ -153,7 +155,7 @@ helm_status h16_chain(helm_ctx* c, const uint16_t* In, uint16_t* T1, float2* z, 
     const float* sc = c->h16s;
     double* d = c->opt.precision == HELM_PREC_FP16 ? c->h16d : nullptr;
     if (d) HELM_CUDA_TRY(cudaMemsetAsync(d, 0, 3 * sizeof(double), s));
-    LaunchChain chain(c, s);
+    LaunchChain chain(c, s, PASS_CLASSES);
     prof_begin(c, s, PROF_XPASS);
     st = tc_xpass_h16(c, 0, In, T1, 1, sc[1], nullptr, 0, s, nb, 0, nullptr, d);
     prof_end(c, s);
@@ -274,7 +276,7 @@ static helm_status precond_base(helm_ctx* c, const float2* r, float2* z, const d
     }
     if (c->opt.precision == HELM_PREC_BF16 || c->opt.precision == HELM_PREC_FP16) return precond_h16(c, r, z, sigma, sidx, s);
     const float hz2 = (float)(c->h[2] * c->h[2]);
-    LaunchChain chain(c, s);
+    LaunchChain chain(c, s, PASS_CLASSES);
     if ((st = xpass(c, 0, r, c->tmp, 1.f, sigma, sidx, s)) != HELM_OK) return st;
     chain.first_done();
     if ((st = ypass(c, 0, c->tmp, z, s)) != HELM_OK) return st;
@@ -337,7 +339,7 @@ helm_status precond_apply_nb(helm_ctx* c, const float2* r, float2* z, int nb, co
         return h16_chain(c, T0, T1, z, c->h16s[5], nullptr, 0, s, nb);
     }
     const float hz2 = (float)(c->h[2] * c->h[2]);
-    LaunchChain chain(c, s);
+    LaunchChain chain(c, s, PASS_CLASSES);
     if ((st = xpass(c, 0, r, c->tmp, 1.f, sigma, sidx, s, nb, sstride)) != HELM_OK) return st;
     chain.first_done();
     if ((st = ypass(c, 0, c->tmp, z, s, nb)) != HELM_OK) return st;

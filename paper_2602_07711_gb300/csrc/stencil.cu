@@ -765,7 +765,7 @@ helm_status launch_stencil_f32_cls(helm_ctx* c, const float2* x, float2* y, cons
         const bool overlap = x < y + c->npts && y < x + c->npts, ring = c->opt.order != 2;
         helm_status st = closure_fill_f32(c, x, overlap || !ring, s);
         if (st == HELM_OK && ring) {
-            LaunchChain chain(c, s);
+            LaunchChain chain(c, s, 0);   // timed as one launch, if at all
             chain.first_done();   // follows the last ghost kernel
             st = launch_stencil_padded(c, overlap ? nullptr : x, y, sigma, sidx, s);
         }
