@@ -174,7 +174,7 @@ struct helm_ctx {
     KrylovWork* kw = nullptr;
     helm_net* net = nullptr;                // attached learned correction (not owned)
     int tune_nb = 0;                        // CTAs of the Arnoldi kernels chosen by helm_autotune (0 = default)
-    int tune_stencil = 0;                   // complex64 matvec variant chosen by helm_autotune (0 = cp.async ring)
+    int tune_stencil = 0;                   // complex64 matvec variant (set-up: 3, two rows per thread; helm_autotune)
     int follows = 0;                        // the next launch of a chain may start early (launch_after)
     int zring_sms = 0;                      // SM count, set with the ring kernel's attributes at set-up
     int zpiv_ready = 0;                     // shared-memory attribute of the pivot-recomputing z-solve set

@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(ZRT) zsolve_ring_kernel(int nx, int ny, int nz
 // EigT form without the factor stream: the pivots depend only on the line's lateral shift
 // s_ij = alpha_x d_{x,i} + alpha_y d_{y,j} and the plane, so the sweeps recompute them step by step (the same
 // operations as zfactor_kernel, one reciprocal per step).  The forward sweep writes no forward values either: it only
-// saves the recurrences' state (c'_{l-1}, d_{l-1}) at the start of every block of ZU2 steps to a small scratch (4
+// saves the recurrences' state (c'_{l-1}, d_{l-1}) at the start of every block of ZU2 steps to a small scratch (2
 // bytes per point, [block][pair] so that a warp's saves are contiguous rows), and the backward sweep recomputes a
 // block's factors and forward values from its checkpoint and from y, read a second time.  HBM and L2 see y read twice
 // and x written: for 16-bit grids 12 bytes a point where forward values in FP32 took 28.
