@@ -180,7 +180,6 @@ struct helm_ctx {
     int zpiv_ready = 0;                     // shared-memory attribute of the pivot-recomputing z-solve set
     void* zck = nullptr;                    // checkpoints of that z-solve ([block][state][line pair] float4)
     int zpiv_off = 0;                       // set while capturing launches that may run concurrently (batch lanes)
-    int zck_slot = 0;                       // first checkpoint slot of the z-solve launches being captured (batch plans)
     size_t zck_bytes = 0;
     int tune_zring = 2;                     // factorised z-solve: CTAs per SM of the L2-resident ring kernel (0 = one thread per line)
     int tune_ypers = 1;                     // y-pass: 1 persistent with double-buffered accumulators, 0 one tile per CTA
@@ -277,6 +276,7 @@ helm_status tc_prepare_sine(helm_ctx* c, const double2* Sx, const double2* Sy, c
                             cudaStream_t s);
 void tc_release(helm_ctx* c);
 // thomas.cu
+size_t zsolve_ck_bytes(const helm_ctx* c, int nb);
 helm_status zsolve_reserve(helm_ctx* c, int nb);
 helm_status launch_zsolve(helm_ctx* c, const float2* in, float2* out, cudaStream_t s, int nb = 1);
 helm_status zsolve_factor(helm_ctx* c, cudaStream_t s);

@@ -1717,9 +1717,18 @@ struct Group {
     float2* tmp = nullptr;          // nb vectors: the group's preconditioner scratch (lane r's own: vector r)
     double* sigma = nullptr;        // nb (m + 1)
     LaneDev* lt = nullptr;          // device table of the lanes' pointers
-    int slot = 0;                   // z-solve checkpoint slot of the group's first lane within its context
+    void* zck = nullptr;            // the group's z-solve checkpoints (groups of a context run concurrently)
+    size_t zck_bytes = 0;
     cudaGraphConditionalHandle* hcyc = nullptr;   // device copy of the lanes' cycle-end handles
 };
+
+// The context's scratch of its preconditioner exchanged for the group's: the captured launches keep the addresses for
+// the plan's life, during which the context may grow its own, and other groups and plans of the context may run.
+void swap_scratch(helm_ctx* c, Group& gr) {
+    std::swap(c->tmp, gr.tmp);
+    std::swap(c->zck, gr.zck);
+    std::swap(c->zck_bytes, gr.zck_bytes);
+}
 
 // The nodes of one group's restart cycle (every conditional node has its own handle, default 0 at each launch):
 //   begin (each lane decides whether it runs the cycle)
@@ -1762,12 +1771,9 @@ helm_status build_group(cudaGraph_t G, Group& gr, std::vector<Lane>& lanes, int*
         const int has_next = j + 1 < m ? 1 : 0;
         const cudaGraphConditionalHandle hn = has_next ? hg[j + 1] : hg[j];
         st = capture_into(gb, nullptr, 0, s, [&]() {
-            float2* save = c->tmp;
-            c->tmp = gr.tmp;
-            c->zck_slot = gr.slot;
+            swap_scratch(c, gr);
             helm_status e = precond_apply_nb(c, vj, zj, nb, gr.sigma, j, m + 1, s);
-            c->zck_slot = 0;
-            c->tmp = save;
+            swap_scratch(c, gr);
             if (e != HELM_OK) return e;
             if ((e = launch_stencil_f32_nb(c, zj, w, nb, s)) != HELM_OK) return e;
             const int nv = j + 1;
@@ -1815,6 +1821,7 @@ void free_group(Group& g) {
     cudaFree(g.sigma);
     cudaFree(g.lt);
     cudaFree(g.hcyc);
+    cudaFree(g.zck);
     g = Group();
 }
 
@@ -1851,9 +1858,8 @@ helm_status plan_build(helm_batch* P) {
     // groups: runs of consecutive lanes of the same context.  Below kGroupMinPoints a problem's right-hand
     // sides run as independent single-lane groups instead: there the operators are latency-bound, and
     // independent chains keep more of the GPU busy than shared launches save (measured on the 64 x 4 batch
-    // of 48^3 .. 160^3 problems).  Each lane has its own z-solve checkpoint slot within its context.
+    // of 48^3 .. 160^3 problems).
     constexpr size_t kGroupMinPoints = (size_t)160 * 160 * 160;
-    std::vector<std::pair<helm_ctx*, int>> nlanes;   // lanes per context so far
     for (size_t i = 0; i < P->lanes.size();) {
         Group g;
         g.c = P->lanes[i].c;
@@ -1864,11 +1870,6 @@ helm_status plan_build(helm_batch* P) {
             ++i;
         }
         g.nb = (int)i - g.first;
-        size_t e = 0;
-        while (e < nlanes.size() && nlanes[e].first != g.c) ++e;
-        if (e == nlanes.size()) nlanes.push_back({g.c, 0});
-        g.slot = nlanes[e].second;   // the context's lanes before this group
-        nlanes[e].second += g.nb;
         P->groups.push_back(g);
     }
     for (Group& g : P->groups) {
@@ -1881,8 +1882,9 @@ helm_status plan_build(helm_batch* P) {
         };
         if (!A((void**)&g.V, vb * (m + 1) * nb) || !A((void**)&g.Z, vb * (flex ? m : 1) * nb) ||
             !A((void**)&g.tmp, vb * nb) || !A((void**)&g.sigma, sizeof(double) * (m + 1) * nb) ||
-            !A((void**)&g.lt, sizeof(LaneDev) * nb) || !A((void**)&g.hcyc, sizeof(cudaGraphConditionalHandle) * nb))
+            !A((void**)&g.lt, sizeof(LaneDev) * nb) || !A((void**)&g.hcyc, sizeof(cudaGraphConditionalHandle) * nb) || !A(&g.zck, zsolve_ck_bytes(c, nb)))
             return HELM_ERR_NOMEM;
+        g.zck_bytes = zsolve_ck_bytes(c, nb);
         std::vector<LaneDev> lt(nb);
         for (int r = 0; r < nb; ++r) {
             Lane& ln = P->lanes[g.first + r];
@@ -1896,7 +1898,7 @@ helm_status plan_build(helm_batch* P) {
             lt[r] = LaneDev{k.V, k.part, k.H, k.cs, k.sn, k.g, k.sigma, k.coef, k.ctrl_d, ln.L_d};
         }
         HELM_CUDA_TRY(cudaMemcpy(g.lt, lt.data(), sizeof(LaneDev) * nb, cudaMemcpyHostToDevice));
-        if ((st = zsolve_reserve(c, g.slot + nb)) != HELM_OK) return st;   // before capture
+        if ((st = zsolve_reserve(c, 1)) != HELM_OK) return st;   // the context's own, for calls captured elsewhere
     }
     HELM_CUDA_TRY(cudaMalloc(&P->flags, sizeof(int) * P->lanes.size()));
     for (size_t i = 0; i < P->lanes.size(); ++i) P->lanes[i].more = P->flags + i;

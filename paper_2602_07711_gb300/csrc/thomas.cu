@@ -791,7 +791,9 @@ size_t zsolve_ck_bytes(const helm_ctx* c, int nb) {
     return (size_t)((c->nz + ZU2 - 1) / ZU2) * 2 * (size_t)(c->nx / 2) * c->ny * nb * sizeof(float4);
 }
 
-// the pivot checkpoints of nb right-hand sides per z-solve launch (device memory of the context)
+// The context's own pivot checkpoints, for nb right-hand sides per z-solve launch.  Growing frees the old block, so
+// launches that are captured to run again later must not hold it: a batch plan brings its own (c->zck swapped while it
+// captures).
 helm_status zsolve_reserve(helm_ctx* c, int nb) {
     const size_t bytes = zsolve_ck_bytes(c, nb);
     if (bytes <= c->zck_bytes) return HELM_OK;
@@ -803,16 +805,16 @@ helm_status zsolve_reserve(helm_ctx* c, int nb) {
     return HELM_OK;
 }
 
-// the pivot-recomputing kernel on checkpoint slots slot .. slot + nb - 1
+// the pivot-recomputing kernel on the checkpoints c->zck
 template <int H>
-static helm_status run_zpiv(helm_ctx* c, const void* in, void* out, int slot, int nb, float oscale, double* h16d, float gain,
+static helm_status run_zpiv(helm_ctx* c, const void* in, void* out, int nb, float oscale, double* h16d, float gain,
                             cudaStream_t s) {
     const int need = (c->nx / 2 * c->ny * nb + ZRT - 1) / ZRT;
     const int cap = c->zring_sms * 2 * (c->tune_zring > 0 ? c->tune_zring : 1);   // tune_zring 1..3: 2, 4 or 6 CTAs per SM
     // lines held whole where all CTAs fit the SMs that way, two on each
     const size_t all = zpiv_smem(c->nz, H != 0, true), ring = zpiv_smem(c->nz, H != 0, false);
     const bool whole = all <= ZPIV_ALL_MAX && need <= 2 * c->zring_sms;
-    float4* ck = reinterpret_cast<float4*>(c->zck) + (size_t)slot * zsolve_ck_bytes(c, 1) / sizeof(float4);
+    float4* ck = reinterpret_cast<float4*>(c->zck);
     const float2 gz = make_float2((float)c->gam[2].x, (float)c->gam[2].y);
     if (!(c->zpiv_ready & (1 << H))) {
         HELM_CUDA_TRY(cudaFuncSetAttribute(zsolve_piv_kernel<H, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -840,19 +842,16 @@ helm_status launch_zsolve(helm_ctx* c, const float2* in, float2* out, cudaStream
     }
     if (in && c->nx % 2 == 0 && c->tune_zring && c->zring_sms > 0 && !c->zpiv_off) {
         // EigT: pivots recomputed from the shifts (the set-up factors' operations), checkpoints in a scratch
-        // of the context (grown here outside stream capture; a capturing caller reserves it beforehand)
-        // (c->zck_slot: the first checkpoint slot of this launch; concurrent solves of one context in a batch
-        // plan each capture with their own slots)
-        const int slot = c->zck_slot;
-        if (zsolve_ck_bytes(c, slot + nb) > c->zck_bytes) {
+        // of the context (grown here outside stream capture; a capturing caller provides it beforehand)
+        if (zsolve_ck_bytes(c, nb) > c->zck_bytes) {
             cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
             HELM_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
             if (cap != cudaStreamCaptureStatusNone) return launch_zsolve_fact(c, c->zfac, in, out, s, nb);
             helm_status st;
-            if ((st = zsolve_reserve(c, slot + nb)) != HELM_OK) return st;
+            if ((st = zsolve_reserve(c, nb)) != HELM_OK) return st;
         }
         prof_begin(c, s, PROF_ZSOLVE);
-        const helm_status st = run_zpiv<0>(c, in, out, slot, nb, 1.f, nullptr, 1.f, s);
+        const helm_status st = run_zpiv<0>(c, in, out, nb, 1.f, nullptr, 1.f, s);
         prof_end(c, s);
         return st;
     }
@@ -866,17 +865,16 @@ helm_status launch_zsolve_h16(helm_ctx* c, const void* in, void* out, float osca
                               double* h16d, float gain) {
     const int H = c->opt.precision == HELM_PREC_FP16 ? 2 : 1;
     if (c->nx % 2 != 0 || c->zring_sms <= 0) return HELM_ERR_UNSUPPORTED;
-    const int slot = c->zck_slot;
-    if (zsolve_ck_bytes(c, slot + nb) > c->zck_bytes) {
+    if (zsolve_ck_bytes(c, nb) > c->zck_bytes) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         HELM_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
         if (cap != cudaStreamCaptureStatusNone) return HELM_ERR_UNSUPPORTED;
         helm_status st;
-        if ((st = zsolve_reserve(c, slot + nb)) != HELM_OK) return st;
+        if ((st = zsolve_reserve(c, nb)) != HELM_OK) return st;
     }
     prof_begin(c, s, PROF_ZSOLVE);
-    const helm_status st = H == 2 ? run_zpiv<2>(c, in, out, slot, nb, oscale, h16d, gain, s)
-                                  : run_zpiv<1>(c, in, out, slot, nb, oscale, nullptr, 1.f, s);
+    const helm_status st = H == 2 ? run_zpiv<2>(c, in, out, nb, oscale, h16d, gain, s)
+                                  : run_zpiv<1>(c, in, out, nb, oscale, nullptr, 1.f, s);
     prof_end(c, s);
     return st;
 }
