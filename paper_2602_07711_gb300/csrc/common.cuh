@@ -92,6 +92,8 @@ cudaError_t launch_after(int follows, void (*kernel)(P...), dim3 grid, dim3 thre
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+constexpr int H16D_COUNT = 8;   // doubles of helm_ctx::h16d
+
 // ---- the context -----------------------------------------------------------------------------
 struct KrylovWork;
 struct helm_net;
@@ -164,7 +166,9 @@ struct helm_ctx {
     int realk = 0;
     float h16s[6] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f};   // FP16 chain: input, four stage scales, final factor
     double* h16n = nullptr;                 // FP16 chain: 1/||r||, ||r|| and partial sums (helm_apply_precond)
-    double* h16d = nullptr;                 // FP16 chain, per application: ||T1||^2, ||T2||^2, ||T3||^2, -, s2, s3, s4, 1/(s2 s3 s4)
+    // FP16 chain, per application: ||T1||^2, ||T2||^2, ||T3||^2, -, s2, s3, s4, 1/(s2 s3 s4).  One application at a time
+    // may use it: groups of a batch plan, which run concurrently, bring their own
+    double* h16d = nullptr;
     float h16g[3] = {1.f, 1.f, 1.f};        // FP16 chain: norm bounds of the y-pass forward, z-solve, y-pass inverse
     cudaEvent_t h16_join = nullptr;         // FP16 basis: an event the chain's last pass waits for (the step's scale)
     void* sfast = nullptr;                  // TMA descriptors of the stencil's fixed operands (stencil_fast.cu)

@@ -1439,11 +1439,11 @@ helm_status tc_prepare(helm_ctx* c, cudaStream_t s) {
         helm_status sst = h16_scales(c, s);
         if (sst != HELM_OK) return sst;
         if (cudaMalloc(&c->h16n, (2 + 1024) * sizeof(double)) != cudaSuccess ||
-            cudaMalloc(&c->h16d, 8 * sizeof(double)) != cudaSuccess) {
+            cudaMalloc(&c->h16d, H16D_COUNT * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             return HELM_ERR_NOMEM;
         }
-        HELM_CUDA_TRY(cudaMemsetAsync(c->h16d, 0, 8 * sizeof(double), s));
+        HELM_CUDA_TRY(cudaMemsetAsync(c->h16d, 0, H16D_COUNT * sizeof(double), s));
     }
     if (t->h16) {
         // the EigT sets in 16 bits (the TF32 sets above serve helm_precond_step and the PFFT passes)

@@ -1719,6 +1719,7 @@ struct Group {
     LaneDev* lt = nullptr;          // device table of the lanes' pointers
     void* zck = nullptr;            // the group's z-solve checkpoints (groups of a context run concurrently)
     size_t zck_bytes = 0;
+    double* h16d = nullptr;         // the stage norms and scales of the group's FP16 chain
     cudaGraphConditionalHandle* hcyc = nullptr;   // device copy of the lanes' cycle-end handles
 };
 
@@ -1728,6 +1729,7 @@ void swap_scratch(helm_ctx* c, Group& gr) {
     std::swap(c->tmp, gr.tmp);
     std::swap(c->zck, gr.zck);
     std::swap(c->zck_bytes, gr.zck_bytes);
+    std::swap(c->h16d, gr.h16d);
 }
 
 // The nodes of one group's restart cycle (every conditional node has its own handle, default 0 at each launch):
@@ -1822,6 +1824,7 @@ void free_group(Group& g) {
     cudaFree(g.lt);
     cudaFree(g.hcyc);
     cudaFree(g.zck);
+    cudaFree(g.h16d);
     g = Group();
 }
 
@@ -1882,7 +1885,8 @@ helm_status plan_build(helm_batch* P) {
         };
         if (!A((void**)&g.V, vb * (m + 1) * nb) || !A((void**)&g.Z, vb * (flex ? m : 1) * nb) ||
             !A((void**)&g.tmp, vb * nb) || !A((void**)&g.sigma, sizeof(double) * (m + 1) * nb) ||
-            !A((void**)&g.lt, sizeof(LaneDev) * nb) || !A((void**)&g.hcyc, sizeof(cudaGraphConditionalHandle) * nb) || !A(&g.zck, zsolve_ck_bytes(c, nb)))
+            !A((void**)&g.lt, sizeof(LaneDev) * nb) || !A((void**)&g.hcyc, sizeof(cudaGraphConditionalHandle) * nb) || !A(&g.zck, zsolve_ck_bytes(c, nb)) ||
+            (c->h16d && !A((void**)&g.h16d, H16D_COUNT * sizeof(double))))
             return HELM_ERR_NOMEM;
         g.zck_bytes = zsolve_ck_bytes(c, nb);
         std::vector<LaneDev> lt(nb);

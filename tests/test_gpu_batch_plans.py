@@ -12,7 +12,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from paper_2602_07711_gb300 import HELM_PREC_FP32, HELM_PREC_TF32, Batch, Solver
+from paper_2602_07711_gb300 import HELM_PREC_FP16, HELM_PREC_FP32, HELM_PREC_TF32, Batch, Solver
 
 
 def _problem(n, nrhs, precision, seed=3):
@@ -54,4 +54,26 @@ def test_two_plans_of_one_context(n, precision):
         assert float((x3[0][r] - xs).norm() / xs.norm()) < 1e-9
     one.close()
     three.close()
+    S.close()
+
+
+@pytest.mark.parametrize("n", [(48, 48, 48), (64, 36, 20), (128, 304, 20)])
+def test_concurrent_fp16_lanes_keep_their_stage_norms_apart(n):
+    """Four right-hand sides of very different sizes of one FP16 context, as independent branches of one graph: each
+    lane is bit for bit what it is alone in a plan (where nothing runs beside it), in every run."""
+    S, B = _problem(n, 4, HELM_PREC_FP16, seed=5)
+    B[1] *= 1e-3
+    B[2, :, :, : n[0] // 4] = 0
+    plan = Batch([S], [B], [torch.zeros_like(B)])
+    runs = [_run(plan) for _ in range(4)]
+    alone = []
+    for r in range(4):
+        one = Batch([S], [B[r:r + 1].contiguous()], [torch.zeros_like(B[:1])])
+        alone.append(_run(one))
+        one.close()
+    for x, it in runs:
+        for r in range(4):
+            assert it[0][r] == alone[r][1][0][0]
+            assert torch.equal(x[0][r], alone[r][0][0][0])
+    plan.close()
     S.close()
