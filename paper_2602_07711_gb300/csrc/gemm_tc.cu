@@ -1011,15 +1011,19 @@ ypass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
 //   y-pass  A = [Wr | Wi], rows 128 rank .. of W (N_y <= 256, K = N_y <= 256); B = 64 + 64 columns of a slice
 //   x-pass  A = 128 + 128 grid rows; B = BN / 2 + BN / 2 rows of the embedding (K = 2 N_x <= 512), BN <= 256 output
 //           columns: a pair keeps to one of the ntn column blocks
-// Barriers: full[s] (own TMA loads), empty[s] and accf[b] (commits of the leader, CTA 0, to both CTAs), and in the leader
-// pfull[s] (the peer's stage has landed: its warp 1 waits for that and arrives), acce[b] (eight arrivals, the
-// epilogue warps of both); resf[kb]: a chunk of the resident operand (the peer's warp 1 waits for its own).  Waits and drains as above; both CTAs
-// meet in a cluster barrier before either frees its tensor memory or exits, and every thread reaches it, because each
-// wait before it is bounded.
-// The streamed operand is bound by the ring's depth (latency of load, relay and commit: six stages of 16 KiB against four,
+// Barriers: empty[s] and accf[b] (commits of the leader, CTA 0, to both CTAs), and in the leader alone full[s] and
+// resf[kb] (a stage, a chunk of the resident operand: the loads of both CTAs complete there, .cta_group::2, and the
+// leader expects the bytes of both) and acce[b] (sixteen arrivals, the epilogue warps of both).  The leader's MMAs read
+// both CTAs' shared memory and write both CTAs' tensor memory, so whatever crosses the pair is ordered at cluster scope:
+// a load's completion is released there, the epilogue warps' arrivals and the waits of this kernel name it.
+// Waits are bounded as above.  Both CTAs meet in a cluster barrier before either frees its tensor memory or exits, and
+// every thread reaches it, because each wait before it is bounded; a failure on either side is known to both by then,
+// and the leader, on whose barriers the loads of both complete, drains them (settle_loads).
+// The streamed operand is bound by the ring's depth (latency of load and commit: six stages of 16 KiB against four,
 // x-pass 32 -> 29 us), the rest by the epilogue: eight warps, as four took 41 us.
-// Measured at 256^3: y-pass 39 -> 30 us, x-pass 40 -> 29 (FP16 out) and 43 -> 42 (FP32 out, 134 MB written on top of a
-// 67 MB grid that is still dirty in L2).
+// Measured at 256^3 (persistent kernels, pairs): y-pass 39, 30 us, x-pass 40, 29 (FP16 out) and 43, 42-46 (FP32 out, 134 MB
+// written on top of a 67 MB grid that is still dirty in L2).  With the peer waiting for its own loads and passing an
+// arrival on to the leader, the times were the same to 1 us.
 // Above 128 points a side (x-pass: 256 real columns): one 128-row tile or one column block leaves a pair half idle and
 // its cluster start costs more than the basis reads.  Whole FP16 preconditioner, persistent kernels against pairs:
 // 96^3 72 and 82 us, 128^3 81 and 94, 160^3 122 and 121, 192^3 150 and 149, 224^3 235 and 218, 256^3 298 and 270.
@@ -1042,14 +1046,63 @@ __device__ __forceinline__ uint32_t cta_rank() {
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// arrive on the barrier at the same offset in CTA 0 of the cluster.  What it orders are accesses of the asynchronous
-// proxy and of tensor memory (a landed TMA load before an MMA, tcgen05.ld behind its fence before the next MMA), no
-// generic ones; with cluster-scope release and acquire on these barriers a stage took 1.2 us instead of 0.7.
-__device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
+// the address of a shared-memory location of this CTA in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// arrive on a barrier of another CTA (a cluster_addr): the epilogue's reads of an accumulator before the MMAs that
+// overwrite it, which the leader issues.  tcgen05.fence::before_thread_sync on this side and ::after_thread_sync on the
+// other order those through any execution ordering of cluster scope, so the arrival is relaxed: a release would also
+// wait for the epilogue's stores to global memory (x-pass 29 -> 36 us, y-pass 30 -> 42 at 256^3)
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, long limit) {
+    for (long it = 0; it < limit; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+// loads into this CTA's shared memory that complete on a barrier of the pair's leader (a cluster_addr)
+__device__ __forceinline__ void tma_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
     asm volatile(
-        "{\n.reg .b32 ra;\nmapa.shared::cluster.u32 ra, %0, 0;\n"
-        "mbarrier.arrive.shared::cluster.b64 _, [ra];\n}\n" ::"r"(bar)
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], "
+        "[%2];" ::"r"(dst),
+        "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1)
         : "memory");
+}
+__device__ __forceinline__ void tma_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, "
+        "%5}], [%2];" ::"r"(dst),
+        "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+}
+// Drain of the pair's loads after an expired wait, by the leader once both CTAs have stopped: `mine` and `theirs` loads
+// of `bytes` were issued in turn on the ns barriers of `full` by the leader (which expected twice the bytes with its own)
+// and by the peer.  Neither is more than ns ahead of the other, since a stage is issued again only after the MMAs
+// consumed it, and those waited for both; so each barrier's last phase is the only one that can be open.  Where only one
+// CTA issued a load, the other's share is settled here: it is expected once, or its completion made up for.
+__device__ __forceinline__ void settle_loads(const uint64_t* full, int ns, uint32_t bytes, long mine, long theirs) {
+    const long last = mine > theirs ? mine : theirs;
+    for (long it = last > ns ? last - ns : 0; it < last; ++it) {
+        const uint32_t bar = su32(&full[it % ns]);
+        if (it >= mine) mbar_expect_tx(bar, bytes);
+        else if (it >= theirs)
+            asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+        mbar_wait_cluster(bar, (uint32_t)((it / ns) & 1), DRAIN_LIMIT);
+    }
 }
 __device__ __forceinline__ uint32_t elect_one() {
     uint32_t r;
@@ -1093,8 +1146,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 1)
 pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmS, const PairArgs a) {
     extern __shared__ uint8_t dsm[];
     constexpr int STAGE = Pair<X>::STAGE;
-    __shared__ __align__(8) uint64_t full[Pair<X>::NS], pfull[Pair<X>::NS], empty[Pair<X>::NS], accf[2], acce[2], resf[8], drainb;
+    __shared__ __align__(8) uint64_t full[Pair<X>::NS], empty[Pair<X>::NS], accf[2], acce[2], resf[8], drainb;
     __shared__ int fail_any;
+    __shared__ uint32_t issued_by[2], resident_by[2];   // in the leader: the loads each CTA issued
     __shared__ uint32_t tslot;
     const uint32_t raw = su32(dsm);
     const uint32_t base = (raw + 1023u) & ~1023u;   // the same offset in both CTAs
@@ -1112,7 +1166,6 @@ pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant_
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; ++s) {
             mbar_init(su32(&full[s]), 1);
-            mbar_init(su32(&pfull[s]), 1);
             mbar_init(su32(&empty[s]), 1);
         }
         for (int b = 0; b < 2; ++b) { mbar_init(su32(&accf[b]), 1); mbar_init(su32(&acce[b]), 16); }
@@ -1133,49 +1186,53 @@ pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant_
     grid_wait();
     grid_trigger();
     bool ok = true;
-    long issued = 0;      // pipeline iterations whose TMA loads the producer issued
-    int rissued = 0;      // resident chunks it issued
+    constexpr uint32_t RBYTES = (X ? 1 : 2) * TILE;   // a CTA's share of a resident chunk
     if (warp == 0) {
         if (lane == 0) {
+            long issued = 0;      // pipeline iterations whose TMA loads this CTA issued
+            int rissued = 0;      // resident chunks it issued
             int s = 0;
             uint32_t ph = 0;
             for (int t = t0; t < ntiles && ok; t += dt)
                 for (int kb = 0; kb < nk; ++kb) {
                     // the resident chunks go out between the first tile's stages, all before the first wait
                     for (; rissued < nk && (rissued <= kb || issued == NS); ++rissued) {
-                        const uint32_t bar = su32(&resf[rissued]);
-                        mbar_expect_tx(bar, (X ? 1 : 2) * TILE);
-                        if (X) tma_2d(base + rissued * TILE, &tmR, bar, rissued * 64, nfix + rank * (a.BNT / 2));
+                        const uint32_t bar = cluster_addr(su32(&resf[rissued]), 0);
+                        if (rank == 0) mbar_expect_tx(su32(&resf[rissued]), 2 * RBYTES);
+                        if (X) tma_2d_pair(base + rissued * TILE, &tmR, bar, rissued * 64, nfix + rank * (a.BNT / 2));
                         else {
-                            tma_3d(base + 2 * rissued * TILE, &tmR, bar, rissued * 64, rank * BM, 0);
-                            tma_3d(base + (2 * rissued + 1) * TILE, &tmR, bar, rissued * 64, rank * BM, 1);
+                            tma_3d_pair(base + 2 * rissued * TILE, &tmR, bar, rissued * 64, rank * BM, 0);
+                            tma_3d_pair(base + (2 * rissued + 1) * TILE, &tmR, bar, rissued * 64, rank * BM, 1);
                         }
                     }
-                    if (issued >= NS && !(ok = mbar_wait(su32(&empty[s]), ph ^ 1, a.wlim))) break;
-                    mbar_expect_tx(su32(&full[s]), STAGE);
-                    if (X) tma_2d(ring + s * STAGE, &tmS, su32(&full[s]), kb * 64, t * 2 * BM + rank * BM);
-                    else tma_3d(ring + s * STAGE, &tmS, su32(&full[s]), (t % ntn) * BN + rank * (BN / 2), kb * 64, t / ntn);
+                    if (issued >= NS && !(ok = mbar_wait_cluster(su32(&empty[s]), ph ^ 1, a.wlim))) break;
+                    const uint32_t bar = cluster_addr(su32(&full[s]), 0);
+                    if (rank == 0) mbar_expect_tx(su32(&full[s]), 2 * STAGE);
+                    if (X) tma_2d_pair(ring + s * STAGE, &tmS, bar, kb * 64, t * 2 * BM + rank * BM);
+                    else tma_3d_pair(ring + s * STAGE, &tmS, bar, (t % ntn) * BN + rank * (BN / 2), kb * 64, t / ntn);
                     ++issued;
                     if (++s == NS) { s = 0; ph ^= 1; }
                 }
             // the last stages' MMAs: no commit is on its way to this CTA when it leaves
             for (long it = issued > NS ? issued - NS : 0; it < issued && ok; ++it)
-                ok = mbar_wait(su32(&empty[it % NS]), (uint32_t)((it / NS) & 1), a.wlim);
+                ok = mbar_wait_cluster(su32(&empty[it % NS]), (uint32_t)((it / NS) & 1), a.wlim);
+            st_cluster(cluster_addr(su32(&issued_by[rank]), 0), (uint32_t)issued);
+            st_cluster(cluster_addr(su32(&resident_by[rank]), 0), (uint32_t)rissued);
         }
-    } else if (warp == 1 && rank == 0) {
+    } else if (warp == 1 && rank == 0) {   // (the peer's warp 1 shares in the tensor memory's allocation alone)
         const uint32_t lead = elect_one();
         const uint32_t idesc = X ? idesc_h16(H, 2 * BM, a.BNT, 0, 0) : idesc_h16(H, 2 * BM, BN, 0, 1);
         int s = 0, lt = 0;
         uint32_t ph = 0;
         for (int t = t0; t < ntiles && ok; t += dt, ++lt) {
             const int b = lt & 1;
-            if (lt >= 2) ok = __all_sync(0xffffffffu, mbar_wait(su32(&acce[b]), (uint32_t)(((lt >> 1) - 1) & 1), a.wlim));
+            if (lt >= 2) ok = __all_sync(0xffffffffu, mbar_wait_cluster(su32(&acce[b]), (uint32_t)(((lt >> 1) - 1) & 1), a.wlim));
             if (!ok) break;
             fence_after();
             const uint32_t acc_t = tmem + (uint32_t)(b * 256);
             for (int kb = 0; kb < nk; ++kb) {
-                ok = __all_sync(0xffffffffu, (lt > 0 || mbar_wait(su32(&resf[kb]), 0, a.wlim)) &&
-                                                 mbar_wait(su32(&full[s]), ph, a.wlim) && mbar_wait(su32(&pfull[s]), ph, a.wlim));
+                ok = __all_sync(0xffffffffu, (lt > 0 || mbar_wait_cluster(su32(&resf[kb]), 0, a.wlim)) &&
+                                                 mbar_wait_cluster(su32(&full[s]), ph, a.wlim));
                 if (!ok) break;
                 fence_after();
                 const uint32_t st = ring + s * STAGE;
@@ -1195,20 +1252,7 @@ pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant_
             }
             if (ok && lead) commit_pair(su32(&accf[b]));
         }
-    } else if (warp == 1) {
-        // the peer: tell the leader which of this CTA's loads have landed
-        if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
-            for (int t = t0; t < ntiles && ok; t += dt)
-                for (int kb = 0; kb < nk; ++kb) {
-                    ok = (t > t0 || mbar_wait(su32(&resf[kb]), 0, a.wlim)) && mbar_wait(su32(&full[s]), ph, a.wlim);
-                    if (!ok) break;
-                    mbar_arrive_leader(su32(&pfull[s]));
-                    if (++s == NS) { s = 0; ph ^= 1; }
-                }
-        }
-    } else {
+    } else if (warp >= 2) {
         // two warps per 32 accumulator rows, which take its 32-column chunks in turn
         const int q = warp & 3, half = (warp - 2) >> 2;
         float* stg = epi + (warp - 2) * 32 * XEPI_LD;
@@ -1237,7 +1281,7 @@ pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant_
                 const int arow = min(rbase + lane, a.dim - 1);
                 al = a.alpha * al2 * (a.alpha_dev ? (float)a.alpha_dev[a.aidx + (arow / a.rows_per) * a.astride] : 1.f);
             }
-            ok = __all_sync(0xffffffffu, mbar_wait(su32(&accf[b]), (uint32_t)((lt >> 1) & 1), a.wlim));
+            ok = __all_sync(0xffffffffu, mbar_wait_cluster(su32(&accf[b]), (uint32_t)((lt >> 1) & 1), a.wlim));
             if (!ok) break;
             fence_after();
             const int nc = X ? a.BNT : BN;
@@ -1258,7 +1302,7 @@ pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant_
             }
             fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_leader(su32(&acce[b]));
+            if (lane == 0) mbar_arrive_cluster(cluster_addr(su32(&acce[b]), 0));
         }
         double* nsq = X ? a.nsq_out : (a.h16d && a.role == 0 ? a.h16d + 1 : nullptr);
         if (nsq) {
@@ -1270,20 +1314,25 @@ pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant_
     if (!ok) {
         atomicOr(a.status, (unsigned)HELM_DEV_WAIT);
         fail_any = 1;
-    }
-    __syncthreads();
-    if (fail_any) {
-        if (warp == 0 && lane == 0) {
-            drain_tma(full, NS, issued);
-            for (int kb = 0; kb < rissued; ++kb) mbar_wait(su32(&resf[kb]), 0, DRAIN_LIMIT);
-        } else if (warp == 1 && rank == 0 && elect_one()) {   // the lane that issued (the election is deterministic)
-            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&drainb)) : "memory");
-            mbar_wait(su32(&drainb), 0, DRAIN_LIMIT);
-        }
+        st_cluster(cluster_addr(su32(&fail_any), rank ^ 1), 1);
     }
     fence_before();
     __syncthreads();
     cluster_sync();
+    if (fail_any) {   // the same in both CTAs, neither of which issues anything more
+        if (warp == 0 && lane == 0 && rank == 0) {
+            settle_loads(full, NS, STAGE, issued_by[0], issued_by[1]);
+            settle_loads(resf, 8, RBYTES, resident_by[0], resident_by[1]);
+        } else if (warp == 1) {   // all MMAs, and with them the commits to both CTAs
+            if (rank == 0) {
+                if (elect_one()) commit_pair(su32(&drainb));   // the lane that issued (the election is deterministic)
+                __syncwarp();
+            }
+            mbar_wait_cluster(su32(&drainb), 0, DRAIN_LIMIT);
+        }
+        __syncthreads();
+        cluster_sync();
+    }
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 
