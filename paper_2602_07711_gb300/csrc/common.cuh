@@ -77,6 +77,9 @@ struct StencilParams {
 // (LaunchChain sets helm_ctx::follows).
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A word that another kernel of the chain writes.  Volatile, and its pointer not __restrict__: an ordinary load that the
+// compiler may take to be the same anywhere in the kernel could be moved ahead of grid_wait().
+__device__ __forceinline__ double chain_value(const double* p) { return *reinterpret_cast<const volatile double*>(p); }
 template <typename... P, typename... A>
 cudaError_t launch_after(int follows, void (*kernel)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchAttribute at;

@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(SPLIT ? 320 : 192, 1)
 xpass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmBl, void* __restrict__ outv, int M, int N2, int K2,
                      float alpha, const double* __restrict__ alpha_dev, int aidx, int rows_per, int astride,
-                     unsigned* status, long wlim, const double* __restrict__ alpha_dev2 = nullptr,
+                     unsigned* status, long wlim, const double* alpha_dev2 = nullptr,
                      double* __restrict__ nsq_out = nullptr) {
     extern __shared__ uint8_t dsm[];
     constexpr int NS = PersX<BNT, SPLIT>::STAGES, BTILE = BNT * BK * 4, STAGE = PersX<BNT, SPLIT>::STAGE_BYTES;
@@ -702,8 +702,7 @@ xpass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const int q = warp & 3;
         int lt = 0;
         float nacc = 0.f;   // squared norm of what this thread stored (OBF, nsq_out)
-        // written by the kernel before this one: not to be read ahead of grid_wait
-        const float al2 = alpha_dev2 ? (float)*(const volatile double*)alpha_dev2 : 1.f;
+        const float al2 = alpha_dev2 ? (float)chain_value(alpha_dev2) : 1.f;
         const bool wide = rows_aligned(outv, N2, OBF ? 2 : 4);
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++lt) {
             const int b = lt & 1;
@@ -789,7 +788,7 @@ template <bool SPLIT, int H = 0>
 __global__ void __launch_bounds__(SPLIT ? 320 : 192, 1)
 ypass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmY,
                      const __grid_constant__ CUtensorMap tmWl, void* __restrict__ outv, int ny, int N2, int nz,
-                     unsigned* status, long wlim, float alpha = 1.f, double* __restrict__ h16d = nullptr,
+                     unsigned* status, long wlim, float alpha = 1.f, double* h16d = nullptr,
                      float gain = 1.f, int role = 0) {
     extern __shared__ uint8_t dsm[];
     constexpr int YPS = PersY<SPLIT>::STAGES, STAGE = PersY<SPLIT>::STAGE_BYTES;
@@ -912,10 +911,10 @@ ypass_tc_pers_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_const
         // scales by that of ||T3|| (h16d[2]), records h16d[6] and the undo factor 1/(s2 s3 s4) in h16d[7]
         float nacc = 0.f;
         if (h16d) {
-            const float sc = stage_scale((double)gain, h16d[role == 0 ? 0 : 2]);
+            const float sc = stage_scale((double)gain, chain_value(h16d + (role == 0 ? 0 : 2)));
             if (blockIdx.x == 0 && threadIdx.x == 64) {
                 h16d[role == 0 ? 4 : 6] = sc;
-                if (role == 1) h16d[7] = 1.0 / (h16d[4] * h16d[5] * (double)sc);
+                if (role == 1) h16d[7] = 1.0 / (chain_value(h16d + 4) * chain_value(h16d + 5) * (double)sc);
             }
             alpha *= sc;
         }
@@ -1262,13 +1261,13 @@ pair_pass_kernel(const __grid_constant__ CUtensorMap tmR, const __grid_constant_
         const bool wide = a.wide;
         float al2 = a.alpha;
         if (X) {
-            if (a.alpha_dev2) al2 = (float)a.alpha_dev2[0];
+            if (a.alpha_dev2) al2 = (float)chain_value(a.alpha_dev2);
             else al2 = 1.f;
         } else if (a.h16d) {
-            const float sc = stage_scale((double)a.gain, a.h16d[a.role == 0 ? 0 : 2]);
+            const float sc = stage_scale((double)a.gain, chain_value(a.h16d + (a.role == 0 ? 0 : 2)));
             if (blockIdx.x == 0 && threadIdx.x == 64) {
                 a.h16d[a.role == 0 ? 4 : 6] = sc;
-                if (a.role == 1) a.h16d[7] = 1.0 / (a.h16d[4] * a.h16d[5] * (double)sc);
+                if (a.role == 1) a.h16d[7] = 1.0 / (chain_value(a.h16d + 4) * chain_value(a.h16d + 5) * (double)sc);
             }
             al2 *= sc;
         }

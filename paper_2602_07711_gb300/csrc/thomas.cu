@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(ZRT, ALL ? 2 : 4) zsolve_piv_kernel(int nx, in
                                                                       const float2* __restrict__ dys,
                                                                       const float2* __restrict__ cz, const void* inv,
                                                                       void* outv, float4* __restrict__ ck, int nb,
-                                                                      float oscale = 1.f, double* __restrict__ h16d = nullptr,
+                                                                      float oscale = 1.f, double* h16d = nullptr,
                                                                       float gain = 1.f) {
     constexpr bool BF = H != 0;
     typedef typename ZPairOf<BF>::T Y;   // a step's input values of a line pair
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(ZRT, ALL ? 2 : 4) zsolve_piv_kernel(int nx, in
     // recorded in h16d[5]; the squared norm of what is stored accumulates into h16d[2]
     float nacc = 0.f;
     if (BF && h16d) {
-        const double n2 = h16d[1];
+        const double n2 = chain_value(h16d + 1);
         float sc = 1.f;
         if (n2 > 0.0) {
             int e = 15 - (int)ceil(log2((double)gain * sqrt(n2)));

@@ -4,7 +4,7 @@ import pathlib
 import re
 
 CSRC = pathlib.Path(__file__).resolve().parent.parent / "paper_2602_07711_gb300" / "csrc"
-SOURCES = {p.name: p.read_text() for p in sorted(CSRC.iterdir()) if p.suffix in (".cu", ".cuh")}
+SOURCES = {p.name: re.sub(r"//.*", "", p.read_text()) for p in sorted(CSRC.iterdir()) if p.suffix in (".cu", ".cuh")}
 
 
 def body(text, name):
@@ -27,3 +27,14 @@ def test_waits_of_the_pair_kernel_acquire_at_cluster_scope():
     for name in ("pair_pass_kernel", "settle_loads"):
         assert not re.search(r"\bmbar_wait\(", body(text, name)), name
     assert "try_wait.parity.acquire.cluster." in body(text, "mbar_wait_cluster")
+
+
+def test_values_of_the_chains_other_kernels_are_not_read_ahead_of_the_wait():
+    """A kernel that may start before its predecessor ends reads what that one writes after grid_wait() alone: no
+    __restrict__ on the pointer, no plain load through it."""
+    for name, text in SOURCES.items():
+        assert not re.search(r"double\*\s+__restrict__\s+(h16d|alpha_dev2)\b", text), name
+        for kernel in re.findall(r"__global__[^;{]*?\b(\w+_kernel)\(", text):
+            code = body(text, kernel)
+            if "grid_wait()" in code:
+                assert not re.search(r"\b(h16d|alpha_dev2)\[[^\]]*\](?!\s*=[^=])", code), (name, kernel)
