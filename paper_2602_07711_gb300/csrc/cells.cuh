@@ -1,7 +1,7 @@
 // Activation layout of the learned correction: cells of 8 channels (BF16, 16 bytes) on a grid with a zero halo
 // of one point, [batch][channel group][Z + 2][Y + 2][pitch] cells, point (z, y, x) at (z + 1, y + 1, x + 1).  The
 // number of groups is even (16-channel chunks); channels beyond the tensor's are zero.  Halo cells are zeroed
-// when the workspace takes a new shape and never written, so a plane can be walked along its flattened index:
+// when the workspace takes a new shape (zero_rest_kernel) and never written, so a plane can be walked along its flattened index:
 // the points (y, x) sit at pitch + 1 + y pitch + x, and what lies between rows is zero.  The pitch is at least 16,
 // so that 15 points beyond the last one (a K step of the weight gradient) are halo too.  Tiles may read past the
 // last plane: CELL_SLACK zeroed cells follow every tensor.  FP32 cells (gradients that are summed further) are 8

@@ -42,10 +42,11 @@ struct helm_net {
     size_t woff[6], boff[6];
     int co[6], ci[6];
     // workspace of the last forward's shape (full-resolution and half-resolution grids); grown on demand, never
-    // shrunk.  `fresh`: the cells have to be zeroed before use (new shape or new memory)
+    // shrunk.  `fresh`: the cells that no kernel writes have to be zeroed before use (new shape or new memory).
+    // `recorded`: a call was recorded into a CUDA graph, whose replays may use the memory in another shape unseen
     int B = 0, Z = 0, Y = 0, X = 0;
     CellGrid gf, gh;
-    bool fresh = false, gfresh = false;
+    bool fresh = false, gfresh = false, recorded = false;
     int gB_ = 0, gZ_ = 0, gY_ = 0, gX_ = 0;                 // shape of the gradient workspace
     Buf xp, y;                                              // channel-first features (BF16) and output (FP32)
     Buf x, a1, u, d1, p, b1, b2;                            // BF16 cells; u holds [up(b2), a2]; p, b1, b2 half resolution
@@ -109,6 +110,40 @@ __device__ __forceinline__ void add_channel_sums(const float* s, float* gb, int 
     if (!(lane & 3)) atomicAdd(&red[lane_fold8_channel(lane)], f);
     __syncthreads();
     if (threadIdx.x < 8 && c0 + threadIdx.x < C) atomicAdd(&gb[c0 + threadIdx.x], red[threadIdx.x]);
+}
+
+// The cells of up to seven tensors that the kernels read but never write are zeroed: the halos, the slack behind each
+// tensor and the groups from Gw on, whose last channels nobody writes.  One warp per row of a padded plane.  Bound by its
+// short scattered writes: 160^3, width 28, 145 us (of a forward pass of 2.1 ms) where a fill of the whole workspace took 480;
+// 96^3 33 us, 16^3 12 us, where the fill took what the largest shape's takes.
+struct Rest {
+    bf16* t;
+    int half, G, Gw;   // a half-resolution tensor; its groups; those that are written whole
+};
+struct Rests { Rest r[7]; };
+__global__ void __launch_bounds__(256) zero_rest_kernel(CellGrid gf, CellGrid gh, const __grid_constant__ Rests rests) {
+    const Rest R = rests.r[blockIdx.y];
+    const CellGrid& g = R.half ? gh : gf;
+    uint4* t = reinterpret_cast<uint4*>(R.t);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the rows of every channel group in `parts` shares of a CTA
+    const int rows = (g.Z + 2) * (g.Y + 2), groups = g.B * R.G, parts = max(1, (int)gridDim.x / groups);
+    for (int c = blockIdx.x; c < groups * parts; c += gridDim.x) {
+        const int group = c / parts;
+        const bool written = group % R.G < R.Gw;
+        for (int q = (c % parts) * 8 + warp; q < rows; q += parts * 8) {
+            const int z = q / (g.Y + 2), y = q - z * (g.Y + 2);
+            uint4* row = t + ((long)group * rows + q) * g.pitch;
+            if (written && z >= 1 && z <= g.Z && y >= 1 && y <= g.Y) {
+                for (int x = lane ? g.X + lane : 0; x < g.pitch; x += 32) row[x] = zero;
+            } else {
+                for (int x = lane; x < g.pitch; x += 32) row[x] = zero;
+            }
+        }
+    }
+    const long end = (long)groups * g.vol;
+    for (long x = blockIdx.x * 256L + threadIdx.x; x < CELL_SLACK; x += gridDim.x * 256L) t[end + x] = zero;
 }
 
 // channel-first features (5 channels) -> cells of group 0 (channels 5-7 zero)
@@ -422,8 +457,8 @@ bool grow(Buf& b, size_t bytes) {
     return true;
 }
 
-// inference workspace for B x Z x Y x X (grown on demand, never shrunk); the cells are zeroed by the next
-// forward when the shape or the memory is new
+// inference workspace for B x Z x Y x X (grown on demand, never shrunk); when the shape or the memory is new, the next
+// forward zeroes the cells that it does not write
 helm_status ensure_ws(helm_net* n, int B, int Z, int Y, int X) {
     if (B < 1 || Z < 2 || Y < 2 || X < 2 || Z % 2 || Y % 2 || X % 2) return HELM_ERR_ARG;
     if (B == n->B && Z == n->Z && Y == n->Y && X == n->X) return HELM_OK;
@@ -459,6 +494,21 @@ dim3 cell_blocks(const CellGrid& g, int C) {
     return dim3((unsigned)(b > 1024 ? 1024 : b), (unsigned)(g.B * ((C + 7) / 8)));
 }
 
+// Zeroes what a forward or backward reads and does not write, where that may hold anything else: in new memory or a new
+// shape (`fresh`, cleared), and always in a graph and once a call was recorded into one, since its replays may lie
+// between any two calls and nothing here sees them.
+helm_status zero_rest(helm_net* n, bool& fresh, cudaStream_t s, const Rests& rests, int count) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    HELM_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+    const bool recording = cap != cudaStreamCaptureStatusNone;
+    n->recorded |= recording;
+    if (!fresh && !n->recorded) return HELM_OK;
+    zero_rest_kernel<<<dim3(1216, count), 256, 0, s>>>(n->gf, n->gh, rests);
+    HELM_CUDA_TRY(cudaGetLastError());
+    if (!recording) fresh = false;
+    return HELM_OK;
+}
+
 // forward of channel-first features xp into y (channel-first FP32); bounded-wait failures OR-ed into *status
 helm_status forward(helm_net* n, const bf16* xp, float* y, unsigned* status, cudaStream_t s) {
     const int c = n->c;
@@ -466,11 +516,13 @@ helm_status forward(helm_net* n, const bf16* xp, float* y, unsigned* status, cud
     const bf16* W = n->Wb;
     const float* F = n->W;
     helm_status st;
-    if (n->fresh) {
-        for (const Buf* b : {&n->x, &n->a1, &n->u, &n->d1, &n->p, &n->b1, &n->b2})
-            HELM_CUDA_TRY(cudaMemsetAsync(b->p, 0, b->cap, s));
-        n->fresh = false;
-    }
+    // (u: where its parts do not meet between cells, its last cell's channels are written one by one)
+    if ((st = zero_rest(n, n->fresh, s, Rests{{{cells(n->x), 0, cell_groups(5), 1}, {cells(n->a1), 0, cell_groups(c), (c + 7) / 8},
+                                              {cells(n->u), 0, cell_groups(3 * c), c % 4 ? 3 * c / 8 : (3 * c + 7) / 8},
+                                              {cells(n->d1), 0, cell_groups(c), (c + 7) / 8}, {cells(n->p), 1, cell_groups(c), (c + 7) / 8},
+                                              {cells(n->b1), 1, cell_groups(2 * c), (2 * c + 7) / 8},
+                                              {cells(n->b2), 1, cell_groups(2 * c), (2 * c + 7) / 8}}}, 7)) != HELM_OK)
+        return st;
     auto conv = [&](const CellGrid& g, int mode, int l, const Buf& in, void* out, int Cout_total, int ooff, int relu) {
         return conv_cells(g, mode, cells(in), n->ci[l], W + n->woff[l], 0, F + n->boff[l], out, n->co[l], Cout_total, ooff, relu,
                           nullptr, nullptr, n->wscr, status, s);
@@ -608,10 +660,11 @@ helm_status helm_net_backward(helm_net* n, const float* gy, void* stream) {
     const CellGrid &gf = n->gf, &gh = n->gh;
     const bf16* W = n->Wb;
     float* G = n->G;
-    if (n->gfresh) {
-        for (const Buf* b : {&n->gy, &n->gC, &n->gD, &n->gH1, &n->gH2}) HELM_CUDA_TRY(cudaMemsetAsync(b->p, 0, b->cap, s));
-        n->gfresh = false;
-    }
+    if ((st = zero_rest(n, n->gfresh, s, Rests{{{cells(n->gy), 0, cell_groups(2), 1}, {cells(n->gC), 0, cell_groups(c), (c + 7) / 8},
+                                               {cells(n->gD), 0, cell_groups(c), (c + 7) / 8},
+                                               {cells(n->gH1), 1, cell_groups(2 * c), (2 * c + 7) / 8},
+                                               {cells(n->gH2), 1, cell_groups(2 * c), (2 * c + 7) / 8}}}, 5)) != HELM_OK)
+        return st;
     auto wgrad = [&](const CellGrid& g, int l, const Buf& in, const Buf& gr) {
         return wgrad_cells(g, cells(in), n->ci[l], cells(gr), n->co[l], G + n->woff[l], n->status, s);
     };
