@@ -158,7 +158,8 @@ enum { HELM_CLOSURE_THREE_POINT = 0, HELM_CLOSURE_HIGH_ORDER = 1 };
  * Each matvec first fills the ghosts in a padded array (six small launches); a complex64 operand of order 4 or 6 is
  * read in place unless the output overlaps it, others are copied into that array.
  * Memory: three padded copies ((N_x+2)(N_y+2)(N_z+2) points as complex64, complex128 and double-float)
- * and two scratch faces, allocated here and freed by helm_destroy or by HELM_CLOSURE_THREE_POINT.  The
+ * and two scratch faces, and for a real k^2 of order 4 or 6 its real fields (4 or 20 bytes a point; left out where
+ * they do not fit), allocated here and freed by helm_destroy or by HELM_CLOSURE_THREE_POINT.  The
  * scratch is shared by every operator call of the context: issue them on one stream (or order them), and
  * do not put the context in a batch (HELM_ERR_UNSUPPORTED there).
  * Errors: HELM_ERR_ARG (bad value), HELM_ERR_UNSUPPORTED (staggered grid, or an N below 8),

@@ -366,6 +366,7 @@ void closure_release(helm_ctx* c) {
     void* ps[] = {c->ho_P32, c->ho_P64, c->ho_Pdf, c->ho_S};
     for (void* p : ps) if (p) cudaFree(p);
     c->ho_P32 = nullptr; c->ho_P64 = nullptr; c->ho_Pdf = nullptr; c->ho_S = nullptr;
+    if (c->ho) stencil_real_release(c);
     c->ho = 0;
 }
 
@@ -391,5 +392,9 @@ extern "C" helm_status helm_set_closure(helm_ctx* c, int closure) {
     HELM_CUDA_TRY(cudaMemset(c->ho_P64, 0, np * sizeof(double2)));
     HELM_CUDA_TRY(cudaMemset(c->ho_Pdf, 0, np * sizeof(float4)));
     c->ho = 1;
-    return HELM_OK;
+    // the real fields of a medium without attenuation; without room for them the matvec reads the complex ones
+    const helm_status st = stencil_real_prepare(c, nullptr);
+    if (st == HELM_OK || st == HELM_ERR_NOMEM) return HELM_OK;
+    closure_release(c);
+    return st;
 }

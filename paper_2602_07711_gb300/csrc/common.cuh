@@ -221,6 +221,7 @@ helm_status launch_rhs(helm_ctx* c, const double2* f, double2* F, float4* fdf, c
 // stencil_fast.cu: the complex64 matvec of orders 4 and 6 (cp.async plane ring, plane-quantity form)
 helm_status stencil_fast_prepare(helm_ctx* c);
 helm_status stencil_real_prepare(helm_ctx* c, cudaStream_t s);
+void stencil_real_release(helm_ctx* c);
 void stencil_fast_release(helm_ctx* c);
 int stencil_variants(const helm_ctx* c);
 helm_status residual_fast_prepare();

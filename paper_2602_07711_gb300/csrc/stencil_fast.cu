@@ -1032,12 +1032,16 @@ helm_status stencil_fast_prepare(helm_ctx* c) {
 void stencil_fast_release(helm_ctx* c) {
     delete (FastMaps*)c->sfast;
     c->sfast = nullptr;
+    stencil_real_release(c);
+    residual_real_release(c);
+}
+
+void stencil_real_release(helm_ctx* c) {
     cudaFree(c->k2r);
     cudaFree(c->fr);
     c->k2r = nullptr;
     c->fr = nullptr;
     c->realk = 0;
-    residual_real_release(c);
 }
 
 namespace {
@@ -1059,9 +1063,10 @@ __global__ void real_fields_kernel(size_t n, int order, const float2* __restrict
 
 // Set-up of the real-medium matvec: when Im k^2 vanishes everywhere (a medium without attenuation), the
 // complex64 matvec stages k^2 as float and reads the four order-6 fields as one real float4 per point
-// (36 instead of 56 bytes per point, real instead of complex products).  Synchronises s.
+// (36 instead of 56 bytes per point, real instead of complex products).  Synchronises s.  Collocated grids: with the
+// high-order closure alone, whose matvec reads them (helm_set_closure).
 helm_status stencil_real_prepare(helm_ctx* c, cudaStream_t s) {
-    if (c->opt.order == 2) return HELM_OK;
+    if (c->opt.order == 2 || (c->colloc && !c->ho)) return HELM_OK;
     unsigned* flag = nullptr;
     unsigned h = 1;
     HELM_CUDA_TRY(cudaMalloc(&flag, sizeof(unsigned)));
