@@ -1,7 +1,8 @@
 // Activation layout of the learned correction: cells of 8 channels (BF16, 16 bytes) on a grid with a zero halo
-// of one point, [batch][channel group][Z + 2][Y + 2][pitch] cells, point (z, y, x) at (z + 1, y + 1, x + 1).  The
-// number of groups is even (16-channel chunks); channels beyond the tensor's are zero.  Halo cells are zeroed
-// when the workspace takes a new shape (zero_rest_kernel) and never written, so a plane can be walked along its flattened index:
+// of one point, [batch][channel group][Z + 2][Y + 2][pitch] cells, point (z, y, x) at (z + 1, y + 1, x + 1).  Channels
+// of the last group beyond the tensor's are zero; where an odd number of groups leaves half of a 16-channel chunk, the
+// kernels stage the zeros that follow the tensor (rounding the groups up to even ones instead took 1.6 times the
+// workspace at width 4).  Halo cells are zeroed when the workspace takes a new shape (zero_rest_kernel) and never written, so a plane can be walked along its flattened index:
 // the points (y, x) sit at pitch + 1 + y pitch + x, and what lies between rows is zero.  The pitch is at least 16,
 // so that 15 points beyond the last one (a K step of the weight gradient) are halo too.  Tiles may read past the
 // last plane: CELL_SLACK zeroed cells follow every tensor.  FP32 cells (gradients that are summed further) are 8
@@ -27,7 +28,7 @@ inline CellGrid cell_grid(int B, int Z, int Y, int X) {
     g.vol = (Z + 2) * g.plane;
     return g;
 }
-__host__ __device__ inline int cell_groups(int C) { return (C + 15) / 16 * 2; }
+__host__ __device__ inline int cell_groups(int C) { return (C + 7) / 8; }
 inline size_t cell_bytes(const CellGrid& g, int C, int elem = 2) {
     return ((size_t)g.B * cell_groups(C) * g.vol + CELL_SLACK) * 8 * elem;
 }

@@ -27,7 +27,8 @@
 //   128-point block each (one warp alone could not issue them fast enough: 118 cycles an MMA), warps 2-9 run the epilogue
 //   of the previous tile.
 //   Measured at 160^3, width 28: the 84 -> 28 layer 4.14 ms before cells, 1.38 with one output plane per MMA, 1.05 with
-//   one MMA warp and four epilogue warps, 0.90 now; the forward pass 9.2, 3.17, 2.46, 2.09 ms.
+//   one MMA warp and four epilogue warps, 0.90 with two and eight; the forward pass 9.2, 3.17, 2.46, 2.09 ms, and 1.89
+//   since a stage's copies are issued without forming their addresses anew.
 // Weight gradient:  gW[o][i][t] = sum_p g[o][p] in[i][p + off_t].
 //   Both operands are read as MN-major cells (channels x points): M = output channels (64, or 128), N = all
 //   input channels of a block (up to 160), K = 256 points of a flattened plane (the gradient's halo is zero, so
@@ -52,6 +53,7 @@ constexpr int CV_THREADS = CT_THREADS + 5 * 32;    // convolutions: eight epilog
                                                    // block (warps 1 and 10)
 constexpr int CT_NST = 8;                          // most stages
 constexpr int CT_CHUNK = 128;                      // cells of a bulk copy at most (whole runs measured the same)
+constexpr int CT_RUN = 3 * (128 * CT_RMAX + 2);    // cells of a staged run at most
 constexpr int CT_SMEM = 229376;                    // dynamic shared memory of a CTA at most (224 KiB)
 constexpr int WG_KT = 256;                         // points of a weight-gradient tile at most
 // Points a CTA sums in tensor memory before it adds to gW.  The accumulators of the tensor cores are FP32 with
@@ -179,7 +181,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) conv_cells_kernel(const __grid_
     __shared__ int fail_any;
     __shared__ float sbias[CT_NPMAX];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nkc = a.Gin / 2;
+    const int nkc = (a.Gin + 1) / 2;
     const uint32_t base = (s32(csm) + 127u) & ~127u;
     const uint32_t wbytes = 27u * 2u * (uint32_t)a.Np * 16u, sbytes = (uint32_t)a.L * 16u;
     const uint32_t ring = base + 2u * wbytes;   // (wbytes is a multiple of 128)
@@ -205,8 +207,17 @@ __global__ void __launch_bounds__(CV_THREADS, 1) conv_cells_kernel(const __grid_
     bool ok = true;
     long issued = 0, wissued = 0;   // stages and weight chunks whose copies were issued
     if (warp == 0) {
-        // a stage's pieces: runs (two channel groups, times three dy in the split form) in chunks of CT_CHUNK cells
+        // a stage's pieces: runs (two channel groups, times three dy in the split form) in chunks of CT_CHUNK cells, one for
+        // each lane (at most 18).  What a lane's copy has in common for all stages is formed here: the time from a free
+        // stage to its copies is on the pipeline's path (a division and a product more per stage cost 3%)
         const int nrun = a.split ? 6 : 2, run = a.split ? a.dstride : a.L, nch = (run + CT_CHUNK - 1) / CT_CHUNK;
+        const int rn = lane / nch, c = (lane - rn * nch) * CT_CHUNK, cg = rn & 1, dy = rn >> 1;
+        const bool copies = rn < nrun;
+        const uint32_t dst = ring + (uint32_t)cg * sbytes + (uint32_t)(dy * a.dstride + c) * 16u;
+        const uint32_t bytes = (uint32_t)min(CT_CHUNK, run - c) * 16u;
+        const bf16* src = a.in + 8 * (cg * g.vol + (long)dy * g.pitch + c);
+        // a second group that does not exist: the zeros behind the tensor, at another place for every CTA
+        const bf16* zeros = a.in + 8 * ((long)g.B * a.Gin * g.vol + blockIdx.x * 24 % (CELL_SLACK - CT_RUN) + c);
         for (int tile = blockIdx.x; tile < a.ntiles && ok; tile += gridDim.x) {
             const int tp = tile % a.ntp, zg = tile / a.ntp, z0 = zg % a.nzg * a.S, b = zg / a.nzg;
             const int planes = min(a.S, g.Z - z0) + 2;   // input planes
@@ -222,19 +233,18 @@ __global__ void __launch_bounds__(CV_THREADS, 1) conv_cells_kernel(const __grid_
                     bulk_g2s(base + (uint32_t)wb * wbytes + o, reinterpret_cast<const unsigned char*>(a.wt) + (size_t)kc * wbytes + o,
                              min(CT_CHUNK * 16u, wbytes - o), s32(&wfull[wb]));
                 ++wissued;
+                const bool none = cg && 2 * kc + 1 == a.Gin;
+                const bf16* from = none ? zeros : src + 8 * (((long)b * a.Gin + 2 * kc) * g.vol + (long)z0 * g.plane + q0);
+                const long step = none ? 0 : 8 * g.plane;
                 for (int zp = 0; zp < planes; ++zp, ++issued) {
                     const int s = (int)(issued % a.nst);
                     if (issued >= a.nst) ok = warp_wait(s32(&empty[s]), (uint32_t)((issued / a.nst - 1) & 1), CT_WAIT);
                     if (!ok) break;
-                    const uint32_t st = ring + (uint32_t)s * (uint32_t)a.stage, fb = s32(&full[s]);
+                    const uint32_t fb = s32(&full[s]);
                     if (lane == 0) bar_expect(fb, 2u * sbytes);
                     __syncwarp();
-                    const bf16* plane = a.in + 8 * (((long)b * a.Gin + 2 * kc) * g.vol + (long)(z0 + zp) * g.plane + q0);
-                    for (int k = lane; k < nrun * nch; k += 32) {
-                        const int rn = k / nch, c = (k - rn * nch) * CT_CHUNK, cg = rn & 1, dy = rn >> 1;
-                        bulk_g2s(st + (uint32_t)cg * sbytes + (uint32_t)(dy * a.dstride + c) * 16u,
-                                 plane + 8 * (cg * g.vol + (long)dy * g.pitch + c), (uint32_t)min(CT_CHUNK, run - c) * 16u, fb);
-                    }
+                    if (copies) bulk_g2s(dst + (uint32_t)s * (uint32_t)a.stage, from, bytes, fb);
+                    from += step;
                 }
             }
         }
@@ -594,7 +604,7 @@ helm_status conv_prepare() {
 helm_status conv_cells(const CellGrid& g, int mode, const bf16* in, int Cin, const bf16* w, int wmode, const float* bias,
                        void* out, int Cout, int Cout_total, int ooff, int relu, const bf16* mask, float* gb, bf16* wscr,
                        unsigned* status, cudaStream_t s) {
-    const int Gin = cell_groups(Cin), nkc = Gin / 2;
+    const int Gin = cell_groups(Cin), nkc = (Gin + 1) / 2;
     const int sms = sm_count();
     // output slices of at most 64 channels (one accumulator width each); the launches follow one another on s
     for (int o0 = 0; o0 < Cout; o0 += CT_NPMAX) {
@@ -658,7 +668,7 @@ helm_status wgrad_cells(const CellGrid& g, const bf16* in, int Cin, const bf16* 
     const int Nin = 8 * a.Gin;
     a.ndy = Nin <= 48 ? 3 : 1;
     a.nblk = (Nin + 159) / 160;
-    a.Nb = (Nin / 16 + a.nblk - 1) / a.nblk * 16;
+    a.Nb = ((Nin + 15) / 16 + a.nblk - 1) / a.nblk * 16;
     // the MMAs read M / 8 groups of gradient rows; those beyond Ggr fall into the staged inputs (their accumulator
     // rows are not used), so a stage is at least as long as all of them
     auto stage = [&](int kt) {
