@@ -679,7 +679,7 @@ helm_status wgrad_cells(const CellGrid& g, const bf16* in, int Cin, const bf16* 
     a.nst = std::min(CT_NST, (CT_SMEM - 128) / a.stage);
     a.ntp = (g.span + a.kt - 1) / a.kt;
     a.ntiles = (int)((long)g.B * g.Z * a.ntp);
-    // whole waves of CTAs (one per SM), each with at most WG_TILES tiles
+    // whole waves of CTAs (one per SM), each with at most WG_POINTS points
     const int groups = (a.ndy == 3 ? 3 : 9) * a.nblk, sms = sm_count();
     const int one = std::max(1, sms / groups), per = WG_POINTS / a.kt;
     const int waves = (a.ntiles + per * one - 1) / (per * one);
