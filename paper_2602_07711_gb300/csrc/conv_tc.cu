@@ -27,8 +27,8 @@
 //   128-point block each (one warp alone could not issue them fast enough: 118 cycles an MMA), warps 2-9 run the epilogue
 //   of the previous tile.
 //   Measured at 160^3, width 28: the 84 -> 28 layer 4.14 ms before cells, 1.38 with one output plane per MMA, 1.05 with
-//   one MMA warp and four epilogue warps, 0.90 with two and eight; the forward pass 9.2, 3.17, 2.46, 2.09 ms, and 1.89
-//   since a stage's copies are issued without forming their addresses anew.
+//   one MMA warp and four epilogue warps, 0.90 with two and eight, 0.80 since a stage's copies
+//   are issued without forming their addresses anew; the forward pass 9.2, 3.17, 2.46, 2.09, 1.89 ms.
 // Weight gradient:  gW[o][i][t] = sum_p g[o][p] in[i][p + off_t].
 //   Both operands are read as MN-major cells (channels x points): M = output channels (64, or 128), N = all
 //   input channels of a block (up to 160), K = 256 points of a flattened plane (the gradient's halo is zero, so
@@ -36,7 +36,7 @@
 //   one dy in tensor memory for its whole share of the points and adds them to gW (FP32 atomics) at the end.
 //   The copies bound it: one warp issues a 4 KiB copy per channel group and tile.  Measured on two 96^3 fields, 84 ->
 //   28 layer: 0.65 ms with tiles of 256 points, 1.19 ms with 128; 7.6 ms with M = 128 rows of which 28 were used, N =
-//   16 inputs at a time and a gathered slab per input chunk.  A training pass: 24.2 -> 4.1 ms.
+//   16 inputs at a time and a gathered slab per input chunk.  A training pass: 24.2 -> 3.9 ms.
 // Every mbarrier wait is bounded; an expired wait raises HELM_DEV_WAIT, the CTA waits (bounded) for its bulk
 // copies and MMAs in flight, frees its tensor memory and exits.
 #include "cells.cuh"
