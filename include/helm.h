@@ -352,7 +352,9 @@ helm_status helm_net_get_grads(helm_net* net, float* host, size_t count);
 /* helm_net_zero_grad - clear the accumulated parameter gradients (stream-ordered). */
 helm_status helm_net_zero_grad(helm_net* net, void* stream);
 /* helm_net_forward - y = N(x) for a batch: x bfloat16 device [B][5][Z][Y][X], y float32 device
- * [B][2][Z][Y][X].  Keeps the activations for helm_net_backward.  Grows the workspace on demand. */
+ * [B][2][Z][Y][X].  Keeps the activations for helm_net_backward.  Grows the workspace on demand, so a call that is
+ * recorded into a CUDA graph needs one of its shape, or a larger one, before it; replays and other calls may alternate,
+ * on one stream, until a larger shape makes the workspace grow. */
 helm_status helm_net_forward(helm_net* net, const void* x, float* y, int B, int Z, int Y, int X, void* stream);
 /* helm_net_backward - accumulates dL/dparams for dL/dy = gy (float32 device, shape of the last forward's y)
  * into the gradients.  Needs a preceding helm_net_forward on the same net. */

@@ -1161,7 +1161,7 @@ template <int ORDER, bool RK, bool PAD>
 void run_two_rows(const FParams& p, dim3 grid, const float2* x, float2* y, const double* sigma, int sidx, cudaStream_t s,
                   int follows = 0) {
     const dim3 block(FTX, FTY / 2);
-    if (PAD)
+    if (PAD)   // (with the constant chunk length where it applies: no gain, 256^3 and 320^3, orders 4 and 6)
         launch_after(follows, stencil_fast2_kernel<ORDER, RK, PAD, true>, grid, block, fast2_smem<RK>(), s, p, x, y, sigma, sidx);
     else if (p.zch != FZCH)
         stencil_fast2_kernel<ORDER, RK, false, true><<<grid, block, fast2_smem<RK>(), s>>>(p, x, y, sigma, sidx);
